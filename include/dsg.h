@@ -239,9 +239,10 @@ void dsg_peel_free(dsg_peel_state* st);
 dsg_status dsg_kcore(const dsg_graph* g, uint32_t* out_core);
 
 /* As dsg_kcore, also writing up to nstats counters of the run into stats:
- *   [0] levels run (the blocks meet once per level, on its work counter)
+ *   [0] levels (core numbers that occur)
  *   [1] row pieces queued to the level-wide work queue
- *   [2] remaining-list entries scanned (sum over levels)
+ *   [2] remaining vertices scanned (sum over levels; for the vertices that
+ *       dsg_set_kcore_tail leaves to the search, what its levels would scan)
  *   [3] remaining-list entries written (sum over levels)
  *   [4] degree atomics issued (decrements plus undos) */
 dsg_status dsg_kcore_stats(const dsg_graph* g, uint32_t* out_core, uint64_t* stats, uint32_t nstats);
@@ -413,12 +414,13 @@ dsg_status dsg_set_local_max(uint32_t local_max, uint32_t local_work);
  * level-wide queue in pieces of at most chunk_len entries, which every block
  * takes from.  Default 256; DSG_INLINE_MAX.  Results never depend on it. */
 dsg_status dsg_set_inline_max(uint32_t inline_max);
-/* Core numbers: once at most max_vertices vertices remain after a level, the
- * remaining graph is compacted (rows cut to the remaining neighbours, which
- * leaves every remaining degree as it is) and one thread-block cluster runs
- * the remaining levels with the degrees in its distributed shared memory.
- * 0 turns it off; at most 131072 (16 blocks of 8192 vertices).  Default
- * 65536; DSG_KCORE_TAIL.  Results never depend on it. */
+/* Core numbers: once at most max_vertices vertices remain after a level (or
+ * from the start, on a graph of no more vertices), their core numbers are
+ * searched bit by bit, all levels at once, instead of level by level; after a
+ * level the remaining graph is compacted first (rows cut to the remaining
+ * neighbours, which leaves every remaining degree as it is).  0 turns it off;
+ * at most 131072.  Default 65536; DSG_KCORE_TAIL.  Results never depend on
+ * it. */
 dsg_status dsg_set_kcore_tail(uint32_t max_vertices);
 /* Peel (Algorithm 1) in a thin tail: once a round removes less than 1/8 of
  * the vertices left, the next round also collects candidates -- every alive

@@ -102,7 +102,6 @@ struct dsg_graph {
     cudaStream_t stream = nullptr;
     uint32_t max_blocks = 0; // cap on the grid of persistent kernels for this handle (0: whole GPU)
     uint32_t force_block = 0; // block size of those kernels regardless of tuning (0: tuned)
-    bool no_tail = false;     // core numbers: keep every level in the grid-wide kernel
 };
 
 // -------------------------------------------------------------- device side
@@ -219,6 +218,10 @@ __device__ __forceinline__ uint32_t atom_add_release_u32(uint32_t* p, uint32_t v
     uint32_t old;
     asm volatile("atom.add.release.gpu.global.u32 %0, [%1], %2;" : "=r"(old) : "l"(p), "r"(v) : "memory");
     return old;
+}
+
+__device__ __forceinline__ void red_add_release_u64(unsigned long long* p, uint64_t v) {
+    asm volatile("red.release.gpu.global.add.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
 }
 
 __device__ __forceinline__ uint64_t ld_volatile_u64(const uint64_t* p) {

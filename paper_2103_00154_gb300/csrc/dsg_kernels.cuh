@@ -82,15 +82,20 @@ dsg_status peel_into(const dsg_graph* g, uint32_t p, uint32_t q, uint8_t* set_de
 dsg_status run_kcore(const dsg_graph* g, uint32_t* core_out, uint64_t* stats, uint32_t nstats,
                      uint64_t* trace_dev = nullptr, uint64_t trace_cap = 0, uint64_t* stamps = nullptr);
 
-// The last levels of the core numbers on the compacted remaining graph (the
-// vertices whose claim bit is clear; deg holds their degrees), by one
-// thread-block cluster; writes their core numbers into deg and adds its
-// levels, scanned remaining entries and atomics into stats5[0], [2], [4];
-// with a trace buffer, block 0 stamps each level's phases there.
-constexpr uint32_t kTailMaxVertices = 16 * 8192;
-dsg_status kcore_tail(uint32_t n, const uint64_t* off, const uint32_t* adj, uint32_t* deg, const uint32_t* claim,
-                      uint32_t cap, cudaStream_t s, uint64_t* stats5, uint64_t* trace = nullptr,
-                      uint64_t trace_cap = 0, uint64_t* stamps = nullptr);
+// The core numbers of the vertices whose claim bit is clear (at most cap of
+// them, none with a core number below lo; deg holds their degrees), on the
+// compacted remaining graph; writes them into deg and adds what a level run
+// would count (levels, remaining entries) and the atomics into stats5[0],
+// [2], [4]; with a trace buffer, block 0 stamps each wave there.
+constexpr uint32_t kTailMaxVertices = 131072;
+dsg_status kcore_tail(const dsg_graph* g, uint32_t* deg, const uint32_t* claim, uint32_t cap, uint32_t lo,
+                      uint64_t* stats5, uint64_t* trace = nullptr, uint64_t trace_cap = 0, uint64_t* stamps = nullptr);
+
+// The same on a whole graph of r <= kTailMaxVertices vertices (rows off, adj;
+// rid nullable: original ids); limits of the grid from g.
+dsg_status core_split(uint32_t r, uint32_t lo, const uint64_t* off, const uint32_t* adj, uint64_t entries,
+                      const uint32_t* rid, uint32_t* core, const dsg_graph* g, Scratch& sc, uint64_t* stats5,
+                      uint64_t* trace, uint64_t trace_cap, uint64_t* stamps);
 
 // Device check that a graph is canonical (sorted rows, no loops, no repeats,
 // symmetric, ids < n).  DSG_EINVAL with a message if not.

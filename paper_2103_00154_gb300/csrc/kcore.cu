@@ -87,7 +87,8 @@ struct __align__(128) CoreCtl {
     unsigned long long levels;
     unsigned long long dbg[4];   // bounds-check builds: first bad access (site, index, capacity, level)
     unsigned long long stamps;
-    unsigned long long tail;     // the level loop stopped with this many vertices left for the cluster tail
+    unsigned long long tail;     // the level loop stopped with this many vertices left ...
+    unsigned long long tail_lo;  // ... none of degree below this
 };
 
 // Bounds checks of the debug build (DSG_DEBUG_BOUNDS): a bad index is
@@ -612,9 +613,12 @@ __global__ void __launch_bounds__(TB, TB == 256 ? 3 : 1) kcore_kernel(CoreArgs a
         ++level;
         if (visited >= n) break;
         if (a.tail_max && (uint64_t)n - visited <= a.tail_max) {
-            // few vertices remain: the cluster finishes them on the compacted graph
+            // few vertices remain: they are finished on the compacted graph
             // (every block sees the same totals, so all leave here together)
-            if (blockIdx.x == 0 && tid == 0) ctl->tail = (uint64_t)n - visited;
+            if (blockIdx.x == 0 && tid == 0) {
+                ctl->tail = (uint64_t)n - visited;
+                ctl->tail_lo = level_min == 0xffffffffu ? k + 1 : level_min;
+            }
             break;
         }
         if (level_min == 0xffffffffu || level_min <= k) {
@@ -662,9 +666,25 @@ dsg_status run_kcore(const dsg_graph* g, uint32_t* core_out, uint64_t* stats, ui
     a.local_max = tu.local_max;
     a.local_work = tu.local_work;
     a.inline_max = tu.inline_max;
-    a.tail_max = g->no_tail ? 0 : (tu.tail_max < kTailMaxVertices ? tu.tail_max : kTailMaxVertices);
+    a.tail_max = tu.tail_max < kTailMaxVertices ? tu.tail_max : kTailMaxVertices;
     a.trace = trace_dev;
     a.trace_cap = trace_cap;
+    const bool direct = is_device_ptr(core_out);
+    if (n <= a.tail_max) {
+        // few enough from the start: no level is run
+        uint64_t vals[5] = {0, 0, 0, 0, 0};
+        uint32_t* core = core_out;
+        if (!direct) DSG_TRY_CUDA(sc.get(&core, n));
+        dsg_status st = core_split(n, 0, g->off, g->adj, 2 * g->m, nullptr, core, g, sc, stats ? vals : nullptr,
+                                   trace_dev, trace_cap, stamps);
+        if (st != DSG_OK) return st;
+        if (!direct) {
+            DSG_TRY_CUDA(copy_any(core_out, core, (size_t)n * 4, s));
+            DSG_TRY_CUDA(cudaStreamSynchronize(s));
+        }
+        for (uint32_t i = 0; stats && i < nstats && i < 5; ++i) stats[i] = vals[i];
+        return DSG_OK;
+    }
     uint32_t grid = 1;
     cudaError_t e;
     switch (tu.block) {
@@ -679,7 +699,6 @@ dsg_status run_kcore(const dsg_graph* g, uint32_t* core_out, uint64_t* stats, ui
     // a level queues at most one piece per chunk_len entries of each row plus
     // one per vertex; blocks may take slots past that and skip them
     a.cap = (uint64_t)n + (2 * g->m) / tu.chunk_len + 1;
-    bool direct = is_device_ptr(core_out);
     if (direct) a.deg = core_out;
     else DSG_TRY_CUDA(sc.get(&a.deg, n));
     DSG_TRY_CUDA(sc.get(&a.claim, ((uint64_t)n + 31) / 32));
@@ -727,7 +746,7 @@ dsg_status run_kcore(const dsg_graph* g, uint32_t* core_out, uint64_t* stats, ui
         // a traced run's tail stamps follow the grid kernel's
         const uint64_t used = trace_dev ? std::min<uint64_t>(2 * c.stamps, trace_cap) : 0;
         uint64_t tail_stamps = 0;
-        st = kcore_tail(n, g->off, g->adj, a.deg, a.claim, (uint32_t)c.tail, s, vals,
+        st = kcore_tail(g, a.deg, a.claim, (uint32_t)c.tail, (uint32_t)c.tail_lo, stats ? vals : nullptr,
                         trace_dev ? trace_dev + used : nullptr, trace_dev ? trace_cap - used : 0, &tail_stamps);
         if (st != DSG_OK) return st;
         if (stamps) *stamps += tail_stamps;

@@ -1,429 +1,420 @@
-// The last levels of Algorithm 2's first phase (core numbers) on a small
-// remaining graph, by one thread-block cluster.
+// The last levels of Algorithm 2's first phase (core numbers), all at once: a
+// bitwise search for every remaining vertex's core number.
 //
 // Once few vertices remain, a level of the grid-wide kernel costs mostly the
-// latency of its cascade (a vertex brought to k by a drain is drained in the
-// same level, and so on, several links deep), and each link there is a few
-// global-memory round trips plus block barriers.  Here the remaining graph is
-// first compacted -- its vertices renumbered 0..r-1 and each row cut down to
-// the neighbours that remain, which changes no degree: a remaining vertex's
-// degree already counts exactly its remaining neighbours, and a drain never
-// lowers the degree of a vertex that is gone -- and then one cluster runs the
-// remaining levels with every vertex's degree, row bounds and queue slot in
-// the distributed shared memory of the cluster: vertex i belongs to block
-// i % C.
+// latency of its cascade: there are hundreds of levels, each with a chain of
+// a few dependent drains, and hardly any work in any of them.  Here the levels
+// are not walked.  A remaining vertex's core number is lo + c, and c is found
+// from its top bit down: for bit b, every group of vertices that agree on the
+// bits above b is peeled at once to its (lo + c + 2^b)-core -- the vertices
+// that stay have the bit set, those that leave do not -- so a remaining graph
+// whose core numbers span K values takes log2 K peels instead of up to K
+// levels, and a peel is a few waves, each of them spread over the whole grid
+// (Chung-Lu, 700,001 vertices, 65,536 remaining: 9 peels and 103 waves
+// instead of 97 levels of about 4.5 dependent drains each).
 //
-// Level k:
-//   scan: each block walks its own vertices not yet taken (a list compacted
-//     every level) and takes those of degree <= k into its queue; the scan
-//     takes are added to a cluster-wide pending count, and a cluster barrier
-//     separates the scan from the drain, so no degree changes while any
-//     block scans;
-//   every block copies the cluster's taken bits (the union of the blocks'
-//     own bitmaps) into its shared memory, so a drain skips a neighbour that
-//     is gone with a local look-up;
-//   drain: each block drains its queue in batches, all its threads spread
-//     over the batch's rows; a neighbour that is not gone loses one degree
-//     (a DSMEM atomic at its owner); if that brought it from k + 1 to k the
-//     decrementer is the one thread that does so: it reads the vertex's row
-//     bounds at the owner, asks L2 for the row, and queues the vertex at its
-//     owner (pending count up, a slot at the owner, one store of the owner's
-//     local index); if it was at or below k already (taken during this
-//     level) the decrement is undone, which leaves the degrees Algorithm 2's
-//     read-then-decrement drain leaves.  A block gives a batch's count back
-//     to the pending count once the batch and the takes it made are
-//     registered, so the count reaches zero only when the level's cascade is
-//     over; the owners drain, so a cascade spreads over the cluster;
-//   the blocks meet at a cluster barrier and sum the level's takes and least
-//   degree above k, so every block takes the same decisions.
+// A vertex's degree d counts its neighbours in its own group (not yet removed
+// in this peel) and in every group above it; those have core numbers at least
+// as large as the group's bound whatever this peel does.  So a removed vertex
+// takes one from each neighbour of its own group only, and the one decrement
+// that takes a neighbour from its bound to below it puts it in the next wave:
+// no claim, no undo.  After the peel a vertex that stayed keeps its d (the
+// groups above it are now its own survivors and those above), one that left
+// gets back the d it had before the peel (ds): everyone it counted is still
+// in its group or above.
+//
+// Bit b, for every vertex: key = c << 1 | first, first = d already below the
+// bound.  The peel's first wave removes the `first` vertices either by
+// pushing (their rows take one from each key == c << 1 neighbour) or by
+// pulling (every other vertex counts its key == c << 1 | 1 neighbours),
+// whichever reads fewer row pieces; the later waves push.  Rows are walked
+// as pieces of at most kPiece entries, as many pieces per warp as spread the
+// wave over all warps, the entries of a warp's pieces dealt out to its lanes
+// (a hub's row is many warps' work, 32 short rows one warp's).
+// key is written to a buffer of its own for every bit, so its look-ups may be
+// cached in L1 although the kernel rewrites it while it runs.
+//
+// The blocks meet after every wave; the word they meet on also sums the
+// pieces that the wave queued, so no block reads the queue's end separately.
+// Two words take turns: a block that is already in the next wave must not add
+// to the sum that a slower block is still to read.
 // Every wait is bounded (ERR_TIMEOUT).
-#include <cooperative_groups.h>
+//
+// What bounds it: the wide waves, L2 gathers (a bit's first wave on Chung-Lu
+// 2^24, 65,287 vertices and about 45 M row entries read: 60 us); the thin ones,
+// a chain of about eight dependent L2 round trips (the meeting, piece, row
+// entry, key, decrement, queue slot, piece written and released): 4.5 us.
+// Measured against one 16-block cluster walking the levels with the degrees
+// in its shared memory: Chung-Lu 2^24 (870 levels left) 18.7 -> 3.6 ms,
+// 700,001 vertices (97 levels) 2.04 -> 0.68 ms, R-MAT scale 18 (129 levels)
+// 2.15 -> 0.76 ms, 10^4 vertices (the whole graph) 0.24 -> 0.16 ms with the
+// compaction and its copies saved.
+// Tried and dropped: a warp that goes on with the vertices it has removed
+// instead of queueing them (1, 2 or 4 rows deep: 0.82, 0.84, 0.88 ms against
+// 0.74 at 700,001 vertices -- the wave waits for the longest chain).
+#include <algorithm>
 
 #include "dsg_common.cuh"
 #include "dsg_kernels.cuh"
 
-namespace cg = cooperative_groups;
-
 namespace dsg {
 
-constexpr uint32_t kTailTB = 1024;
-constexpr uint32_t kTailC = 16;                       // blocks in the cluster
-constexpr uint32_t kTailVPC = kTailMaxVertices / kTailC;  // vertices per block at most
-constexpr uint32_t kTailWPB = kTailVPC / 32;          // bitmap words per block
-constexpr uint16_t kSlotEmpty = 0xffffu;
-constexpr uint32_t kOffMax = 0xffffffffu;             // compacted row offsets must stay below this
+constexpr uint32_t kSplitTB = 1024;
+constexpr uint32_t kPiece = 128;  // entries per row piece: one step of a warp, 4 loads per lane in flight
+constexpr uint32_t kSplitBits = 17;  // kTailMaxVertices vertices have core numbers below 2^17
+// A vertex's key: pieces of its row above kKeyBits (a row has fewer than
+// kTailMaxVertices entries, 1,024 pieces), its c, and the `first` bit.
+constexpr uint32_t kKeyBits = kSplitBits + 1;
+constexpr uint32_t kKeyMask = (1u << kKeyBits) - 1u;
+constexpr uint32_t kPiecesMax = (1u << (32 - kKeyBits)) - 1u;
 
-struct TailStats {
-    unsigned long long levels, rem_scanned, atomics, claims, stamps;
+__device__ __forceinline__ uint32_t pieces_of(uint64_t len) {
+    const uint64_t np = (len + kPiece - 1) / kPiece;
+    return np < kPiecesMax ? (uint32_t)np : kPiecesMax;
+}
+
+struct __align__(128) SplitCtl {
+    unsigned long long bar[2][16];  // arrivals (low half) and pieces queued (high half), by parity
+    unsigned long long tail[3][16];  // next queue slot, by bit modulo 3
+    uint32_t above[32];  // vertices with degree >= lo + 2^b at the start
+    unsigned long long npieces;
+    unsigned long long atomics, waves, stamps;
     uint32_t err;
 };
 
-struct TailArgs {
-    uint32_t r;                 // remaining vertices, numbered 0..r-1
-    const uint64_t* off;        // compacted rows, r + 1 (every offset below 2^32 - 1)
-    const uint32_t* adj;        // compacted neighbour numbers
-    const uint32_t* cdeg;       // degree of each remaining vertex when the tail starts
-    const uint32_t* rid;        // original id of each remaining vertex
-    uint32_t* core;             // core numbers by original id (written for the remaining vertices)
-    TailStats* stats;
-    uint64_t limit_ns;          // bound of every wait
-    uint64_t* trace;            // nullable: block 0 stamps (%globaltimer, kind << 32 | k) per level phase
-    uint64_t trace_cap;         // words of trace
+struct SplitArgs {
+    uint32_t r;           // vertices, numbered 0..r-1
+    uint32_t lo;          // no core number is below lo
+    const uint64_t* off;  // rows, r + 1
+    const uint32_t* adj;
+    const uint32_t* rid;  // original ids (nullable: the numbers themselves)
+    uint32_t* d;          // degrees in the running peel
+    uint32_t* ds;         // degrees before it
+    uint32_t* key;        // kSplitBits + 1 buffers of kstride entries
+    uint64_t kstride;
+    uint4* pieces;        // every row's pieces: first entry (low word), vertex, entries | first entry >> 32 << 16
+    uint4* queue;         // the waves' pieces, the vertex's c in the last word
+    uint64_t cap;         // slots of each
+    uint32_t* core;       // core numbers by original id
+    SplitCtl* ctl;
+    uint64_t limit_ns;
+    uint64_t* trace;      // nullable: block 0 stamps (%globaltimer, kind << 32 | bit) per phase
+    uint64_t trace_cap;
 };
 
-struct TailSmem {
-    uint32_t deg[kTailVPC];            // this block's vertices' degrees (other blocks decrement them)
-    uint32_t rbeg[kTailVPC];           // ... their row starts and lengths in the compacted adjacency
-    uint32_t rlen[kTailVPC];
-    uint32_t taken[kTailWPB];          // this block's vertices taken into a level (written by this block)
-    uint32_t gone[kTailC * kTailWPB];  // copy of every block's taken bits, block b's at [b * kTailWPB]
-    uint16_t rem[2][kTailVPC];         // this block's vertices still to scan, by level parity
-    uint16_t q[kTailVPC];              // this level's queue of own vertices (local index); kSlotEmpty until
-                                       // the taker has written it
-    uint32_t start[kTailTB];           // a batch's rows: exclusive prefix of lengths ...
-    uint32_t beg[kTailTB];             // ... row starts
-    uint32_t red[33];
-    uint64_t red64[33];
-    uint32_t qtail, nkeep, batch_n, batch_total, stop;
-    uint32_t pending;                  // block 0's copy: taken vertices of the level not yet drained
-    uint32_t pub_min[2], pub_claims[2], pub_err[2];  // a level's totals of this block, by level parity
-    uint32_t tot_min, tot_err;
-    unsigned long long tot_claims;
+struct SplitSmem {
+    uint32_t pushed;                  // pieces queued by this block in the running phase
+    uint32_t got;                     // pieces queued by the whole grid
+    uint32_t ok;
+    uint32_t above[32];
+    uint32_t cnt[kSplitTB / 32][32];  // pull: a warp's counts, per piece
 };
 
-// Ask L2 to fetch adj[b, b + l) (rounded out to 16-byte boundaries; the
-// adjacency allocation is padded to 256 bytes, so the rounding stays inside it).
-__device__ __forceinline__ void prefetch_row(const uint32_t* adj, uint32_t b, uint32_t l) {
-    if (l == 0) return;
-    const uint64_t lo = (uint64_t)b & ~3ull, hi = ((uint64_t)b + l + 3) & ~3ull;
-    asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(__cvta_generic_to_global(adj + lo)),
-                 "r"((uint32_t)((hi - lo) * 4))
-                 : "memory");
+// Write the pieces of the rows u[j] (bit j of hit; np[j] pieces each, c[j] to
+// go with them) to list, at slots reserved at *tail: one atomic per warp, its
+// round trip running beside the loads of the row bounds.  All lanes call it.
+template <int K>
+__device__ __forceinline__ void put_rows(const SplitArgs& a, uint4* list, unsigned long long* tail, uint32_t* pushed,
+                                         uint32_t hit, const uint32_t (&u)[K], const uint32_t (&c)[K],
+                                         const uint32_t (&np)[K]) {
+    const uint32_t lane = lane_id();
+    uint32_t mine = 0;
+#pragma unroll
+    for (int j = 0; j < K; ++j) mine += hit >> j & 1u ? np[j] : 0u;
+    const uint32_t inc = warp_incl_scan(mine);
+    const uint32_t total = __shfl_sync(kFullMask, inc, 31);
+    unsigned long long base = 0;
+    if (lane == 0 && total) {
+        base = atomicAdd(tail, (unsigned long long)total);
+        atomicAdd(pushed, total);
+    }
+    uint64_t beg[K], end[K];
+#pragma unroll
+    for (int j = 0; j < K; ++j) {
+        beg[j] = hit >> j & 1u ? a.off[u[j]] : 0;
+        end[j] = hit >> j & 1u ? a.off[u[j] + 1] : 0;
+    }
+    base = __shfl_sync(kFullMask, base, 0) + inc - mine;
+    auto put = [&](unsigned long long at, uint64_t b, uint64_t e, uint32_t v, uint32_t vc, uint32_t k) {
+        b += (uint64_t)k * kPiece;
+        if (at + k < a.cap && b < e)
+            list[at + k] = make_uint4((uint32_t)b, v, (uint32_t)min((uint64_t)kPiece, e - b) | (uint32_t)(b >> 32) << 16,
+                                      vc);
+    };
+#pragma unroll
+    for (int j = 0; j < K; ++j) {
+        const uint32_t n_ = hit >> j & 1u ? np[j] : 0u;
+        if (n_ <= 4)
+            for (uint32_t k = 0; k < n_; ++k) put(base, beg[j], end[j], u[j], c[j], k);
+        // a long row's pieces are written by the whole warp
+        for (uint32_t pend = __ballot_sync(kFullMask, n_ > 4); pend; pend &= pend - 1) {
+            const uint32_t o = __ffs(pend) - 1;
+            const unsigned long long ob = __shfl_sync(kFullMask, base, o);
+            const uint64_t bb = __shfl_sync(kFullMask, beg[j], o), be = __shfl_sync(kFullMask, end[j], o);
+            const uint32_t ov = __shfl_sync(kFullMask, u[j], o), oc = __shfl_sync(kFullMask, c[j], o);
+            const uint32_t on = __shfl_sync(kFullMask, n_, o);
+            for (uint32_t k = lane; k < on; k += 32) put(ob, bb, be, ov, oc, k);
+        }
+        base += n_;
+    }
 }
 
-__global__ void __launch_bounds__(kTailTB, 1) kcore_tail_kernel(TailArgs a) {
-    extern __shared__ __align__(16) unsigned char tail_smem_raw[];
-    TailSmem& sm = *reinterpret_cast<TailSmem*>(tail_smem_raw);
-    cg::cluster_group cluster = cg::this_cluster();
-    const uint32_t C = cluster.num_blocks();
-    const uint32_t rank = cluster.block_rank();
+// All blocks meet (epoch counts the meetings); returns the pieces queued by
+// the grid since the last one.  sm.ok is false once a wait ran out.
+__device__ __forceinline__ uint32_t split_meet(const SplitArgs& a, SplitSmem& sm, uint32_t& epoch, uint32_t seen[2]) {
+    __syncthreads();
+    const uint32_t par = epoch & 1u;
+    ++epoch;
+    if (threadIdx.x == 0) {
+        const uint32_t mine = sm.pushed;
+        sm.pushed = 0;
+        if (gridDim.x == 1) {
+            sm.got = mine;
+        } else {
+            unsigned long long* word = &a.ctl->bar[par][0];
+            const uint32_t target = ((epoch + 1) >> 1) * gridDim.x;  // odd and even meetings have a word each
+            red_add_release_u64(word, (uint64_t)mine << 32 | 1ull);
+            uint64_t w;
+            uint32_t polls = 0;
+            const uint64_t t0 = global_ns();
+            while ((int32_t)((uint32_t)(w = ld_acquire_u64(word)) - target) < 0) {
+                if ((++polls & 63u) == 0) {
+                    if (global_ns() - t0 > a.limit_ns) atomicOr(&a.ctl->err, ERR_TIMEOUT);
+                    if (ld_volatile_u32(&a.ctl->err) & ERR_TIMEOUT) {
+                        sm.ok = 0;
+                        break;
+                    }
+                }
+            }
+            sm.got = (uint32_t)(w >> 32) - seen[par];
+        }
+    }
+    __syncthreads();
+    const uint32_t got = sm.got;
+    seen[par] += got;
+    return got;
+}
+
+__global__ void __launch_bounds__(kSplitTB, 1) core_split_kernel(SplitArgs a) {
+    __shared__ SplitSmem sm;
+    SplitCtl* const ctl = a.ctl;
     const uint32_t tid = threadIdx.x, lane = tid & 31u;
-    const uint32_t r = a.r;
-    const uint32_t V = r > rank ? (r - rank + C - 1) / C : 0;  // this block's vertices: i = li * C + rank
-    const uint32_t wmax = ((r + C - 1) / C + 31) / 32;         // taken words in use per block
-    // ---- degrees, row bounds, the list of this block's vertices; least degree
-    uint32_t mn = 0xffffffffu;
-    for (uint32_t li = tid; li < V; li += kTailTB) {
-        const uint32_t i = li * C + rank;
-        const uint32_t d = a.cdeg[i];
-        const uint64_t b0 = a.off[i], b1 = a.off[i + 1];
-        sm.deg[li] = d;
-        sm.rbeg[li] = (uint32_t)b0;
-        sm.rlen[li] = (uint32_t)(b1 - b0);
-        sm.rem[0][li] = (uint16_t)li;
-        mn = min(mn, d);
-    }
-    for (uint32_t w = tid; w < kTailWPB; w += kTailTB) sm.taken[w] = 0;
-    for (uint32_t i = tid; i < kTailVPC; i += kTailTB) sm.q[i] = kSlotEmpty;
-    mn = block_min_u32(mn, sm.red);
-    if (tid == 0) {
-        sm.pub_min[1] = mn;
-        sm.qtail = 0;
-        sm.pending = 0;
-    }
-    cluster.sync();
-    uint32_t k = 0xffffffffu;
-    for (uint32_t b = 0; b < C; ++b) k = min(k, *cluster.map_shared_rank(&sm.pub_min[1], (int)b));
-    uint32_t* const pending0 = cluster.map_shared_rank(&sm.pending, 0);
-    uint64_t visited = 0, level = 0, scanned = 0, natom = 0, nstamp = 0;
-    uint32_t nrem = V;
-    bool bad = false, timeout = false;
-    // trace pairs: kind 11 scan done, 12 drain done, 13 level over (block 0), 14 the level's claims;
-    // block 0's batches: 15 batch taken (time), 16 its vertices << 32 | its entries, 17 batch drained (time)
-    auto stamp = [&](uint32_t kind, uint64_t val) {
-        if (a.trace && rank == 0 && tid == 0 && 2 * nstamp + 1 < a.trace_cap) {
+    const uint32_t r = a.r, lo = a.lo;
+    const uint32_t gw = (blockIdx.x * kSplitTB + tid) >> 5, nw = gridDim.x * (kSplitTB / 32);
+    const uint32_t nth = gridDim.x * kSplitTB;
+    const uint32_t rpad = (r + 31u) & ~31u;  // whole warps in the per-vertex loops
+    uint32_t epoch = 0, seen[2] = {0, 0};
+    uint64_t natom = 0, nwaves = 0, nstamp = 0;
+    // trace pairs: kind 11 keys written, 12 first wave over, 13 a later wave over, 14 its pieces (value)
+    auto stamp = [&](uint32_t kind, uint32_t b, uint64_t val) {
+        if (!a.trace) return;
+        if (blockIdx.x == 0 && tid == 0 && 2 * nstamp + 1 < a.trace_cap) {
             a.trace[2 * nstamp] = val;
-            a.trace[2 * nstamp + 1] = ((uint64_t)kind << 32) | k;
+            a.trace[2 * nstamp + 1] = (uint64_t)kind << 32 | b;
         }
         ++nstamp;
     };
-    while (visited < r) {
-        const uint32_t par = (uint32_t)(level & 1);
-        const uint16_t* cur = sm.rem[par];
-        uint16_t* nxt = sm.rem[par ^ 1u];
-        uint32_t lmin = 0xffffffffu;
-        if (tid == 0) sm.nkeep = 0;
-        __syncthreads();
-        // ---- scan: take degree <= k (queued here), keep degree > k; nothing changes a degree meanwhile
-        uint32_t lclaims = 0;
-        for (uint32_t j0 = 0; j0 < nrem; j0 += kTailTB) {
-            const uint32_t j = j0 + tid;
-            bool keep = false;
-            uint32_t li = 0;
-            if (j < nrem) {
-                li = cur[j];
-                const uint32_t bit = 1u << (li & 31u);
-                if (!(sm.taken[li >> 5] & bit)) {
-                    const uint32_t d = sm.deg[li];
-                    if (d > k) {
-                        keep = true;
-                        lmin = min(lmin, d);
-                    } else {
-                        atomicOr(&sm.taken[li >> 5], bit);
-                        prefetch_row(a.adj, sm.rbeg[li], sm.rlen[li]);
-                        sm.q[atomicAdd(&sm.qtail, 1u)] = (uint16_t)li;
-                        ++lclaims;
-                    }
-                }
-            }
-            const uint32_t bal = __ballot_sync(kFullMask, keep);
-            uint32_t base = 0;
-            if (lane == 0 && bal) base = atomicAdd(&sm.nkeep, (uint32_t)__popc(bal));
-            base = __shfl_sync(kFullMask, base, 0);
-            if (keep) nxt[base + __popc(bal & lanemask_lt())] = (uint16_t)li;
+    if (tid < 32) sm.above[tid] = 0;
+    if (tid == 0) {
+        sm.pushed = 0;
+        sm.ok = 1;
+    }
+    for (uint32_t i = tid; i < kSplitTB; i += kSplitTB) sm.cnt[i >> 5][i & 31u] = 0;
+    __syncthreads();
+    // ---- every row's pieces, and how many vertices reach lo + 2^b: in a simple graph a
+    // (lo + 2^b)-core needs more vertices than that of at least that degree, which bounds the bits
+    for (uint32_t i = blockIdx.x * kSplitTB + tid; i < rpad; i += nth) {
+        uint32_t d = 0, top = 0;
+        const uint32_t v1[1] = {i}, c1[1] = {0u};
+        if (i < r) {
+            d = (uint32_t)(a.off[i + 1] - a.off[i]);
+            a.d[i] = d;
+            a.ds[i] = d;
+            top = d > lo ? 32u - (uint32_t)__clz(d - lo) : 0u;  // d >= lo + 2^b for b < top
         }
-        if (tid == 0) scanned += nrem;
-        {
-            const uint32_t c = (uint32_t)block_sum<uint64_t>((uint64_t)lclaims, sm.red64);
-            if (tid == 0 && c) atomicAdd(pending0, c);
+#pragma unroll 1
+        for (uint32_t b = 0; b < kSplitBits; ++b) {
+            const uint32_t m = __ballot_sync(kFullMask, top > b);
+            if (m == 0) break;
+            if (lane == 0) atomicAdd(&sm.above[b], (uint32_t)__popc(m));
         }
-        cluster.sync();  // every scan take is counted and every taken bit of the scan is set
-        // ---- the cluster's taken bits, for the drain's look-ups
-        for (uint32_t w = tid; w < C * wmax; w += kTailTB) {
-            const uint32_t b = w / wmax, ww = w - b * wmax;
-            sm.gone[b * kTailWPB + ww] =
-                *reinterpret_cast<volatile uint32_t*>(cluster.map_shared_rank(&sm.taken[ww], (int)b));
-        }
-        __syncthreads();
-        stamp(11, global_ns());
-        // ---- drain: a neighbour not gone loses one degree at its owner; the one decrement
-        // that takes it from k + 1 to k queues it there; one that finds it at or below k
-        // (taken during this level) is undone
-        auto visit = [&](const uint32_t* u, uint32_t valid) {
-            uint32_t old[kBatch], live = 0;
-            uint32_t* dp[kBatch];
-#pragma unroll
-            for (uint32_t jj = 0; jj < kBatch; ++jj) {
-                dp[jj] = nullptr;
-                old[jj] = 0;
-                if (!(valid >> jj & 1u)) continue;
-                if (u[jj] >= r) {
-                    bad = true;
-                    continue;
-                }
-                const uint32_t ru = u[jj] % C, lu = u[jj] / C;
-                if (sm.gone[ru * kTailWPB + (lu >> 5)] >> (lu & 31u) & 1u) continue;
-                dp[jj] = cluster.map_shared_rank(&sm.deg[lu], (int)ru);
-                old[jj] = atomicSub(dp[jj], 1u);
-                ++natom;
-                live |= 1u << jj;
-            }
-            uint32_t claim = 0;
-#pragma unroll
-            for (uint32_t jj = 0; jj < kBatch; ++jj) {
-                if (!(live >> jj & 1u)) continue;
-                if (old[jj] <= k) {
-                    atomicAdd(dp[jj], 1u);
-                    ++natom;
-                } else if (old[jj] == k + 1) {
-                    claim |= 1u << jj;
+        const uint32_t np1[1] = {pieces_of(d)};
+        put_rows<1>(a, a.pieces, &ctl->npieces, &sm.pushed, d ? 1u : 0u, v1, c1, np1);
+    }
+    __syncthreads();
+    if (tid < 32 && sm.above[tid]) atomicAdd(&ctl->above[tid], sm.above[tid]);
+    const uint32_t npieces = split_meet(a, sm, epoch, seen);
+    if (!sm.ok) return;
+    uint32_t bits = 0;
+    {
+        const uint32_t cnt = ld_relaxed_u32(&ctl->above[lane]);
+        const uint32_t m = __ballot_sync(kFullMask, lane < kSplitBits && cnt > lo + (1u << lane));
+        bits = m ? 32u - (uint32_t)__clz(m) : 0u;
+    }
+    // ---- one wave over list[from, to): push the rows' removal, or pull it
+    // (first: list holds every row's pieces, only those of (push) the first or (pull) the
+    // other vertices count)
+    auto wave = [&](const uint4* list, uint32_t from, uint32_t to, const uint32_t* key, uint32_t bound, bool first,
+                    bool pull, unsigned long long* tail) {
+        const uint32_t n_ = to - from;
+        uint32_t G = (n_ + nw - 1) / nw;
+        if (G > 32) G = 32;
+        uint32_t* const cnt = sm.cnt[tid >> 5];
+        // lane l takes piece g0 + l nw + gw: neighbouring pieces (a hub's) go to different warps
+        for (uint64_t g0 = 0; g0 < n_; g0 += (uint64_t)nw * G) {
+            uint32_t len = 0, kv = 0, kc = 0, v = 0;
+            uint64_t b0 = 0;
+            const uint64_t at = g0 + (uint64_t)lane * nw + gw;
+            if (lane < G && at < n_) {
+                const uint4 it = __ldcg(list + from + at);
+                v = it.y;
+                len = it.z & 0xffffu;
+                b0 = (uint64_t)(it.z >> 16) << 32 | it.x;
+                if (first) {
+                    kv = __ldca(key + v);
+                    // push: neighbours of v's group that are not removed yet; pull: those removed first
+                    kc = pull ? (kv | 1u) & kKeyMask : kv & (kKeyMask - 1u);
+                    if ((kv & 1u) == (pull ? 1u : 0u)) len = 0;
                 } else {
-                    lmin = min(lmin, old[jj] - 1);
+                    kc = it.w << 1;
                 }
             }
-            // the warp's takes: one pending increment by a leader, a slot at each owner and the
-            // row bounds there, then the row asked into L2 and the slot written (the count never
-            // reads zero while a take is unqueued)
-            const uint32_t wsum = warp_sum((uint32_t)__popc(claim));
-            if (wsum == 0) return;
-            uint32_t was = 0;
-            if (lane == 0) was = atomicAdd(pending0, wsum);
-            uint32_t slot[kBatch], rb[kBatch], rl[kBatch];
-#pragma unroll
-            for (uint32_t jj = 0; jj < kBatch; ++jj) {
-                if (!(claim >> jj & 1u)) continue;
-                const uint32_t ru = u[jj] % C, lu = u[jj] / C;
-                slot[jj] = atomicAdd(cluster.map_shared_rank(&sm.qtail, (int)ru), 1u);
-                rb[jj] = *cluster.map_shared_rank(&sm.rbeg[lu], (int)ru);
-                rl[jj] = *cluster.map_shared_rank(&sm.rlen[lu], (int)ru);
-            }
-#pragma unroll
-            for (uint32_t jj = 0; jj < kBatch; ++jj)
-                if (claim >> jj & 1u) prefetch_row(a.adj, rb[jj], rl[jj]);
-            was = __shfl_sync(kFullMask, was, 0);
-            if (was == 0xffffffffu) bad = true;
-#pragma unroll
-            for (uint32_t jj = 0; jj < kBatch; ++jj) {
-                if (!(claim >> jj & 1u)) continue;
-                if (slot[jj] >= kTailVPC) {
-                    bad = true;
-                    continue;
-                }
-                volatile uint16_t* sp = cluster.map_shared_rank(&sm.q[slot[jj]], (int)(u[jj] % C));
-                *sp = (uint16_t)(u[jj] / C);
-            }
-        };
-        // ---- drain this block's queue until the cluster has nothing pending
-        uint32_t qhead = 0;
-        uint64_t wait_start = global_ns();
-        for (;;) {
-            if (tid == 0) {
-                // wait here, alone, for queued work or the level's end: the queue tail is local and
-                // polled tightly, the cluster's pending count every few polls
-                uint32_t take = 0, stop = 0;
-                for (uint32_t spins = 0;; ++spins) {
-                    const uint32_t t = *reinterpret_cast<volatile uint32_t*>(&sm.qtail);
-                    if (t != qhead) {
-                        take = min(t - qhead, kTailTB);
-                        break;
-                    }
-                    if ((spins & 7u) == 7u) {
-                        if (*reinterpret_cast<volatile uint32_t*>(pending0) == 0) {
-                            // nothing queued here (re-read: a take may have landed meanwhile)
-                            if (*reinterpret_cast<volatile uint32_t*>(&sm.qtail) == qhead) {
-                                stop = 1;
-                                break;
-                            }
-                            continue;
-                        }
-                        if (global_ns() - wait_start > a.limit_ns) {
-                            stop = 1;
-                            timeout = true;
-                            break;
-                        }
-                    }
-                }
-                sm.stop = stop;
-                sm.batch_n = take;
-            }
-            __syncthreads();
-            const uint32_t nb = sm.batch_n;
-            if (sm.stop) break;
-            // the batch's vertices: slots qhead .. qhead + nb, each written by its taker right
-            // after it reserved the slot: wait for it, bounded
-            uint32_t len = 0, bg = 0;
-            if (tid < nb) {
-                volatile uint16_t* sl = &sm.q[qhead + tid];
-                uint16_t x = *sl;
-                const uint64_t s0 = global_ns();
-                while (x == kSlotEmpty) {
-                    if (global_ns() - s0 > a.limit_ns) { timeout = true; break; }
-                    x = *sl;
-                }
-                if (x != kSlotEmpty && x < V) {
-                    atomicOr(&sm.taken[x >> 5], 1u << (x & 31u));
-                    bg = sm.rbeg[x];
-                    len = sm.rlen[x];
-                } else if (x != kSlotEmpty) {
-                    bad = true;
-                }
-            }
-            uint32_t total;
-            if (nb == 1) {
-                // one row (the common case in the last levels): no scan
-                if (tid == 0) {
-                    sm.start[0] = 0;
-                    sm.beg[0] = bg;
-                    sm.batch_total = len;
-                }
-                __syncthreads();
-                total = sm.batch_total;
-            } else {
-                const uint32_t st = block_excl_scan<uint32_t>(len, sm.red, &total);
-                sm.start[tid] = st;
-                sm.beg[tid] = bg;
-                __syncthreads();
-            }
-            if (a.trace) {
-                stamp(15, global_ns());
-                stamp(16, ((uint64_t)nb << 32) | total);
-            }
-            for (uint32_t w0 = tid & ~31u; w0 < total; w0 += kBatch * kTailTB) {
-                uint32_t bu[kBatch], valid = 0;
+            const uint32_t inc = warp_incl_scan(len);
+            const uint32_t total = __shfl_sync(kFullMask, inc, 31);
+            const uint32_t st = inc - len;
+            b0 -= st;  // entry e of the warp's pieces is adj[b0 + e] for its owner's b0
+            for (uint32_t e0 = lane; e0 < ((total + 31u) & ~31u); e0 += 32 * kBatch) {
+                uint32_t u[kBatch], kk[kBatch], ow[kBatch], ku[kBatch], old[kBatch];
 #pragma unroll
                 for (uint32_t j = 0; j < kBatch; ++j) {
-                    const uint32_t e = w0 + lane + j * kTailTB;
-                    bu[j] = 0;
-                    if (e < total) {
-                        uint32_t lo = 0, hi = nb;  // row = last whose start is <= e
-                        while (hi - lo > 1) {
-                            const uint32_t mid = (lo + hi) >> 1;
-                            if (sm.start[mid] <= e) lo = mid; else hi = mid;
+                    const uint32_t e = e0 + 32 * j;
+                    uint32_t o = 0;
+                    if (G > 1) {
+#pragma unroll
+                        for (uint32_t step = 16; step > 0; step >>= 1) {
+                            const uint32_t s = __shfl_sync(kFullMask, st, o + step);
+                            if (o + step < 32 && s <= e) o += step;
                         }
-                        bu[j] = a.adj[sm.beg[lo] + (e - sm.start[lo])];
-                        valid |= 1u << j;
                     }
+                    const uint64_t ob = __shfl_sync(kFullMask, b0, o);
+                    kk[j] = __shfl_sync(kFullMask, kc, o);
+                    ow[j] = o;
+                    u[j] = e < total ? __ldg(a.adj + ob + e) : 0xffffffffu;
                 }
-                visit(bu, valid);
+#pragma unroll
+                for (uint32_t j = 0; j < kBatch; ++j) ku[j] = u[j] < r ? __ldca(key + u[j]) : ~kk[j];
+                if (pull) {
+#pragma unroll
+                    for (uint32_t j = 0; j < kBatch; ++j)
+                        if ((ku[j] & kKeyMask) == kk[j]) atomicAdd(&cnt[ow[j]], 1u);
+                } else {
+                    uint32_t hit = 0;
+#pragma unroll
+                    for (uint32_t j = 0; j < kBatch; ++j) {
+                        old[j] = 0;
+                        if ((ku[j] & kKeyMask) == kk[j]) {
+                            old[j] = atomicSub(&a.d[u[j]], 1u);
+                            ++natom;
+                        }
+                    }
+#pragma unroll
+                    for (uint32_t j = 0; j < kBatch; ++j) {
+                        if ((ku[j] & kKeyMask) == kk[j] && old[j] == bound + (kk[j] >> 1)) hit |= 1u << j;
+                        ku[j] >>= kKeyBits;  // its pieces
+                        kk[j] >>= 1;         // its c
+                    }
+                    if (__any_sync(kFullMask, hit != 0))
+                        put_rows<kBatch>(a, a.queue, tail, &sm.pushed, hit, u, kk, ku);
+                }
             }
-            __syncthreads();  // every drain of the batch is done and its takes are counted
-            if (a.trace) stamp(17, global_ns());
-            if (tid == 0) atomicSub(pending0, nb);
-            qhead += nb;
-            wait_start = global_ns();
-        }
-        stamp(12, global_ns());
-        // ---- the level's totals over the cluster; queue slots back to empty for the next level
-        for (uint32_t i = tid; i < qhead; i += kTailTB) sm.q[i] = kSlotEmpty;
-        lmin = block_min_u32(lmin, sm.red);
-        const uint32_t to = __syncthreads_or(timeout || bad);
-        if (tid == 0) {
-            // (level parity: a block writes these again two levels on, after every block passed the
-            // next level's barriers and so has read them)
-            sm.pub_min[par] = lmin;
-            sm.pub_claims[par] = qhead;  // every vertex this block took at this level went through its queue
-            sm.pub_err[par] = to;
-            sm.qtail = 0;
-        }
-        nrem = sm.nkeep;
-        cluster.sync();  // every block's drains of this level are done and its totals published
-        if (tid < 32) {  // one warp gathers the cluster's totals
-            uint32_t m_ = 0xffffffffu, e_ = 0, c_ = 0;
-            if (tid < C) {
-                m_ = *cluster.map_shared_rank(&sm.pub_min[par], (int)tid);
-                c_ = *cluster.map_shared_rank(&sm.pub_claims[par], (int)tid);
-                e_ = *cluster.map_shared_rank(&sm.pub_err[par], (int)tid);
-            }
-            m_ = warp_min(m_);
-            const uint64_t cs_ = warp_sum<uint64_t>((uint64_t)c_);
-            e_ = __reduce_or_sync(kFullMask, e_);
-            if (tid == 0) {
-                sm.tot_min = m_;
-                sm.tot_claims = cs_;
-                sm.tot_err = e_;
+            if (pull) {
+                __syncwarp();
+                const uint32_t take = cnt[lane];
+                cnt[lane] = 0;
+                const uint32_t v1[1] = {v}, c1[1] = {kc >> 1}, np1[1] = {kv >> kKeyBits};
+                uint32_t hit = 0;
+                if (take) {
+                    const uint32_t old = atomicSub(&a.d[v], take);
+                    ++natom;
+                    const uint32_t mid = bound + c1[0];
+                    hit = old >= mid && old - take < mid ? 1u : 0u;
+                }
+                if (__any_sync(kFullMask, hit != 0)) put_rows<1>(a, a.queue, tail, &sm.pushed, hit, v1, c1, np1);
+                __syncwarp();
             }
         }
-        __syncthreads();
-        const uint32_t kmin = sm.tot_min, err = sm.tot_err;
-        const uint64_t claims = sm.tot_claims;
-        visited += claims;
-        stamp(13, global_ns());
-        stamp(14, claims);
-        ++level;
-        if (visited >= r) break;
-        if (err || kmin == 0xffffffffu || kmin <= k) {  // a wait ran out, or an inconsistent remaining graph
-            bad = bad || !timeout;
-            break;
+    };
+    uint32_t* key = a.key;  // buffer of the running bit
+    bool bad = false;
+    for (uint32_t b = bits; b-- > 0;) {
+        // ---- what the bit above decided, and this bit's keys
+        const uint32_t bound = lo + (1u << b);
+        const bool top = b + 1 == bits;
+        unsigned long long* const tail = &ctl->tail[b % 3][0];
+        if (blockIdx.x == 0 && tid == 0) ctl->tail[(b + 2) % 3][0] = 0;  // the next bit's, last used two bits ago
+        uint32_t nfirst = 0;  // pieces of the first vertices
+        for (uint32_t i = blockIdx.x * kSplitTB + tid; i < r; i += nth) {
+            uint32_t c = 0, d = __ldcg(a.d + i);
+            if (!top) {
+                c = (__ldca(key - a.kstride + i) & kKeyMask) >> 1;
+                if (d >= bound + (1u << b) + c) {
+                    c += 2u << b;
+                    a.ds[i] = d;
+                } else {
+                    d = a.ds[i];
+                    a.d[i] = d;
+                }
+            }
+            const bool first = d < bound + c;
+            const uint32_t np = pieces_of(a.off[i + 1] - a.off[i]);
+            key[i] = np << kKeyBits | c << 1 | (first ? 1u : 0u);
+            if (first) nfirst += np;
         }
-        k = kmin;
+        nfirst = warp_sum(nfirst);
+        if (lane == 0 && nfirst) atomicAdd(&sm.pushed, nfirst);
+        const uint32_t np = split_meet(a, sm, epoch, seen);
+        if (!sm.ok) return;
+        stamp(11, b, global_ns());
+        if (np != 0 && np != npieces) {
+            const bool pull = npieces - np < np;
+            wave(a.pieces, 0, npieces, key, bound, true, pull, tail);
+            ++nwaves;
+            uint32_t from = 0, to = split_meet(a, sm, epoch, seen);
+            if (!sm.ok) return;
+            stamp(12, b, global_ns());
+            stamp(14, b, to);
+            while (from < to && to <= a.cap) {
+                wave(a.queue, from, to, key, bound, false, false, tail);
+                ++nwaves;
+                from = to;
+                to += split_meet(a, sm, epoch, seen);
+                if (!sm.ok) return;
+                stamp(13, b, global_ns());
+                stamp(14, b, to - from);
+            }
+            if (to > a.cap) {  // cannot happen: a row is queued once per bit
+                bad = true;
+                break;
+            }
+        }
+        key += a.kstride;
     }
-    // ---- core numbers of this block's vertices; then no block may leave
-    // while another could still read its shared memory
-    for (uint32_t li = tid; li < V; li += kTailTB) a.core[a.rid[li * C + rank]] = sm.deg[li];
+    // ---- the last bit's decision; core numbers out
+    for (uint32_t i = blockIdx.x * kSplitTB + tid; i < r; i += nth) {
+        uint32_t c = 0;
+        if (bits) {
+            c = (__ldca(key - a.kstride + i) & kKeyMask) >> 1;
+            if (__ldcg(a.d + i) >= lo + 1u + c) c += 1u;
+        }
+        a.core[a.rid ? a.rid[i] : i] = lo + c;
+    }
     natom = warp_sum(natom);
-    scanned = warp_sum(scanned);
-    if (lane == 0) {
-        if (natom) atomicAdd(&a.stats->atomics, (unsigned long long)natom);
-        if (scanned) atomicAdd(&a.stats->rem_scanned, (unsigned long long)scanned);
+    if (lane == 0 && natom) atomicAdd(&ctl->atomics, (unsigned long long)natom);
+    if (blockIdx.x == 0 && tid == 0) {
+        ctl->waves = nwaves;
+        ctl->stamps = nstamp;
+        if (bad) atomicOr(&ctl->err, ERR_CAPACITY);
     }
-    if (bad) atomicOr(&a.stats->err, ERR_RANGE);
-    if (timeout) atomicOr(&a.stats->err, ERR_TIMEOUT);
-    if (rank == 0 && tid == 0) {
-        a.stats->levels = level;
-        a.stats->claims = visited;
-        a.stats->stamps = nstamp;
-    }
-    cluster.sync();
 }
 
 // ---------------------------------------------------------------- compaction
@@ -509,19 +500,108 @@ __global__ void __launch_bounds__(256) tail_fill_kernel(uint32_t r, const uint64
     walk_all_entries(roff, r, pre, put);
 }
 
-// core[rid[i]] = ccore[i]: core numbers of the compacted graph back to original ids.
-__global__ void tail_scatter_kernel(uint32_t r, const uint32_t* __restrict__ rid, const uint32_t* __restrict__ ccore,
-                                    uint32_t* __restrict__ core) {
-    const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < r) core[rid[i]] = ccore[i];
+// What a level-by-level run would count on these vertices: levels[0] = distinct
+// core numbers, levels[1] = sum over them of the vertices at or above.  One
+// block; hist (kmax + 1 bins, zero beforehand) is filled first.
+__global__ void __launch_bounds__(1024) tail_levels_kernel(uint32_t r, const uint32_t* __restrict__ rid,
+                                                           const uint32_t* __restrict__ core, uint32_t bins,
+                                                           uint32_t* hist, unsigned long long* levels) {
+    __shared__ uint64_t tmp[33];
+    for (uint32_t i = threadIdx.x; i < r; i += 1024) {
+        const uint32_t c = core[rid ? rid[i] : i];
+        if (c < bins) atomicAdd(&hist[c], 1u);
+    }
+    __syncthreads();
+    uint64_t above = 0, nl = 0, ns = 0;
+    for (int64_t top = (int64_t)bins - 1; top >= 0; top -= 1024) {
+        const int64_t k = top - (int64_t)threadIdx.x;
+        const uint64_t x = k >= 0 ? __ldcg(hist + k) : 0;
+        uint64_t tot;
+        const uint64_t pre = block_excl_scan<uint64_t>(x, tmp, &tot);
+        if (x) {
+            ++nl;
+            ns += above + pre + x;
+        }
+        above += tot;
+    }
+    nl = block_sum<uint64_t>(nl, tmp);
+    ns = block_sum<uint64_t>(ns, tmp);
+    if (threadIdx.x == 0) {
+        levels[0] = nl;
+        levels[1] = ns;
+    }
+}
+
+// The bitwise search on a graph of r <= kTailMaxVertices vertices (rows off,
+// adj), none with a core number below lo; core numbers to core (by original
+// id through rid, nullable: the vertices' own numbers).
+dsg_status core_split(uint32_t r, uint32_t lo, const uint64_t* off, const uint32_t* adj, uint64_t entries,
+                      const uint32_t* rid, uint32_t* core, const dsg_graph* g, Scratch& sc, uint64_t* stats5,
+                      uint64_t* trace, uint64_t trace_cap, uint64_t* stamps) {
+    cudaStream_t s = g->stream;
+    SplitArgs a;
+    a.r = r;
+    a.lo = lo;
+    a.off = off;
+    a.adj = adj;
+    a.rid = rid;
+    a.core = core;
+    a.limit_ns = wait_limit_ns();
+    a.trace = trace;
+    a.trace_cap = trace ? trace_cap : 0;
+    a.kstride = ((uint64_t)r + 63) & ~uint64_t(63);
+    a.cap = (uint64_t)r + entries / kPiece;
+    DSG_TRY_CUDA(sc.get(&a.d, r));
+    DSG_TRY_CUDA(sc.get(&a.ds, r));
+    DSG_TRY_CUDA(sc.get(&a.key, a.kstride * (kSplitBits + 1)));
+    DSG_TRY_CUDA(sc.get(&a.pieces, a.cap));
+    DSG_TRY_CUDA(sc.get(&a.queue, a.cap));
+    DSG_TRY_CUDA(sc.get(&a.ctl, 1));
+    DSG_TRY_CUDA(cudaMemsetAsync(a.ctl, 0, sizeof(SplitCtl), s));
+    uint32_t grid = 1;
+    DSG_TRY_CUDA(coop_grid(core_split_kernel, kSplitTB, 0, (uint64_t)r + entries / 16, 1, &grid, g->max_blocks));
+    {
+        void* params[] = {&a};
+        LaunchScope ls("kcore_split", s);
+        DSG_TRY_CUDA(cudaLaunchCooperativeKernel((const void*)core_split_kernel, dim3(grid), dim3(kSplitTB), params, 0,
+                                                 s));
+    }
+    unsigned long long* lev = nullptr;
+    if (stats5) {
+        uint32_t* hist;
+        const uint32_t bins = std::min<uint64_t>((uint64_t)lo + (1ull << kSplitBits), 1ull << 31);
+        DSG_TRY_CUDA(sc.get(&hist, bins));
+        DSG_TRY_CUDA(sc.get(&lev, 2));
+        DSG_TRY_CUDA(cudaMemsetAsync(hist, 0, (size_t)bins * 4, s));
+        LaunchScope ls("kcore_tail_levels", s);
+        tail_levels_kernel<<<1, 1024, 0, s>>>(r, rid, core, bins, hist, lev);
+        DSG_TRY_CUDA(cudaGetLastError());
+    }
+    SplitCtl h;
+    unsigned long long hl[2] = {0, 0};
+    DSG_TRY_CUDA(cudaMemcpyAsync(&h, a.ctl, sizeof(h), cudaMemcpyDeviceToHost, s));
+    if (lev) DSG_TRY_CUDA(cudaMemcpyAsync(hl, lev, sizeof(hl), cudaMemcpyDeviceToHost, s));
+    DSG_TRY_CUDA(cudaStreamSynchronize(s));
+    dsg_status st = status_from_err(h.err, "kcore tail");
+    if (st != DSG_OK) return st;
+    if (stats5) {
+        stats5[0] += hl[0];
+        stats5[2] += hl[1];
+        stats5[4] += h.atomics;
+    }
+    if (stamps) *stamps = h.stamps;
+    return DSG_OK;
 }
 
 // Scan of n uint32 values into out[0..n] (exclusive, out[n] = total).
 dsg_status scan_u32(const uint32_t* in, uint64_t n, uint64_t* out, Scratch& sc, cudaStream_t s);
 
-dsg_status kcore_tail(uint32_t n, const uint64_t* off, const uint32_t* adj, uint32_t* deg, const uint32_t* claim,
-                      uint32_t cap, cudaStream_t s, uint64_t* stats5, uint64_t* trace, uint64_t trace_cap,
-                      uint64_t* stamps) {
+dsg_status kcore_tail(const dsg_graph* g, uint32_t* deg, const uint32_t* claim, uint32_t cap, uint32_t lo,
+                      uint64_t* stats5, uint64_t* trace, uint64_t trace_cap, uint64_t* stamps) {
+    cudaStream_t s = g->stream;
+    const uint32_t n = g->n;
+    const uint64_t* off = g->off;
+    const uint32_t* adj = g->adj;
     Scratch sc(s);
     uint32_t *rid, *newid, *cdeg, *flen, *cnt;
     DSG_TRY_CUDA(sc.get(&rid, cap));
@@ -532,9 +612,9 @@ dsg_status kcore_tail(uint32_t n, const uint64_t* off, const uint32_t* adj, uint
     DSG_TRY_CUDA(cudaMemsetAsync(cnt, 0, sizeof(uint32_t), s));
     {
         const uint32_t words = (n + 31) >> 5;
-        const uint32_t g = (uint32_t)std::min<uint64_t>(((uint64_t)words + 255) / 256, (uint64_t)dev_info().sms * 8);
+        const uint32_t gb = (uint32_t)std::min<uint64_t>(((uint64_t)words + 255) / 256, (uint64_t)dev_info().sms * 8);
         LaunchScope ls("kcore_tail_collect", s);
-        tail_collect_kernel<<<g ? g : 1, 256, 0, s>>>(n, claim, deg, off, rid, newid, cdeg, flen, cnt, cap);
+        tail_collect_kernel<<<gb ? gb : 1, 256, 0, s>>>(n, claim, deg, off, rid, newid, cdeg, flen, cnt, cap);
     }
     DSG_TRY_CUDA(cudaGetLastError());
     uint32_t r = 0;
@@ -570,96 +650,15 @@ dsg_status kcore_tail(uint32_t n, const uint64_t* off, const uint32_t* adj, uint
                                                                                     newid, coff, fill, cadj, cnt);
     }
     DSG_TRY_CUDA(cudaGetLastError());
-    if (ecount >= (uint64_t)kOffMax) {
-        // row offsets do not fit the cluster's 32-bit row starts: finish with the grid-wide
-        // kernel on the compacted graph instead, then put its core numbers in place
-        uint32_t* ccore;
-        DSG_TRY_CUDA(sc.get(&ccore, r));
-        dsg_graph view;
-        view.n = r;
-        view.m = ecount / 2;
-        view.off = coff;
-        view.adj = cadj;
-        view.owns = false;
-        DSG_TRY_CUDA(cudaGetDevice(&view.device));
-        view.stream = s;
-        view.no_tail = true;
-        uint64_t sub[5] = {0, 0, 0, 0, 0};
-        dsg_status st2 = run_kcore(&view, ccore, sub, 5);
-        if (st2 != DSG_OK) return st2;
-        {
-            LaunchScope ls("kcore_tail_scatter", s);
-            tail_scatter_kernel<<<(r + 255) / 256, 256, 0, s>>>(r, rid, ccore, deg);
-        }
-        DSG_TRY_CUDA(cudaGetLastError());
-        DSG_TRY_CUDA(cudaStreamSynchronize(s));
-        if (stats5) {
-            stats5[0] += sub[0];
-            stats5[2] += sub[2];
-            stats5[4] += sub[4];
-        }
-        if (stamps) *stamps = 0;
-        return DSG_OK;
-    }
-    // ---- the cluster: 16 blocks (each holds at most kTailVPC vertices, so 16 always suffice)
-    const uint32_t C = kTailC;
-    const size_t smem = sizeof(TailSmem);
-    DSG_TRY_CUDA(cudaFuncSetAttribute(kcore_tail_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    if (cudaFuncSetAttribute(kcore_tail_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) {
-        cudaGetLastError();
-        set_error("kcore tail: %u vertices need a cluster of %u blocks, which this device does not allow", r, C);
-        return DSG_ECUDA;
-    }
-    TailArgs ta;
-    ta.r = r;
-    ta.off = coff;
-    ta.adj = cadj;
-    ta.cdeg = cdeg;
-    ta.rid = rid;
-    ta.core = deg;
-    ta.limit_ns = wait_limit_ns();
-    DSG_TRY_CUDA(sc.get(&ta.stats, 1));
-    DSG_TRY_CUDA(cudaMemsetAsync(ta.stats, 0, sizeof(TailStats), s));
-    ta.trace = trace;
-    ta.trace_cap = trace ? trace_cap : 0;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(C);
-    cfg.blockDim = dim3(kTailTB);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = s;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = C;
-    attr[0].val.clusterDim.y = 1;
-    attr[0].val.clusterDim.z = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    int clusters = 0;
-    DSG_TRY_CUDA(cudaOccupancyMaxActiveClusters(&clusters, kcore_tail_kernel, &cfg));
-    if (clusters < 1) {
-        set_error("kcore tail: a cluster of %u blocks with %zu bytes of shared memory each does not fit", C, smem);
-        return DSG_ECUDA;
-    }
-    {
-        LaunchScope ls("kcore_tail", s);
-        DSG_TRY_CUDA(cudaLaunchKernelEx(&cfg, kcore_tail_kernel, ta));
-    }
-    TailStats h;
+    dsg_status st3 = core_split(r, lo, coff, cadj, ecount, rid, deg, g, sc, stats5, trace, trace_cap, stamps);
+    if (st3 != DSG_OK) return st3;
     uint32_t fill_err = 0;
-    DSG_TRY_CUDA(cudaMemcpyAsync(&h, ta.stats, sizeof(h), cudaMemcpyDeviceToHost, s));
     DSG_TRY_CUDA(cudaMemcpyAsync(&fill_err, cnt, sizeof(uint32_t), cudaMemcpyDeviceToHost, s));
     DSG_TRY_CUDA(cudaStreamSynchronize(s));
-    if (h.err & ERR_TIMEOUT) return status_from_err(h.err, "kcore tail");
-    if (h.err || fill_err || h.claims != r) {
-        set_error("kcore tail: inconsistent remaining graph (err %u, %llu of %u vertices placed)", h.err, h.claims, r);
+    if (fill_err) {
+        set_error("kcore tail: inconsistent remaining graph (err %u)", fill_err);
         return DSG_ECUDA;
     }
-    if (stats5) {
-        stats5[0] += h.levels;
-        stats5[2] += h.rem_scanned;
-        stats5[4] += h.atomics;
-    }
-    if (stamps) *stamps = h.stamps;
     return DSG_OK;
 }
 
