@@ -414,13 +414,13 @@ dsg_status dsg_set_local_max(uint32_t local_max, uint32_t local_work);
  * level-wide queue in pieces of at most chunk_len entries, which every block
  * takes from.  Default 256; DSG_INLINE_MAX.  Results never depend on it. */
 dsg_status dsg_set_inline_max(uint32_t inline_max);
-/* Core numbers: once at most max_vertices vertices remain after a level (or
- * from the start, on a graph of no more vertices), their core numbers are
- * searched bit by bit, all levels at once, instead of level by level; after a
- * level the remaining graph is compacted first (rows cut to the remaining
- * neighbours, which leaves every remaining degree as it is).  0 turns it off;
- * at most 131072.  Default 65536; DSG_KCORE_TAIL.  Results never depend on
- * it. */
+/* Core numbers: once at most 4 max_vertices vertices remain after a level,
+ * their core numbers are searched bit by bit, all levels at once, instead of
+ * level by level, on the compacted remaining graph (rows cut to the remaining
+ * neighbours, which leaves every remaining degree as it is); a graph of at
+ * most 16 max_vertices vertices is searched whole, without levels.  0 turns
+ * it off; at most 131072.  Default 65536; DSG_KCORE_TAIL.  Results never
+ * depend on it. */
 dsg_status dsg_set_kcore_tail(uint32_t max_vertices);
 /* Peel (Algorithm 1) in a thin tail: once a round removes less than 1/8 of
  * the vertices left, the next round also collects candidates -- every alive

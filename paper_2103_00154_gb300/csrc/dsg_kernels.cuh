@@ -27,8 +27,8 @@ struct Tuning {
     uint32_t local_work = 16384; // k-core: ... while that block's local share of the sub-round stays within this
     uint32_t inline_max = 256;   // k-core: rows up to this length claimed by a block's level scan are drained by
                                  // that block; longer ones by every warp in the next sub-round
-    uint32_t tail_max = 65536;   // k-core: once at most this many vertices remain, one thread-block cluster
-                                 // finishes the levels on the compacted remaining graph (0: never)
+    uint32_t tail_max = 65536;   // k-core: scale of the graphs and remaining graphs whose core numbers are searched
+                                 // bit by bit instead of level by level (kTailHandOver, kTailWhole; 0: never)
     uint32_t batch_split = 0;    // batches: a graph whose work (2m + n) exceeds this is solved by the
                                  // grid-wide kernels (0: above twice a block's share and 2^20)
     uint32_t batch_block = 512;  // batches: threads per block of the block-per-graph kernel
@@ -87,11 +87,22 @@ dsg_status run_kcore(const dsg_graph* g, uint32_t* core_out, uint64_t* stats, ui
 // compacted remaining graph; writes them into deg and adds what a level run
 // would count (levels, remaining entries) and the atomics into stats5[0],
 // [2], [4]; with a trace buffer, block 0 stamps each wave there.
-constexpr uint32_t kTailMaxVertices = 131072;
+constexpr uint32_t kTailMaxVertices = 131072;  // largest Tuning::tail_max
+// The search takes over from the levels once at most kTailHandOver * tail_max
+// vertices remain, and takes graphs of up to kTailWhole * tail_max vertices
+// whole (core numbers, ms, at hand-overs of 65,536 / 131,072 / 262,144 /
+// 524,288 vertices: Chung-Lu 2^24 20.5 / 18.7 / 17.7 / 18.0, 3 10^6 4.93 /
+// 4.43 / 4.31 / 4.45, 2 10^6 4.13 / 3.74 / 3.55 / 3.78; whole against the best
+// hand-over: Chung-Lu 7 10^5 1.29 / 1.52, 3 10^5 0.98 / 1.16, 10^5 0.65 / 0.91,
+// R-MAT 2^20 2.37 / 2.36, 2^18 0.84 / 1.04, Erdos-Renyi 10^6 0.86 / 1.41;
+// at 2 10^6 vertices of mean degree 30 it no longer wins: 3.71 / 3.55).
+constexpr uint64_t kTailHandOver = 4;
+constexpr uint64_t kTailWhole = 16;
+constexpr uint64_t kTailMaxEntries = 1ull << 36;  // beyond: levels only
 dsg_status kcore_tail(const dsg_graph* g, uint32_t* deg, const uint32_t* claim, uint32_t cap, uint32_t lo,
                       uint64_t* stats5, uint64_t* trace = nullptr, uint64_t trace_cap = 0, uint64_t* stamps = nullptr);
 
-// The same on a whole graph of r <= kTailMaxVertices vertices (rows off, adj;
+// The same on a whole graph of r vertices (rows off, adj;
 // rid nullable: original ids); limits of the grid from g.
 dsg_status core_split(uint32_t r, uint32_t lo, const uint64_t* off, const uint32_t* adj, uint64_t entries,
                       const uint32_t* rid, uint32_t* core, const dsg_graph* g, Scratch& sc, uint64_t* stats5,

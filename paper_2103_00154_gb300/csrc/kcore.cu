@@ -666,11 +666,12 @@ dsg_status run_kcore(const dsg_graph* g, uint32_t* core_out, uint64_t* stats, ui
     a.local_max = tu.local_max;
     a.local_work = tu.local_work;
     a.inline_max = tu.inline_max;
-    a.tail_max = tu.tail_max < kTailMaxVertices ? tu.tail_max : kTailMaxVertices;
+    const uint64_t tail = 2 * g->m < kTailMaxEntries ? tu.tail_max : 0;
+    a.tail_max = (uint32_t)(kTailHandOver * std::min<uint64_t>(tail, kTailMaxVertices));
     a.trace = trace_dev;
     a.trace_cap = trace_cap;
     const bool direct = is_device_ptr(core_out);
-    if (n <= a.tail_max) {
+    if (n <= kTailWhole * std::min<uint64_t>(tail, kTailMaxVertices)) {
         // few enough from the start: no level is run
         uint64_t vals[5] = {0, 0, 0, 0, 0};
         uint32_t* core = core_out;

@@ -45,10 +45,10 @@
 // a chain of about eight dependent L2 round trips (the meeting, piece, row
 // entry, key, decrement, queue slot, piece written and released): 4.5 us.
 // Measured against one 16-block cluster walking the levels with the degrees
-// in its shared memory: Chung-Lu 2^24 (870 levels left) 18.7 -> 3.6 ms,
-// 700,001 vertices (97 levels) 2.04 -> 0.68 ms, R-MAT scale 18 (129 levels)
-// 2.15 -> 0.76 ms, 10^4 vertices (the whole graph) 0.24 -> 0.16 ms with the
-// compaction and its copies saved.
+// in its shared memory, 65,536 vertices left to either: Chung-Lu 2^24 (870
+// levels) 18.7 -> 3.6 ms, 700,001 vertices (97 levels) 2.04 -> 0.68 ms, R-MAT
+// scale 18 (129 levels) 2.15 -> 0.76 ms.  Where it takes over:
+// kTailHandOver and kTailWhole.
 // Tried and dropped: a warp that goes on with the vertices it has removed
 // instead of queueing them (1, 2 or 4 rows deep: 0.82, 0.84, 0.88 ms against
 // 0.74 at 700,001 vertices -- the wave waits for the longest chain).
@@ -61,17 +61,14 @@ namespace dsg {
 
 constexpr uint32_t kSplitTB = 1024;
 constexpr uint32_t kPiece = 128;  // entries per row piece: one step of a warp, 4 loads per lane in flight
-constexpr uint32_t kSplitBits = 17;  // kTailMaxVertices vertices have core numbers below 2^17
-// A vertex's key: pieces of its row above kKeyBits (a row has fewer than
-// kTailMaxVertices entries, 1,024 pieces), its c, and the `first` bit.
+constexpr uint32_t kSplitBits = 18;  // bits of c (a core number k takes k (k + 1) row entries: enough below 2^36)
+// A vertex's key: pieces of its row above kKeyBits (kPiecesMax: that many or
+// more, count them from the row), its c, and the `first` bit.
 constexpr uint32_t kKeyBits = kSplitBits + 1;
 constexpr uint32_t kKeyMask = (1u << kKeyBits) - 1u;
 constexpr uint32_t kPiecesMax = (1u << (32 - kKeyBits)) - 1u;
 
-__device__ __forceinline__ uint32_t pieces_of(uint64_t len) {
-    const uint64_t np = (len + kPiece - 1) / kPiece;
-    return np < kPiecesMax ? (uint32_t)np : kPiecesMax;
-}
+__device__ __forceinline__ uint32_t pieces_of(uint64_t len) { return (uint32_t)((len + kPiece - 1) / kPiece); }
 
 struct __align__(128) SplitCtl {
     unsigned long long bar[2][16];  // arrivals (low half) and pieces queued (high half), by parity
@@ -90,7 +87,7 @@ struct SplitArgs {
     const uint32_t* rid;  // original ids (nullable: the numbers themselves)
     uint32_t* d;          // degrees in the running peel
     uint32_t* ds;         // degrees before it
-    uint32_t* key;        // kSplitBits + 1 buffers of kstride entries
+    uint32_t* key;        // a buffer of kstride entries for every bit
     uint64_t kstride;
     uint4* pieces;        // every row's pieces: first entry (low word), vertex, entries | first entry >> 32 << 16
     uint4* queue;         // the waves' pieces, the vertex's c in the last word
@@ -116,9 +113,12 @@ struct SplitSmem {
 template <int K>
 __device__ __forceinline__ void put_rows(const SplitArgs& a, uint4* list, unsigned long long* tail, uint32_t* pushed,
                                          uint32_t hit, const uint32_t (&u)[K], const uint32_t (&c)[K],
-                                         const uint32_t (&np)[K]) {
+                                         uint32_t (&np)[K]) {
     const uint32_t lane = lane_id();
     uint32_t mine = 0;
+#pragma unroll
+    for (int j = 0; j < K; ++j)
+        if ((hit >> j & 1u) && np[j] == kPiecesMax) np[j] = pieces_of(a.off[u[j] + 1] - a.off[u[j]]);
 #pragma unroll
     for (int j = 0; j < K; ++j) mine += hit >> j & 1u ? np[j] : 0u;
     const uint32_t inc = warp_incl_scan(mine);
@@ -238,7 +238,7 @@ __global__ void __launch_bounds__(kSplitTB, 1) core_split_kernel(SplitArgs a) {
             if (m == 0) break;
             if (lane == 0) atomicAdd(&sm.above[b], (uint32_t)__popc(m));
         }
-        const uint32_t np1[1] = {pieces_of(d)};
+        uint32_t np1[1] = {pieces_of(d)};
         put_rows<1>(a, a.pieces, &ctl->npieces, &sm.pushed, d ? 1u : 0u, v1, c1, np1);
     }
     __syncthreads();
@@ -331,7 +331,8 @@ __global__ void __launch_bounds__(kSplitTB, 1) core_split_kernel(SplitArgs a) {
                 __syncwarp();
                 const uint32_t take = cnt[lane];
                 cnt[lane] = 0;
-                const uint32_t v1[1] = {v}, c1[1] = {kc >> 1}, np1[1] = {kv >> kKeyBits};
+                const uint32_t v1[1] = {v}, c1[1] = {kc >> 1};
+                uint32_t np1[1] = {kv >> kKeyBits};
                 uint32_t hit = 0;
                 if (take) {
                     const uint32_t old = atomicSub(&a.d[v], take);
@@ -367,7 +368,7 @@ __global__ void __launch_bounds__(kSplitTB, 1) core_split_kernel(SplitArgs a) {
             }
             const bool first = d < bound + c;
             const uint32_t np = pieces_of(a.off[i + 1] - a.off[i]);
-            key[i] = np << kKeyBits | c << 1 | (first ? 1u : 0u);
+            key[i] = min(np, kPiecesMax) << kKeyBits | c << 1 | (first ? 1u : 0u);
             if (first) nfirst += np;
         }
         nfirst = warp_sum(nfirst);
@@ -532,8 +533,7 @@ __global__ void __launch_bounds__(1024) tail_levels_kernel(uint32_t r, const uin
     }
 }
 
-// The bitwise search on a graph of r <= kTailMaxVertices vertices (rows off,
-// adj), none with a core number below lo; core numbers to core (by original
+// The bitwise search on a graph of r vertices (rows off, adj), none with a core number below lo; core numbers to core (by original
 // id through rid, nullable: the vertices' own numbers).
 dsg_status core_split(uint32_t r, uint32_t lo, const uint64_t* off, const uint32_t* adj, uint64_t entries,
                       const uint32_t* rid, uint32_t* core, const dsg_graph* g, Scratch& sc, uint64_t* stats5,
@@ -553,7 +553,10 @@ dsg_status core_split(uint32_t r, uint32_t lo, const uint64_t* off, const uint32
     a.cap = (uint64_t)r + entries / kPiece;
     DSG_TRY_CUDA(sc.get(&a.d, r));
     DSG_TRY_CUDA(sc.get(&a.ds, r));
-    DSG_TRY_CUDA(sc.get(&a.key, a.kstride * (kSplitBits + 1)));
+    // the bits searched: (lo + 2^b)^2 stays below the row entries
+    uint64_t nbuf = 1;
+    while (nbuf < kSplitBits && (1ull << (2 * nbuf)) <= entries) ++nbuf;
+    DSG_TRY_CUDA(sc.get(&a.key, a.kstride * nbuf));
     DSG_TRY_CUDA(sc.get(&a.pieces, a.cap));
     DSG_TRY_CUDA(sc.get(&a.queue, a.cap));
     DSG_TRY_CUDA(sc.get(&a.ctl, 1));
@@ -569,7 +572,7 @@ dsg_status core_split(uint32_t r, uint32_t lo, const uint64_t* off, const uint32
     unsigned long long* lev = nullptr;
     if (stats5) {
         uint32_t* hist;
-        const uint32_t bins = std::min<uint64_t>((uint64_t)lo + (1ull << kSplitBits), 1ull << 31);
+        const uint32_t bins = (uint32_t)std::min<uint64_t>((uint64_t)lo + (1ull << kSplitBits), 1ull << 31);
         DSG_TRY_CUDA(sc.get(&hist, bins));
         DSG_TRY_CUDA(sc.get(&lev, 2));
         DSG_TRY_CUDA(cudaMemsetAsync(hist, 0, (size_t)bins * 4, s));

@@ -2,7 +2,8 @@
 graph when it is small enough): rows at the edges of a row piece (128 entries)
 and of a warp's 32 pieces, graphs whose core numbers need one to eleven bits,
 one block up to the whole grid, the largest graph it takes whole and the
-smallest it does not, thin and wide cascades.  Every core number against the
+smallest it does not, rows of more pieces than a key can say, thin and wide
+cascades.  Every core number against the
 oracle, the level counters against the core numbers."""
 import numpy as np
 import pytest
@@ -38,12 +39,12 @@ CASES = [
     _bipartite(3, 127), _bipartite(3, 128), _bipartite(2, 129), _bipartite(5, 32 * 128 + 1),
     inputs.star(127), inputs.star(128), inputs.star(129), inputs.star(4 * 128 + 1), inputs.star(131070),
     inputs.path(700), inputs.cycle(1000), inputs.onion(6000, 16, 40), inputs.empty(131072),
-    inputs.rmat(12, 1 << 17, seed=5), inputs.chung_lu(131072, 1 << 20, 2.1, 16.0, 20000.0, 9),
-    inputs.chung_lu(131073, 1 << 20, 2.1, 16.0, 20000.0, 9), inputs.random_small(400, 0.5, 3),
+    inputs.star((8191 * 128) + 1), inputs.star(1_200_000), inputs.rmat(12, 1 << 17, seed=5), inputs.chung_lu(32768, 1 << 18, 2.1, 16.0, 9000.0, 9),
+    inputs.chung_lu(32769, 1 << 18, 2.1, 16.0, 9000.0, 9), inputs.random_small(400, 0.5, 3),
 ]
 
 
-@pytest.mark.parametrize("tail", [131072, 65536, 500])
+@pytest.mark.parametrize("tail", [131072, 65536, 2048, 100])
 @pytest.mark.parametrize("raw", CASES, ids=lambda r: r.name)
 def test_core_numbers(raw, tail):
     c = oracle.from_raw(raw)
