@@ -386,9 +386,11 @@ void dsg_serve_destroy(dsg_server* s);
  * Launch parameters of the round kernels (not part of the method):
  *   block          threads per block of the persistent kernels: 256, 512, 1024
  *   blocks_per_sm  resident blocks per SM (0 = as many as fit)
- *   short_max      rows up to this length are scanned edge-balanced inside a
- *                  block; longer rows are cut into chunk items
- *   chunk_len      entries per chunk item (one warp each), >= 32
+ *                  (until this call or DSG_BLOCK gives it, it is picked by
+ *                  the graph's size and the kernel)
+ *   short_max      has no effect any more (rows of all lengths are walked
+ *                  edge-balanced)
+ *   chunk_len      rows are cut into pieces of at most this many entries, >= 32
  * Process-wide; also read from DSG_BLOCK, DSG_BLOCKS_PER_SM, DSG_SHORT_MAX and
  * DSG_CHUNK_LEN at first use.  Results never depend on these.
  */
@@ -434,12 +436,8 @@ dsg_status dsg_set_kcore_tail(uint32_t max_vertices);
  * (dsg_trace.tested).  1 (default) on, 0 off; DSG_PEEL_LAZY.  Results never
  * depend on it. */
 dsg_status dsg_set_peel_lazy(uint32_t on);
-/* Peel (Algorithm 1): 1 reads the long rows' chunks as aligned 16-byte
- * groups, four consecutive entries per lane (one 128-bit load each, entries
- * outside the chunk masked off); 0 (default) reads one entry per lane, 32
- * consecutive entries per warp load, four loads in flight.  Used only when
- * the adjacency array is 16-byte aligned.  DSG_PEEL_VEC.  Results never
- * depend on it. */
+/* Has no effect any more: the 128-bit row loads it chose in the peel were
+ * slower than one entry per lane and are gone. */
 dsg_status dsg_set_peel_vec(uint32_t on);
 
 /*

@@ -29,13 +29,6 @@ struct BatchSmem {
     uint32_t item;
 };
 
-__device__ __forceinline__ uint32_t b_threshold(uint64_t p, uint64_t q, uint64_t E, uint64_t S) {
-    unsigned __int128 num = (unsigned __int128)2 * (unsigned __int128)(p + q) * (unsigned __int128)E;
-    unsigned __int128 den = (unsigned __int128)q * (unsigned __int128)S;
-    unsigned __int128 t = num / den;
-    return t > (unsigned __int128)0xffffffffu ? 0xffffffffu : (uint32_t)t;
-}
-
 // Algorithm 1 on one graph by one block.
 template <int TB>
 __device__ void peel_block(const BatchArgs& a, uint32_t g, BatchSmem<TB>& sm) {
@@ -55,7 +48,10 @@ __device__ void peel_block(const BatchArgs& a, uint32_t g, BatchSmem<TB>& sm) {
     const uint32_t* alive = nullptr;
     uint32_t* next = alive_a;
     while (S > 0) {
-        const uint32_t T = b_threshold(p, q, E, S);
+        // one thread divides for the block: the division is a few hundred instructions
+        if (tid == 0) sm.u32[1] = peel_threshold(p, q, E, S);
+        __syncthreads();
+        const uint32_t T = sm.u32[1];
         const uint32_t mark = kDeadB | (uint32_t)(r + 1);
         uint32_t nf = 0, ns = 0;
         if (tid == 0) sum_S += S;

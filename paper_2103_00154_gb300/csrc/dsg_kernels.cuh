@@ -18,8 +18,8 @@ __device__ __forceinline__ uint32_t ld_stream(const uint32_t* p) { return __ldcs
 struct Tuning {
     uint32_t block = 512;       // threads per block of the persistent kernels
     uint32_t blocks_per_sm = 0; // 0: as many as fit
-    uint32_t short_max = 32;    // rows up to this length go through the tile path
-    uint32_t chunk_len = 256;   // long rows are cut into items of this many entries
+    uint32_t short_max = 32;    // kept for saved tables and callers; no kernel tells short rows apart any more
+    uint32_t chunk_len = 256;   // rows are cut into pieces of at most this many entries
     uint32_t hot_deg = 0;       // decrements of vertices at or above this degree are combined in shared memory
                                 // (0: four times the number of blocks, i.e. hubs expected to be hit
                                 // several times by every block)
@@ -34,8 +34,7 @@ struct Tuning {
     uint32_t batch_block = 512;  // batches: threads per block of the block-per-graph kernel
     uint32_t peel_lazy = 1;      // peel: thin-tail rounds test only the candidate list (0: every round
                                  // tests the whole alive list); read from the global tuning only
-    uint32_t peel_vec = 0;       // peel: long rows read as aligned 128-bit groups (0: one entry per lane);
-                                 // read from the global tuning only
+    uint32_t peel_vec = 0;       // kept for callers; the 128-bit row loads it chose were slower and are gone
 };
 
 // Tuning of a batch of G graphs with `work` = sum of (2m + n): the autotuned
@@ -108,6 +107,20 @@ dsg_status core_split(uint32_t r, uint32_t lo, const uint64_t* off, const uint32
                       const uint32_t* rid, uint32_t* core, const dsg_graph* g, Scratch& sc, uint64_t* stats5,
                       uint64_t* trace, uint64_t trace_cap, uint64_t* stamps);
 
+// floor(2(p+q)E / (qS)) clamped to 32 bits; S > 0 (Algorithm 1's threshold).
+// A division of two 64-bit numbers unless one of them needs 128 bits.
+__device__ __forceinline__ uint32_t peel_threshold(uint64_t p, uint64_t q, uint64_t E, uint64_t S) {
+    const uint64_t a = 2 * (p + q);
+    uint64_t t;
+    if (__umul64hi(a, E) == 0 && __umul64hi(q, S) == 0) {
+        t = a * E / (q * S);
+    } else {
+        const unsigned __int128 w = (unsigned __int128)a * E / ((unsigned __int128)q * S);
+        t = w > 0xffffffffu ? 0xffffffffu : (uint64_t)w;
+    }
+    return t > 0xffffffffu ? 0xffffffffu : (uint32_t)t;
+}
+
 // Device check that a graph is canonical (sorted rows, no loops, no repeats,
 // symmetric, ids < n).  DSG_EINVAL with a message if not.
 dsg_status validate_csr(const dsg_graph* g);
@@ -142,6 +155,55 @@ __device__ __forceinline__ uint32_t ld_relaxed_u32(const uint32_t* p) {
     uint32_t v;
     asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
     return v;
+}
+
+// The blocks of a co-resident grid meet, on a word that also sums a count:
+// low half arrivals, high half the blocks' `mine`.  The grid's sum comes back
+// with the wait, so nothing is read for it afterwards.  Two words take turns:
+// a block that is already on its way to the next meeting must not add to the
+// sum that a slower block is still to read (to come back to the same word it
+// has to pass the other, which needs the slower block).  The words start at
+// zero.  Every thread of the block calls it; thread 0's `mine` counts.  A wait
+// above limit_ns records ERR_TIMEOUT and clears sm.ok, as does seeing the
+// error of another block.  With one block (nblocks == 1) it is a block barrier.
+struct MeetState {
+    uint32_t epoch = 0, seen0 = 0, seen1 = 0;
+};
+struct MeetSmem {
+    uint32_t got, ok;
+};
+
+__device__ __forceinline__ uint32_t grid_meet(unsigned long long (*bar)[16], uint32_t* err, uint64_t limit_ns,
+                                              uint32_t nblocks, uint32_t mine, MeetState& st, MeetSmem& sm) {
+    __syncthreads();
+    const uint32_t par = st.epoch & 1u;
+    ++st.epoch;
+    if (threadIdx.x == 0) {
+        if (nblocks == 1) {
+            sm.got = mine;
+        } else {
+            unsigned long long* word = &bar[par][0];
+            const uint32_t target = ((st.epoch + 1) >> 1) * nblocks;  // odd and even meetings have a word each
+            red_add_release_u64(word, (uint64_t)mine << 32 | 1ull);
+            uint64_t w;
+            uint32_t polls = 0;
+            const uint64_t t0 = global_ns();
+            while ((int32_t)((uint32_t)(w = ld_acquire_u64(word)) - target) < 0) {
+                if ((++polls & 63u) == 0) {
+                    if (global_ns() - t0 > limit_ns) atomicOr(err, ERR_TIMEOUT);
+                    if (ld_volatile_u32(err) & ERR_TIMEOUT) {
+                        sm.ok = 0;
+                        break;
+                    }
+                }
+            }
+            sm.got = (uint32_t)(w >> 32) - (par ? st.seen1 : st.seen0);
+        }
+    }
+    __syncthreads();
+    const uint32_t got = sm.got;
+    if (par) st.seen1 += got; else st.seen0 += got;
+    return got;
 }
 
 // Per-block table that combines degree decrements aimed at the same
@@ -428,155 +490,6 @@ __device__ __forceinline__ void walk_all_entries(const uint64_t* __restrict__ of
         r = __shfl_sync(kFullMask, last, 31);
         if (!__shfl_sync(kFullMask, valid >> (kWalkU - 1) & 1u, 31)) break;  // span's final step
     }
-}
-
-// Walk every adjacency entry of a frontier, handing entries to the visitor
-// four at a time per thread so the visitor can issue four independent loads
-// (then four independent atomics) before it waits on any of them.  No block
-// barrier is used: every warp works on its own share.
-//   short rows: F[lo, hi), one vertex per entry; a warp takes 32 of them,
-//     prefix-sums their lengths with shuffles and spreads the concatenated
-//     entries over its lanes (consecutive lanes read consecutive entries); a
-//     lane finds the row owning an entry by a 5-step shuffle binary search.
-//   long rows: C[clo, chi), items (v << 32 | c) standing for entries
-//     [off[v] + c*chunk_len, min(off[v+1], off[v] + (c+1)*chunk_len)); one warp
-//     per item, 32 consecutive entries per step, four steps in flight.
-// fn(u[4], v[4], valid) is called with bit j of `valid` set for each filled
-// slot j (u = neighbour, v = row owner).  All lanes of a warp call fn
-// together (valid may be 0).
-// LOCAL = true: F is this block's own list (e.g. in shared memory) and only
-// this block's warps walk it; C is ignored.
-// FB / FL (nullable): row starts and lengths stored beside F, saving the
-// offset loads of the short rows.
-// vec_end (0: off): adj is 16-byte aligned and holds at least vec_end
-// entries; long rows are then read with 128-bit loads.
-template <int TB, bool LOCAL = false, class Fn>
-__device__ __forceinline__ void scan_frontier(const uint64_t* __restrict__ off, const uint32_t* __restrict__ adj,
-                                              const uint32_t* F, uint64_t lo, uint64_t hi,
-                                              const uint64_t* __restrict__ C, uint64_t clo, uint64_t chi,
-                                              uint32_t chunk_len, Fn& fn, uint32_t dbg_n = 0,
-                                              const uint64_t* FB = nullptr, const uint32_t* FL = nullptr,
-                                              uint64_t vec_end = 0) {
-    const uint32_t tid = threadIdx.x;
-    const uint32_t lane = tid & 31u;
-    const uint64_t gw = LOCAL ? (uint64_t)(tid >> 5) : ((uint64_t)blockIdx.x * TB + tid) >> 5;
-    const uint64_t nw = LOCAL ? (uint64_t)(TB >> 5) : ((uint64_t)gridDim.x * TB) >> 5;
-    // ---- short rows, 32 per warp, edge-balanced over the warp's lanes
-    auto short_group = [&](uint64_t g0) {
-        uint64_t i = g0 + lane;
-        uint32_t v = 0, len = 0;
-        uint64_t b = 0;
-        if (i < hi) {
-            v = F[i];
-#ifdef DSG_DEBUG_BOUNDS
-            if (v >= dbg_n) {
-                uint32_t bu[kBatch] = {0xfffffffeu}, bv[kBatch] = {v};
-                fn(bu, bv, 1u);
-                v = 0;
-            }
-#endif
-            if (FB) {
-                b = FB[i];
-                len = FL[i];
-            } else {
-                b = off[v];
-                len = (uint32_t)(off[v + 1] - b);
-            }
-        }
-        const uint32_t inc = warp_incl_scan(len);
-        const uint32_t total = __shfl_sync(kFullMask, inc, 31);
-        const uint32_t st = inc - len;
-        for (uint32_t e0 = lane; e0 < ((total + 31u) & ~31u); e0 += 32 * kBatch) {
-            uint32_t bu[kBatch], bv[kBatch], valid = 0;
-#pragma unroll
-            for (uint32_t j = 0; j < kBatch; ++j) {
-                const uint32_t e = e0 + 32 * j;
-                // owner = last lane whose start is <= e (all lanes take part in the shuffles)
-                uint32_t a = 0;
-#pragma unroll
-                for (uint32_t step = 16; step > 0; step >>= 1) {
-                    uint32_t s_mid = __shfl_sync(kFullMask, st, a + step);
-                    if (a + step < 32 && s_mid <= e) a += step;
-                }
-                const uint32_t ost = __shfl_sync(kFullMask, st, a);
-                const uint64_t ob = __shfl_sync(kFullMask, b, a);
-                const uint32_t ov = __shfl_sync(kFullMask, v, a);
-                bu[j] = 0;
-                bv[j] = ov;
-                if (e < total) {
-                    uint64_t pos = ob + (e - ost);
-#ifdef DSG_DEBUG_BOUNDS
-                    if (pos >= off[dbg_n]) { bu[j] = 0xffffffffu; bv[j] = 0xffffffffu; valid |= 1u << j; continue; }
-#endif
-                    bu[j] = ld_stream(adj + pos);
-                    valid |= 1u << j;
-                }
-            }
-            fn(bu, bv, valid);
-        }
-    };
-    // ---- long rows, one warp per chunk item
-    auto chunk_item = [&](uint64_t it) {
-        uint64_t item = C[it];
-        uint32_t v = (uint32_t)(item >> 32);
-#ifdef DSG_DEBUG_BOUNDS
-        if (v >= dbg_n) {
-            uint32_t bu[kBatch] = {0xfffffffdu}, bv[kBatch] = {v};
-            fn(bu, bv, 1u);
-            return;
-        }
-#endif
-        uint64_t c = item & 0xffffffffull;
-        uint64_t b = off[v], e_end = off[v + 1];
-        uint64_t beg = b + c * chunk_len;
-        uint64_t end = min(e_end, beg + chunk_len);
-        if (vec_end) {
-            // 128-bit loads: lane l takes the aligned group of four entries 4g..4g+3, g = g0 + l
-            // (+ 32 per step); entries of a group outside [beg, end) are masked off, and a
-            // group that reaches past vec_end is read entry by entry
-            static_assert(kBatch == 4, "one 16-byte group per visitor call");
-            const uint64_t g0 = beg >> 2, g1 = (end + 3) >> 2;
-            for (uint64_t gb = g0; gb < g1; gb += 32) {
-                const uint64_t g = gb + lane;
-                uint32_t bu[kBatch] = {0u, 0u, 0u, 0u}, bv[kBatch] = {v, v, v, v}, valid = 0;
-                if (g < g1) {
-                    const uint64_t e0 = g * 4;
-                    if (e0 + 4 <= vec_end) {
-                        const uint4 q = __ldcs(reinterpret_cast<const uint4*>(adj) + g);
-                        bu[0] = q.x;
-                        bu[1] = q.y;
-                        bu[2] = q.z;
-                        bu[3] = q.w;
-                    } else {
-#pragma unroll
-                        for (uint32_t j = 0; j < kBatch; ++j)
-                            if (e0 + j >= beg && e0 + j < end) bu[j] = ld_stream(adj + e0 + j);
-                    }
-#pragma unroll
-                    for (uint32_t j = 0; j < kBatch; ++j)
-                        if (e0 + j >= beg && e0 + j < end) valid |= 1u << j;
-                }
-                fn(bu, bv, valid);
-            }
-            return;
-        }
-        for (uint64_t j0 = beg + lane; j0 < end; j0 += 32 * kBatch) {
-            uint32_t bu[kBatch], bv[kBatch], valid = 0;
-#pragma unroll
-            for (uint32_t j = 0; j < kBatch; ++j) {
-                uint64_t jj = j0 + 32 * j;
-                bu[j] = 0;
-                bv[j] = v;
-                if (jj < end) {
-                    bu[j] = ld_stream(adj + jj);
-                    valid |= 1u << j;
-                }
-            }
-            fn(bu, bv, valid);
-        }
-    };
-    for (uint64_t g0 = lo + gw * 32; g0 < hi; g0 += nw * 32) short_group(g0);
-    for (uint64_t it = LOCAL ? chi : clo + gw; it < chi; it += nw) chunk_item(it);
 }
 
 }  // namespace dsg

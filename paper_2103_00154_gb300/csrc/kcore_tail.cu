@@ -34,10 +34,8 @@
 // key is written to a buffer of its own for every bit, so its look-ups may be
 // cached in L1 although the kernel rewrites it while it runs.
 //
-// The blocks meet after every wave; the word they meet on also sums the
-// pieces that the wave queued, so no block reads the queue's end separately.
-// Two words take turns: a block that is already in the next wave must not add
-// to the sum that a slower block is still to read.
+// The blocks meet after every wave (grid_meet: the pieces that the wave queued
+// come back with the wait).
 // Every wait is bounded (ERR_TIMEOUT).
 //
 // What bounds it: the wide waves, L2 gathers (a bit's first wave on Chung-Lu
@@ -101,8 +99,7 @@ struct SplitArgs {
 
 struct SplitSmem {
     uint32_t pushed;                  // pieces queued by this block in the running phase
-    uint32_t got;                     // pieces queued by the whole grid
-    uint32_t ok;
+    MeetSmem meet;
     uint32_t above[32];
     uint32_t cnt[kSplitTB / 32][32];  // pull: a warp's counts, per piece
 };
@@ -159,40 +156,15 @@ __device__ __forceinline__ void put_rows(const SplitArgs& a, uint4* list, unsign
     }
 }
 
-// All blocks meet (epoch counts the meetings); returns the pieces queued by
-// the grid since the last one.  sm.ok is false once a wait ran out.
-__device__ __forceinline__ uint32_t split_meet(const SplitArgs& a, SplitSmem& sm, uint32_t& epoch, uint32_t seen[2]) {
+// All blocks meet; returns the pieces queued by the grid since the last time.
+__device__ __forceinline__ uint32_t split_meet(const SplitArgs& a, SplitSmem& sm, MeetState& st) {
     __syncthreads();
-    const uint32_t par = epoch & 1u;
-    ++epoch;
+    uint32_t mine = 0;
     if (threadIdx.x == 0) {
-        const uint32_t mine = sm.pushed;
+        mine = sm.pushed;
         sm.pushed = 0;
-        if (gridDim.x == 1) {
-            sm.got = mine;
-        } else {
-            unsigned long long* word = &a.ctl->bar[par][0];
-            const uint32_t target = ((epoch + 1) >> 1) * gridDim.x;  // odd and even meetings have a word each
-            red_add_release_u64(word, (uint64_t)mine << 32 | 1ull);
-            uint64_t w;
-            uint32_t polls = 0;
-            const uint64_t t0 = global_ns();
-            while ((int32_t)((uint32_t)(w = ld_acquire_u64(word)) - target) < 0) {
-                if ((++polls & 63u) == 0) {
-                    if (global_ns() - t0 > a.limit_ns) atomicOr(&a.ctl->err, ERR_TIMEOUT);
-                    if (ld_volatile_u32(&a.ctl->err) & ERR_TIMEOUT) {
-                        sm.ok = 0;
-                        break;
-                    }
-                }
-            }
-            sm.got = (uint32_t)(w >> 32) - seen[par];
-        }
     }
-    __syncthreads();
-    const uint32_t got = sm.got;
-    seen[par] += got;
-    return got;
+    return grid_meet(a.ctl->bar, &a.ctl->err, a.limit_ns, gridDim.x, mine, st, sm.meet);
 }
 
 __global__ void __launch_bounds__(kSplitTB, 1) core_split_kernel(SplitArgs a) {
@@ -203,7 +175,7 @@ __global__ void __launch_bounds__(kSplitTB, 1) core_split_kernel(SplitArgs a) {
     const uint32_t gw = (blockIdx.x * kSplitTB + tid) >> 5, nw = gridDim.x * (kSplitTB / 32);
     const uint32_t nth = gridDim.x * kSplitTB;
     const uint32_t rpad = (r + 31u) & ~31u;  // whole warps in the per-vertex loops
-    uint32_t epoch = 0, seen[2] = {0, 0};
+    MeetState ms;
     uint64_t natom = 0, nwaves = 0, nstamp = 0;
     // trace pairs: kind 11 keys written, 12 first wave over, 13 a later wave over, 14 its pieces (value)
     auto stamp = [&](uint32_t kind, uint32_t b, uint64_t val) {
@@ -217,7 +189,7 @@ __global__ void __launch_bounds__(kSplitTB, 1) core_split_kernel(SplitArgs a) {
     if (tid < 32) sm.above[tid] = 0;
     if (tid == 0) {
         sm.pushed = 0;
-        sm.ok = 1;
+        sm.meet.ok = 1;
     }
     for (uint32_t i = tid; i < kSplitTB; i += kSplitTB) sm.cnt[i >> 5][i & 31u] = 0;
     __syncthreads();
@@ -243,8 +215,8 @@ __global__ void __launch_bounds__(kSplitTB, 1) core_split_kernel(SplitArgs a) {
     }
     __syncthreads();
     if (tid < 32 && sm.above[tid]) atomicAdd(&ctl->above[tid], sm.above[tid]);
-    const uint32_t npieces = split_meet(a, sm, epoch, seen);
-    if (!sm.ok) return;
+    const uint32_t npieces = split_meet(a, sm, ms);
+    if (!sm.meet.ok) return;
     uint32_t bits = 0;
     {
         const uint32_t cnt = ld_relaxed_u32(&ctl->above[lane]);
@@ -373,23 +345,23 @@ __global__ void __launch_bounds__(kSplitTB, 1) core_split_kernel(SplitArgs a) {
         }
         nfirst = warp_sum(nfirst);
         if (lane == 0 && nfirst) atomicAdd(&sm.pushed, nfirst);
-        const uint32_t np = split_meet(a, sm, epoch, seen);
-        if (!sm.ok) return;
+        const uint32_t np = split_meet(a, sm, ms);
+        if (!sm.meet.ok) return;
         stamp(11, b, global_ns());
         if (np != 0 && np != npieces) {
             const bool pull = npieces - np < np;
             wave(a.pieces, 0, npieces, key, bound, true, pull, tail);
             ++nwaves;
-            uint32_t from = 0, to = split_meet(a, sm, epoch, seen);
-            if (!sm.ok) return;
+            uint32_t from = 0, to = split_meet(a, sm, ms);
+            if (!sm.meet.ok) return;
             stamp(12, b, global_ns());
             stamp(14, b, to);
             while (from < to && to <= a.cap) {
                 wave(a.queue, from, to, key, bound, false, false, tail);
                 ++nwaves;
                 from = to;
-                to += split_meet(a, sm, epoch, seen);
-                if (!sm.ok) return;
+                to += split_meet(a, sm, ms);
+                if (!sm.meet.ok) return;
                 stamp(13, b, global_ns());
                 stamp(14, b, to - from);
             }

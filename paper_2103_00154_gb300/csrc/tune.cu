@@ -14,6 +14,7 @@ namespace dsg {
 static std::mutex g_tune_mu;
 static Tuning g_tune;
 static bool g_tune_set = false;
+static bool g_block_given = false;  // by dsg_set_tuning or DSG_BLOCK: then no rule of its own picks the block size
 
 static uint32_t env_u32(const char* name, uint32_t dflt) {
     const char* e = getenv(name);
@@ -25,6 +26,8 @@ Tuning current_tuning() {
     std::lock_guard<std::mutex> lk(g_tune_mu);
     if (!g_tune_set) {
         Tuning t;
+        const char* eb = getenv("DSG_BLOCK");
+        g_block_given = eb && *eb;
         t.block = env_u32("DSG_BLOCK", t.block);
         t.blocks_per_sm = env_u32("DSG_BLOCKS_PER_SM", t.blocks_per_sm);
         t.short_max = env_u32("DSG_SHORT_MAX", t.short_max);
@@ -58,6 +61,7 @@ extern "C" dsg_status dsg_set_tuning(uint32_t block, uint32_t blocks_per_sm, uin
     DSG_CHECK_ARG(short_max >= 1 && short_max <= 4096, "short_max must be in [1, 4096]");
     std::lock_guard<std::mutex> lk(g_tune_mu);
     g_tune.block = block;
+    g_block_given = true;
     g_tune.blocks_per_sm = blocks_per_sm;
     g_tune.short_max = short_max;
     g_tune.chunk_len = chunk_len;
@@ -234,10 +238,24 @@ static void ensure_table_loaded_locked() {
     if (e && *e) load_table_locked(e);
 }
 
+// Block size where nobody has given one.  Peel: 1,024 threads, one block per
+// SM, from 2^19 vertices (half the blocks to meet, and a hub table twice as
+// many decrements share: 3 10^6 vertices 0.73 against 0.79 ms, Chung-Lu 2^24
+// 3.31 against 3.39, Erdos-Renyi 10^6 0.244 against 0.252), 512 below (the
+// meetings and short lists weigh more: nested shells of 265,100 vertices 2.85
+// against 3.05 ms, 10^4 vertices 93 against 108 us).  Core-number levels: 256,
+// three blocks per SM (an idle warp holds up seven others instead of fifteen:
+// Chung-Lu 2^24 levels 9.6 against 10.9 ms, Erdos-Renyi 10^6 0.66 against 1.08).
+static uint32_t default_block(const dsg_graph* g, int kernel) {
+    if (kernel != 0) return 256;
+    return g->n >= (1u << 19) ? 1024 : 512;
+}
+
 Tuning tuning_for(const dsg_graph* g, int kernel) {
     if (g_forced) return *g_forced;
     Tuning base = current_tuning();
     std::lock_guard<std::mutex> lk(g_tune_mu);
+    if (!g_block_given) base.block = default_block(g, kernel);
     ensure_table_loaded_locked();
     if (g_table.empty()) return base;
     auto it = g_table.find(class_key(g, kernel));
@@ -346,8 +364,7 @@ extern "C" dsg_status dsg_autotune(const dsg_graph* g, uint32_t eps_num, uint32_
         };
         const Knob peel_knobs[] = {{&Tuning::block, {256, 512, 1024}, 3},
                                    {&Tuning::hot_deg, {0, 1024, 4096, 16384}, 4},
-                                   {&Tuning::chunk_len, {128, 256, 1024}, 3},
-                                   {&Tuning::short_max, {16, 32, 64}, 3}};
+                                   {&Tuning::chunk_len, {128, 256, 1024}, 3}};
         const Knob core_knobs[] = {{&Tuning::block, {256, 512, 1024}, 3},
                                    {&Tuning::local_max, {256, 1024, 4096}, 3},
                                    {&Tuning::local_work, {4096, 16384, 65536}, 3},
@@ -355,7 +372,7 @@ extern "C" dsg_status dsg_autotune(const dsg_graph* g, uint32_t eps_num, uint32_
                                    {&Tuning::chunk_len, {256, 1024, 2048}, 3},
                                    {&Tuning::tail_max, {0, 16384, 32768, 131072}, 4}};
         const Knob* knobs = kernel == 0 ? peel_knobs : core_knobs;
-        const int nknobs = kernel == 0 ? 4 : 6;
+        const int nknobs = kernel == 0 ? 3 : 6;
         for (int kk = 0; kk < nknobs; ++kk) {
             for (int vi = 0; vi < knobs[kk].count; ++vi) {
                 Tuning cand = best;
