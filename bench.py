@@ -21,6 +21,7 @@ from __future__ import annotations
 import argparse
 import json
 import os
+import re
 import statistics
 import subprocess
 import sys
@@ -291,12 +292,16 @@ def kernel_source_sha(name: str, read=None) -> str:
     import hashlib
     csrc = os.path.join(ROOT, "paper_2103_00154_gb300", "csrc")
     h = hashlib.sha256()
-    for f in KERNEL_SOURCES[name] + ["dsg_kernels.cuh", "dsg_common.cuh"]:
+    files = KERNEL_SOURCES[name] + ["dsg_kernels.cuh", "dsg_common.cuh"]
+    for f in files:
         if read is not None:
             data = read(f)
         else:
             with open(os.path.join(csrc, f), "rb") as fh:
                 data = fh.read()
+        # a file's own headers belong to it (dsg_*.cuh are shared and listed)
+        files += [h_ for h_ in re.findall(r'^#include "([a-z_]+\.cuh)"', data.decode(), re.M)
+                  if not h_.startswith("dsg_") and h_ not in files]
         h.update(code_only(data))
     return h.hexdigest()[:16]
 

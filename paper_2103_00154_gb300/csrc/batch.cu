@@ -7,159 +7,53 @@
 // largest first, so the long ones start early) and solves it alone: the
 // Bahmani peel of Algorithm 1 and, when asked, the core numbers of
 // Algorithm 2's first phase.  A round's (or level's) barrier is the block's
-// __syncthreads, so a graph costs no grid-wide synchronisation; per-graph
-// state lives in the concatenated scratch arrays at the graph's vertex slots.
+// __syncthreads, so a graph costs no grid-wide synchronisation.
+// Graphs that would keep one block busy long after the others are done get a
+// thread-block cluster each instead, from a queue of their own.  Both run the
+// body of the grid-wide peel, the clusters that of the bitwise core-number
+// search too, with the block's or the cluster's barrier between rounds and
+// waves, on a slab of scratch per team.
 #include <algorithm>
 #include <vector>
 
+#include "core_split.cuh"
 #include "dsg_batch.cuh"
 #include "dsg_common.cuh"
 #include "dsg_kernels.cuh"
+#include "peel_body.cuh"
 
 namespace dsg {
-
-constexpr uint32_t kDeadB = 0x80000000u;
-
-template <int TB>
-struct BatchSmem {
-    BlockTile<TB> tile;
-    TileSmem<TB> red;
-    uint64_t u64[4];
-    uint32_t u32[4];
-    uint32_t item;
-};
-
-// Algorithm 1 on one graph by one block.
-template <int TB>
-__device__ void peel_block(const BatchArgs& a, uint32_t g, BatchSmem<TB>& sm) {
-    const uint32_t tid = threadIdx.x;
-    const uint64_t vb = a.slot[g];
-    const uint32_t n = a.gn[g];
-    const uint64_t* off = a.goff[g];
-    const uint32_t* adj = a.gadj[g];
-    uint32_t* st = a.st + vb;
-    uint32_t* alive_a = a.la + vb;
-    uint32_t* alive_b = a.lb + vb;
-    uint32_t* failed = a.lf + vb;
-    const uint64_t p = a.p[g], q = a.q[g];
-    uint64_t S = n, E = n ? (off[n] - off[0]) / 2 : 0;
-    uint64_t best_E = E, best_V = S, best_round = 0, r = 0;
-    uint64_t sum_S = 0, ndec = 0;  // byte-model counters (thread-local; summed at the end)
-    const uint32_t* alive = nullptr;
-    uint32_t* next = alive_a;
-    while (S > 0) {
-        // one thread divides for the block: the division is a few hundred instructions
-        if (tid == 0) sm.u32[1] = peel_threshold(p, q, E, S);
-        __syncthreads();
-        const uint32_t T = sm.u32[1];
-        const uint32_t mark = kDeadB | (uint32_t)(r + 1);
-        uint32_t nf = 0, ns = 0;
-        if (tid == 0) sum_S += S;
-        // part 1: test every alive vertex against the round-start degrees
-        for (uint64_t t = 0; t < S; t += TB) {
-            uint64_t i = t + tid;
-            bool valid = i < S, fail = false;
-            uint32_t v = 0;
-            if (valid) {
-                uint32_t d;
-                if (r == 0) {
-                    v = (uint32_t)i;
-                    d = (uint32_t)(off[v + 1] - off[v]);
-                } else {
-                    v = alive[i];
-                    d = st[v];
-                }
-                fail = d <= T;
-                if (fail) st[v] = mark;
-                else if (r == 0) st[v] = d;
-            }
-            uint64_t tot;
-            uint64_t pk = (uint64_t)(valid && fail) | ((uint64_t)(valid && !fail) << 32);
-            uint64_t pre = block_excl_scan<uint64_t>(pk, sm.red.scan_tmp64, &tot);
-            if (valid && fail) failed[nf + (uint32_t)pre] = v;
-            if (valid && !fail) next[ns + (uint32_t)(pre >> 32)] = v;
-            nf += (uint32_t)tot;
-            ns += (uint32_t)(tot >> 32);
-        }
-        __syncthreads();
-        // part 2: remove the failed vertices' edges
-        uint64_t dE = 0;
-        auto visit = [&](const uint32_t* u, const uint32_t* v, uint32_t valid) {
-            uint32_t w[kBatch];
-#pragma unroll
-            for (uint32_t j = 0; j < kBatch; ++j) w[j] = (valid >> j & 1u) ? st[u[j]] : kDeadB;
-#pragma unroll
-            for (uint32_t j = 0; j < kBatch; ++j) {
-                if (!(valid >> j & 1u)) continue;
-                if (!(w[j] & kDeadB)) {
-                    atomicSub(&st[u[j]], 1u);
-                    ++dE;
-                    ++ndec;
-                } else if (w[j] == mark && u[j] > v[j]) {
-                    ++dE;
-                }
-            }
-        };
-        scan_block_list<TB>(off, adj, failed, 0, nf, sm.tile, visit);
-        dE = block_sum<uint64_t>(dE, sm.red.scan_tmp64);
-        ++r;
-        S -= nf;
-        E -= dE;
-        if (S > 0 && (unsigned __int128)E * best_V > (unsigned __int128)best_E * S) {
-            best_round = r;
-            best_E = E;
-            best_V = S;
-        }
-        alive = next;
-        next = (next == alive_a) ? alive_b : alive_a;
-    }
-    if (a.stats) {
-        ndec = warp_sum(ndec);
-        if ((tid & 31u) == 0 && ndec) atomicAdd(&a.stats[1], (unsigned long long)ndec);
-        if (tid == 0) {
-            atomicAdd(&a.stats[0], (unsigned long long)sum_S);
-            atomicAdd(&a.stats[2], (unsigned long long)(n ? off[n] - off[0] : 0));
-        }
-    }
-    if (tid == 0) {
-        a.res[4 * (uint64_t)g + 0] = n ? best_E : 0;
-        a.res[4 * (uint64_t)g + 1] = n ? best_V : 0;
-        a.res[4 * (uint64_t)g + 2] = r;
-        a.res[4 * (uint64_t)g + 3] = best_round;
-    }
-    if (a.out_set)
-        for (uint32_t v = tid; v < n; v += TB) a.out_set[vb + v] = (st[v] & ~kDeadB) > best_round ? 1 : 0;
-    __syncthreads();
-}
 
 // Algorithm 2, first phase, on one graph by one block: level k collects the
 // remaining vertices of degree k, then drains them (atomicSub on every
 // neighbour; a == k+1 joins the level; a <= k is undone, so a vertex already
 // at or below k never reads k+1 again); the level's frontier is one FIFO in
-// global memory with a shared-memory cursor.
+// global memory with a shared-memory cursor.  One block alone reads every row
+// once here; the bitwise search reads it about seven times, which pays only
+// where its waves are spread over several blocks (600 graphs of 1,000 to
+// 100,000 vertices with core numbers: 7.2 ms against 14.1 ms).
 template <int TB>
-__device__ void kcore_block(const BatchArgs& a, uint32_t g, BatchSmem<TB>& sm) {
+struct LevelSmem {
+    BlockTile<TB> tile;
+    uint32_t scan_tmp[33];
+    uint32_t cursor;
+};
+
+template <int TB>
+__device__ void kcore_block(uint32_t n, const uint64_t* off, const uint32_t* adj, uint32_t* deg, uint32_t* rem_a,
+                            uint32_t* rem_b, uint32_t* Q, LevelSmem<TB>& sm) {
     const uint32_t tid = threadIdx.x;
-    const uint64_t vb = a.slot[g];
-    const uint32_t n = a.gn[g];
-    const uint64_t* off = a.goff[g];
-    const uint32_t* adj = a.gadj[g];
-    uint32_t* deg = a.core + vb;
-    uint32_t* rem_a = a.la + vb;
-    uint32_t* rem_b = a.lb + vb;
-    uint32_t* Q = a.lf + vb;
-    if (n == 0) return;
     uint32_t mn = 0xffffffffu;
     for (uint32_t v = tid; v < n; v += TB) {
         uint32_t d = (uint32_t)(off[v + 1] - off[v]);
         deg[v] = d;
         mn = min(mn, d);
     }
-    uint32_t k = block_min_u32(mn, sm.red.scan_tmp);
+    uint32_t k = block_min_u32(mn, sm.scan_tmp);
     const uint32_t* rem = nullptr;
     uint32_t* rem_next = rem_a;
     uint32_t rem_n = n, visited = 0;
-    if (tid == 0) sm.u32[0] = 0;  // FIFO cursor
+    if (tid == 0) sm.cursor = 0;  // FIFO cursor
     __syncthreads();
     for (;;) {
         uint32_t kept = 0, mnext = 0xffffffffu;
@@ -170,19 +64,19 @@ __device__ void kcore_block(const BatchArgs& a, uint32_t g, BatchSmem<TB>& sm) {
             if (i < rem_n) {
                 v = rem ? rem[i] : i;
                 uint32_t d = deg[v];
-                if (d == k) Q[atomicAdd(&sm.u32[0], 1u)] = v;
+                if (d == k) Q[atomicAdd(&sm.cursor, 1u)] = v;
                 else if (d > k) {
                     keep = true;
                     mnext = min(mnext, d);
                 }
             }
             uint32_t tot;
-            uint32_t pre = block_excl_scan<uint32_t>(keep ? 1u : 0u, sm.red.scan_tmp, &tot);
+            uint32_t pre = block_excl_scan<uint32_t>(keep ? 1u : 0u, sm.scan_tmp, &tot);
             if (keep) rem_next[kept + pre] = v;
             kept += tot;
         }
         __syncthreads();
-        uint32_t q_lo = visited, q_hi = sm.u32[0];
+        uint32_t q_lo = visited, q_hi = sm.cursor;
         __syncthreads();
         while (q_lo < q_hi) {
             // every neighbour loses one degree at once (no read first); one
@@ -198,19 +92,19 @@ __device__ void kcore_block(const BatchArgs& a, uint32_t g, BatchSmem<TB>& sm) {
 #pragma unroll
                 for (uint32_t j = 0; j < kBatch; ++j) {
                     if (!(need >> j & 1u)) continue;
-                    if (old[j] == k + 1) Q[atomicAdd(&sm.u32[0], 1u)] = u[j];
+                    if (old[j] == k + 1) Q[atomicAdd(&sm.cursor, 1u)] = u[j];
                     else if (old[j] <= k) atomicAdd(&deg[u[j]], 1u);
                     else mnext = min(mnext, old[j] - 1);
                 }
             };
             scan_block_list<TB>(off, adj, Q, q_lo, q_hi, sm.tile, visit);
             q_lo = q_hi;
-            q_hi = sm.u32[0];
+            q_hi = sm.cursor;
             __syncthreads();
         }
         visited = q_hi;
         if (visited >= n) break;
-        k = block_min_u32(mnext, sm.red.scan_tmp);
+        k = block_min_u32(mnext, sm.scan_tmp);
         if (k == 0xffffffffu) break;
         rem_n = kept;
         rem = rem_next;
@@ -219,57 +113,308 @@ __device__ void kcore_block(const BatchArgs& a, uint32_t g, BatchSmem<TB>& sm) {
     __syncthreads();
 }
 
+// Blocks of a cluster: 16 while there are at most kFewGraphs graphs (8 graphs of
+// 100,000 to 300,000 vertices with core numbers 2.9 against 4.5 ms), else 8,
+// of which 15 clusters fit the GPU against 7 (60 graphs to 300,000 vertices
+// 5.0 against 5.6 ms).
+constexpr uint32_t kClusterBlocks = 8, kClusterBlocksFew = 16, kFewGraphs = 14;
+constexpr uint32_t kClusterTB = 1024;
+
+struct BatchKernelArgs {
+    BatchArgs b;
+    unsigned char* slabs;  // after the error word, one slab per team
+    uint64_t slab;         // bytes of one
+    // offsets inside a slab (the peel's arrays and the search's share the space)
+    uint64_t o_listA, o_listB, o_items, o_map;
+    uint64_t o_ds, o_key, o_pieces, o_queue;
+    uint64_t cap;          // row pieces of the largest graph
+    uint32_t chunk_len;
+    uint32_t size;         // blocks of a team
+};
+
 template <int TB>
-__global__ void __launch_bounds__(TB) batch_kernel(BatchArgs a) {
+struct BatchSmem {
+    union {
+        PeelSmem<TB> peel;
+        SplitSmem<TB> split;
+        LevelSmem<TB> level;
+    };
+    union {  // the running graph's arguments: read from here, not held in registers
+        PeelArgs pargs;
+        SplitArgs sargs;
+    };
+    PeelCtl pctl;
+    SplitCtl sctl;
+    uint32_t item;
+};
+
+__device__ __forceinline__ uint32_t cluster_rank() {
+    uint32_t r;
+    asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+    return r;
+}
+
+// p, as the address of the same object in block 0 of the cluster.
+template <class T>
+__device__ __forceinline__ T* at_block0(T* p) {
+    uint64_t q;
+    asm("mapa.u64 %0, %1, 0;" : "=l"(q) : "l"(reinterpret_cast<uint64_t>(p)));
+    return reinterpret_cast<T*>(q);
+}
+
+// The two bodies as functions of their own: inlined into one kernel they spill
+// each other's registers.
+template <int TB, bool CL>
+__device__ __noinline__ PeelOut team_peel(const PeelArgs& a, PeelSmem<TB>& sm, uint32_t rank, uint32_t size) {
+    return peel_body<TB, CL>(a, Team<CL>{rank, size, a.ctl->bar, &a.ctl->err, 0, {}}, sm);
+}
+template <int TB, bool CL>
+__device__ __noinline__ void team_split(const SplitArgs& a, SplitSmem<TB>& sm, uint32_t rank, uint32_t size) {
+    split_body<TB, CL>(a, Team<CL>{rank, size, a.ctl->bar, &a.ctl->err, 0, {}}, sm);
+}
+
+// A team -- one block, or (CL) a cluster -- takes graphs from
+// the queue until none is left: Algorithm 1, then the core numbers if asked.
+// What bounds it: as the grid-wide kernels, L2 gathers in the wide waves and
+// dependent round trips in the thin ones, but a meeting is the block's barrier
+// or the cluster's and two accesses to a neighbour's shared memory.
+template <int TB, bool CL>
+__global__ void __launch_bounds__(TB, 1024 / TB) batch_kernel(BatchKernelArgs c) {
     __shared__ BatchSmem<TB> sm;
+    const BatchArgs& b = c.b;
+    const uint32_t size = CL ? c.size : 1;
+    const uint32_t tid = threadIdx.x, rank = CL ? cluster_rank() : 0;
+    PeelCtl* const pctl = CL ? at_block0(&sm.pctl) : &sm.pctl;
+    SplitCtl* const sctl = CL ? at_block0(&sm.sctl) : &sm.sctl;
+    uint32_t* const item0 = CL ? at_block0(&sm.item) : &sm.item;
+    unsigned char* const slab = c.slabs + 256 + (uint64_t)(blockIdx.x / size) * c.slab;
+    uint32_t* const err = reinterpret_cast<uint32_t*>(c.slabs);
+    auto sync = [] {
+        if constexpr (CL) cluster_sync();
+        else __syncthreads();
+    };
     for (;;) {
-        if (threadIdx.x == 0) sm.item = (uint32_t)atomicAdd(a.next, 1ull);
+        if (rank == 0) {
+            static_assert(sizeof(PeelCtl) % 4 == 0 && sizeof(SplitCtl) % 4 == 0, "cleared word by word");
+            for (uint32_t i = tid; i < sizeof(PeelCtl) / 4; i += TB) reinterpret_cast<uint32_t*>(&sm.pctl)[i] = 0;
+            for (uint32_t i = tid; i < sizeof(SplitCtl) / 4; i += TB) reinterpret_cast<uint32_t*>(&sm.sctl)[i] = 0;
+            if (tid == 0) sm.item = (uint32_t)min(atomicAdd(b.next, 1ull), (unsigned long long)b.G);
+        }
+        sync();
+        const uint32_t item = ld_volatile_u32(item0);
+        if (item >= b.G) break;
+        const uint32_t g = b.order[item];
+        const uint64_t vb = b.slot[g];
+        const uint32_t n = b.gn[g];
+        const uint64_t* off = b.goff[g];
+        if (tid == 0) {
+            PeelArgs& a = sm.pargs;
+            a.n = n;
+            a.m = n ? (off[n] - off[0]) / 2 : 0;
+            a.p = b.p[g];
+            a.q = b.q[g];
+            a.off = off;
+            a.adj = b.gadj[g];
+            a.st = reinterpret_cast<uint32_t*>(slab);
+            a.listA = reinterpret_cast<uint32_t*>(slab + c.o_listA);
+            a.listB = reinterpret_cast<uint32_t*>(slab + c.o_listB);
+            a.items = reinterpret_cast<uint64_t*>(slab + c.o_items);
+            a.map = reinterpret_cast<uint32_t*>(slab + c.o_map);
+            a.candA = a.candB = nullptr;
+            a.hist_S = a.hist_E = nullptr;
+            a.hist_cap = ~0ull;
+            a.ctl = pctl;
+            a.limit_ns = 0;
+            a.chunk_len = c.chunk_len;
+            a.hot_deg = b.hot_deg;
+            a.trace = nullptr;
+            a.trace_cap = 0;
+            a.r0 = a.S0 = a.E0 = a.best_round0 = a.best_E0 = a.best_V0 = a.max_rounds = 0;
+        }
         __syncthreads();
-        const uint32_t item = sm.item;
-        __syncthreads();
-        if (item >= a.G) break;
-        const uint32_t g = a.order[item];
-        peel_block<TB>(a, g, sm);
-        if (a.core && (!a.want_core || a.want_core[g])) kcore_block<TB>(a, g, sm);
+        {
+            const PeelOut o = team_peel<TB, CL>(sm.pargs, sm.peel, rank, size);
+            if (rank == 0 && tid == 0) {
+                b.res[4 * (uint64_t)g + 0] = n ? o.best_E : 0;
+                b.res[4 * (uint64_t)g + 1] = n ? o.best_V : 0;
+                b.res[4 * (uint64_t)g + 2] = o.rounds;
+                b.res[4 * (uint64_t)g + 3] = o.best_round;
+                if (b.stats) {
+                    atomicAdd(&b.stats[0], pctl->tested);
+                    atomicAdd(&b.stats[1], pctl->dec);
+                    atomicAdd(&b.stats[2], (unsigned long long)(2 * sm.pargs.m));
+                }
+                if (pctl->err) atomicOr(err, pctl->err);
+            }
+            if (b.out_set) {
+                const uint32_t* st = reinterpret_cast<const uint32_t*>(slab);
+                for (uint32_t v = rank * TB + tid; v < n; v += size * TB)
+                    b.out_set[vb + v] = (__ldcg(st + v) & ~kDead) > o.best_round ? 1 : 0;
+            }
+        }
+        sync();  // the peel's arrays and arguments are read before the search takes their place
+        if (b.core && (!b.want_core || b.want_core[g]) && n) {
+            if constexpr (CL) {
+                if (tid == 0) {
+                    SplitArgs& a = sm.sargs;
+                    a.r = n;
+                    a.lo = 0;
+                    a.off = off;
+                    a.adj = b.gadj[g];
+                    a.rid = nullptr;
+                    a.d = reinterpret_cast<uint32_t*>(slab);
+                    a.ds = reinterpret_cast<uint32_t*>(slab + c.o_ds);
+                    a.key = reinterpret_cast<uint32_t*>(slab + c.o_key);
+                    a.kstride = ((uint64_t)n + 63) & ~uint64_t(63);
+                    a.pieces = reinterpret_cast<uint4*>(slab + c.o_pieces);
+                    a.queue = reinterpret_cast<uint4*>(slab + c.o_queue);
+                    a.cap = c.cap;
+                    a.core = b.core + vb;
+                    a.ctl = sctl;
+                    a.limit_ns = 0;
+                    a.trace = nullptr;
+                    a.trace_cap = 0;
+                }
+                __syncthreads();
+                team_split<TB, CL>(sm.sargs, sm.split, rank, size);
+                sync();  // its keys are read, its counters written
+                if (rank == 0 && tid == 0 && sctl->err) atomicOr(err, sctl->err);
+                __syncthreads();
+            } else {
+                kcore_block<TB>(n, off, b.gadj[g], b.core + vb, reinterpret_cast<uint32_t*>(slab),
+                                reinterpret_cast<uint32_t*>(slab + c.o_listA),
+                                reinterpret_cast<uint32_t*>(slab + c.o_listB), sm.level);
+            }
+        }
     }
+    sync();  // no block leaves while another reads block 0's shared memory
+}
+
+// The slab layout for graphs of at most n_max vertices and e_max row entries.
+static BatchKernelArgs batch_layout(const BatchArgs& b, uint32_t n_max, uint64_t e_max, bool search) {
+    BatchKernelArgs c = {};
+    c.b = b;
+    c.chunk_len = 256;
+    uint64_t o = 0;
+    auto carve = [&](uint64_t bytes) { const uint64_t at = o; o += (bytes + 255) & ~uint64_t(255); return at; };
+    const uint64_t n = n_max;
+    carve(4 * n);  // the peel's states (a block's level lists: this and the two after it)
+    c.o_listA = carve(4 * n);
+    c.o_listB = carve(4 * n);
+    c.o_items = carve(8 * (n + e_max / c.chunk_len + 1));
+    c.o_map = carve((n + 15) / 16 * 4);
+    c.slab = o;
+    if (b.core && search) {
+        o = 0;
+        c.cap = n + e_max / kPiece + 1;
+        carve(4 * n);  // the search's degrees
+        c.o_ds = carve(4 * n);
+        c.o_key = carve(4 * ((n + 63) & ~uint64_t(63)) * split_key_buffers(e_max));
+        c.o_pieces = carve(16 * c.cap);
+        c.o_queue = carve(16 * c.cap);
+        c.slab = std::max(c.slab, o);
+    }
+    c.slab = std::max<uint64_t>(c.slab, 256);
+    return c;
+}
+
+// Scratch for `teams` teams (fewer if they would take more than scratch_max bytes), cleared error word.
+static cudaError_t batch_slabs(BatchKernelArgs& c, uint64_t* teams, size_t scratch_max, cudaStream_t s, void** slabs) {
+    *teams = std::max<uint64_t>(1, std::min<uint64_t>(*teams, scratch_max / c.slab));
+    void* p = nullptr;
+    cudaError_t e = dev_alloc(&p, 256 + *teams * c.slab, s);
+    if (e != cudaSuccess) return e;
+    *slabs = p;
+    c.slabs = static_cast<unsigned char*>(p);
+    return cudaMemsetAsync(p, 0, 256, s);
 }
 
 template <int TB>
-static cudaError_t batch_launch_tb(const BatchArgs& a, cudaStream_t s, uint32_t max_grid) {
+static uint32_t slots_tb() {
     int per_sm = 0;
-    cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, batch_kernel<TB>, TB, 0);
-    if (e != cudaSuccess) return e;
-    uint32_t slots = (uint32_t)(per_sm > 0 ? per_sm : 1) * (uint32_t)dev_info().sms;
-    if (max_grid && slots > max_grid) slots = max_grid;
-    uint32_t grid = slots < a.G ? slots : a.G;
-    LaunchScope ls("batch_solve", s);
-    batch_kernel<TB><<<grid, TB, 0, s>>>(a);
-    return cudaGetLastError();
-}
-
-cudaError_t batch_launch(const BatchArgs& a, cudaStream_t s, uint32_t block, uint32_t max_grid) {
-    if (a.G == 0) return cudaSuccess;
-    switch (block) {
-        case 256: return batch_launch_tb<256>(a, s, max_grid);
-        case 1024: return batch_launch_tb<1024>(a, s, max_grid);
-        default: return batch_launch_tb<512>(a, s, max_grid);
-    }
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, batch_kernel<TB, false>, TB, 0) != cudaSuccess ||
+        per_sm < 1)
+        per_sm = 1;
+    return (uint32_t)per_sm * (uint32_t)dev_info().sms;
 }
 
 // Block slots of the block-per-graph kernel at `block` threads.
 static uint32_t batch_slots(uint32_t block) {
-    int per_sm = 0;
-    cudaError_t e;
     switch (block) {
-        case 256: e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, batch_kernel<256>, 256, 0); break;
-        case 1024: e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, batch_kernel<1024>, 1024, 0); break;
-        default: e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, batch_kernel<512>, 512, 0); break;
+        case 256: return slots_tb<256>();
+        case 1024: return slots_tb<1024>();
+        default: return slots_tb<512>();
     }
-    if (e != cudaSuccess || per_sm < 1) per_sm = 1;
-    return (uint32_t)per_sm * (uint32_t)dev_info().sms;
 }
 
 uint32_t batch_slots_for(uint32_t block) { return batch_slots(block); }
+
+cudaError_t batch_launch(const BatchArgs& a, uint32_t n_max, uint64_t e_max, size_t scratch_max, cudaStream_t s,
+                         void** slabs, uint32_t block, uint32_t max_grid) {
+    BatchKernelArgs c = batch_layout(a, n_max, e_max, false);
+    uint64_t teams = std::min<uint64_t>(batch_slots(block), a.G);
+    if (max_grid) teams = std::min<uint64_t>(teams, max_grid);
+    cudaError_t e = batch_slabs(c, &teams, scratch_max, s, slabs);
+    if (e != cudaSuccess) return e;
+    const uint32_t grid = (uint32_t)teams;
+    LaunchScope ls("batch_solve", s);
+    switch (block) {
+        case 256: batch_kernel<256, false><<<grid, 256, 0, s>>>(c); break;
+        case 1024: batch_kernel<1024, false><<<grid, 1024, 0, s>>>(c); break;
+        default: batch_kernel<512, false><<<grid, 512, 0, s>>>(c); break;
+    }
+    return cudaGetLastError();
+}
+
+cudaError_t batch_cluster_launch(const BatchArgs& a, uint32_t n_max, uint64_t e_max, size_t scratch_max, cudaStream_t s,
+                                 void** slabs, uint32_t max_sms) {
+    BatchKernelArgs c = batch_layout(a, n_max, e_max, true);
+    // (only the attribute's failure, not its value, is of interest: without it 8 blocks still fit)
+    const bool few = a.G <= kFewGraphs && cudaFuncSetAttribute(batch_kernel<kClusterTB, true>,
+                                                              cudaFuncAttributeNonPortableClusterSizeAllowed,
+                                                              1) == cudaSuccess;
+    c.size = few ? kClusterBlocksFew : kClusterBlocks;
+    cudaLaunchConfig_t cfg = {};
+    cfg.blockDim = dim3(kClusterTB);
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = c.size;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    cfg.gridDim = dim3(c.size);
+    int fit = 0;
+    cudaError_t e = cudaOccupancyMaxActiveClusters(&fit, batch_kernel<kClusterTB, true>, &cfg);
+    if (e != cudaSuccess) return e;
+    uint64_t teams = std::min<uint64_t>(fit > 0 ? fit : 1, a.G);
+    if (max_sms) teams = std::min<uint64_t>(teams, std::max<uint32_t>(1, max_sms / c.size));
+    e = batch_slabs(c, &teams, scratch_max, s, slabs);
+    if (e != cudaSuccess) return e;
+    cfg.gridDim = dim3((uint32_t)teams * c.size);
+    LaunchScope ls("batch_clusters", s);
+    return cudaLaunchKernelEx(&cfg, batch_kernel<kClusterTB, true>, c);
+}
+
+// A cluster for a graph of more than twice a block's share of the batch (it
+// would be the last to end; at one share the clusters hold SMs that the blocks
+// use better: 600 graphs with core numbers 7.2 against 9.2 ms) and of more than
+// 2^17 units of work (40 graphs of 3,000 to 35,000 vertices: 0.44 ms against
+// 0.53 from 2^15 and 0.69 from 2^18).  The whole GPU for one that is more than
+// a quarter of the batch (8 graphs of 100,000 to 300,000 vertices: all in
+// clusters 4.4 ms, three of them on the whole GPU first 5.7) or too large for
+// the search to take it whole.
+void batch_classes(const uint64_t* work, const uint32_t* n, uint32_t G, uint32_t* grid, uint32_t* cluster) {
+    uint64_t total = 0;
+    for (uint32_t i = 0; i < G; ++i) total += work[i];
+    const uint64_t share = total / batch_slots(512);
+    uint32_t k = 0;
+    while (k < G && ((work[k] > (1u << 20) && work[k] > total / 4) || n[k] > kTailWhole * 65536)) ++k;
+    *grid = k;
+    while (k < G && work[k] > (1u << 17) && work[k] > 2 * share) ++k;
+    *cluster = k;
+}
 
 // want_core[g] read from host or device memory.
 static bool host_want_core(const uint8_t* want_core, uint32_t g, cudaStream_t s) {
@@ -303,6 +448,29 @@ __global__ void gather_ends_kernel(const uint64_t* __restrict__ off, const uint6
                                    uint64_t* __restrict__ ends) {
     const uint32_t g = blockIdx.x * blockDim.x + threadIdx.x;
     if (g < G1) ends[g] = off[vb[g]];
+}
+
+// A second stream and two events per calling thread and device, made once.
+struct BatchSide {
+    int device = -1;
+    cudaStream_t s = nullptr;
+    cudaEvent_t fork = nullptr, join = nullptr;
+};
+
+static cudaError_t batch_side(BatchSide** out) {
+    static thread_local BatchSide cache[16];
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    BatchSide& b = cache[dev & 15];
+    if (b.device != dev) {
+        if ((e = cudaStreamCreateWithFlags(&b.s, cudaStreamNonBlocking)) != cudaSuccess) return e;
+        if ((e = cudaEventCreateWithFlags(&b.fork, cudaEventDisableTiming)) != cudaSuccess) return e;
+        if ((e = cudaEventCreateWithFlags(&b.join, cudaEventDisableTiming)) != cudaSuccess) return e;
+        b.device = dev;
+    }
+    *out = &b;
+    return cudaSuccess;
 }
 
 }  // namespace dsg
@@ -396,10 +564,6 @@ extern "C" dsg_status dsg_batch_solve(const dsg_batch* b, dsg_batch_result* r, v
     DSG_TRY_CUDA(sc.get(&d_order, G));
     DSG_TRY_CUDA(copy_any(d_order, order.data(), G * sizeof(uint32_t), s));
     a.order = d_order;
-    DSG_TRY_CUDA(sc.get(&a.st, N ? N : 1));
-    DSG_TRY_CUDA(sc.get(&a.la, N ? N : 1));
-    DSG_TRY_CUDA(sc.get(&a.lb, N ? N : 1));
-    DSG_TRY_CUDA(sc.get(&a.lf, N ? N : 1));
     bool core_direct = r->core && is_device_ptr(r->core);
     bool set_direct = r->out_set && is_device_ptr(r->out_set);
     a.core = nullptr;
@@ -420,15 +584,11 @@ extern "C" dsg_status dsg_batch_solve(const dsg_batch* b, dsg_batch_result* r, v
     DSG_TRY_CUDA(sc.get(&a.res, 4 * (size_t)G));
     DSG_TRY_CUDA(sc.get(&a.next, 1));
     DSG_TRY_CUDA(cudaMemsetAsync(a.next, 0, sizeof(unsigned long long), s));
-    // Scheduling: a graph whose work is well above one block's share of the
-    // batch would alone set the batch's makespan, so it is solved first by
-    // the grid-wide kernels; the rest share one block-per-graph launch.
     uint64_t total_work = 0;
     for (uint32_t g = 0; g < G; ++g) total_work += work(g);
     const Tuning tu = tuning_for_batch(G, total_work);
     a.hot_deg = tu.hot_deg;
     const uint32_t block = tu.batch_block ? tu.batch_block : 512;
-    const uint32_t slots = batch_slots(block);
     unsigned long long* d_stats = nullptr;
     if (r->stats) {
         DSG_TRY_CUDA(sc.get(&d_stats, 3));
@@ -436,12 +596,20 @@ extern "C" dsg_status dsg_batch_solve(const dsg_batch* b, dsg_batch_result* r, v
     }
     a.stats = d_stats;
     uint64_t big_sum_S = 0, big_dec = 0, big_entries = 0;
-    const uint64_t share = total_work / slots;
-    uint32_t nbig = 0;
-    if (tu.batch_split)
+    // which graphs run on the whole GPU one after the other, which get a cluster, which a block
+    uint32_t nbig = 0, ncl = 0;
+    if (tu.batch_split) {
         while (nbig < G && work(order[nbig]) > tu.batch_split) ++nbig;
-    else
-        while (nbig < G && work(order[nbig]) > 2 * share && work(order[nbig]) > (1u << 20)) ++nbig;
+        ncl = nbig;
+    } else {
+        std::vector<uint64_t> w(G);
+        std::vector<uint32_t> wn(G);
+        for (uint32_t i = 0; i < G; ++i) {
+            w[i] = work(order[i]);
+            wn[i] = (uint32_t)(vb[order[i] + 1] - vb[order[i]]);
+        }
+        batch_classes(w.data(), wn.data(), G, &nbig, &ncl);
+    }
     std::vector<uint64_t> res(4 * (size_t)G, 0);
     for (uint32_t i = 0; i < nbig; ++i) {
         const uint32_t g = order[i];
@@ -466,16 +634,59 @@ extern "C" dsg_status dsg_batch_solve(const dsg_batch* b, dsg_batch_result* r, v
             if (st != DSG_OK) return st;
         }
     }
-    const uint32_t nsmall = G - nbig;
-    a.order = d_order + nbig;
-    a.G = nsmall;
-    if (nsmall) DSG_TRY_CUDA(batch_launch(a, s, block));
-    DSG_TRY_CUDA(cudaGetLastError());
+    // clusters and blocks run side by side: the blocks fill the SMs the clusters leave
+    auto largest = [&](uint32_t lo, uint32_t hi, uint32_t* n_max, uint64_t* e_max) {
+        *n_max = 0;
+        *e_max = 0;
+        for (uint32_t i = lo; i < hi; ++i) {
+            const uint32_t g = order[i];
+            *n_max = std::max<uint32_t>(*n_max, (uint32_t)(vb[g + 1] - vb[g]));
+            *e_max = std::max<uint64_t>(*e_max, hoff_ends[g + 1] - hoff_ends[g]);
+        }
+    };
+    uint32_t n_max = 0, h_err[2] = {0, 0};
+    uint64_t e_max = 0;
+    BatchSide* side = nullptr;
+    void *slabs_cl = nullptr, *slabs_bl = nullptr;
+    if (ncl > nbig) {
+        BatchArgs ca = a;
+        ca.order = d_order + nbig;
+        ca.G = ncl - nbig;
+        DSG_TRY_CUDA(sc.get(&ca.next, 1));
+        DSG_TRY_CUDA(cudaMemsetAsync(ca.next, 0, sizeof(unsigned long long), s));
+        largest(nbig, ncl, &n_max, &e_max);
+        if (ncl < G) {
+            DSG_TRY_CUDA(batch_side(&side));
+            DSG_TRY_CUDA(cudaEventRecord(side->fork, s));
+            DSG_TRY_CUDA(cudaStreamWaitEvent(side->s, side->fork, 0));
+        }
+        const cudaError_t e = batch_cluster_launch(ca, n_max, e_max, SIZE_MAX, s, &slabs_cl);
+        if (slabs_cl) sc.adopt(slabs_cl);
+        DSG_TRY_CUDA(e);
+    }
+    a.order = d_order + ncl;
+    a.G = G - ncl;
+    if (a.G) {
+        largest(ncl, G, &n_max, &e_max);
+        cudaStream_t sb = side ? side->s : s;
+        cudaError_t e = batch_launch(a, n_max, e_max, SIZE_MAX, sb, &slabs_bl, block);
+        if (slabs_bl && e == cudaSuccess)
+            e = cudaMemcpyAsync(&h_err[1], slabs_bl, sizeof(uint32_t), cudaMemcpyDeviceToHost, sb);
+        if (slabs_bl) dev_free(slabs_bl, sb);
+        if (side) {
+            // the caller's stream waits for the blocks whatever became of the launch
+            cudaEventRecord(side->join, sb);
+            cudaStreamWaitEvent(s, side->join, 0);
+        }
+        DSG_TRY_CUDA(e);
+    }
+    if (slabs_cl) DSG_TRY_CUDA(cudaMemcpyAsync(&h_err[0], slabs_cl, sizeof(uint32_t), cudaMemcpyDeviceToHost, s));
     std::vector<uint64_t> res_dev(4 * (size_t)G);
     DSG_TRY_CUDA(cudaMemcpyAsync(res_dev.data(), a.res, res_dev.size() * sizeof(uint64_t), cudaMemcpyDeviceToHost, s));
     if (r->core && !core_direct) DSG_TRY_CUDA(copy_any(r->core, a.core, N * sizeof(uint32_t), s));
     if (r->out_set && !set_direct) DSG_TRY_CUDA(copy_any(r->out_set, a.out_set, N, s));
     DSG_TRY_CUDA(cudaStreamSynchronize(s));
+    if (h_err[0] | h_err[1]) return status_from_err(h_err[0] | h_err[1], "batch");
     for (uint32_t i = nbig; i < G; ++i) {
         const uint32_t g = order[i];
         for (int k = 0; k < 4; ++k) res[4 * (size_t)g + k] = res_dev[4 * (size_t)g + k];

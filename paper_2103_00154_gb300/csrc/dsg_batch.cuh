@@ -17,10 +17,6 @@ struct BatchArgs {
     const uint32_t* q;
     const uint8_t* want_core;
     const uint32_t* order;  // graph ids, largest first
-    uint32_t* st;           // peel state per vertex slot
-    uint32_t* la;           // scratch lists per vertex slot (x3)
-    uint32_t* lb;
-    uint32_t* lf;
     uint32_t* core;         // core numbers per vertex slot (nullable)
     uint8_t* out_set;       // membership in the densest set found (nullable)
     uint64_t* res;          // 4 per graph: E, V, rounds, best_round
@@ -34,8 +30,24 @@ struct BatchArgs {
 // Launch the block-per-graph kernel over a.order[0, a.G) on stream s
 // (asynchronous) with `block` threads per block (256, 512 or 1024; 0: 512),
 // at most max_grid blocks (0: as many as fit).  a.next must be zeroed and
-// every table filled.
-cudaError_t batch_launch(const BatchArgs& a, cudaStream_t s, uint32_t block = 0, uint32_t max_grid = 0);
+// every table filled.  The kernel works on slabs of scratch, one per block,
+// sized by the largest graph (n_max vertices, e_max row entries); at most
+// scratch_max bytes of them, at least one.  *slabs gets them, to be freed by
+// the caller in stream order; the first word is an error word to read when
+// the launch is done.
+cudaError_t batch_launch(const BatchArgs& a, uint32_t n_max, uint64_t e_max, size_t scratch_max, cudaStream_t s,
+                         void** slabs, uint32_t block = 0, uint32_t max_grid = 0);
+
+// The same with a thread-block cluster per graph (on at most max_sms SMs; 0:
+// all), for the graphs too large for a block of their own to keep the launch
+// short.
+cudaError_t batch_cluster_launch(const BatchArgs& a, uint32_t n_max, uint64_t e_max, size_t scratch_max, cudaStream_t s,
+                                 void** slabs, uint32_t max_sms = 0);
+
+// Which graphs of a batch, sorted largest first by work (2m + n), go where:
+// [0, *grid) one at a time on the whole GPU, [*grid, *cluster) a cluster each,
+// the rest a block each.
+void batch_classes(const uint64_t* work, const uint32_t* n, uint32_t G, uint32_t* grid, uint32_t* cluster);
 
 // Blocks of `block` threads the block-per-graph kernel can keep resident on the GPU.
 uint32_t batch_slots_for(uint32_t block);

@@ -76,6 +76,7 @@ struct Scratch {
     ~Scratch() {
         for (int i = 0; i < n; ++i) dev_free(ptrs[i], s);
     }
+    void adopt(void* p) { ptrs[n++] = p; }  // an allocation made elsewhere on the same stream
     template <class T>
     cudaError_t get(T** p, size_t count) {
         void* q = nullptr;
@@ -278,6 +279,12 @@ __device__ __forceinline__ bool wait_flag(const uint32_t* flag, uint32_t* err, u
         }
     }
     return true;
+}
+
+// Barrier of the thread-block cluster: every thread of every block; what any
+// of them wrote before is visible to all after.
+__device__ __forceinline__ void cluster_sync() {
+    asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
 }
 
 // Mask of the lanes below this one.

@@ -157,7 +157,7 @@ __device__ __forceinline__ uint32_t ld_relaxed_u32(const uint32_t* p) {
     return v;
 }
 
-// The blocks of a co-resident grid meet, on a word that also sums a count:
+// Several blocks meet, on a word that also sums a count:
 // low half arrivals, high half the blocks' `mine`.  The grid's sum comes back
 // with the wait, so nothing is read for it afterwards.  Two words take turns:
 // a block that is already on its way to the next meeting must not add to the
@@ -165,7 +165,7 @@ __device__ __forceinline__ uint32_t ld_relaxed_u32(const uint32_t* p) {
 // has to pass the other, which needs the slower block).  The words start at
 // zero.  Every thread of the block calls it; thread 0's `mine` counts.  A wait
 // above limit_ns records ERR_TIMEOUT and clears sm.ok, as does seeing the
-// error of another block.  With one block (nblocks == 1) it is a block barrier.
+// error of another block.  With one block (size == 1) it is a block barrier.
 struct MeetState {
     uint32_t epoch = 0, seen0 = 0, seen1 = 0;
 };
@@ -173,38 +173,56 @@ struct MeetSmem {
     uint32_t got, ok;
 };
 
-__device__ __forceinline__ uint32_t grid_meet(unsigned long long (*bar)[16], uint32_t* err, uint64_t limit_ns,
-                                              uint32_t nblocks, uint32_t mine, MeetState& st, MeetSmem& sm) {
-    __syncthreads();
-    const uint32_t par = st.epoch & 1u;
-    ++st.epoch;
-    if (threadIdx.x == 0) {
-        if (nblocks == 1) {
-            sm.got = mine;
-        } else {
+// The blocks that work on one graph: a co-resident grid (CL = false), or one
+// thread-block cluster (CL = true: the words are in a block's shared memory,
+// the wait is the cluster's barrier).
+template <bool CL>
+struct Team {
+    uint32_t rank, size;  // this block among them, and how many (1: meet is a block barrier)
+    unsigned long long (*bar)[16];
+    uint32_t* err;
+    uint64_t limit_ns;
+    MeetState st;
+
+    __device__ __forceinline__ uint32_t meet(uint32_t mine, MeetSmem& sm) {
+        const uint32_t par = st.epoch & 1u;
+        ++st.epoch;
+        if constexpr (CL) {
             unsigned long long* word = &bar[par][0];
-            const uint32_t target = ((st.epoch + 1) >> 1) * nblocks;  // odd and even meetings have a word each
-            red_add_release_u64(word, (uint64_t)mine << 32 | 1ull);
-            uint64_t w;
-            uint32_t polls = 0;
-            const uint64_t t0 = global_ns();
-            while ((int32_t)((uint32_t)(w = ld_acquire_u64(word)) - target) < 0) {
-                if ((++polls & 63u) == 0) {
-                    if (global_ns() - t0 > limit_ns) atomicOr(err, ERR_TIMEOUT);
-                    if (ld_volatile_u32(err) & ERR_TIMEOUT) {
-                        sm.ok = 0;
-                        break;
+            if (threadIdx.x == 0 && mine) atomicAdd(word, (unsigned long long)mine);
+            cluster_sync();
+            if (threadIdx.x == 0) sm.got = (uint32_t)ld_volatile_u64((const uint64_t*)word) - (par ? st.seen1 : st.seen0);
+        } else {
+            __syncthreads();
+            if (threadIdx.x == 0) {
+                if (size == 1) {
+                    sm.got = mine;
+                } else {
+                    unsigned long long* word = &bar[par][0];
+                    const uint32_t target = ((st.epoch + 1) >> 1) * size;  // odd and even meetings have a word each
+                    red_add_release_u64(word, (uint64_t)mine << 32 | 1ull);
+                    uint64_t w;
+                    uint32_t polls = 0;
+                    const uint64_t t0 = global_ns();
+                    while ((int32_t)((uint32_t)(w = ld_acquire_u64(word)) - target) < 0) {
+                        if ((++polls & 63u) == 0) {
+                            if (global_ns() - t0 > limit_ns) atomicOr(err, ERR_TIMEOUT);
+                            if (ld_volatile_u32(err) & ERR_TIMEOUT) {
+                                sm.ok = 0;
+                                break;
+                            }
+                        }
                     }
+                    sm.got = (uint32_t)(w >> 32) - (par ? st.seen1 : st.seen0);
                 }
             }
-            sm.got = (uint32_t)(w >> 32) - (par ? st.seen1 : st.seen0);
         }
+        __syncthreads();
+        const uint32_t got = sm.got;
+        if (par) st.seen1 += got; else st.seen0 += got;
+        return got;
     }
-    __syncthreads();
-    const uint32_t got = sm.got;
-    if (par) st.seen1 += got; else st.seen0 += got;
-    return got;
-}
+};
 
 // Per-block table that combines degree decrements aimed at the same
 // high-degree vertex, so a hub adjacent to thousands of failing vertices
@@ -215,10 +233,10 @@ constexpr uint32_t kAggBits = 11;
 constexpr uint32_t kAggSlots = 1u << kAggBits;
 constexpr uint32_t kAggEmpty = 0xffffffffu;
 
-// The degree at which combining pays: a vertex takes about deg / gridDim.x
+// The degree at which combining pays: a vertex takes about deg / blocks
 // decrements per block, so combining helps once that is well above one.
-__device__ __forceinline__ uint32_t hot_threshold(uint32_t hot_deg) {
-    return hot_deg ? hot_deg : 4u * gridDim.x;
+__device__ __forceinline__ uint32_t hot_threshold(uint32_t hot_deg, uint32_t blocks) {
+    return hot_deg ? hot_deg : 4u * blocks;
 }
 
 struct AggTable {

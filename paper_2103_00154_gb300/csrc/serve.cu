@@ -6,9 +6,9 @@
 //   worker  (one host thread per server) admits queued requests while their
 //           device-memory charge fits the budget and hands them to the
 //           ingest threads, and whenever one of its max_inflight solve
-//           streams is free launches one block-per-graph launch over
-//           everything ingested so far on that stream; while batches run,
-//           new arrivals keep being admitted and ingested, and form the next
+//           streams is free launches everything ingested so far on that
+//           stream (a cluster of blocks each for the large graphs, a block
+//           each for the rest); while batches run, new arrivals keep being admitted and ingested, and form the next
 //           batch; a finished batch's results are copied out, its graphs
 //           freed and their charge returned to the budget;
 //   ingest  (ingest_threads host threads, each with its own stream) turn
@@ -20,7 +20,7 @@
 //           a batch of small ones back;
 //   poll    waits (bounded) for one ticket's completion.
 // A request's results do not depend on what it is batched with: each graph is
-// solved by its own block with its own state.
+// solved by its own block or cluster with its own state.
 #include <stdlib.h>
 #include <string.h>
 
@@ -77,7 +77,8 @@ struct dsg_server {
     size_t in_use = 0;
     bool stop = false;
     std::thread worker;
-    std::vector<cudaStream_t> s_solve;  // one per batch that may be in flight
+    std::vector<cudaStream_t> s_solve;  // one per batch that may be in flight ...
+    std::vector<cudaStream_t> s_side;   // ... and one for its small graphs beside its large ones
     // ingest threads and the big-request thread
     std::condition_variable cv_ingest, cv_big;
     std::deque<dsg::ServeReq*> to_ingest, big;
@@ -106,12 +107,22 @@ struct Inflight {
     std::vector<ServeReq*> reqs;
     BatchArgs a;
     uint64_t* d_res = nullptr;
-    uint32_t* d_tables = nullptr;  // one allocation for every table and scratch array
+    uint32_t* d_tables = nullptr;  // one allocation for every table and output array
+    void *slabs_cl = nullptr, *slabs_bl = nullptr;  // scratch of the two launches (first word: an error word)
     size_t tables_bytes = 0;
     std::vector<uint64_t> slot;
     uint64_t N = 0;
-    cudaEvent_t start_ev = nullptr, done_ev = nullptr;
+    cudaEvent_t start_ev = nullptr, done_ev = nullptr, fork_ev = nullptr, join_ev = nullptr;
 };
+
+// A batch's device memory and events, after its streams are done with them.
+static void release_batch(Inflight& f, cudaStream_t ss) {
+    for (void* p : {(void*)f.d_tables, f.slabs_cl, f.slabs_bl})
+        if (p) dev_free(p, ss);
+    for (cudaEvent_t e : {f.start_ev, f.done_ev, f.fork_ev, f.join_ev})
+        if (e) cudaEventDestroy(e);
+    f = Inflight();
+}
 
 static void finish_request(dsg_server* s, ServeReq* r, dsg_status st) {
     r->status = st;
@@ -226,8 +237,9 @@ static void big_main(dsg_server* s, cudaStream_t sb) {
     }
 }
 
-// Build the tables of one batch and launch it on the solve stream.
-static dsg_status launch_batch(dsg_server* s, Inflight& f, cudaStream_t ss) {
+// Build the tables of one batch and launch it on the solve stream: a cluster
+// each for its large graphs, a block each for the rest, side by side.
+static dsg_status launch_batch(dsg_server* s, Inflight& f, cudaStream_t ss, cudaStream_t side) {
     const uint32_t G = (uint32_t)f.reqs.size();
     // largest first inside the batch
     std::stable_sort(f.reqs.begin(), f.reqs.end(), [](ServeReq* x, ServeReq* y) {
@@ -243,12 +255,11 @@ static dsg_status launch_batch(dsg_server* s, Inflight& f, cudaStream_t ss) {
     auto carve = [&](size_t bytes) { size_t o = off; off += (bytes + 255) & ~size_t(255); return o; };
     const size_t o_goff = carve(G * sizeof(void*)), o_gadj = carve(G * sizeof(void*)), o_slot = carve(G * 8),
                  o_gn = carve(G * 4), o_p = carve(G * 4), o_q = carve(G * 4), o_wc = carve(G), o_order = carve(G * 4),
-                 o_st = carve(N * 4), o_la = carve(N * 4), o_lb = carve(N * 4), o_lf = carve(N * 4),
-                 o_core = carve(N * 4), o_set = carve(N), o_res = carve(4 * (size_t)G * 8), o_next = carve(8);
+                 o_core = carve(N * 4), o_set = carve(N), o_res = carve(4 * (size_t)G * 8), o_next = carve(16);
     f.tables_bytes = off;
     DSG_TRY_CUDA(dev_alloc((void**)&f.d_tables, off, ss));
     unsigned char* base = reinterpret_cast<unsigned char*>(f.d_tables);
-    std::vector<unsigned char> host(o_st, 0);
+    std::vector<unsigned char> host(o_core, 0);
     auto put = [&](size_t o, const void* src, size_t bytes) { memcpy(host.data() + o, src, bytes); };
     std::vector<const uint64_t*> goff(G);
     std::vector<const uint32_t*> gadj(G);
@@ -272,8 +283,8 @@ static dsg_status launch_batch(dsg_server* s, Inflight& f, cudaStream_t ss) {
     put(o_q, gq.data(), G * 4);
     put(o_wc, wc.data(), G);
     put(o_order, order.data(), G * 4);
-    DSG_TRY_CUDA(cudaMemcpyAsync(base, host.data(), o_st, cudaMemcpyHostToDevice, ss));
-    DSG_TRY_CUDA(cudaMemsetAsync(base + o_next, 0, 8, ss));
+    DSG_TRY_CUDA(cudaMemcpyAsync(base, host.data(), o_core, cudaMemcpyHostToDevice, ss));
+    DSG_TRY_CUDA(cudaMemsetAsync(base + o_next, 0, 16, ss));
     DSG_TRY_CUDA(cudaEventCreate(&f.start_ev));
     DSG_TRY_CUDA(cudaEventRecord(f.start_ev, ss));
     BatchArgs& a = f.a;
@@ -286,10 +297,6 @@ static dsg_status launch_batch(dsg_server* s, Inflight& f, cudaStream_t ss) {
     a.q = reinterpret_cast<const uint32_t*>(base + o_q);
     a.want_core = reinterpret_cast<const uint8_t*>(base + o_wc);
     a.order = reinterpret_cast<const uint32_t*>(base + o_order);
-    a.st = reinterpret_cast<uint32_t*>(base + o_st);
-    a.la = reinterpret_cast<uint32_t*>(base + o_la);
-    a.lb = reinterpret_cast<uint32_t*>(base + o_lb);
-    a.lf = reinterpret_cast<uint32_t*>(base + o_lf);
     a.core = reinterpret_cast<uint32_t*>(base + o_core);
     a.out_set = reinterpret_cast<uint8_t*>(base + o_set);
     a.res = reinterpret_cast<uint64_t*>(base + o_res);
@@ -301,8 +308,45 @@ static dsg_status launch_batch(dsg_server* s, Inflight& f, cudaStream_t ss) {
     const uint32_t sms = (uint32_t)dev_info().sms;
     const uint32_t big_sms =
         s->cfg.big_work == UINT64_MAX ? 0 : (uint32_t)std::min<uint64_t>((uint64_t)s->cfg.big_sms * s->cfg.big_threads, sms - 1);
-    const uint32_t cap = (uint32_t)((uint64_t)batch_slots_for(512) * (sms - big_sms) / sms);
-    DSG_TRY_CUDA(batch_launch(a, ss, 512, cap ? cap : 1));
+    uint32_t grid = 0, ncl = 0;
+    {
+        std::vector<uint64_t> w(G);
+        for (uint32_t i = 0; i < G; ++i) w[i] = 2 * f.reqs[i]->m + f.reqs[i]->n;
+        batch_classes(w.data(), gn.data(), G, &grid, &ncl);  // (none runs on the whole GPU here)
+    }
+    // a launch's scratch stays within what its requests were admitted with
+    auto launch = [&](uint32_t lo, uint32_t hi, bool clusters, cudaStream_t st) {
+        BatchArgs b = a;
+        b.order = a.order + lo;
+        b.G = hi - lo;
+        b.next = a.next + (clusters ? 1 : 0);
+        uint32_t n_max = 0;
+        uint64_t e_max = 0;
+        size_t room = 0;
+        for (uint32_t i = lo; i < hi; ++i) {
+            n_max = std::max(n_max, f.reqs[i]->n);
+            e_max = std::max<uint64_t>(e_max, 2 * f.reqs[i]->m);
+            room += f.reqs[i]->charge;
+        }
+        if (clusters) return batch_cluster_launch(b, n_max, e_max, room, st, &f.slabs_cl, std::max(1u, sms - big_sms));
+        const uint32_t cap = (uint32_t)((uint64_t)batch_slots_for(512) * (sms - big_sms) / sms);
+        return batch_launch(b, n_max, e_max, room, st, &f.slabs_bl, 512, cap ? cap : 1);
+    };
+    cudaError_t e = cudaSuccess;
+    if (ncl == 0 || ncl == G) {
+        e = launch(0, G, ncl == G, ss);
+    } else {
+        DSG_TRY_CUDA(cudaEventCreateWithFlags(&f.fork_ev, cudaEventDisableTiming));
+        DSG_TRY_CUDA(cudaEventCreateWithFlags(&f.join_ev, cudaEventDisableTiming));
+        DSG_TRY_CUDA(cudaEventRecord(f.fork_ev, ss));
+        DSG_TRY_CUDA(cudaStreamWaitEvent(side, f.fork_ev, 0));
+        e = launch(0, ncl, true, ss);
+        if (e == cudaSuccess) e = launch(ncl, G, false, side);
+        // the solve stream waits for the small graphs whatever became of the launches
+        cudaEventRecord(f.join_ev, side);
+        cudaStreamWaitEvent(ss, f.join_ev, 0);
+    }
+    DSG_TRY_CUDA(e);
     DSG_TRY_CUDA(cudaEventCreate(&f.done_ev));
     DSG_TRY_CUDA(cudaEventRecord(f.done_ev, ss));
     // (the pageable staging vector may go: a host-to-device copy from pageable
@@ -314,7 +358,11 @@ static dsg_status launch_batch(dsg_server* s, Inflight& f, cudaStream_t ss) {
 static void complete_batch(dsg_server* s, Inflight& f, cudaStream_t ss) {
     const uint32_t G = (uint32_t)f.reqs.size();
     std::vector<uint64_t> res(4 * (size_t)G);
+    uint32_t err[2] = {0, 0};
     dsg_status st = DSG_OK;
+    if ((f.slabs_cl && cudaMemcpyAsync(&err[0], f.slabs_cl, 4, cudaMemcpyDeviceToHost, ss) != cudaSuccess) ||
+        (f.slabs_bl && cudaMemcpyAsync(&err[1], f.slabs_bl, 4, cudaMemcpyDeviceToHost, ss) != cudaSuccess))
+        st = DSG_ECUDA;
     if (cudaMemcpyAsync(res.data(), f.d_res, res.size() * 8, cudaMemcpyDeviceToHost, ss) != cudaSuccess)
         st = DSG_ECUDA;
     for (uint32_t i = 0; i < G && st == DSG_OK; ++i) {
@@ -328,6 +376,7 @@ static void complete_batch(dsg_server* s, Inflight& f, cudaStream_t ss) {
             st = DSG_ECUDA;
     }
     if (cudaStreamSynchronize(ss) != cudaSuccess) st = DSG_ECUDA;
+    if (st == DSG_OK) st = status_from_err(err[0] | err[1], "serve batch");
     for (uint32_t i = 0; i < G; ++i) {
         ServeReq* r = f.reqs[i];
         for (int k = 0; k < 4; ++k) r->res[k] = res[4 * (size_t)i + k];
@@ -335,10 +384,7 @@ static void complete_batch(dsg_server* s, Inflight& f, cudaStream_t ss) {
     }
     float dev_ms = 0;
     if (cudaEventElapsedTime(&dev_ms, f.start_ev, f.done_ev) != cudaSuccess) dev_ms = 0;
-    dev_free(f.d_tables, ss);
-    cudaEventDestroy(f.start_ev);
-    cudaEventDestroy(f.done_ev);
-    f = Inflight();
+    release_batch(f, ss);
     std::lock_guard<std::mutex> lk(s->mu);
     s->batches++;
     s->batch_dev_ms += dev_ms;
@@ -404,13 +450,12 @@ static void worker_main(dsg_server* s) {
             }
             if (batch.empty()) break;
             fl[k].reqs = batch;
-            dsg_status st = launch_batch(s, fl[k], s->s_solve[k]);
+            dsg_status st = launch_batch(s, fl[k], s->s_solve[k], s->s_side[k]);
             if (st != DSG_OK) {
+                // one of the two launches may be running: its graphs are freed after it
+                cudaStreamSynchronize(s->s_solve[k]);
                 for (ServeReq* r : fl[k].reqs) finish_request(s, r, st);
-                if (fl[k].d_tables) dev_free(fl[k].d_tables, s->s_solve[k]);
-                if (fl[k].start_ev) cudaEventDestroy(fl[k].start_ev);
-                if (fl[k].done_ev) cudaEventDestroy(fl[k].done_ev);
-                fl[k] = Inflight();
+                release_batch(fl[k], s->s_solve[k]);
             } else {
                 running[k] = true;
             }
@@ -461,6 +506,9 @@ dsg_status dsg_serve_create(const dsg_serve_config* cfg, dsg_server** out) {
     s->s_solve.assign(s->cfg.max_inflight, nullptr);
     for (uint32_t k = 0; k < s->cfg.max_inflight && e == cudaSuccess; ++k)
         e = cudaStreamCreateWithFlags(&s->s_solve[k], cudaStreamNonBlocking);
+    s->s_side.assign(s->cfg.max_inflight, nullptr);
+    for (uint32_t k = 0; k < s->cfg.max_inflight && e == cudaSuccess; ++k)
+        e = cudaStreamCreateWithFlags(&s->s_side[k], cudaStreamNonBlocking);
     if (e != cudaSuccess) {
         set_error("serve_create: %s", cudaGetErrorString(e));
         for (cudaStream_t st : s->s_ingest)
@@ -468,6 +516,8 @@ dsg_status dsg_serve_create(const dsg_serve_config* cfg, dsg_server** out) {
         for (cudaStream_t st : s->s_big)
             if (st) cudaStreamDestroy(st);
         for (cudaStream_t st : s->s_solve)
+            if (st) cudaStreamDestroy(st);
+        for (cudaStream_t st : s->s_side)
             if (st) cudaStreamDestroy(st);
         delete s;
         return DSG_ECUDA;
@@ -628,6 +678,8 @@ void dsg_serve_destroy(dsg_server* s) {
     for (cudaStream_t st : s->s_big)
         if (st) cudaStreamDestroy(st);
     for (cudaStream_t st : s->s_solve)
+        if (st) cudaStreamDestroy(st);
+    for (cudaStream_t st : s->s_side)
         if (st) cudaStreamDestroy(st);
     delete s;
 }
