@@ -129,7 +129,6 @@ struct BatchKernelArgs {
     uint64_t o_ds, o_key, o_pieces, o_queue;
     uint64_t cap;          // row pieces of the largest graph
     uint32_t chunk_len;
-    uint32_t size;         // blocks of a team
 };
 
 template <int TB>
@@ -148,29 +147,15 @@ struct BatchSmem {
     uint32_t item;
 };
 
-__device__ __forceinline__ uint32_t cluster_rank() {
-    uint32_t r;
-    asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
-    return r;
-}
-
-// p, as the address of the same object in block 0 of the cluster.
-template <class T>
-__device__ __forceinline__ T* at_block0(T* p) {
-    uint64_t q;
-    asm("mapa.u64 %0, %1, 0;" : "=l"(q) : "l"(reinterpret_cast<uint64_t>(p)));
-    return reinterpret_cast<T*>(q);
-}
-
 // The two bodies as functions of their own: inlined into one kernel they spill
 // each other's registers.
-template <int TB, bool CL>
-__device__ __noinline__ PeelOut team_peel(const PeelArgs& a, PeelSmem<TB>& sm, uint32_t rank, uint32_t size) {
-    return peel_body<TB, CL>(a, Team<CL>{rank, size, a.ctl->bar, &a.ctl->err, 0, {}}, sm);
+template <int TB, uint32_t size>
+__device__ __noinline__ PeelOut team_peel(const PeelArgs& a, PeelSmem<TB>& sm, uint32_t rank) {
+    return peel_body<TB, (size > 1)>(a, Team<(size > 1)>{rank, size, a.ctl->bar, &a.ctl->err, 0, {}}, sm);
 }
-template <int TB, bool CL>
-__device__ __noinline__ void team_split(const SplitArgs& a, SplitSmem<TB>& sm, uint32_t rank, uint32_t size) {
-    split_body<TB, CL>(a, Team<CL>{rank, size, a.ctl->bar, &a.ctl->err, 0, {}}, sm);
+template <int TB, uint32_t size>
+__device__ __noinline__ void team_split(const SplitArgs& a, SplitSmem<TB>& sm, uint32_t rank) {
+    split_body<TB, (size > 1)>(a, Team<(size > 1)>{rank, size, a.ctl->bar, &a.ctl->err, 0, {}}, sm);
 }
 
 // A team -- one block, or (CL) a cluster -- takes graphs from
@@ -178,11 +163,11 @@ __device__ __noinline__ void team_split(const SplitArgs& a, SplitSmem<TB>& sm, u
 // What bounds it: as the grid-wide kernels, L2 gathers in the wide waves and
 // dependent round trips in the thin ones, but a meeting is the block's barrier
 // or the cluster's and two accesses to a neighbour's shared memory.
-template <int TB, bool CL>
+template <int TB, uint32_t size>  // size: blocks of the team
 __global__ void __launch_bounds__(TB, 1024 / TB) batch_kernel(BatchKernelArgs c) {
+    constexpr bool CL = size > 1;
     __shared__ BatchSmem<TB> sm;
     const BatchArgs& b = c.b;
-    const uint32_t size = CL ? c.size : 1;
     const uint32_t tid = threadIdx.x, rank = CL ? cluster_rank() : 0;
     PeelCtl* const pctl = CL ? at_block0(&sm.pctl) : &sm.pctl;
     SplitCtl* const sctl = CL ? at_block0(&sm.sctl) : &sm.sctl;
@@ -233,7 +218,7 @@ __global__ void __launch_bounds__(TB, 1024 / TB) batch_kernel(BatchKernelArgs c)
         }
         __syncthreads();
         {
-            const PeelOut o = team_peel<TB, CL>(sm.pargs, sm.peel, rank, size);
+            const PeelOut o = team_peel<TB, size>(sm.pargs, sm.peel, rank);
             if (rank == 0 && tid == 0) {
                 b.res[4 * (uint64_t)g + 0] = n ? o.best_E : 0;
                 b.res[4 * (uint64_t)g + 1] = n ? o.best_V : 0;
@@ -276,7 +261,7 @@ __global__ void __launch_bounds__(TB, 1024 / TB) batch_kernel(BatchKernelArgs c)
                     a.trace_cap = 0;
                 }
                 __syncthreads();
-                team_split<TB, CL>(sm.sargs, sm.split, rank, size);
+                team_split<TB, size>(sm.sargs, sm.split, rank);
                 sync();  // its keys are read, its counters written
                 if (rank == 0 && tid == 0 && sctl->err) atomicOr(err, sctl->err);
                 __syncthreads();
@@ -332,7 +317,7 @@ static cudaError_t batch_slabs(BatchKernelArgs& c, uint64_t* teams, size_t scrat
 template <int TB>
 static uint32_t slots_tb() {
     int per_sm = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, batch_kernel<TB, false>, TB, 0) != cudaSuccess ||
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, batch_kernel<TB, 1>, TB, 0) != cudaSuccess ||
         per_sm < 1)
         per_sm = 1;
     return (uint32_t)per_sm * (uint32_t)dev_info().sms;
@@ -359,9 +344,9 @@ cudaError_t batch_launch(const BatchArgs& a, uint32_t n_max, uint64_t e_max, siz
     const uint32_t grid = (uint32_t)teams;
     LaunchScope ls("batch_solve", s);
     switch (block) {
-        case 256: batch_kernel<256, false><<<grid, 256, 0, s>>>(c); break;
-        case 1024: batch_kernel<1024, false><<<grid, 1024, 0, s>>>(c); break;
-        default: batch_kernel<512, false><<<grid, 512, 0, s>>>(c); break;
+        case 256: batch_kernel<256, 1><<<grid, 256, 0, s>>>(c); break;
+        case 1024: batch_kernel<1024, 1><<<grid, 1024, 0, s>>>(c); break;
+        default: batch_kernel<512, 1><<<grid, 512, 0, s>>>(c); break;
     }
     return cudaGetLastError();
 }
@@ -369,32 +354,33 @@ cudaError_t batch_launch(const BatchArgs& a, uint32_t n_max, uint64_t e_max, siz
 cudaError_t batch_cluster_launch(const BatchArgs& a, uint32_t n_max, uint64_t e_max, size_t scratch_max, cudaStream_t s,
                                  void** slabs, uint32_t max_sms) {
     BatchKernelArgs c = batch_layout(a, n_max, e_max, true);
-    // (only the attribute's failure, not its value, is of interest: without it 8 blocks still fit)
-    const bool few = a.G <= kFewGraphs && cudaFuncSetAttribute(batch_kernel<kClusterTB, true>,
+    // (16 blocks need leave of the device; without it 8 do)
+    const bool few = a.G <= kFewGraphs && cudaFuncSetAttribute(batch_kernel<kClusterTB, kClusterBlocksFew>,
                                                               cudaFuncAttributeNonPortableClusterSizeAllowed,
                                                               1) == cudaSuccess;
-    c.size = few ? kClusterBlocksFew : kClusterBlocks;
+    const uint32_t size = few ? kClusterBlocksFew : kClusterBlocks;
+    auto* const kernel = few ? batch_kernel<kClusterTB, kClusterBlocksFew> : batch_kernel<kClusterTB, kClusterBlocks>;
     cudaLaunchConfig_t cfg = {};
     cfg.blockDim = dim3(kClusterTB);
     cfg.stream = s;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = c.size;
+    attr[0].val.clusterDim.x = size;
     attr[0].val.clusterDim.y = 1;
     attr[0].val.clusterDim.z = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    cfg.gridDim = dim3(c.size);
+    cfg.gridDim = dim3(size);
     int fit = 0;
-    cudaError_t e = cudaOccupancyMaxActiveClusters(&fit, batch_kernel<kClusterTB, true>, &cfg);
+    cudaError_t e = cudaOccupancyMaxActiveClusters(&fit, kernel, &cfg);
     if (e != cudaSuccess) return e;
     uint64_t teams = std::min<uint64_t>(fit > 0 ? fit : 1, a.G);
-    if (max_sms) teams = std::min<uint64_t>(teams, std::max<uint32_t>(1, max_sms / c.size));
+    if (max_sms) teams = std::min<uint64_t>(teams, std::max<uint32_t>(1, max_sms / size));
     e = batch_slabs(c, &teams, scratch_max, s, slabs);
     if (e != cudaSuccess) return e;
-    cfg.gridDim = dim3((uint32_t)teams * c.size);
+    cfg.gridDim = dim3((uint32_t)teams * size);
     LaunchScope ls("batch_clusters", s);
-    return cudaLaunchKernelEx(&cfg, batch_kernel<kClusterTB, true>, c);
+    return cudaLaunchKernelEx(&cfg, kernel, c);
 }
 
 // A cluster for a graph of more than twice a block's share of the batch (it
