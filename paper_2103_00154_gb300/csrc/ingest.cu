@@ -17,11 +17,14 @@
 //                 each, by a stable LSD radix sort on 8-bit digits
 //   6. scan       final row lengths -> off
 //   7. copy       unique entries into adj
+// Small inputs (at most kDirectPairs pairs) go through all of it in one launch
+// instead (direct_kernel).
 // The result is byte-identical to sorting the (min, max) keys and removing
 // repeats, because a canonical CSR of a given edge set is unique.
 #include <cooperative_groups.h>
 
 #include <algorithm>
+#include <atomic>
 
 #include "dsg_common.cuh"
 #include "dsg_kernels.cuh"
@@ -1266,6 +1269,433 @@ __global__ void expand_rows(uint32_t n, const uint64_t* __restrict__ off, uint32
         for (uint64_t j = off[v] + lane; j < off[v + 1]; j += 32) src[j] = (uint32_t)v;
 }
 
+// ------------------------------------------------------ small inputs, at once
+// One launch, of a thread-block cluster or a co-resident grid, does the whole
+// ingest: the entries' counts and ranks in their rows by returning atomics on
+// the counts (the rank saves a second atomic when the entry is placed), row
+// starts by a scan over the blocks' shares, entries to their rows, rows sorted
+// and de-duplicated (at most 32 entries: several rows a warp; 1,024: a warp
+// each; kDirectRow: a block each), final lengths scanned, unique entries
+// copied out.  The other path's fourteen launches and two waits cost more than
+// all the work here.  What bounds this one: up to about 10^5 pairs its
+// dependent round trips (eight phases of one to three between meetings, 3 to
+// 10 us each), then the atomics on the counts (10^6 uniform pairs: 21 of 110
+// us; with hubs 82 of 230) and the row sorts.
+constexpr uint32_t kDirectTB = 512;
+constexpr uint32_t kDirectBlocks = 16;   // of the cluster
+constexpr uint32_t kDirectGridMax = 512;  // blocks of the grid at most
+constexpr uint32_t kDirectRow = 16 * 1024;  // longest row (repeats counted) a block sorts
+// Pairs at most: above, hubs' counts contend and rows that no block can sort
+// appear (us for this path / the other: Erdos-Renyi 50,000 pairs 73 / 242,
+// 10^6 154 / 356, 8 10^6 765 / 809; Chung-Lu 80,000 118 / 309, 960,000
+// 270 / 466, 4 10^6 764 / 837, 8 10^6 1167 / 1099; R-MAT 131,072 141 / 363,
+// 524,288 217 / 565, 2^21 925 / 865, 2^22 1371 / 1185).
+constexpr uint64_t kDirectPairs = 1500000;
+// Up to here one cluster, above a grid of a block per 1,024 pairs (12,000
+// pairs: 63 against 74 us; 50,000: 96 against 73 us).
+constexpr uint64_t kDirectClusterPairs = 16384;
+
+struct DirectArgs {
+    uint32_t n, m;
+    const uint32_t *src, *dst;
+    uint32_t *cnt, *newlen;          // n each
+    uint64_t* start;                 // n + 1
+    uint32_t* rows;                  // n: rows for a warp from the front, for a block from the back
+    uint32_t* giant;                 // n: rows too long for a block
+    uint32_t *rank_u, *rank_v;       // m each: the entry's place in its row (kPad: none)
+    uint32_t* tmp;                   // 2m
+    uint64_t* off;                   // n + 1
+    uint32_t* adj;                   // 2m
+    uint64_t* out;                   // entries kept, error bits, giant rows (if any, the rest is the caller's)
+    struct DirectCtl* ctl;           // of a grid (zero beforehand); a cluster has its own
+    uint64_t limit_ns;
+};
+
+struct DirectCtl {
+    unsigned long long bar[2][16];
+    unsigned long long part[2][kDirectGridMax];  // the blocks' sums of the two scans
+    uint32_t warp_rows, block_rows, giants, err;
+};
+
+struct DirectSmem {
+    BlockSortSmem<kDirectTB / 32> sort;
+    DirectCtl ctl;
+    MeetSmem meet;
+    uint32_t scan_tmp[33];
+    uint32_t before, all;
+};
+
+template <int E>
+__device__ __forceinline__ uint32_t sort_row_warp(uint32_t* row, uint32_t len, uint32_t lane) {
+    uint32_t x[E];
+#pragma unroll
+    for (int e = 0; e < E; ++e) {
+        const uint32_t i = (uint32_t)e * 32 + lane;
+        x[e] = i < len ? row[i] : kPad;
+    }
+    bitonic_sort<E, 32 * E>(x, 0, lane);
+    return warp_unique_write<E>(x, kPad, lane, row);
+}
+
+// Exclusive prefix sums of in[0, n), each block its share of whole tiles:
+// put(i, prefix) for every i of the block; the total to every thread.
+template <bool CL, class Put>
+__device__ __forceinline__ uint32_t direct_scan(const uint32_t* in, uint32_t n, unsigned long long* part,
+                                                Team<CL>& team, DirectSmem& sm, Put put) {
+    const uint32_t tid = threadIdx.x;
+    const uint32_t share = ((n + team.size - 1) / team.size + kDirectTB - 1) / kDirectTB * kDirectTB;
+    const uint32_t lo = min(n, team.rank * share), hi = min(n, lo + share);
+    uint32_t mine = 0;
+    for (uint32_t i = lo + tid; i < hi; i += kDirectTB) mine += __ldcg(in + i);
+    uint32_t tot;
+    block_excl_scan<uint32_t>(mine, sm.scan_tmp, &tot);
+    if (tid == 0) part[team.rank] = tot;
+    team.meet(0u, sm.meet);
+    if (tid < 32) {
+        uint32_t before = 0, all = 0;
+        for (uint32_t b = tid; b < team.size; b += 32) {
+            const uint32_t x = (uint32_t)ld_volatile_u64((const uint64_t*)&part[b]);
+            if (b < team.rank) before += x;
+            all += x;
+        }
+        before = warp_sum(before);
+        all = warp_sum(all);
+        if (tid == 0) {
+            sm.before = before;
+            sm.all = all;
+        }
+    }
+    __syncthreads();
+    uint32_t run = sm.before;
+    const uint32_t all = sm.all;
+    for (uint32_t t = lo; t < hi; t += kDirectTB) {
+        const uint32_t i = t + tid;
+        const uint32_t c = i < hi ? __ldcg(in + i) : 0u;
+        const uint32_t pre = block_excl_scan<uint32_t>(c, sm.scan_tmp, &tot);
+        if (i < hi) put(i, run + pre);
+        run += tot;
+    }
+    return all;
+}
+
+template <bool CL>
+__global__ void __launch_bounds__(kDirectTB, 1) direct_kernel(DirectArgs a) {
+    extern __shared__ __align__(16) unsigned char direct_smem_raw[];
+    DirectSmem& sm = *reinterpret_cast<DirectSmem*>(direct_smem_raw);
+    const uint32_t tid = threadIdx.x, lane = tid & 31u, n = a.n;
+    DirectCtl* const ctl = CL ? at_block0(&sm.ctl) : a.ctl;
+    Team<CL> team{CL ? cluster_rank() : blockIdx.x, gridDim.x, ctl->bar, &ctl->err, a.limit_ns, {}};
+    const uint32_t gt = team.rank * kDirectTB + tid, nt = team.size * kDirectTB;
+    const uint32_t gw = gt >> 5, nw = nt >> 5;
+    // no block of a cluster leaves while another reads block 0's shared memory
+    auto leave = [&]() {
+        if constexpr (CL) cluster_sync();
+    };
+    if (tid == 0) sm.meet.ok = 1;
+    if (CL && team.rank == 0)
+        for (uint32_t i = tid; i < sizeof(DirectCtl) / 4; i += kDirectTB) reinterpret_cast<uint32_t*>(&sm.ctl)[i] = 0;
+    for (uint32_t i = gt; i < n; i += nt) a.cnt[i] = 0;
+    if constexpr (CL) {
+        cluster_sync();
+    } else {
+        team.meet(0u, sm.meet);
+        if (!sm.meet.ok) return;
+    }
+    // ---- counts and ranks
+    {
+        constexpr uint32_t kU = 4;
+        bool bad = false;
+        for (uint32_t i0 = gt; i0 < a.m; i0 += kU * nt) {
+            uint32_t u[kU], v[kU], ru[kU], rv[kU];
+#pragma unroll
+            for (uint32_t j = 0; j < kU; ++j) {
+                const uint32_t i = i0 + j * nt;
+                u[j] = i < a.m ? a.src[i] : 0u;
+                v[j] = i < a.m ? a.dst[i] : 0u;
+            }
+#pragma unroll
+            for (uint32_t j = 0; j < kU; ++j) {
+                ru[j] = rv[j] = kPad;
+                if (u[j] >= n || v[j] >= n) bad |= i0 + j * nt < a.m;
+                else if (u[j] != v[j]) {
+                    ru[j] = atomicAdd(&a.cnt[u[j]], 1u);
+                    rv[j] = atomicAdd(&a.cnt[v[j]], 1u);
+                }
+            }
+#pragma unroll
+            for (uint32_t j = 0; j < kU; ++j)
+                if (i0 + j * nt < a.m) {
+                    a.rank_u[i0 + j * nt] = ru[j];
+                    a.rank_v[i0 + j * nt] = rv[j];
+                }
+        }
+        if (bad) atomicOr(&ctl->err, ERR_RANGE);
+    }
+    team.meet(0u, sm.meet);
+    if (!sm.meet.ok) return;
+    // ---- row starts
+    direct_scan(a.cnt, n, ctl->part[0], team, sm, [&](uint32_t i, uint32_t pre) { a.start[i] = pre; });
+    if (!sm.meet.ok) return;
+    team.meet(0u, sm.meet);
+    if (!sm.meet.ok) return;
+    if (ld_volatile_u32(&ctl->err)) {
+        if (team.rank == 0 && tid == 0) a.out[1] = ld_volatile_u32(&ctl->err);
+        leave();
+        return;
+    }
+    // ---- entries to their rows
+    for (uint32_t i = gt; i < a.m; i += nt) {
+        const uint32_t ru = a.rank_u[i];
+        if (ru == kPad) continue;
+        const uint32_t u = a.src[i], v = a.dst[i];
+        a.tmp[__ldcg(a.start + u) + ru] = v;
+        a.tmp[__ldcg(a.start + v) + a.rank_v[i]] = u;
+    }
+    team.meet(0u, sm.meet);
+    if (!sm.meet.ok) return;
+    // ---- rows of at most 32 entries; the longer ones listed
+    const uint32_t per = min(32u, max(4u, (n + nw - 1) / nw));  // rows per warp and turn
+    for (uint32_t v0 = gw * per; v0 < n; v0 += nw * per) {
+        const uint32_t vl = lane < per ? v0 + lane : n;
+        const uint32_t len = vl < n ? __ldcg(a.cnt + vl) : 0u;
+        const uint64_t st = vl < n ? __ldcg(a.start + vl) : 0u;
+        const uint32_t wrow = __ballot_sync(kFullMask, len > 32 && len <= 1024);
+        const uint32_t brow = __ballot_sync(kFullMask, len > 1024 && len <= kDirectRow);
+        uint32_t base = 0;
+        if (len > kDirectRow) a.giant[atomicAdd(&ctl->giants, 1u)] = vl;
+        if (lane == 0 && wrow) base = atomicAdd(&ctl->warp_rows, (uint32_t)__popc(wrow));
+        if (lane == 1 && brow) base = atomicAdd(&ctl->block_rows, (uint32_t)__popc(brow));
+        const uint32_t wb = __shfl_sync(kFullMask, base, 0), bb = __shfl_sync(kFullMask, base, 1);
+        if (wrow >> lane & 1u) a.rows[wb + __popc(wrow & lanemask_lt())] = vl;
+        if (brow >> lane & 1u) a.rows[n - 1 - bb - __popc(brow & lanemask_lt())] = vl;
+        if (vl < n && len == 0) a.newlen[vl] = 0;
+        sort_small_batches<8>(__ballot_sync(kFullMask, len && len <= 8), v0, len, st, a.tmp, a.newlen, lane);
+        sort_small_batches<16>(__ballot_sync(kFullMask, len > 8 && len <= 16), v0, len, st, a.tmp, a.newlen, lane);
+        sort_small_batches<32>(__ballot_sync(kFullMask, len > 16 && len <= 32), v0, len, st, a.tmp, a.newlen, lane);
+    }
+    team.meet(0u, sm.meet);
+    if (!sm.meet.ok) return;
+    // ---- the longer rows, a warp or a block each
+    {
+        const uint32_t nb = ld_volatile_u32(&ctl->block_rows), nwr = ld_volatile_u32(&ctl->warp_rows);
+        for (uint32_t r = team.rank; r < nb; r += team.size) {
+            const uint32_t v = __ldcg(a.rows + (n - 1 - r));
+            uint32_t* row = a.tmp + __ldcg(a.start + v);
+            const uint32_t kept = block_sort_unique<kDirectTB / 32>(row, __ldcg(a.cnt + v), row, sm.sort);
+            if (tid == 0) a.newlen[v] = kept;
+        }
+        for (uint32_t r = gw; r < nwr; r += nw) {
+            const uint32_t v = __ldcg(a.rows + r), len = __ldcg(a.cnt + v);
+            uint32_t* row = a.tmp + __ldcg(a.start + v);
+            uint32_t kept;
+            if (len <= 64) kept = sort_row_warp<2>(row, len, lane);
+            else if (len <= 128) kept = sort_row_warp<4>(row, len, lane);
+            else if (len <= 256) kept = sort_row_warp<8>(row, len, lane);
+            else if (len <= 512) kept = sort_row_warp<16>(row, len, lane);
+            else kept = sort_row_warp<32>(row, len, lane);
+            if (lane == 0) a.newlen[v] = kept;
+        }
+    }
+    team.meet(0u, sm.meet);
+    if (!sm.meet.ok) return;
+    if (const uint32_t giants = ld_volatile_u32(&ctl->giants)) {
+        if (team.rank == 0 && tid == 0) {
+            a.out[1] = 0;
+            a.out[2] = giants;
+        }
+        leave();
+        return;
+    }
+    // ---- row offsets and unique entries
+    const uint32_t total = direct_scan(a.newlen, n, ctl->part[1], team, sm, [&](uint32_t i, uint32_t pre) {
+        a.off[i] = pre;
+    });
+    if (!sm.meet.ok) return;
+    if (team.rank == 0 && tid == 0) {
+        a.off[n] = total;
+        a.out[0] = total;
+        a.out[1] = a.out[2] = 0;
+    }
+    team.meet(0u, sm.meet);
+    if (!sm.meet.ok) return;
+    auto pre = [&](uint64_t) { return 0u; };
+    auto put = [&](const uint32_t* v, const uint64_t* j, const uint32_t*, uint32_t valid) {
+        uint32_t val[kWalkU];
+#pragma unroll
+        for (uint32_t t = 0; t < kWalkU; ++t)
+            if (valid >> t & 1u) val[t] = __ldcg(a.tmp + (__ldcg(a.start + v[t]) + (j[t] - a.off[v[t]])));
+#pragma unroll
+        for (uint32_t t = 0; t < kWalkU; ++t)
+            if (valid >> t & 1u) a.adj[j[t]] = val[t];
+    };
+    walk_all_entries(a.off, n, pre, put);  // (the launch is this team alone: its blocks are the walker's)
+    leave();
+}
+
+// Giant rows (list of ng, device) sorted and de-duplicated in tmp: split by
+// splitters, the skewed ones by radix.  spare: as many entries as tmp.
+static dsg_status sort_giants(const uint32_t* glist, uint32_t ng, uint32_t n, const uint64_t* start, const uint32_t* cnt,
+                              uint32_t* tmp, uint32_t* spare, uint32_t* newlen, Scratch& sc, cudaStream_t s) {
+    const uint32_t sms = (uint32_t)dev_info().sms;
+    uint32_t nbits = 1;
+    while (nbits < 32 && ((uint64_t)n - 1) >> nbits) ++nbits;
+    const uint32_t passes = (nbits + 7) / 8;
+    uint32_t *gticket, *skewed;  // gticket[0]: split rows taken, [1]: skewed rows listed, [2]: radix rows taken
+    DSG_TRY_CUDA(sc.get(&gticket, 3));
+    DSG_TRY_CUDA(sc.get(&skewed, ng));
+    DSG_TRY_CUDA(cudaMemsetAsync(gticket, 0, 3 * sizeof(uint32_t), s));
+    {
+        LaunchScope ls_("ingest_giant_rows", s);
+        giant_split_kernel<<<std::min<uint32_t>(ng, 2 * sms), 256, 0, s>>>(glist, ng, start, cnt, tmp, spare, newlen,
+                                                                         gticket, skewed, gticket + 1);
+    }
+    DSG_TRY_CUDA(cudaGetLastError());
+    {
+        LaunchScope ls_("ingest_giant_skewed", s);
+        giant_radix_kernel<<<std::min<uint32_t>(ng, sms), kRadixTB, 0, s>>>(skewed, gticket + 1, start, cnt, tmp, spare,
+                                                                          passes, newlen, gticket + 2);
+    }
+    DSG_TRY_CUDA(cudaGetLastError());
+    return DSG_OK;
+}
+
+// The graph from sorted rows (row v: newlen[v] entries at tmp[start[v]]).
+static dsg_status finish_rows(uint32_t n, const uint64_t* start, const uint32_t* tmp, const uint32_t* newlen,
+                              uint64_t* sums, int dev, cudaStream_t s, dsg_graph** out) {
+    dsg_graph* g = new dsg_graph();
+    g->n = n;
+    g->device = dev;
+    g->stream = s;
+    cudaError_t e = dev_alloc((void**)&g->off, ((size_t)n + 1) * sizeof(uint64_t), s);
+    if (e == cudaSuccess) e = device_scan(newlen, n, g->off, sums, s);
+    uint64_t total2 = 0;
+    if (e == cudaSuccess) e = cudaMemcpyAsync(&total2, g->off + n, sizeof(uint64_t), cudaMemcpyDeviceToHost, s);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+    if (e == cudaSuccess) e = dev_alloc((void**)&g->adj, (size_t)(total2 ? total2 : 1) * sizeof(uint32_t), s);
+    if (e == cudaSuccess) {
+        if (total2) {
+            // one resident wave: every warp walks an equal share of the positions
+            int per_sm = 0;
+            if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, copy_rows, 256, 0) != cudaSuccess || per_sm < 1)
+                per_sm = 1;
+            LaunchScope ls_("ingest_copy_rows", s);
+            copy_rows<<<(uint32_t)dev_info().sms * (uint32_t)per_sm, 256, 0, s>>>(n, start, tmp, g->off, g->adj);
+        }
+        e = cudaGetLastError();
+    }
+    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+    if (e != cudaSuccess) {
+        set_error("graph_from_edges: %s", cudaGetErrorString(e));
+        g->owns = true;
+        dsg_graph_free(g);
+        return e == cudaErrorMemoryAllocation ? DSG_ENOMEM : DSG_ECUDA;
+    }
+    g->m = total2 / 2;
+    *out = g;
+    return DSG_OK;
+}
+
+// The small-input path.  shared: other work is on the GPU (the server's
+// ingest threads): few blocks, which find room beside it.
+static dsg_status ingest_direct(uint32_t n, uint32_t m, const uint32_t* src, const uint32_t* dst, bool shared,
+                                cudaStream_t s, dsg_graph** out) {
+    int dev = 0;
+    DSG_TRY_CUDA(cudaGetDevice(&dev));
+    const bool cluster = m <= kDirectClusterPairs;
+    static std::atomic<bool> ready[64] = {};  // the attributes are per function and device, set once (idempotent)
+    if (!ready[dev & 63]) {
+        for (auto* k : {direct_kernel<true>, direct_kernel<false>})
+            DSG_TRY_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(DirectSmem)));
+        DSG_TRY_CUDA(cudaFuncSetAttribute(direct_kernel<true>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+        ready[dev & 63] = true;
+    }
+    Scratch sc(s);
+    DirectArgs a;
+    a.n = n;
+    a.m = m;
+    a.src = src;
+    a.dst = dst;
+    const uint64_t nn = ((uint64_t)n + 64) & ~uint64_t(63), mm = ((uint64_t)m + 63) & ~uint64_t(63);
+    uint32_t* w;
+    constexpr size_t kCtlWords = (sizeof(DirectCtl) + 255) / 256 * 64;
+    DSG_TRY_CUDA(sc.get(&w, 64 + kCtlWords + 6 * nn + 4 * mm));
+    a.out = reinterpret_cast<uint64_t*>(w);
+    a.ctl = reinterpret_cast<DirectCtl*>(w + 64);
+    a.limit_ns = wait_limit_ns();
+    a.start = reinterpret_cast<uint64_t*>(w + 64 + kCtlWords);
+    a.cnt = w + 64 + kCtlWords + 2 * nn;
+    a.newlen = a.cnt + nn;
+    a.rows = a.newlen + nn;
+    a.giant = a.rows + nn;
+    a.rank_u = a.giant + nn;
+    a.rank_v = a.rank_u + mm;
+    a.tmp = a.rank_v + mm;
+    dsg_graph* g = new dsg_graph();
+    g->n = n;
+    g->device = dev;
+    g->stream = s;
+    uint64_t h[3] = {0, ERR_TIMEOUT, 0};  // (the error stays set if a wait runs out: the kernel leaves before it writes it)
+    cudaError_t e = dev_alloc((void**)&g->off, ((size_t)n + 1) * sizeof(uint64_t), s);
+    if (e == cudaSuccess) e = dev_alloc((void**)&g->adj, (size_t)(m ? 2 * (uint64_t)m : 1) * sizeof(uint32_t), s);
+    if (e == cudaSuccess) {
+        a.off = g->off;
+        a.adj = g->adj;
+        if (cluster) {
+            cudaLaunchConfig_t cfg = {};
+            cfg.gridDim = dim3(kDirectBlocks);
+            cfg.blockDim = dim3(kDirectTB);
+            cfg.dynamicSmemBytes = sizeof(DirectSmem);
+            cfg.stream = s;
+            cudaLaunchAttribute attr[1];
+            attr[0].id = cudaLaunchAttributeClusterDimension;
+            attr[0].val.clusterDim.x = kDirectBlocks;
+            attr[0].val.clusterDim.y = 1;
+            attr[0].val.clusterDim.z = 1;
+            cfg.attrs = attr;
+            cfg.numAttrs = 1;
+            e = cudaMemsetAsync(a.out, 0, sizeof(h), s);
+            LaunchScope ls("ingest_direct", s);
+            if (e == cudaSuccess) e = cudaLaunchKernelEx(&cfg, direct_kernel<true>, a);
+        } else {
+            uint32_t grid = 1;
+            const uint64_t pairs_per_block = shared ? 16384 : 1024;
+            e = cudaMemsetAsync(a.ctl, 0, sizeof(DirectCtl), s);
+            if (e == cudaSuccess) e = cudaMemcpyAsync(a.out, h, sizeof(h), cudaMemcpyHostToDevice, s);
+            if (e == cudaSuccess)
+                e = coop_grid(direct_kernel<false>, kDirectTB, sizeof(DirectSmem), (uint64_t)m * kDirectTB / pairs_per_block, 1,
+                              &grid, kDirectGridMax);
+            if (e == cudaSuccess) {
+                void* params[] = {&a};
+                LaunchScope ls("ingest_direct", s);
+                e = cudaLaunchCooperativeKernel((const void*)direct_kernel<false>, dim3(grid), dim3(kDirectTB), params,
+                                                sizeof(DirectSmem), s);
+            }
+        }
+    }
+    if (e == cudaSuccess) e = cudaMemcpyAsync(h, a.out, sizeof(h), cudaMemcpyDeviceToHost, s);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+    if (e == cudaSuccess && !h[1] && !h[2]) {
+        g->m = h[0] / 2;
+        *out = g;
+        return DSG_OK;
+    }
+    dsg_graph_free(g);
+    if (e != cudaSuccess) {
+        set_error("graph_from_edges: %s", cudaGetErrorString(e));
+        return e == cudaErrorMemoryAllocation ? DSG_ENOMEM : DSG_ECUDA;
+    }
+    if (h[1] & ERR_TIMEOUT) return status_from_err(ERR_TIMEOUT, "graph_from_edges");
+    if (h[1]) {
+        set_error("graph_from_edges: a vertex id is >= n");
+        return DSG_EINVAL;
+    }
+    // giant rows: sorted by kernels of their own, then the rows are put together like a large input's
+    uint64_t* sums;
+    DSG_TRY_CUDA(sc.get(&sums, (size_t)n / kScanTile + 2));
+    const dsg_status st = sort_giants(a.giant, (uint32_t)h[2], n, a.start, a.cnt, a.tmp, a.rank_u, a.newlen, sc, s);
+    return st == DSG_OK ? finish_rows(n, a.start, a.tmp, a.newlen, sums, dev, s, out) : st;
+}
+
 static uint32_t grid_for(uint64_t work, uint32_t block) {
     uint64_t g = (work + block - 1) / block;
     uint64_t cap = (uint64_t)dev_info().sms * 16;
@@ -1274,8 +1704,10 @@ static uint32_t grid_for(uint64_t work, uint32_t block) {
 }
 
 // Core ingest on device arrays src/dst (m_raw pairs).  Allocates the graph.
-static dsg_status ingest_device(uint32_t n, uint64_t m_raw, const uint32_t* src, const uint32_t* dst,
+static dsg_status ingest_device(uint32_t n, uint64_t m_raw, const uint32_t* src, const uint32_t* dst, bool shared,
                                 cudaStream_t s, dsg_graph** out) {
+    if (n && m_raw <= kDirectPairs && n <= 4 * kDirectPairs)
+        return ingest_direct(n, (uint32_t)m_raw, src, dst, shared, s, out);
     int dev = 0;
     DSG_TRY_CUDA(cudaGetDevice(&dev));
     Scratch sc(s);
@@ -1444,60 +1876,13 @@ static dsg_status ingest_device(uint32_t n, uint64_t m_raw, const uint32_t* src,
     DSG_TRY_CUDA(cudaGetLastError());
     if (hc.cls_count[kGiant]) {
         const uint32_t ng = hc.cls_count[kGiant];
-        const uint32_t* glist = lists.rows + lists.base[kGiant];
-        uint32_t nbits = 1;
-        while (nbits < 32 && ((uint64_t)n - 1) >> nbits) ++nbits;
-        const uint32_t passes = (nbits + 7) / 8;
         // the bucket entries are no longer needed: their space is the spare buffer of both sorts
-        uint32_t* spare = reinterpret_cast<uint32_t*>(E1);
-        uint32_t *gticket, *skewed;  // gticket[0]: split rows taken, [1]: skewed rows listed, [2]: radix rows taken
-        DSG_TRY_CUDA(sc.get(&gticket, 3));
-        DSG_TRY_CUDA(sc.get(&skewed, ng));
-        DSG_TRY_CUDA(cudaMemsetAsync(gticket, 0, 3 * sizeof(uint32_t), s));
-        {
-            LaunchScope ls_("ingest_giant_rows", s);
-            giant_split_kernel<<<std::min<uint32_t>(ng, 2 * sms), 256, 0, s>>>(glist, ng, start, cnt, tmp, spare,
-                                                                             newlen, gticket, skewed, gticket + 1);
-        }
-        DSG_TRY_CUDA(cudaGetLastError());
-        {
-            LaunchScope ls_("ingest_giant_skewed", s);
-            giant_radix_kernel<<<std::min<uint32_t>(ng, sms), kRadixTB, 0, s>>>(skewed, gticket + 1, start, cnt, tmp,
-                                                                              spare, passes, newlen, gticket + 2);
-        }
+        const dsg_status st = sort_giants(lists.rows + lists.base[kGiant], ng, n, start, cnt, tmp,
+                                          reinterpret_cast<uint32_t*>(E1), newlen, sc, s);
+        if (st != DSG_OK) return st;
     }
     DSG_TRY_CUDA(cudaGetLastError());
-    dsg_graph* g = new dsg_graph();
-    g->n = n;
-    g->device = dev;
-    g->stream = s;
-    cudaError_t e = dev_alloc((void**)&g->off, ((size_t)n + 1) * sizeof(uint64_t), s);
-    if (e == cudaSuccess) e = device_scan(newlen, n, g->off, sums, s);
-    uint64_t total2 = 0;
-    if (e == cudaSuccess) e = cudaMemcpyAsync(&total2, g->off + n, sizeof(uint64_t), cudaMemcpyDeviceToHost, s);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-    if (e == cudaSuccess) e = dev_alloc((void**)&g->adj, (size_t)(total2 ? total2 : 1) * sizeof(uint32_t), s);
-    if (e == cudaSuccess) {
-        if (total2) {
-            // one resident wave: every warp walks an equal share of the positions
-            int per_sm = 0;
-            if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, copy_rows, 256, 0) != cudaSuccess || per_sm < 1)
-                per_sm = 1;
-            LaunchScope ls_("ingest_copy_rows", s);
-            copy_rows<<<(uint32_t)dev_info().sms * (uint32_t)per_sm, 256, 0, s>>>(n, start, tmp, g->off, g->adj);
-        }
-        e = cudaGetLastError();
-    }
-    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-    if (e != cudaSuccess) {
-        set_error("graph_from_edges: %s", cudaGetErrorString(e));
-        g->owns = true;
-        dsg_graph_free(g);
-        return e == cudaErrorMemoryAllocation ? DSG_ENOMEM : DSG_ECUDA;
-    }
-    g->m = total2 / 2;
-    *out = g;
-    return DSG_OK;
+    return finish_rows(n, start, tmp, newlen, sums, dev, s, out);
 }
 
 dsg_status ingest_from_csr_entries(uint32_t n, const uint64_t* off, const uint32_t* adj, uint64_t total,
@@ -1536,7 +1921,7 @@ dsg_status ingest_from_csr_entries(uint32_t n, const uint64_t* off, const uint32
     DSG_TRY_CUDA(sc.get(&src, total ? total : 1));
     { LaunchScope ls_("ingest_expand_rows", s); expand_rows<<<grid_for((uint64_t)n * 32, 256), 256, 0, s>>>(n, doff, src); }
     DSG_TRY_CUDA(cudaGetLastError());
-    dsg_status st = ingest_device(n, total, src, dadj, s, out);
+    dsg_status st = ingest_device(n, total, src, dadj, false, s, out);
     if (st == DSG_OK && (flags & DSG_CSR_VALIDATE)) {
         st = validate_csr(*out);
         if (st != DSG_OK) {
@@ -1612,8 +1997,8 @@ dsg_status validate_csr(const dsg_graph* g) {
 
 using namespace dsg;
 
-extern "C" dsg_status dsg_graph_from_edges(uint32_t n, uint64_t m_raw, const uint32_t* src, const uint32_t* dst,
-                                           uint32_t flags, void* stream, dsg_graph** out) {
+dsg_status dsg::graph_from_edges(uint32_t n, uint64_t m_raw, const uint32_t* src, const uint32_t* dst, uint32_t flags,
+                                 bool shared, void* stream, dsg_graph** out) {
     clear_error();
     DSG_CHECK_ARG(out, "out is NULL");
     DSG_CHECK_ARG(n < 0x80000000u, "n must be below 2^31");
@@ -1634,7 +2019,7 @@ extern "C" dsg_status dsg_graph_from_edges(uint32_t n, uint64_t m_raw, const uin
         dsrc = a;
         ddst = b;
     }
-    dsg_status st = ingest_device(n, m_raw, dsrc, ddst, s, out);
+    dsg_status st = ingest_device(n, m_raw, dsrc, ddst, shared, s, out);
     if (st == DSG_OK && (flags & DSG_CSR_VALIDATE)) {
         st = validate_csr(*out);
         if (st != DSG_OK) {
@@ -1643,4 +2028,9 @@ extern "C" dsg_status dsg_graph_from_edges(uint32_t n, uint64_t m_raw, const uin
         }
     }
     return st;
+}
+
+extern "C" dsg_status dsg_graph_from_edges(uint32_t n, uint64_t m_raw, const uint32_t* src, const uint32_t* dst,
+                                           uint32_t flags, void* stream, dsg_graph** out) {
+    return graph_from_edges(n, m_raw, src, dst, flags, false, stream, out);
 }

@@ -153,7 +153,7 @@ static bool is_big(const dsg_server* s, const ServeReq* r) {
 static void ingest_one(dsg_server* s, ServeReq* r, cudaStream_t st_ing) {
     const double t_in = now_us();
     dsg_graph* g = nullptr;
-    dsg_status st = dsg_graph_from_edges(r->n, r->m_raw, r->src, r->dst, 0, st_ing, &g);
+    dsg_status st = graph_from_edges(r->n, r->m_raw, r->src, r->dst, 0, true, st_ing, &g);
     if (r->owned) {
         free(r->src);
         free(r->dst);
