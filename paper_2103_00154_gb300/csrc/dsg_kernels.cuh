@@ -149,6 +149,30 @@ cudaError_t coop_grid(K kernel, uint32_t block, size_t smem, uint64_t work_items
     return cudaSuccess;
 }
 
+// A launch of one thread-block cluster of `blocks` blocks (16 need the
+// kernel's non-portable attribute).
+template <class... P, class... A>
+cudaError_t launch_cluster(void (*kernel)(P...), uint32_t blocks, uint32_t threads, size_t smem, cudaStream_t s,
+                           A... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(blocks);
+    cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = blocks;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, args...);
+}
+
+// Graphs that one cluster of 16 blocks handles sooner than a grid does: the
+// meetings are the cluster's barrier instead of a word in L2.
+constexpr uint32_t kSmallBlocks = 16;
+
 __device__ __forceinline__ uint64_t ld_relaxed_u64(const unsigned long long* p) {
     uint64_t v;
     asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");

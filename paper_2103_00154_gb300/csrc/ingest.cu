@@ -1641,21 +1641,10 @@ static dsg_status ingest_direct(uint32_t n, uint32_t m, const uint32_t* src, con
         a.off = g->off;
         a.adj = g->adj;
         if (cluster) {
-            cudaLaunchConfig_t cfg = {};
-            cfg.gridDim = dim3(kDirectBlocks);
-            cfg.blockDim = dim3(kDirectTB);
-            cfg.dynamicSmemBytes = sizeof(DirectSmem);
-            cfg.stream = s;
-            cudaLaunchAttribute attr[1];
-            attr[0].id = cudaLaunchAttributeClusterDimension;
-            attr[0].val.clusterDim.x = kDirectBlocks;
-            attr[0].val.clusterDim.y = 1;
-            attr[0].val.clusterDim.z = 1;
-            cfg.attrs = attr;
-            cfg.numAttrs = 1;
             e = cudaMemsetAsync(a.out, 0, sizeof(h), s);
             LaunchScope ls("ingest_direct", s);
-            if (e == cudaSuccess) e = cudaLaunchKernelEx(&cfg, direct_kernel<true>, a);
+            if (e == cudaSuccess)
+                e = launch_cluster(direct_kernel<true>, kDirectBlocks, kDirectTB, sizeof(DirectSmem), s, a);
         } else {
             uint32_t grid = 1;
             const uint64_t pairs_per_block = shared ? 16384 : 1024;

@@ -14,6 +14,25 @@ __global__ void __launch_bounds__(kSplitTB, 1) core_split_kernel(SplitArgs a) {
     split_body<kSplitTB, false>(a, team, sm);
 }
 
+// The same by one cluster, its control block in shared memory (copied to
+// a.ctl at the end).
+__global__ void __launch_bounds__(kSplitTB, 1) core_split_cluster_kernel(SplitArgs a) {
+    __shared__ SplitSmem<kSplitTB> sm;
+    __shared__ SplitCtl ctl;
+    SplitCtl* const global = a.ctl;
+    a.ctl = at_block0(&ctl);
+    const uint32_t rank = cluster_rank();
+    uint32_t* const words = reinterpret_cast<uint32_t*>(&ctl);
+    if (rank == 0)
+        for (uint32_t i = threadIdx.x; i < sizeof(SplitCtl) / 4; i += kSplitTB) words[i] = 0;
+    cluster_sync();
+    split_body<kSplitTB, true>(a, Team<true>{rank, kSmallBlocks, a.ctl->bar, &a.ctl->err, 0, {}}, sm);
+    cluster_sync();  // every block's counts are in; no block leaves while another reads block 0's shared memory
+    if (rank == 0)
+        for (uint32_t i = threadIdx.x; i < sizeof(SplitCtl) / 4; i += kSplitTB)
+            reinterpret_cast<uint32_t*>(global)[i] = words[i];
+}
+
 // ---------------------------------------------------------------- compaction
 
 // The vertices not yet taken (claim bit clear), numbered in the order warps
@@ -129,6 +148,11 @@ __global__ void __launch_bounds__(1024) tail_levels_kernel(uint32_t r, const uin
     }
 }
 
+// Vertices plus row entries up to which one cluster searches (us, cluster /
+// grid: work of 28,000 140 / 165, 113,000 164 / 179, 168,000 323 / 353,
+// 244,000 363 / 378, 337,000 449 / 442, 372,000 300 / 251).
+constexpr uint64_t kSmallCore = 250000;
+
 // The bitwise search on a graph of r vertices (rows off, adj), none with a core number below lo; core numbers to core (by original
 // id through rid, nullable: the vertices' own numbers).
 dsg_status core_split(uint32_t r, uint32_t lo, const uint64_t* off, const uint32_t* adj, uint64_t entries,
@@ -147,16 +171,28 @@ dsg_status core_split(uint32_t r, uint32_t lo, const uint64_t* off, const uint32
     a.trace_cap = trace ? trace_cap : 0;
     a.kstride = ((uint64_t)r + 63) & ~uint64_t(63);
     a.cap = (uint64_t)r + entries / kPiece;
-    DSG_TRY_CUDA(sc.get(&a.d, r));
-    DSG_TRY_CUDA(sc.get(&a.ds, r));
-    DSG_TRY_CUDA(sc.get(&a.key, a.kstride * split_key_buffers(entries)));
-    DSG_TRY_CUDA(sc.get(&a.pieces, a.cap));
-    DSG_TRY_CUDA(sc.get(&a.queue, a.cap));
-    DSG_TRY_CUDA(sc.get(&a.ctl, 1));
-    DSG_TRY_CUDA(cudaMemsetAsync(a.ctl, 0, sizeof(SplitCtl), s));
-    uint32_t grid = 1;
-    DSG_TRY_CUDA(coop_grid(core_split_kernel, kSplitTB, 0, (uint64_t)r + entries / 16, 1, &grid, g->max_blocks));
-    {
+    // one allocation for all of it
+    const uint64_t nbuf = split_key_buffers(entries);
+    const uint64_t words = 16 * 64 + a.kstride * (2 + nbuf);
+    static_assert(sizeof(SplitCtl) <= 16 * 64 * 4, "the control block's share of the allocation");
+    uint32_t* w;
+    DSG_TRY_CUDA(sc.get(&w, words + 8 * a.cap));
+    a.ctl = reinterpret_cast<SplitCtl*>(w);
+    a.d = w + 16 * 64;
+    a.ds = a.d + a.kstride;
+    a.key = a.ds + a.kstride;
+    a.pieces = reinterpret_cast<uint4*>(w + words);
+    a.queue = a.pieces + a.cap;
+    const bool small = r + entries <= kSmallCore && (g->max_blocks == 0 || g->max_blocks >= kSmallBlocks) &&
+                       cudaFuncSetAttribute(core_split_cluster_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed,
+                                            1) == cudaSuccess;
+    if (small) {
+        LaunchScope ls("kcore_split", s);
+        DSG_TRY_CUDA(launch_cluster(core_split_cluster_kernel, kSmallBlocks, kSplitTB, 0, s, a));
+    } else {
+        DSG_TRY_CUDA(cudaMemsetAsync(a.ctl, 0, sizeof(SplitCtl), s));
+        uint32_t grid = 1;
+        DSG_TRY_CUDA(coop_grid(core_split_kernel, kSplitTB, 0, (uint64_t)r + entries / 16, 1, &grid, g->max_blocks));
         void* params[] = {&a};
         LaunchScope ls("kcore_split", s);
         DSG_TRY_CUDA(cudaLaunchCooperativeKernel((const void*)core_split_kernel, dim3(grid), dim3(kSplitTB), params, 0,

@@ -20,6 +20,39 @@ __global__ void __launch_bounds__(TB, 1024 / TB) peel_kernel(PeelArgs a) {
     peel_body<TB, false>(a, team, sm);
 }
 
+// The whole peel of a small graph by one cluster: the control block in shared
+// memory (copied to a.ctl at the end), and the results written in the same
+// launch (peel_round, set: nullable).
+constexpr uint32_t kSmallTB = 512;
+
+__global__ void __launch_bounds__(kSmallTB, 2) peel_cluster_kernel(PeelArgs a, uint32_t* peel_round, uint8_t* set) {
+    __shared__ PeelSmem<kSmallTB> sm;
+    __shared__ PeelCtl ctl;
+    PeelCtl* const global = a.ctl;
+    a.ctl = at_block0(&ctl);
+    const uint32_t rank = cluster_rank(), tid = threadIdx.x;
+    uint32_t* const words = reinterpret_cast<uint32_t*>(&ctl);
+    if (rank == 0)
+        for (uint32_t i = tid; i < sizeof(PeelCtl) / 4; i += kSmallTB) words[i] = 0;
+    cluster_sync();
+    const PeelOut o =
+        peel_body<kSmallTB, true>(a, Team<true>{rank, kSmallBlocks, a.ctl->bar, &a.ctl->err, 0, {}}, sm);
+    for (uint32_t v = rank * kSmallTB + tid; v < a.n; v += kSmallBlocks * kSmallTB) {
+        const uint32_t pr = __ldcg(a.st + v) & ~kDead;
+        if (peel_round) peel_round[v] = pr;
+        if (set) set[v] = pr > o.best_round ? 1 : 0;
+    }
+    cluster_sync();  // no block leaves while another reads block 0's shared memory
+    if (rank == 0)
+        for (uint32_t i = tid; i < sizeof(PeelCtl) / 4; i += kSmallTB) reinterpret_cast<uint32_t*>(global)[i] = words[i];
+}
+
+// Vertices plus row entries up to which one cluster peels (us, cluster / grid
+// with its second launch for the results: work of 28,000 73 / 83, 113,000
+// 81 / 86, 168,000 94 / 100, 244,000 81 / 83, 337,000 107 / 112, 372,000
+// 106 / 89, 929,000 143 / 95).
+constexpr uint64_t kSmallPeel = 250000;
+
 // peel_round[v] = round v failed; set[v] = peel_round > best_round.
 __global__ void peel_finish_kernel(uint32_t n, const uint32_t* __restrict__ st, const PeelCtl* __restrict__ ctl,
                                    uint32_t* __restrict__ peel_round, uint8_t* __restrict__ set) {
@@ -107,47 +140,58 @@ static dsg_status run_peel(const dsg_graph* g, uint32_t p, uint32_t q, uint64_t*
     a.trace = trace_dev;
     a.trace_cap = trace_cap;
     a.r0 = a.S0 = a.E0 = a.best_round0 = a.best_E0 = a.best_V0 = a.max_rounds = 0;
-    DSG_TRY_CUDA(sc.get(&a.st, n));
-    DSG_TRY_CUDA(sc.get(&a.listA, n));
-    DSG_TRY_CUDA(sc.get(&a.listB, n));
-    DSG_TRY_CUDA(sc.get(&a.items, item_cap));
-    DSG_TRY_CUDA(sc.get(&a.map, ((size_t)n + 15) / 16));
-    a.candA = a.candB = nullptr;
-    if (current_tuning().peel_lazy) {
-        DSG_TRY_CUDA(sc.get(&a.candA, n));
-        DSG_TRY_CUDA(sc.get(&a.candB, n));
+    const bool lazy = current_tuning().peel_lazy != 0;
+    const bool pr_direct = peel_round_out && is_device_ptr(peel_round_out);
+    const bool set_direct = set_out && is_device_ptr(set_out);
+    uint32_t* pr_dev = peel_round_out && pr_direct ? peel_round_out : nullptr;
+    uint8_t* set_dev = set_out && set_direct ? set_out : nullptr;
+    {
+        // one allocation for all of it
+        size_t o = 0;
+        auto carve = [&](size_t bytes) { const size_t at = o; o += (bytes + 255) & ~size_t(255); return at; };
+        const size_t nb = (size_t)n * 4;
+        const size_t o_ctl = carve(sizeof(PeelCtl)), o_st = carve(nb), o_a = carve(nb), o_b = carve(nb),
+                     o_items = carve(item_cap * 8), o_map = carve(((size_t)n + 15) / 16 * 4),
+                     o_ca = carve(lazy ? nb : 0), o_cb = carve(lazy ? nb : 0), o_hs = carve(cap * 8),
+                     o_he = carve(cap * 8), o_pr = carve(peel_round_out && !pr_direct ? nb : 0),
+                     o_set = carve(set_out && !set_direct ? n : 0);
+        unsigned char* w;
+        DSG_TRY_CUDA(sc.get(&w, o));
+        a.ctl = reinterpret_cast<PeelCtl*>(w + o_ctl);
+        a.st = reinterpret_cast<uint32_t*>(w + o_st);
+        a.listA = reinterpret_cast<uint32_t*>(w + o_a);
+        a.listB = reinterpret_cast<uint32_t*>(w + o_b);
+        a.items = reinterpret_cast<uint64_t*>(w + o_items);
+        a.map = reinterpret_cast<uint32_t*>(w + o_map);
+        a.candA = lazy ? reinterpret_cast<uint32_t*>(w + o_ca) : nullptr;
+        a.candB = lazy ? reinterpret_cast<uint32_t*>(w + o_cb) : nullptr;
+        a.hist_S = reinterpret_cast<uint64_t*>(w + o_hs);
+        a.hist_E = reinterpret_cast<uint64_t*>(w + o_he);
+        if (peel_round_out && !pr_direct) pr_dev = reinterpret_cast<uint32_t*>(w + o_pr);
+        if (set_out && !set_direct) set_dev = w + o_set;
     }
-    DSG_TRY_CUDA(sc.get(&a.hist_S, cap));
-    DSG_TRY_CUDA(sc.get(&a.hist_E, cap));
-    DSG_TRY_CUDA(sc.get(&a.ctl, 1));
-    DSG_TRY_CUDA(cudaMemsetAsync(a.ctl, 0, sizeof(PeelCtl), s));
-    cudaError_t e;
-    switch (tu.block) {
-        case 256: e = launch_peel<256>(a, tu.blocks_per_sm, s, g->max_blocks); break;
-        case 1024: e = launch_peel<1024>(a, tu.blocks_per_sm, s, g->max_blocks); break;
-        default: e = launch_peel<512>(a, tu.blocks_per_sm, s, g->max_blocks); break;
-    }
-    DSG_TRY_CUDA(e);
-    uint32_t* pr_dev = nullptr;
-    uint8_t* set_dev = nullptr;
-    bool pr_direct = peel_round_out && is_device_ptr(peel_round_out);
-    bool set_direct = set_out && is_device_ptr(set_out);
-    if (peel_round_out) {
-        if (pr_direct) pr_dev = peel_round_out;
-        else DSG_TRY_CUDA(sc.get(&pr_dev, n));
-    }
-    if (set_out) {
-        if (set_direct) set_dev = set_out;
-        else DSG_TRY_CUDA(sc.get(&set_dev, n));
-    }
-    if (pr_dev || set_dev) {
-        uint64_t want = ((uint64_t)n + 255) / 256, cap_b = (uint64_t)dev_info().sms * 8;
-        uint32_t blocks = (uint32_t)(want < cap_b ? want : cap_b);
-        {
+    const bool small = n + 2 * g->m <= kSmallPeel && (g->max_blocks == 0 || g->max_blocks >= kSmallBlocks) &&
+                       cudaFuncSetAttribute(peel_cluster_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) ==
+                           cudaSuccess;
+    if (small) {
+        LaunchScope ls("peel_rounds", s);
+        DSG_TRY_CUDA(launch_cluster(peel_cluster_kernel, kSmallBlocks, kSmallTB, 0, s, a, pr_dev, set_dev));
+    } else {
+        DSG_TRY_CUDA(cudaMemsetAsync(a.ctl, 0, sizeof(PeelCtl), s));
+        cudaError_t e;
+        switch (tu.block) {
+            case 256: e = launch_peel<256>(a, tu.blocks_per_sm, s, g->max_blocks); break;
+            case 1024: e = launch_peel<1024>(a, tu.blocks_per_sm, s, g->max_blocks); break;
+            default: e = launch_peel<512>(a, tu.blocks_per_sm, s, g->max_blocks); break;
+        }
+        DSG_TRY_CUDA(e);
+        if (pr_dev || set_dev) {
+            uint64_t want = ((uint64_t)n + 255) / 256, cap_b = (uint64_t)dev_info().sms * 8;
+            uint32_t blocks = (uint32_t)(want < cap_b ? want : cap_b);
             LaunchScope ls("peel_finish", s);
             peel_finish_kernel<<<blocks, 256, 0, s>>>(n, a.st, a.ctl, pr_dev, set_dev);
+            DSG_TRY_CUDA(cudaGetLastError());
         }
-        DSG_TRY_CUDA(cudaGetLastError());
     }
     DSG_TRY_CUDA(cudaMemcpyAsync(ctl_host, a.ctl, sizeof(PeelCtl), cudaMemcpyDeviceToHost, s));
     DSG_TRY_CUDA(cudaStreamSynchronize(s));

@@ -382,7 +382,7 @@ __device__ __forceinline__ PeelOut peel_body(const PeelArgs& a, Team<CL> team, P
                 __syncthreads();  // the tile's totals are read before the next tile writes its own
             }
         };
-        if (by_id || span >= 4 * threads) test(std::integral_constant<uint32_t, 4>{});
+        if (span >= 4 * threads) test(std::integral_constant<uint32_t, 4>{});
         else test(std::integral_constant<uint32_t, 1>{});
         {
             X = warp_sum(X);
