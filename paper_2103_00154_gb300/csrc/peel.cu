@@ -295,8 +295,11 @@ dsg_status dsg_solve(const dsg_graph* g, uint32_t count, const uint32_t* eps_num
     va.force_block = vb.force_block = 1024;
     // the peels' share of the SMs: DSG_SOLVE_PEEL_PERMILLE if set, else from
     // the autotuned times (each side's share of the summed time, within
-    // [1/4, 3/4]), else half
-    double peel_frac = 0.5;
+    // [1/4, 3/4]), else as if the core numbers took as long as eight peels
+    // (R-MAT 2^20, three peels, from host memory: 6.72 ms at 0.25, 6.82 at 0.3,
+    // 7.49 at half; Chung-Lu 3 10^6 9.48 / 8.98 / 9.63; Erdos-Renyi 5 10^5
+    // 1.80 / 1.78 / 1.89)
+    double peel_frac = std::min(0.5, std::max(0.15, count / (count + 8.0)));
     if (tuned && count * peel_ms + core_ms > 0)
         peel_frac = std::min(0.75, std::max(0.25, count * peel_ms / (count * peel_ms + core_ms)));
     if (const char* e = getenv("DSG_SOLVE_PEEL_PERMILLE")) {
