@@ -167,6 +167,7 @@ __device__ __forceinline__ PeelOut peel_body(const PeelArgs& a, Team<CL> team, P
     uint32_t* next_cand = a.candB;
     uint64_t cand_n = 0, cand_base = 0, S_prev = S;
     bool have_cands = false;
+    uint64_t cand_from = 0, cand_rest = 2;  // no candidates are collected before round cand_from
     uint32_t B = 0;
     uint64_t best_E = resume ? a.best_E0 : E, best_V = resume ? a.best_V0 : S;
     uint64_t best_round = resume ? a.best_round0 : 0;
@@ -229,15 +230,16 @@ __device__ __forceinline__ PeelOut peel_body(const PeelArgs& a, Team<CL> team, P
         const bool by_id = fresh || scan_all;
         // thin: the last round removed less than 1/8 of the vertices; then this round collects the
         // next round's candidates (bound Bn), and it is lazy when the current list covers T
-        const bool thin = lazy_ok && !solo && !fresh && (S_prev - S) * 8 < S_prev;
+        // (unless the last collections were too long to be of use: see below)
+        const bool thin = lazy_ok && !solo && !fresh && (S_prev - S) * 8 < S_prev && r >= cand_from;
         const bool lazy = thin && have_cands && !by_id && T <= B && cand_n * 4 < S;
         const uint32_t Bn = lazy ? B : (thin ? T + T / 128u : 0u);
         const uint64_t span = by_id ? (scan_all ? a.n : S) : (lazy ? cand_n : alive_len);
         const uint32_t* src = lazy ? cur_cand : alive;
         tested += span;
         lazy_rounds += lazy ? 1u : 0u;
-        // a tile is `items` slices of TB (thread tid takes i = t + j TB + tid for j < items), four
-        // where there is enough to test (their loads in flight together), else one; a list shorter
+        // a tile is `items` slices of TB (thread tid takes i = t + j TB + tid for j < items), four or
+        // two where there is enough to test (their loads in flight together), else one; a list shorter
         // than the blocks' threads is spread over the blocks, `width` entries each (a hub's pieces
         // are written by its warp).  The first pass tests and marks, the second writes the lists at
         // the tile's reserved places
@@ -383,6 +385,7 @@ __device__ __forceinline__ PeelOut peel_body(const PeelArgs& a, Team<CL> team, P
             }
         };
         if (span >= 4 * threads) test(std::integral_constant<uint32_t, 4>{});
+        else if (!CL && span > threads) test(std::integral_constant<uint32_t, 2>{});
         else test(std::integral_constant<uint32_t, 1>{});
         {
             X = warp_sum(X);
@@ -559,6 +562,16 @@ __device__ __forceinline__ PeelOut peel_body(const PeelArgs& a, Team<CL> team, P
                 next_cand = t_;
                 cand_n = cand_hi - cand_base;
                 B = Bn;
+                // a list that is no use to the next round (most degrees lie just above the threshold)
+                // costs more than testing everyone: an atomic per warp of the alive list (nested shells
+                // of 265,100 vertices: 12.5 us a round's test against 8).  Rest before the next try,
+                // longer each time
+                if (cand_n * 4 >= S1) {
+                    cand_from = r + cand_rest;
+                    cand_rest = min(2 * cand_rest, (uint64_t)64);
+                } else {
+                    cand_rest = 2;
+                }
             }
             have_cands = thin;
             cand_base = cand_hi;

@@ -52,3 +52,20 @@ def test_rounds(raw, pq, block):
     np.testing.assert_array_equal(tr.peel_round, want.peel_round)
     np.testing.assert_array_equal(tr.mask, want.mask)
     g.close()
+
+
+@pytest.mark.parametrize("d,core", [(64, 160), (16, 60)])
+def test_candidate_lists_that_are_no_use(d, core):
+    # nested shells whose degrees all lie just above the threshold: every candidate list would hold
+    # nearly every vertex, so collecting rests; the rounds stay the same, with lists on and off
+    raw = inputs.onion(40_000, d, core)
+    c = oracle.from_raw(raw)
+    want = oracle.bahmani(c, 1, 1000)
+    for lazy in (True, False):
+        dsg.set_tuning(peel_lazy=lazy)
+        g = dsg.Graph.from_csr(raw.n, c.off, c.adj)
+        tr = g.bahmani_trace(1, 1000)
+        assert (tr.rounds, tr.best_round, tr.E, tr.V) == (want.rounds, want.best_round, want.E, want.V)
+        np.testing.assert_array_equal(tr.peel_round, want.peel_round)
+        np.testing.assert_array_equal(tr.hist_E, want.hist_E)
+        g.close()
