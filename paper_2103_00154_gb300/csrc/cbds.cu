@@ -55,14 +55,13 @@ struct __align__(128) CbdsCtl {
     uint64_t n_elig_items, n_legit_items;
 };
 
-// Warp-aggregated histogram increment: lanes holding the same key combine
-// their counts before one atomic.  key == ~0u means "no increment".
+// Histogram increment; key == ~0u means "no increment".  In shared memory a
+// plain +1 without a result: the hardware counts the lanes of a word itself.
 __device__ __forceinline__ void hist_add_shared(uint32_t* h, uint32_t key) {
-    const uint32_t peers = __match_any_sync(kFullMask, key);
-    const uint32_t leader = __ffs(peers) - 1;
-    if (key != ~0u && (threadIdx.x & 31u) == leader) atomicAdd(&h[key], (uint32_t)__popc(peers));
+    if (key != ~0u) atomicAdd(&h[key], 1u);
 }
 
+// In global memory the lanes holding the same key combine their counts before one atomic.
 __device__ __forceinline__ void hist_add_global(unsigned long long* h, uint32_t key) {
     const uint32_t peers = __match_any_sync(kFullMask, key);
     const uint32_t leader = __ffs(peers) - 1;

@@ -475,17 +475,20 @@ __device__ __forceinline__ void walk_all_entries(const uint64_t* off, uint32_t n
         {
             const uint32_t base = r;
             const uint32_t idx = base + 1 + lane;
-            const uint64_t w = off[idx < n ? idx : n];
-            const uint64_t w31 = __shfl_sync(kFullMask, w, 31);
+            // row starts relative to the step (none lies before it: row r holds the position before
+            // jb or jb itself), clamped to what a position of the step can be compared with
+            const uint32_t w = (uint32_t)min(off[idx < n ? idx : n] - jb, (uint64_t)kStep);
+            const uint32_t w31 = __shfl_sync(kFullMask, w, 31);
 #pragma unroll
             for (uint32_t t = 0; t < kWalkU; ++t) {
+                const uint32_t e = lane + 32 * t;
                 uint32_t c = 0;
 #pragma unroll
                 for (uint32_t step = 16; step > 0; step >>= 1) {
-                    const uint64_t wv = __shfl_sync(kFullMask, w, c + step - 1);
-                    if (wv <= j[t]) c += step;
+                    const uint32_t wv = __shfl_sync(kFullMask, w, c + step - 1);
+                    if (wv <= e) c += step;
                 }
-                if (c == 31 && w31 <= j[t]) c = 32;
+                if (c == 31 && w31 <= e) c = 32;
                 if (!(done >> t & 1u) && c < 32) {
                     owner[t] = base + c;
                     done |= 1u << t;
