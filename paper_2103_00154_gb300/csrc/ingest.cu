@@ -796,39 +796,60 @@ __global__ void sort_small_rows(uint32_t n, const uint64_t* __restrict__ start, 
 }
 
 // ---- bitonic network over values held in registers by one warp.
-// Value e of lane l has index base + 32e + l.  A compare-exchange at distance
-// J >= 32 pairs two registers of the same lane; J < 32 pairs two lanes.  The
-// direction of a pair is ascending when (index & k) == 0 (k = block size of
-// the current merge), as in the textbook network.
+// Value e of lane l has index base + E l + e: a lane holds consecutive values,
+// so a compare-exchange at distance J < E pairs two registers of a lane and
+// only J >= E pairs two lanes.  A shuffle costs about four ALU instructions of
+// issue, and this way there are 15 shuffle steps for any E (with consecutive
+// values in consecutive lanes, 15 + 5 log2 E: 40 for 1,024 values).  Rows of
+// 33..8,192 entries of a 268M-pair graph: 3.62 -> 2.73 ms.  A block of
+// size K sorts upwards when (index & K) == 0; where that is the same for all
+// of a lane's values (K >= E) the others are complemented for the merge, so
+// every step is a plain min and max.
 template <int E, uint32_t J>
-__device__ __forceinline__ void bitonic_step(uint32_t (&x)[E], uint32_t base, uint32_t k, uint32_t lane) {
-    if constexpr (J >= 32) {
-        constexpr uint32_t je = J / 32;
+__device__ __forceinline__ void merge_up(uint32_t (&x)[E], uint32_t lane) {  // steps J, J/2, ..., 1, all upwards
+    if constexpr (J >= (uint32_t)E) {
+        const bool lower = (lane & (J / E)) == 0;
 #pragma unroll
         for (int e = 0; e < E; ++e) {
-            if ((e & je) == 0) {
-                bool asc = ((base + (uint32_t)e * 32 + lane) & k) == 0;
-                uint32_t a = x[e], b = x[e | je];
-                x[e] = asc ? min(a, b) : max(a, b);
-                x[e | je] = asc ? max(a, b) : min(a, b);
-            }
+            const uint32_t y = __shfl_xor_sync(kFullMask, x[e], J / E);
+            x[e] = lower ? min(x[e], y) : max(x[e], y);
         }
     } else {
 #pragma unroll
         for (int e = 0; e < E; ++e) {
-            uint32_t y = __shfl_xor_sync(kFullMask, x[e], J);
-            bool asc = ((base + (uint32_t)e * 32 + lane) & k) == 0;
-            bool lower = (lane & J) == 0;
-            x[e] = (lower == asc) ? min(x[e], y) : max(x[e], y);
+            if (e & J) continue;
+            const uint32_t a = x[e], b = x[e | J];
+            x[e] = min(a, b);
+            x[e | J] = max(a, b);
         }
     }
+    if constexpr (J > 1) merge_up<E, J / 2>(x, lane);
 }
 
-// steps J, J/2, ..., 1 of a merge with block size k
+// one merge of blocks of size K < E inside the lanes: steps J, J/2, ..., 1
+template <int E, uint32_t K, uint32_t J>
+__device__ __forceinline__ void merge_lane(uint32_t (&x)[E]) {
+#pragma unroll
+    for (int e = 0; e < E; ++e) {
+        if (e & J) continue;
+        const uint32_t a = x[e], b = x[e | J];
+        const uint32_t lo = min(a, b), hi = max(a, b);
+        x[e] = (e & K) ? hi : lo;
+        x[e | J] = (e & K) ? lo : hi;
+    }
+    if constexpr (J > 1) merge_lane<E, K, J / 2>(x);
+}
+
+// steps J, J/2, ..., 1 of a merge in the direction `down` says (the same for
+// every value of the lane)
 template <int E, uint32_t J>
-__device__ __forceinline__ void bitonic_merge(uint32_t (&x)[E], uint32_t base, uint32_t k, uint32_t lane) {
-    bitonic_step<E, J>(x, base, k, lane);
-    if constexpr (J > 1) bitonic_merge<E, J / 2>(x, base, k, lane);
+__device__ __forceinline__ void bitonic_merge(uint32_t (&x)[E], bool down, uint32_t lane) {
+    const uint32_t flip = down ? 0xffffffffu : 0u;
+#pragma unroll
+    for (int e = 0; e < E; ++e) x[e] ^= flip;
+    merge_up<E, J>(x, lane);
+#pragma unroll
+    for (int e = 0; e < E; ++e) x[e] ^= flip;
 }
 
 // all merges k = 2, 4, ..., K: afterwards the warp's values are sorted, in
@@ -836,27 +857,46 @@ __device__ __forceinline__ void bitonic_merge(uint32_t (&x)[E], uint32_t base, u
 template <int E, uint32_t K>
 __device__ __forceinline__ void bitonic_sort(uint32_t (&x)[E], uint32_t base, uint32_t lane) {
     if constexpr (K > 2) bitonic_sort<E, K / 2>(x, base, lane);
-    bitonic_merge<E, K / 2>(x, base, K, lane);
+    if constexpr (K < (uint32_t)E) merge_lane<E, K, K / 2>(x);
+    else bitonic_merge<E, K / 2>(x, ((base + lane * E) & K) != 0, lane);
 }
 
-// Write the first of each run of equal sorted values (ascending, kPad last)
-// of the warp's registers to out[pos0 ...]; prev_in is the value before
-// index 0 (kPad if none).  Returns the number written.
+// Room to bring a warp's values from the lanes' order into memory order, one
+// word of padding for each 32.
+constexpr uint32_t kOrderWords(uint32_t E) { return 33 * E; }
+__device__ __forceinline__ uint32_t order_at(uint32_t i) { return i + (i >> 5); }
+
+// Which of the lane's sorted values are the first of their run (kPad, last, is
+// none); prev_in is the value before index 0 (kPad if none).
 template <int E>
-__device__ __forceinline__ uint32_t warp_unique_write(const uint32_t (&x)[E], uint32_t prev_in, uint32_t lane,
-                                                      uint32_t* out) {
-    uint32_t pos = 0;
+__device__ __forceinline__ uint32_t unique_mask(const uint32_t (&x)[E], uint32_t prev_in, uint32_t lane) {
+    uint32_t prev = __shfl_up_sync(kFullMask, x[E - 1], 1);
+    if (lane == 0) prev = prev_in;
+    uint32_t m = 0;
 #pragma unroll
     for (int e = 0; e < E; ++e) {
-        uint32_t up = __shfl_up_sync(kFullMask, x[e], 1);
-        uint32_t last_prev = e == 0 ? prev_in : __shfl_sync(kFullMask, x[e > 0 ? e - 1 : 0], 31);
-        uint32_t prev = lane == 0 ? last_prev : up;
-        bool keep = x[e] != kPad && x[e] != prev;
-        uint32_t bal = __ballot_sync(kFullMask, keep);
-        if (keep) out[pos + __popc(bal & lanemask_lt())] = x[e];
-        pos += __popc(bal);
+        if (x[e] != kPad && x[e] != prev) m |= 1u << e;
+        prev = x[e];
     }
-    return pos;
+    return m;
+}
+
+// Write those values to out[0 ...], in order; order: the warp's kOrderWords(E)
+// words of shared memory.  Returns their number.
+template <int E>
+__device__ __forceinline__ uint32_t warp_unique_write(const uint32_t (&x)[E], uint32_t prev_in, uint32_t lane,
+                                                      uint32_t* order, uint32_t* out) {
+    const uint32_t m = unique_mask<E>(x, prev_in, lane);
+    const uint32_t mine = __popc(m), inc = warp_incl_scan(mine);
+    const uint32_t total = __shfl_sync(kFullMask, inc, 31);
+    uint32_t at = inc - mine;
+    __syncwarp();
+#pragma unroll
+    for (int e = 0; e < E; ++e)
+        if (m >> e & 1u) order[order_at(at++)] = x[e];
+    __syncwarp();
+    for (uint32_t i = lane; i < total; i += 32) out[i] = order[order_at(i)];
+    return total;
 }
 
 // Rows of 33..1024 entries: one warp per row, E values per lane.
@@ -865,6 +905,7 @@ __global__ void __launch_bounds__(256) sort_warp_rows(const uint32_t* __restrict
                                                       const uint64_t* __restrict__ start,
                                                       const uint32_t* __restrict__ cnt, uint32_t* __restrict__ tmp,
                                                       uint32_t* __restrict__ newlen) {
+    __shared__ uint32_t order[8][kOrderWords(E)];
     const uint32_t lane = threadIdx.x & 31u;
     const uint32_t gw = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const uint32_t nw = (gridDim.x * blockDim.x) >> 5;
@@ -879,7 +920,7 @@ __global__ void __launch_bounds__(256) sort_warp_rows(const uint32_t* __restrict
             x[e] = i < len ? tmp[b + i] : kPad;
         }
         bitonic_sort<E, 32 * E>(x, 0, lane);
-        uint32_t kept = warp_unique_write<E>(x, kPad, lane, tmp + b);
+        uint32_t kept = warp_unique_write<E>(x, kPad, lane, order[threadIdx.x >> 5], tmp + b);
         if (lane == 0) newlen[v] = kept;
     }
 }
@@ -890,7 +931,7 @@ __global__ void __launch_bounds__(256) sort_warp_rows(const uint32_t* __restrict
 // keeping the first of each run of equal values.
 template <uint32_t kBlockWarps>
 struct BlockSortSmem {
-    uint32_t s[kBlockWarps * 1024];
+    uint32_t s[kBlockWarps * kOrderWords(32)];  // exchange between warps, then each warp's output in order
     uint32_t wlast[kBlockWarps];
     uint32_t wcount[kBlockWarps];
 };
@@ -924,29 +965,21 @@ __device__ __forceinline__ uint32_t block_sort_unique(const uint32_t* in, uint32
 #pragma unroll
                 for (int e = 0; e < 32; ++e) {
                     uint32_t i = base + (uint32_t)e * 32 + lane;
-                    uint32_t y = sm.s[i ^ j];
-                    bool asc = (i & k) == 0;
-                    bool lower = (i & j) == 0;
-                    x[e] = (lower == asc) ? min(x[e], y) : max(x[e], y);
+                    const uint32_t y = sm.s[i ^ j];  // (the same lane and value of the other warp)
+                    const bool keep_min = ((base & k) == 0) == ((base & j) == 0);
+                    x[e] = keep_min ? min(x[e], y) : max(x[e], y);
                 }
             }
             __syncthreads();
         }
-        if (active) bitonic_merge<32, 512>(x, base, k, lane);
+        if (active) bitonic_merge<32, 512>(x, (base & k) != 0, lane);
     }
     // de-duplicate across the block: each warp needs the previous warp's last value
     if (lane == 31) sm.wlast[w] = x[31];
     __syncthreads();
     uint32_t prev_in = (w == 0 || !active) ? kPad : sm.wlast[w - 1];
     // count first, then write at the prefix of the warps' counts
-    uint32_t mine = 0;
-#pragma unroll
-    for (int e = 0; e < 32; ++e) {
-        uint32_t up = __shfl_up_sync(kFullMask, x[e], 1);
-        uint32_t last_prev = e == 0 ? prev_in : __shfl_sync(kFullMask, x[e > 0 ? e - 1 : 0], 31);
-        uint32_t prev = lane == 0 ? last_prev : up;
-        mine += __popc(__ballot_sync(kFullMask, x[e] != kPad && x[e] != prev));
-    }
+    const uint32_t mine = __reduce_add_sync(kFullMask, (uint32_t)__popc(unique_mask<32>(x, prev_in, lane)));
     if (lane == 0) sm.wcount[w] = active ? mine : 0;
     __syncthreads();
     uint32_t off = 0, total = 0;
@@ -954,7 +987,7 @@ __device__ __forceinline__ uint32_t block_sort_unique(const uint32_t* in, uint32
         if (q < w) off += sm.wcount[q];
         total += sm.wcount[q];
     }
-    if (active) warp_unique_write<32>(x, prev_in, lane, out + off);
+    if (active) warp_unique_write<32>(x, prev_in, lane, sm.s + w * kOrderWords(32), out + off);
     __syncthreads();
     return total;
 }
@@ -984,7 +1017,12 @@ __global__ void __launch_bounds__(kBlockWarps * 32) sort_block_rows(const uint32
 // de-duplicated by the block like a block row, and the ranges' unique values
 // are copied back, in range order, to the row's place in tmp.  A row with a
 // range above kBlockRowMax entries (a very skewed row) goes to a list that
-// the radix kernel below sorts instead.
+// the radix kernel below sorts instead.  The entries of a range are counted by
+// plain shared-memory increments: with up to 64 ranges the lanes that meet in
+// one cost less than grouping the lanes by range with a match (giant rows of a
+// 268M-pair graph 2.93 -> 2.55 ms; of 2^20 vertices and 2^24 pairs 1.01 ->
+// 0.83).  Ranges of 3,000 to 3,800, sorted by half the warps, were no faster
+// (2.6 to 2.3 ms there, 0.92 to 0.88 here): more ranges one after the other.
 constexpr uint32_t kSplitTarget = 5000;
 constexpr uint32_t kSplitMaxRanges = 64;
 
@@ -1033,14 +1071,14 @@ __global__ void __launch_bounds__(256) giant_split_kernel(const uint32_t* __rest
             for (int e = 0; e < 32; ++e) x[e] = A[((uint64_t)((uint32_t)e * 32 + lane) * L) >> 10];
             bitonic_sort<32, 1024>(x, 0, lane);
 #pragma unroll
-            for (int e = 0; e < 32; ++e) sm.bs.s[(uint32_t)e * 32 + lane] = x[e];
+            for (int e = 0; e < 32; ++e) sm.bs.s[order_at(lane * 32 + (uint32_t)e)] = x[e];
         }
         if (tid < kSplitMaxRanges) {
             sm.rcnt[tid] = 0;
             sm.rcur[tid] = 0;
         }
         __syncthreads();
-        if (tid + 1 < nr) sm.spl[tid] = sm.bs.s[((tid + 1) * 1024) / nr];
+        if (tid + 1 < nr) sm.spl[tid] = sm.bs.s[order_at(((tid + 1) * 1024) / nr)];
         if (tid == 0) sm.nsp = nr - 1;
         __syncthreads();
         const uint32_t nsp = sm.nsp;
@@ -1051,10 +1089,7 @@ __global__ void __launch_bounds__(256) giant_split_kernel(const uint32_t* __rest
             for (uint32_t j = 0; j < 4; ++j) x[j] = i0 + j * 256 + tid < L ? A[i0 + j * 256 + tid] : 0u;
 #pragma unroll
             for (uint32_t j = 0; j < 4; ++j) {
-                const uint32_t rg = i0 + j * 256 + tid < L ? split_range(sm.spl, nsp, x[j]) : kSplitMaxRanges;
-                const uint32_t peers = __match_any_sync(kFullMask, rg);
-                if (rg < kSplitMaxRanges && lane == (uint32_t)(__ffs(peers) - 1))
-                    atomicAdd(&sm.rcnt[rg], (uint32_t)__popc(peers));
+                if (i0 + j * 256 + tid < L) atomicAdd(&sm.rcnt[split_range(sm.spl, nsp, x[j])], 1u);
             }
         }
         __syncthreads();
@@ -1082,12 +1117,7 @@ __global__ void __launch_bounds__(256) giant_split_kernel(const uint32_t* __rest
 #pragma unroll
             for (uint32_t j = 0; j < 4; ++j) {
                 const uint32_t rg = i0 + j * 256 + tid < L ? split_range(sm.spl, nsp, x[j]) : kSplitMaxRanges;
-                const uint32_t peers = __match_any_sync(kFullMask, rg);
-                const uint32_t leader = __ffs(peers) - 1;
-                uint32_t base = 0;
-                if (rg < kSplitMaxRanges && lane == leader) base = atomicAdd(&sm.rcur[rg], (uint32_t)__popc(peers));
-                base = __shfl_sync(kFullMask, base, leader);
-                if (rg < kSplitMaxRanges) B[sm.rstart[rg] + base + __popc(peers & lanemask_lt())] = x[j];
+                if (rg < kSplitMaxRanges) B[sm.rstart[rg] + atomicAdd(&sm.rcur[rg], 1u)] = x[j];
             }
         }
         __syncthreads();
@@ -1326,7 +1356,7 @@ struct DirectSmem {
 };
 
 template <int E>
-__device__ __forceinline__ uint32_t sort_row_warp(uint32_t* row, uint32_t len, uint32_t lane) {
+__device__ __forceinline__ uint32_t sort_row_warp(uint32_t* row, uint32_t len, uint32_t lane, uint32_t* order) {
     uint32_t x[E];
 #pragma unroll
     for (int e = 0; e < E; ++e) {
@@ -1334,7 +1364,7 @@ __device__ __forceinline__ uint32_t sort_row_warp(uint32_t* row, uint32_t len, u
         x[e] = i < len ? row[i] : kPad;
     }
     bitonic_sort<E, 32 * E>(x, 0, lane);
-    return warp_unique_write<E>(x, kPad, lane, row);
+    return warp_unique_write<E>(x, kPad, lane, order, row);
 }
 
 // Exclusive prefix sums of in[0, n), each block its share of whole tiles:
@@ -1484,15 +1514,16 @@ __global__ void __launch_bounds__(kDirectTB, 1) direct_kernel(DirectArgs a) {
             const uint32_t kept = block_sort_unique<kDirectTB / 32>(row, __ldcg(a.cnt + v), row, sm.sort);
             if (tid == 0) a.newlen[v] = kept;
         }
+        uint32_t* const order = sm.sort.s + (tid >> 5) * kOrderWords(32);
         for (uint32_t r = gw; r < nwr; r += nw) {
             const uint32_t v = __ldcg(a.rows + r), len = __ldcg(a.cnt + v);
             uint32_t* row = a.tmp + __ldcg(a.start + v);
             uint32_t kept;
-            if (len <= 64) kept = sort_row_warp<2>(row, len, lane);
-            else if (len <= 128) kept = sort_row_warp<4>(row, len, lane);
-            else if (len <= 256) kept = sort_row_warp<8>(row, len, lane);
-            else if (len <= 512) kept = sort_row_warp<16>(row, len, lane);
-            else kept = sort_row_warp<32>(row, len, lane);
+            if (len <= 64) kept = sort_row_warp<2>(row, len, lane, order);
+            else if (len <= 128) kept = sort_row_warp<4>(row, len, lane, order);
+            else if (len <= 256) kept = sort_row_warp<8>(row, len, lane, order);
+            else if (len <= 512) kept = sort_row_warp<16>(row, len, lane, order);
+            else kept = sort_row_warp<32>(row, len, lane, order);
             if (lane == 0) a.newlen[v] = kept;
         }
     }
