@@ -378,29 +378,25 @@ __device__ __forceinline__ void scan_block_list(const uint64_t* __restrict__ off
 }
 
 // scan_block_list over rows whose starts and lengths are already known:
-// rows F[0, cnt) with row starts B[] and lengths L[].
-template <int TB, class Fn>
-__device__ __forceinline__ void scan_block_rows(const uint32_t* __restrict__ adj, const uint32_t* F,
-                                                const uint64_t* B, const uint32_t* L, uint32_t cnt_all,
+// row(i, v, beg, len) gives row i of cnt_all (its thread's, once; a row left
+// out has length 0).
+template <int TB, class Row, class Fn>
+__device__ __forceinline__ void scan_block_rows(const uint32_t* __restrict__ adj, uint32_t cnt_all, Row row,
                                                 BlockTile<TB>& sm, Fn& fn) {
     const uint32_t tid = threadIdx.x;
     for (uint32_t t = 0; t < cnt_all; t += TB) {
         const uint32_t cnt = min((uint32_t)TB, cnt_all - t);
         uint32_t v = 0, len = 0;
         uint64_t b = 0;
-        if (tid < cnt) {
-            v = F[t + tid];
-            b = B[t + tid];
-            len = L[t + tid];
-        }
+        if (tid < cnt) row(t + tid, v, b, len);
         uint32_t total;
         const uint32_t st = block_excl_scan<uint32_t>(len, sm.scan_tmp, &total);
         sm.start[tid] = st;
         sm.beg[tid] = b;
         sm.v[tid] = v;
         __syncthreads();
-        for (uint32_t e0 = tid; e0 < total; e0 += kBatch * TB) {
-            uint32_t bu[kBatch], bv[kBatch], valid = 0;
+        auto fetch = [&](uint32_t e0, uint32_t (&bu)[kBatch], uint32_t (&bv)[kBatch]) {
+            uint32_t valid = 0;
 #pragma unroll
             for (uint32_t j = 0; j < kBatch; ++j) {
                 const uint32_t e = e0 + j * TB;
@@ -417,6 +413,11 @@ __device__ __forceinline__ void scan_block_rows(const uint32_t* __restrict__ adj
                     valid |= 1u << j;
                 }
             }
+            return valid;
+        };
+        for (uint32_t e0 = tid; e0 < total; e0 += kBatch * TB) {
+            uint32_t bu[kBatch], bv[kBatch];
+            const uint32_t valid = fetch(e0, bu, bv);
             fn(bu, bv, valid);
         }
         __syncthreads();

@@ -4,8 +4,8 @@
 //
 // Level k (Alg. 2 first phase):
 //   scan: every block walks its own segment of the remaining vertices; degree
-//     <= k joins the level's frontier (Algorithm 2's per-thread buffer),
-//     degree > k stays in the (compacted) segment;
+//     <= k joins the block's list (Algorithm 2's per-thread buffer), degree > k
+//     stays in the (compacted) segment;
 //   drain: for every frontier vertex v and every neighbour u,
 //     a = atomicSub(deg[u], 1); a == k+1 puts u in the frontier (it just
 //     reached k); a <= k is undone with atomicAdd (u was already at or below
@@ -14,7 +14,8 @@
 //     memory round trip per link of a cascade and leaves the same degrees.
 //     A block drains the rows its scan found
 //     (up to inline_max entries each) and the vertices that reach k while it
-//     drains (rows up to local_max entries, while its local budget lasts:
+//     drains, which it collects and claims between two drains (rows up to
+//     local_max entries, while its local budget lasts:
 //     PKC's thread-local buffer); everything else goes to a level-wide queue
 //     of row pieces (at most chunk_len entries each) that blocks with no
 //     work of their own take from as it comes, so neither hub rows nor
@@ -29,8 +30,15 @@
 //     the next level as soon as it sees that, with no grid barrier;
 //   the count of visited vertices grows by the frontier size (as in Algorithm 2).
 // Scan and drain overlap, so a vertex is taken into the frontier by claiming
-// its bit in a bitmap (atomicOr): whichever of the scan and the decrement that
-// brought it to k claims it first drains it, exactly once.  A scanned degree
+// its bit in a bitmap (atomicOr): whichever of the block that scanned it and
+// the one whose decrement brought it to k claims it first drains it, exactly
+// once.  Both claim as they load the row bounds for a drain, a whole tile of
+// vertices at a time, so the scan itself waits for nothing but the list and
+// the degrees (2^24 vertices, 2^28 pairs: the scans of 103 levels 2.11 -> 1.01
+// ms, the level kernel 9.5 -> 8.3).  What is left is bound by the drains' two
+// random accesses per entry, claim word and degree: 263M edges are taken off
+// by 300M atomics, which alone need 2.2 ms at the rate such atomics were
+// measured to reach (135 10^9/s over 64 MB).  A scanned degree
 // below k can only be such a vertex caught between a decrement and its undo:
 // every vertex whose degree was below k at the level's start was claimed at an
 // earlier level.
@@ -118,9 +126,7 @@ struct CoreArgs {
     uint32_t* claim;  // one bit per vertex: taken into a frontier
     uint32_t* remA;   // per-block segments: the vertices each block's scan keeps
     uint32_t* remB;
-    uint32_t* QA;     // per-block segments: vertices the block's scan claimed ...
-    uint64_t* QB;     // ... their row starts
-    uint32_t* QL;     // ... and row lengths
+    uint32_t* QA;     // per-block segments: vertices of degree <= k the block's scan found
     uint64_t seg;     // segment length per block
     uint32_t* IV;     // level queue (cap slots) of row pieces: row owner ...
     uint64_t* IB;     // ... first entry
@@ -138,11 +144,12 @@ struct CoreArgs {
     uint64_t trace_cap;
 };
 
+constexpr uint32_t kNone = 0xffffffffu;  // no vertex
+
 // Block-local frontier: vertices that reach k while this block drains are
 // drained by the same block (PKC's thread-local buff, Algorithm 2), so a
 // chain of degree-k vertices costs no queue round trip per link.
-template <int TB>
-constexpr uint32_t local_q_cap() { return TB >= 1024 ? 640 : 1024; }
+constexpr uint32_t kLocalQ = 1024;
 
 #ifndef DSG_TAKE_SLOTS
 #define DSG_TAKE_SLOTS 32
@@ -152,12 +159,9 @@ static_assert(kTakeSlots >= 1 && kTakeSlots <= 32, "a block takes 1..32 queue sl
 
 template <int TB>
 struct CoreSmem {
-    static constexpr uint32_t kLocalQ = local_q_cap<TB>();
     TileSmem<TB> tile;
     BlockTile<TB> btile;
-    uint32_t lq[kLocalQ];   // vertices ...
-    uint64_t lqb[kLocalQ];  // ... their row starts
-    uint32_t lql[kLocalQ];  // ... and row lengths
+    uint32_t lq[kLocalQ];   // vertices that reached k, not yet claimed
     uint32_t lq_tail;
     uint32_t lq_work;       // row entries this block has taken on locally in this batch
     uint32_t own;           // vertices this block's scan claimed
@@ -262,8 +266,6 @@ __global__ void __launch_bounds__(TB, TB == 256 ? 3 : 1) kcore_kernel(CoreArgs a
     const uint32_t* my_rem = nullptr;  // level 0: identity
     uint32_t* my_rem_next = a.remA + segoff;
     uint32_t* const myQA = a.QA + segoff;
-    uint64_t* const myQB = a.QB + segoff;
-    uint32_t* const myQL = a.QL + segoff;
     uint64_t visited = 0, level = 0;
     uint32_t* deg = a.deg;
     for (;;) {
@@ -282,25 +284,31 @@ __global__ void __launch_bounds__(TB, TB == 256 ? 3 : 1) kcore_kernel(CoreArgs a
         }
         uint32_t dmn = 0xffffffffu;
         uint64_t claimed = 0, natom = 0, npieces = 0, nscan_claims = 0;
-        // u reached k: drain it in this block if there is room, else queue it
-        // (a scan still running elsewhere may have taken it first)
-        auto reach_k = [&](uint32_t u) {
+        // Claim u, which reached k (a scan still running elsewhere may have taken it first): true if this
+        // block drains its row, which is queued if it is long or the block has enough.
+        auto take = [&](uint32_t u, uint64_t& beg, uint32_t& row_len, auto fits) {
             // the row bounds are loaded alongside the claim (one round trip)
-            const uint64_t beg = a.off[u];
+            beg = a.off[u];
             const uint64_t end = a.off[u + 1];
-            if (!claim_vertex(a.claim, u)) return;
+            if (!claim_vertex(a.claim, u)) return false;
             ++claimed;
             const uint64_t len = end - beg;
-            if (len <= a.local_max && atomicAdd(&sm.lq_work, (uint32_t)len) + len <= a.local_work) {
-                uint32_t pos = atomicAdd(&sm.lq_tail, 1u);
-                if (pos < CoreSmem<TB>::kLocalQ) {
-                    sm.lq[pos] = u;
-                    sm.lqb[pos] = beg;
-                    sm.lql[pos] = (uint32_t)len;
-                    return;
-                }
-            }
+            row_len = (uint32_t)len;
+            if (fits(len)) return true;
             if (len) npieces += queue_row(a, P, tag, u, beg, len);
+            return false;
+        };
+        // u reached k: noted, to be claimed with the block's others between two drains (claiming it at
+        // once would hold the whole warp for a memory round trip at every such vertex)
+        auto reach_k = [&](uint32_t u) {
+            const uint32_t pos = atomicAdd(&sm.lq_tail, 1u);
+            if (pos < kLocalQ) {
+                sm.lq[pos] = u;
+                return;
+            }
+            uint64_t beg;
+            uint32_t len;
+            take(u, beg, len, [](uint64_t) { return false; });
         };
         // one unit was just taken from u's degree, which was old: a degree
         // already at or below k gets it back (Algorithm 2's undo); reaching k
@@ -349,14 +357,22 @@ __global__ void __launch_bounds__(TB, TB == 256 ? 3 : 1) kcore_kernel(CoreArgs a
             for (uint32_t jj = 0; jj < kBatch; ++jj)
                 if (need >> jj & 1u) settle(u[jj], old[jj]);
         };
+        // a row the block drains itself, beside the others it has taken on
+        auto local_room = [&](uint64_t len) {
+            return len <= a.local_max && atomicAdd(&sm.lq_work, (uint32_t)len) + len <= a.local_work;
+        };
         // drain what this block found, until it finds nothing more
         auto local_loop = [&]() {
             for (uint32_t lq_lo = 0;;) {
-                uint32_t lq_hi = min(sm.lq_tail, CoreSmem<TB>::kLocalQ);
+                uint32_t lq_hi = min(sm.lq_tail, kLocalQ);
                 __syncthreads();
                 if (lq_lo >= lq_hi) break;
-                scan_block_rows<TB>(a.adj, sm.lq + lq_lo, sm.lqb + lq_lo, sm.lql + lq_lo, lq_hi - lq_lo, sm.btile,
-                                    visit);
+                scan_block_rows<TB>(a.adj, lq_hi - lq_lo,
+                                    [&](uint32_t i, uint32_t& v, uint64_t& beg, uint32_t& len) {
+                                        v = sm.lq[lq_lo + i];
+                                        if (!take(v, beg, len, local_room)) len = 0;
+                                    },
+                                    sm.btile, visit);
                 lq_lo = lq_hi;
             }
         };
@@ -392,90 +408,48 @@ __global__ void __launch_bounds__(TB, TB == 256 ? 3 : 1) kcore_kernel(CoreArgs a
             sm.acc_pieces = 0;
         }
         __syncthreads();
-        // ---- scan: claim degree <= k, keep degree > k, drop the claimed.
-        // kScanU tiles per step, their loads issued together.
+        // ---- scan: degree <= k joins the block's own list (to be claimed when it is drained: most
+        // are free, the others were taken at an earlier level or by a drain of this one), degree > k
+        // is kept.  kScanU tiles per step, their loads issued together.
         {
-            constexpr uint32_t kScanU = TB >= 1024 ? 2 : 4;  // 1024-thread blocks have 64 registers
+            constexpr uint32_t kScanU = TB >= 1024 ? 4 : 8;  // 1024-thread blocks have 64 registers
             uint32_t mn = 0xffffffffu;
             const uint64_t lim = my_rem ? my_n : n;
             const uint64_t stride = my_rem ? TB : (uint64_t)gridDim.x * TB;
             uint64_t scanned = 0;
             for (uint64_t t = my_rem ? 0 : (uint64_t)blockIdx.x * TB; t < lim; t += kScanU * stride) {
-                uint32_t v[kScanU], dv[kScanU], cw[kScanU];
-                bool in[kScanU];
+                uint32_t v[kScanU], dv[kScanU];
 #pragma unroll
                 for (uint32_t u = 0; u < kScanU; ++u) {
                     const uint64_t i = t + u * stride + tid;
-                    in[u] = i < lim;
-                    v[u] = in[u] ? (my_rem ? my_rem[i] : (uint32_t)i) : 0u;
+                    v[u] = i < lim ? (my_rem ? my_rem[i] : (uint32_t)i) : kNone;
                 }
-                // the degree first; the claim word only where the degree is at or
-                // below k (a vertex taken at an earlier level ended at its core
-                // number, below k, so one above k is never taken)
 #pragma unroll
-                for (uint32_t u = 0; u < kScanU; ++u) dv[u] = in[u] ? deg[v[u]] : 0u;
-#pragma unroll
-                for (uint32_t u = 0; u < kScanU; ++u) cw[u] = (in[u] && dv[u] <= k) ? a.claim[v[u] >> 5] : 0u;
-                bool keep[kScanU], mine[kScanU];
+                for (uint32_t u = 0; u < kScanU; ++u) dv[u] = v[u] != kNone ? deg[v[u]] : kNone;
+                // a warp ballot and one shared-memory atomic per warp, tile and list
 #pragma unroll
                 for (uint32_t u = 0; u < kScanU; ++u) {
-                    keep[u] = false;
-                    mine[u] = false;
-                    if (!in[u]) continue;
-                    ++scanned;
-                    if (cw[u] >> (v[u] & 31u) & 1u) continue;  // taken earlier
-                    if (dv[u] > k) {
-                        keep[u] = true;
+                    const bool in = v[u] != kNone, keep = in && dv[u] > k, mine = in && dv[u] <= k;
+                    const uint32_t kb = __ballot_sync(kFullMask, keep), mb = __ballot_sync(kFullMask, mine);
+                    uint32_t at = 0;
+                    if (lane == 0 && kb) at = atomicAdd(&sm.kept, (uint32_t)__popc(kb));
+                    if (lane == 1 && mb) at = atomicAdd(&sm.own, (uint32_t)__popc(mb));
+                    const uint32_t ka = __shfl_sync(kFullMask, at, 0) + __popc(kb & lanemask_lt());
+                    const uint32_t ma = __shfl_sync(kFullMask, at, 1) + __popc(mb & lanemask_lt());
+                    if (lane == 0) scanned += __popc(kb) + __popc(mb);
+                    if (keep) {
                         mn = min(mn, dv[u]);
-                    } else {
-                        mine[u] = true;  // a candidate: claimed below
-                    }
-                }
-                // row bounds of the candidates, loaded alongside their claims
-                uint64_t beg[kScanU], len[kScanU];
-#pragma unroll
-                for (uint32_t u = 0; u < kScanU; ++u) {
-                    beg[u] = mine[u] ? a.off[v[u]] : 0;
-                    len[u] = mine[u] ? a.off[v[u] + 1] : 0;
-                }
-#pragma unroll
-                for (uint32_t u = 0; u < kScanU; ++u)
-                    if (mine[u]) mine[u] = claim_vertex(a.claim, v[u]);
-#pragma unroll
-                for (uint32_t u = 0; u < kScanU; ++u) {
-                    if (!mine[u]) continue;
-                    ++claimed;
-                    ++nscan_claims;
-                    const uint64_t ln = len[u] - beg[u];
-                    // drained by this block, or, for rows above inline_max,
-                    // queued in pieces for every block
-                    if (ln <= a.inline_max) {
-                        uint32_t pos = atomicAdd(&sm.own, 1u);
-                        DSG_BOUND(ctl, 5, pos, a.seg, level, pos = 0);
-                        myQA[pos] = v[u];
-                        myQB[pos] = beg[u];
-                        myQL[pos] = (uint32_t)ln;
-                    } else {
-                        npieces += queue_row(a, P, tag, v[u], beg[u], ln);
-                    }
-                }
-                // keep: warp ballot, one shared-memory atomic per warp and tile
-#pragma unroll
-                for (uint32_t u = 0; u < kScanU; ++u) {
-                    const uint32_t bal = __ballot_sync(kFullMask, keep[u]);
-                    uint32_t base = 0;
-                    if (lane == 0 && bal) base = atomicAdd(&sm.kept, (uint32_t)__popc(bal));
-                    base = __shfl_sync(kFullMask, base, 0);
-                    if (keep[u]) {
-                        uint64_t at = base + __popc(bal & lanemask_lt());
                         bool ok = true;
-                        DSG_BOUND(ctl, 3, at, a.seg, level, ok = false);
-                        if (ok) my_rem_next[at] = v[u];
+                        DSG_BOUND(ctl, 3, ka, a.seg, level, ok = false);
+                        if (ok) my_rem_next[ka] = v[u];
+                    } else if (mine) {
+                        bool ok = true;
+                        DSG_BOUND(ctl, 5, ma, a.seg, level, ok = false);
+                        if (ok) myQA[ma] = v[u];
                     }
                 }
             }
             dmn = min(dmn, mn);
-            scanned = warp_sum(scanned);
             if (lane == 0 && scanned) atomicAdd(&ctl->rem_scanned, (unsigned long long)scanned);
         }
         __syncthreads();
@@ -483,7 +457,14 @@ __global__ void __launch_bounds__(TB, TB == 256 ? 3 : 1) kcore_kernel(CoreArgs a
         // ---- drain what this block's scan claimed, and what that leads to locally
         {
             const uint32_t own = (uint32_t)min((uint64_t)sm.own, a.seg);
-            scan_block_rows<TB>(a.adj, myQA, myQB, myQL, own, sm.btile, visit);
+            scan_block_rows<TB>(a.adj, own,
+                                [&](uint32_t i, uint32_t& v, uint64_t& beg, uint32_t& len) {
+                                    v = myQA[i];
+                                    const uint64_t was = claimed;
+                                    if (!take(v, beg, len, [&](uint64_t l) { return l <= a.inline_max; })) len = 0;
+                                    nscan_claims += claimed - was;
+                                },
+                                sm.btile, visit);
             local_loop();
         }
         // the block adds nothing more except from queue pieces: give back its token
@@ -541,7 +522,13 @@ __global__ void __launch_bounds__(TB, TB == 256 ? 3 : 1) kcore_kernel(CoreArgs a
                 __syncthreads();
                 const uint32_t got = sm.tcount;
                 if (got) {
-                    scan_block_rows<TB>(a.adj, sm.tv, sm.tb, sm.tl, got, sm.btile, visit);
+                    scan_block_rows<TB>(a.adj, got,
+                                        [&](uint32_t i, uint32_t& v, uint64_t& beg, uint32_t& len) {
+                                            v = sm.tv[i];
+                                            beg = sm.tb[i];
+                                            len = sm.tl[i];
+                                        },
+                                        sm.btile, visit);
                     local_loop();
                     // drained, and whatever they queued is counted: publish, then give them back
                     publish();
@@ -706,8 +693,6 @@ dsg_status run_kcore(const dsg_graph* g, uint32_t* core_out, uint64_t* stats, ui
     DSG_TRY_CUDA(sc.get(&a.remA, a.seg * grid));
     DSG_TRY_CUDA(sc.get(&a.remB, a.seg * grid));
     DSG_TRY_CUDA(sc.get(&a.QA, a.seg * grid));
-    DSG_TRY_CUDA(sc.get(&a.QB, a.seg * grid));
-    DSG_TRY_CUDA(sc.get(&a.QL, a.seg * grid));
     DSG_TRY_CUDA(sc.get(&a.IV, a.cap));
     DSG_TRY_CUDA(sc.get(&a.IB, a.cap));
     DSG_TRY_CUDA(sc.get(&a.IL, a.cap));
