@@ -1021,31 +1021,39 @@ __global__ void __launch_bounds__(kBlockWarps * 32) sort_block_rows(const uint32
     }
 }
 
-// ---- giant rows (> kBlockRowMax entries), one block of 8 warps per row:
-// splitters taken from a sorted sample of the row (1,024 values spread over
-// it) cut its values into ranges of about kSplitTarget entries; the row is
-// counted and scattered by range into the spare buffer (equal values share a
-// range, so no run of equal ids crosses two ranges), each range is sorted and
-// de-duplicated by the block like a block row, and the ranges' unique values
-// are copied back, in range order, to the row's place in tmp.  A row with a
-// range above kBlockRowMax entries (a very skewed row) goes to a list that
-// the radix kernel below sorts instead.  The entries of a range are counted by
-// plain shared-memory increments: with up to 64 ranges the lanes that meet in
-// one cost less than grouping the lanes by range with a match (giant rows of a
-// 268M-pair graph 2.93 -> 2.55 ms; of 2^20 vertices and 2^24 pairs 1.01 ->
-// 0.83).  Ranges of 3,000 to 3,800, sorted by half the warps, were no faster
-// (2.6 to 2.3 ms there, 0.92 to 0.88 here): more ranges one after the other.
+// ---- giant rows (> kBlockRowMax entries), in three launches.  Split: one
+// block per row takes splitters from a sorted sample of the row (1,024 values
+// spread over it) that cut its values into ranges of about kSplitTarget
+// entries, counts the row by range and scatters it by range into the spare
+// buffer (equal values share a range, so no run of equal ids crosses two
+// ranges).  Sort: each range of any row is a block's task, sorted and
+// de-duplicated like a block row.  Copy: the ranges' unique values go back, in
+// range order, to the row's place in tmp.  A row with a range above
+// kBlockRowMax entries (a very skewed row) goes to a list that the radix
+// kernel below sorts instead.  (With a row's ranges sorted one after the other
+// by the block that split it, the longest row set the time: rows of a graph of
+// 2^20 vertices and 2^24 pairs 0.83 -> 0.23 ms, of 2^24 and 2^28 2.4 -> 2.2.)
+// The entries of a range are counted by plain shared-memory increments: with
+// up to 64 ranges the lanes that meet in one cost less than grouping the lanes
+// by range with a match (2.93 -> 2.55 ms and 1.01 -> 0.83 then).  Ranges of
+// 3,000 to 3,800, sorted by half the warps, were no faster.
 constexpr uint32_t kSplitTarget = 5000;
 constexpr uint32_t kSplitMaxRanges = 64;
+constexpr uint32_t kSplitTB = 1024;
+
+struct SplitRow {                          // what the later launches need of a split row
+    uint32_t nr;                           // ranges
+    uint32_t start[kSplitMaxRanges + 1];   // first slot of each range
+    uint32_t kept[kSplitMaxRanges];        // unique values of each
+};
 
 struct SplitSmem {
-    BlockSortSmem<8> bs;
+    uint32_t sample[kOrderWords(32)];
     uint32_t spl[kSplitMaxRanges];         // splitters: range of x = number of splitters <= x
     uint32_t rcnt[kSplitMaxRanges];        // entries per range ...
     uint32_t rcur[kSplitMaxRanges];        // ... scatter cursors ...
     uint32_t rstart[kSplitMaxRanges + 1];  // ... first slot of each range
-    uint32_t kept[kSplitMaxRanges + 1];    // unique values per range, then their exclusive prefix
-    uint32_t row, nsp, too_big;
+    uint32_t row, too_big, task0;
 };
 
 __device__ __forceinline__ uint32_t split_range(const uint32_t* spl, uint32_t nsp, uint32_t x) {
@@ -1057,25 +1065,27 @@ __device__ __forceinline__ uint32_t split_range(const uint32_t* spl, uint32_t ns
     return lo;
 }
 
-__global__ void __launch_bounds__(256) giant_split_kernel(const uint32_t* __restrict__ list, uint32_t count,
-                                                          const uint64_t* __restrict__ start,
-                                                          const uint32_t* __restrict__ cnt, uint32_t* __restrict__ tmp,
-                                                          uint32_t* __restrict__ spare, uint32_t* __restrict__ newlen,
-                                                          uint32_t* __restrict__ ticket,
-                                                          uint32_t* __restrict__ skewed, uint32_t* __restrict__ nskewed) {
+// ctr: [0] rows taken, [1] skewed rows listed, [3] tasks listed (row * kSplitMaxRanges + range)
+__global__ void __launch_bounds__(kSplitTB) giant_split_kernel(const uint32_t* __restrict__ list, uint32_t count,
+                                                               const uint64_t* __restrict__ start,
+                                                               const uint32_t* __restrict__ cnt,
+                                                               const uint32_t* __restrict__ tmp,
+                                                               uint32_t* __restrict__ spare,
+                                                               SplitRow* __restrict__ rows, uint32_t* __restrict__ tasks,
+                                                               uint32_t* __restrict__ skewed, uint32_t* ctr) {
     __shared__ SplitSmem sm;
     const uint32_t tid = threadIdx.x, lane = tid & 31u, w = tid >> 5;
     for (;;) {
         __syncthreads();
-        if (tid == 0) sm.row = atomicAdd(ticket, 1u);
+        if (tid == 0) sm.row = atomicAdd(&ctr[0], 1u);
         __syncthreads();
         const uint32_t r = sm.row;
         if (r >= count) break;
         const uint32_t v = list[r];
         const uint32_t L = cnt[v];
-        uint32_t* A = tmp + start[v];
+        const uint32_t* A = tmp + start[v];
         uint32_t* B = spare + start[v];
-        const uint32_t nr = min(kSplitMaxRanges, (L + kSplitTarget - 1) / kSplitTarget);
+        const uint32_t nr = min(kSplitMaxRanges, (L + kSplitTarget - 1) / kSplitTarget), nsp = nr - 1;
         // ---- the sample, sorted by warp 0; splitters at its nr-quantiles
         if (w == 0) {
             uint32_t x[32];
@@ -1083,85 +1093,97 @@ __global__ void __launch_bounds__(256) giant_split_kernel(const uint32_t* __rest
             for (int e = 0; e < 32; ++e) x[e] = A[((uint64_t)((uint32_t)e * 32 + lane) * L) >> 10];
             bitonic_sort<32, 1024>(x, 0, lane);
 #pragma unroll
-            for (int e = 0; e < 32; ++e) sm.bs.s[order_at(lane * 32 + (uint32_t)e)] = x[e];
-        }
-        if (tid < kSplitMaxRanges) {
-            sm.rcnt[tid] = 0;
-            sm.rcur[tid] = 0;
+            for (int e = 0; e < 32; ++e) sm.sample[order_at(lane * 32 + (uint32_t)e)] = x[e];
+        } else if (w == 1) {
+            for (uint32_t i = lane; i < kSplitMaxRanges; i += 32) sm.rcnt[i] = sm.rcur[i] = 0;
         }
         __syncthreads();
-        if (tid + 1 < nr) sm.spl[tid] = sm.bs.s[order_at(((tid + 1) * 1024) / nr)];
-        if (tid == 0) sm.nsp = nr - 1;
+        if (tid < nsp) sm.spl[tid] = sm.sample[order_at(((tid + 1) * 1024) / nr)];
         __syncthreads();
-        const uint32_t nsp = sm.nsp;
         // ---- entries per range
-        for (uint32_t i0 = 0; i0 < L; i0 += 4 * 256) {
+        for (uint32_t i0 = 0; i0 < L; i0 += 4 * kSplitTB) {
             uint32_t x[4];
 #pragma unroll
-            for (uint32_t j = 0; j < 4; ++j) x[j] = i0 + j * 256 + tid < L ? A[i0 + j * 256 + tid] : 0u;
+            for (uint32_t j = 0; j < 4; ++j) x[j] = i0 + j * kSplitTB + tid < L ? A[i0 + j * kSplitTB + tid] : 0u;
 #pragma unroll
-            for (uint32_t j = 0; j < 4; ++j) {
-                if (i0 + j * 256 + tid < L) atomicAdd(&sm.rcnt[split_range(sm.spl, nsp, x[j])], 1u);
-            }
+            for (uint32_t j = 0; j < 4; ++j)
+                if (i0 + j * kSplitTB + tid < L) atomicAdd(&sm.rcnt[split_range(sm.spl, nsp, x[j])], 1u);
         }
         __syncthreads();
         if (w == 0) {
-            const uint32_t c0 = lane < nr ? sm.rcnt[lane] : 0u, c1 = lane + 32 < nr ? sm.rcnt[lane + 32] : 0u;
+            const uint32_t c0 = sm.rcnt[lane], c1 = sm.rcnt[lane + 32];  // 0 past nr
             const uint32_t i0 = warp_incl_scan(c0), i1 = warp_incl_scan(c1);
             const uint32_t t0 = __shfl_sync(kFullMask, i0, 31);
-            const uint32_t tot = t0 + __shfl_sync(kFullMask, i1, 31);
             sm.rstart[lane] = i0 - c0;
             sm.rstart[lane + 32] = t0 + i1 - c1;
-            if (lane == 0) sm.rstart[kSplitMaxRanges] = tot;
+            if (lane == 0) sm.rstart[kSplitMaxRanges] = L;
             const uint32_t big = __ballot_sync(kFullMask, c0 > kBlockRowMax || c1 > kBlockRowMax);
-            if (lane == 0) sm.too_big = big != 0;
+            if (lane == 0) {
+                sm.too_big = big != 0;
+                if (big) skewed[atomicAdd(&ctr[1], 1u)] = v;
+                else sm.task0 = atomicAdd(&ctr[3], nr);
+            }
         }
         __syncthreads();
-        if (sm.too_big) {
-            if (tid == 0) skewed[atomicAdd(nskewed, 1u)] = v;
-            continue;
-        }
+        if (sm.too_big) continue;
+        if (tid <= nr) rows[r].start[tid] = sm.rstart[tid];
+        if (tid < nr) tasks[sm.task0 + tid] = r * kSplitMaxRanges + tid;
+        if (tid == 0) rows[r].nr = nr;
         // ---- scatter by range (order inside a range does not matter: it is sorted next)
-        for (uint32_t i0 = 0; i0 < L; i0 += 4 * 256) {
+        for (uint32_t i0 = 0; i0 < L; i0 += 4 * kSplitTB) {
             uint32_t x[4];
 #pragma unroll
-            for (uint32_t j = 0; j < 4; ++j) x[j] = i0 + j * 256 + tid < L ? A[i0 + j * 256 + tid] : 0u;
+            for (uint32_t j = 0; j < 4; ++j) x[j] = i0 + j * kSplitTB + tid < L ? A[i0 + j * kSplitTB + tid] : 0u;
 #pragma unroll
             for (uint32_t j = 0; j < 4; ++j) {
-                const uint32_t rg = i0 + j * 256 + tid < L ? split_range(sm.spl, nsp, x[j]) : kSplitMaxRanges;
-                if (rg < kSplitMaxRanges) B[sm.rstart[rg] + atomicAdd(&sm.rcur[rg], 1u)] = x[j];
+                if (i0 + j * kSplitTB + tid >= L) continue;
+                const uint32_t rg = split_range(sm.spl, nsp, x[j]);
+                B[sm.rstart[rg] + atomicAdd(&sm.rcur[rg], 1u)] = x[j];
             }
         }
+    }
+}
+
+// ctr: [3] tasks, [4] tasks taken
+__global__ void __launch_bounds__(256) giant_sort_kernel(const uint32_t* __restrict__ list,
+                                                         const uint64_t* __restrict__ start,
+                                                         uint32_t* __restrict__ spare, SplitRow* __restrict__ rows,
+                                                         const uint32_t* __restrict__ tasks, uint32_t* ctr) {
+    __shared__ BlockSortSmem<8> bs;
+    __shared__ uint32_t s_task;
+    for (;;) {
         __syncthreads();
-        // ---- each range sorted and de-duplicated in place
-        for (uint32_t g = 0; g < nr; ++g) {
-            const uint32_t c = sm.rcnt[g];
-            uint32_t k = 0;
-            if (c) k = block_sort_unique<8>(B + sm.rstart[g], c, B + sm.rstart[g], sm.bs);
-            if (tid == 0) sm.kept[g] = k;
-        }
+        if (threadIdx.x == 0) s_task = atomicAdd(&ctr[4], 1u);
         __syncthreads();
-        if (w == 0) {
-            const uint32_t c0 = lane < nr ? sm.kept[lane] : 0u, c1 = lane + 32 < nr ? sm.kept[lane + 32] : 0u;
-            const uint32_t i0 = warp_incl_scan(c0), i1 = warp_incl_scan(c1);
-            const uint32_t t0 = __shfl_sync(kFullMask, i0, 31);
-            const uint32_t tot = t0 + __shfl_sync(kFullMask, i1, 31);
-            __syncwarp();
-            sm.kept[lane] = i0 - c0;
-            sm.kept[lane + 32] = t0 + i1 - c1;
-            if (lane == 0) {
-                sm.kept[kSplitMaxRanges] = tot;
-                newlen[v] = tot;
-            }
-        }
-        __syncthreads();
-        // ---- the ranges' unique values back to the row, in order
-        for (uint32_t g = 0; g < nr; ++g) {
-            const uint32_t k = (g + 1 < nr ? sm.kept[g + 1] : sm.kept[kSplitMaxRanges]) - sm.kept[g];
-            const uint32_t* src = B + sm.rstart[g];
-            uint32_t* dst = A + sm.kept[g];
-            for (uint32_t j = tid; j < k; j += 256) dst[j] = src[j];
-        }
+        const uint32_t t = s_task;
+        if (t >= ctr[3]) break;
+        const uint32_t r = tasks[t] / kSplitMaxRanges, g = tasks[t] % kSplitMaxRanges;
+        uint32_t* row = spare + start[list[r]] + rows[r].start[g];
+        const uint32_t c = rows[r].start[g + 1] - rows[r].start[g];
+        uint32_t k = 0;
+        if (c) k = block_sort_unique<8>(row, c, row, bs);
+        if (threadIdx.x == 0) rows[r].kept[g] = k;
+    }
+}
+
+__global__ void __launch_bounds__(256) giant_copy_kernel(const uint32_t* __restrict__ list,
+                                                         const uint64_t* __restrict__ start,
+                                                         const uint32_t* __restrict__ spare, uint32_t* __restrict__ tmp,
+                                                         const SplitRow* __restrict__ rows,
+                                                         const uint32_t* __restrict__ tasks, const uint32_t* ctr,
+                                                         uint32_t* __restrict__ newlen) {
+    const uint32_t lane = threadIdx.x & 31u, total = ctr[3];
+    for (uint32_t t = blockIdx.x; t < total; t += gridDim.x) {
+        const uint32_t r = tasks[t] / kSplitMaxRanges, g = tasks[t] % kSplitMaxRanges;
+        const uint32_t v = list[r];
+        // unique values of the ranges before this one (each warp for itself)
+        const uint32_t at = __reduce_add_sync(kFullMask, (lane < g ? rows[r].kept[lane] : 0u) +
+                                                             (lane + 32 < g ? rows[r].kept[lane + 32] : 0u));
+        const uint32_t k = rows[r].kept[g];
+        const uint32_t* src = spare + start[v] + rows[r].start[g];
+        uint32_t* dst = tmp + start[v] + at;
+        for (uint32_t j = threadIdx.x; j < k; j += 256) dst[j] = src[j];
+        if (threadIdx.x == 0 && g + 1 == rows[r].nr) newlen[v] = at + k;
     }
 }
 
@@ -1583,14 +1605,30 @@ static dsg_status sort_giants(const uint32_t* glist, uint32_t ng, uint32_t n, co
     uint32_t nbits = 1;
     while (nbits < 32 && ((uint64_t)n - 1) >> nbits) ++nbits;
     const uint32_t passes = (nbits + 7) / 8;
-    uint32_t *gticket, *skewed;  // gticket[0]: split rows taken, [1]: skewed rows listed, [2]: radix rows taken
-    DSG_TRY_CUDA(sc.get(&gticket, 3));
+    // gticket: [0] split rows taken, [1] skewed rows listed, [2] radix rows taken, [3] ranges listed, [4] ranges taken
+    uint32_t *gticket, *skewed, *tasks;
+    SplitRow* rows;
+    DSG_TRY_CUDA(sc.get(&gticket, 5));
     DSG_TRY_CUDA(sc.get(&skewed, ng));
-    DSG_TRY_CUDA(cudaMemsetAsync(gticket, 0, 3 * sizeof(uint32_t), s));
+    DSG_TRY_CUDA(sc.get(&tasks, (uint64_t)ng * kSplitMaxRanges));
+    DSG_TRY_CUDA(sc.get(&rows, ng));
+    DSG_TRY_CUDA(cudaMemsetAsync(gticket, 0, 5 * sizeof(uint32_t), s));
     {
-        LaunchScope ls_("ingest_giant_rows", s);
-        giant_split_kernel<<<std::min<uint32_t>(ng, 2 * sms), 256, 0, s>>>(glist, ng, start, cnt, tmp, spare, newlen,
-                                                                         gticket, skewed, gticket + 1);
+        LaunchScope ls_("ingest_giant_split", s);
+        giant_split_kernel<<<std::min<uint32_t>(ng, 2 * sms), kSplitTB, 0, s>>>(glist, ng, start, cnt, tmp, spare, rows,
+                                                                             tasks, skewed, gticket);
+    }
+    DSG_TRY_CUDA(cudaGetLastError());
+    // (a row has at least two ranges)
+    const uint32_t grid = (uint32_t)std::min<uint64_t>((uint64_t)ng * kSplitMaxRanges, 4 * sms);
+    {
+        LaunchScope ls_("ingest_giant_sort", s);
+        giant_sort_kernel<<<grid, 256, 0, s>>>(glist, start, spare, rows, tasks, gticket);
+    }
+    DSG_TRY_CUDA(cudaGetLastError());
+    {
+        LaunchScope ls_("ingest_giant_copy", s);
+        giant_copy_kernel<<<grid, 256, 0, s>>>(glist, start, spare, tmp, rows, tasks, gticket, newlen);
     }
     DSG_TRY_CUDA(cudaGetLastError());
     {
