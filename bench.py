@@ -269,7 +269,7 @@ KERNEL_SOURCES = {
 }
 
 # Roofline units: the peel is one kernel launch; the core numbers are the
-# level kernel plus the tail (compaction and the cluster), whose launches
+# level kernel plus the tail (compaction and the bitwise search), whose launches
 # together compute what the byte model counts.
 ROOF_GROUPS = {
     "peel_rounds": lambda name: name == "peel_rounds",

@@ -166,8 +166,8 @@ uint64_t dsg_round_bound(uint32_t n, uint32_t eps_num, uint32_t eps_den);
  *                waits for this stream twice: it reads off[n] back before
  *                the launch and the results after it.
  * Limits: the scratch is nine arrays, each rounded up to a multiple of 256
- * bytes: four of 4n bytes (vertex state, two alive lists, failed list), the
- * chunk items 8(n + 2m/chunk_len + 1) bytes, the status map 4 ceil(n/16)
+ * bytes: four of 4n bytes (vertex state, two alive lists, one spare), the row
+ * pieces 8(n + 2m/chunk_len + 1) bytes, the status map 4 ceil(n/16)
  * bytes, two round histories of 8(dsg_round_bound(n, p, q) + 1) bytes, and a
  * control block of about 1 KB; chunk_len is the current tuning's
  * (dsg_set_tuning; 256 by default).  A graph whose scratch exceeds 64 MiB is
@@ -281,16 +281,20 @@ typedef struct {
 } dsg_batch_result;
 
 /*
- * Solve a batch in one persistent launch: blocks pull graphs largest first
- * and each block solves its graph alone (block barriers instead of grid
+ * Solve a batch in two persistent launches side by side: the graphs that
+ * would keep one block busy long after the others are done get a cluster of 8
+ * or 16 blocks each, the rest a block each; clusters and blocks pull their
+ * next graph largest first (cluster and block barriers instead of grid
  * barriers).  Results equal those of dsg_bahmani / dsg_kcore on each graph
  * alone.  DSG_EINVAL on malformed offsets or eps_den == 0.
  */
 dsg_status dsg_batch_solve(const dsg_batch* b, dsg_batch_result* r, void* stream);
-/* Which graphs of a batch the grid-wide kernels solve (before the
- * block-per-graph launch): those whose work 2m + n exceeds min_work; 0 (the
- * default) means those above twice one block's share of the batch's work and
- * above 2^20; 0xffffffff keeps every graph in the block-per-graph launch.
+/* Which graphs of a batch the grid-wide kernels solve (before the other
+ * launches): those whose work 2m + n exceeds min_work, the rest getting a
+ * block each; 0 (the default) means those above 2^20 that hold over a quarter
+ * of the batch's work or over 2^20 vertices, while of the rest those above
+ * 2^17 and twice one block's share get a cluster; 0xffffffff keeps every graph
+ * in the block-per-graph launch.
  * DSG_BATCH_SPLIT.  Results never depend on it. */
 dsg_status dsg_set_batch_split(uint32_t min_work);
 /* Autotune dsg_batch_solve for this batch's class (device, floor(log2 G),
@@ -307,7 +311,7 @@ dsg_status dsg_batch_autotune(const dsg_batch* b, uint32_t* trials);
  * A serving loop on one GPU: requests (raw pairs + eps) are admitted while
  * their device-memory charge fits a budget, ingested into resident graphs,
  * and solved by continuous batching -- whatever was ingested while the
- * previous batch ran forms the next block-per-graph launch (see
+ * previous batch ran forms the next launches of clusters and blocks (see
  * dsg_batch_solve), so arrivals overlap with work already on the device.  A
  * request's results do not depend on what it is batched with.  All calls
  * are thread-safe.
@@ -399,7 +403,8 @@ dsg_status dsg_get_tuning(uint32_t* block, uint32_t* blocks_per_sm, uint32_t* sh
 /* Bahmani peel: degree at or above which decrements of a vertex are first
  * combined in a per-block shared-memory table (one global atomic per block and
  * phase for a hub instead of one per edge).  0 (the default) means four times
- * the number of blocks of the launch; DSG_HOT_DEG.  Results never depend on
+ * the number of blocks of the launch and at least 1,024, or 4,096 where a graph
+ * has at most 16 blocks; DSG_HOT_DEG.  Results never depend on
  * it.  The core numbers decrement every neighbour at once and ignore it. */
 dsg_status dsg_set_hot_degree(uint32_t hot_deg);
 /* Core numbers: a vertex whose row has at most local_max entries and that

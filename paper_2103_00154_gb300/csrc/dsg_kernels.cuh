@@ -21,8 +21,7 @@ struct Tuning {
     uint32_t short_max = 32;    // kept for saved tables and callers; no kernel tells short rows apart any more
     uint32_t chunk_len = 256;   // rows are cut into pieces of at most this many entries
     uint32_t hot_deg = 0;       // decrements of vertices at or above this degree are combined in shared memory
-                                // (0: four times the number of blocks, i.e. hubs expected to be hit
-                                // several times by every block)
+                                // (0: by the number of blocks, hot_threshold)
     uint32_t local_max = 1024;  // k-core: rows up to this length reached while draining stay in the block
     uint32_t local_work = 16384; // k-core: ... while that block's local share of the sub-round stays within this
     uint32_t inline_max = 256;   // k-core: rows up to this length claimed by a block's level scan are drained by
@@ -30,7 +29,7 @@ struct Tuning {
     uint32_t tail_max = 65536;   // k-core: scale of the graphs and remaining graphs whose core numbers are searched
                                  // bit by bit instead of level by level (kTailHandOver, kTailWhole; 0: never)
     uint32_t batch_split = 0;    // batches: a graph whose work (2m + n) exceeds this is solved by the
-                                 // grid-wide kernels (0: above twice a block's share and 2^20)
+                                 // grid-wide kernels, the others by a block each (0: batch_classes)
     uint32_t batch_block = 512;  // batches: threads per block of the block-per-graph kernel
     uint32_t peel_lazy = 1;      // peel: thin-tail rounds test only the candidate list (0: every round
                                  // tests the whole alive list); read from the global tuning only

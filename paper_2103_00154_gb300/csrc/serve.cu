@@ -8,9 +8,10 @@
 //           ingest threads, and whenever one of its max_inflight solve
 //           streams is free launches everything ingested so far on that
 //           stream (a cluster of blocks each for the large graphs, a block
-//           each for the rest); while batches run, new arrivals keep being admitted and ingested, and form the next
-//           batch; a finished batch's results are copied out, its graphs
-//           freed and their charge returned to the budget;
+//           each for the rest); while batches run, new arrivals keep being
+//           admitted and ingested, and form the next batch; a finished batch's
+//           results are copied out, its graphs freed and their charge returned
+//           to the budget;
 //   ingest  (ingest_threads host threads, each with its own stream) turn
 //           admitted requests into resident graphs; a request above
 //           big_work goes to the big-request thread, the rest to the batches;
