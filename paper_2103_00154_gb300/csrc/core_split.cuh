@@ -50,7 +50,10 @@
 // kTailHandOver and kTailWhole.
 // Tried and dropped: a warp that goes on with the vertices it has removed
 // instead of queueing them (1, 2 or 4 rows deep: 0.82, 0.84, 0.88 ms against
-// 0.74 at 700,001 vertices -- the wave waits for the longest chain).
+// 0.74 at 700,001 vertices -- the wave waits for the longest chain); waves of
+// at most 32, 64 or 160 pieces by block 0 alone while the others wait at one
+// meeting (1.288, 1.295, 1.365 ms against 1.274 there, 5.43, 5.39, 5.51
+// against 5.07 on Chung-Lu 2^24).
 #pragma once
 
 #include "dsg_common.cuh"
