@@ -31,7 +31,11 @@
 // whichever reads fewer row pieces; the later waves push.  Rows are walked
 // as pieces of at most kPiece entries, as many pieces per warp as spread the
 // wave over all warps, the entries of a warp's pieces dealt out to its lanes
-// (a hub's row is many warps' work, 32 short rows one warp's).
+// (a hub's row is many warps' work, 32 short rows one warp's); the lanes find
+// an entry's piece by counting piece starts in a bit map and look it up in
+// shared memory (with a shuffle search and three shuffles per entry, a quarter
+// of the wide waves' load-store work, 0.85 ms on R-MAT scale 18 and 2.73 on
+// scale 20 beside its peels; 0.81 and 2.63 this way).
 // key is written to a buffer of its own for every bit, so its look-ups may be
 // cached in L1 although the kernel rewrites it while it runs.
 //
@@ -107,6 +111,7 @@ struct SplitSmem {
     MeetSmem meet;
     uint32_t above[32];
     uint32_t cnt[TB / 32][32];  // pull: a warp's counts, per piece
+    uint4 own[TB / 32][32];     // a warp's pieces that have entries: row position to add an entry to, key looked for
 };
 
 // Write the pieces of the rows u[j] (bit j of hit; np[j] pieces each, c[j] to
@@ -263,23 +268,30 @@ __device__ __forceinline__ void split_body(const SplitArgs& a, Team<CL> team, Sp
             const uint32_t total = __shfl_sync(kFullMask, inc, 31);
             const uint32_t st = inc - len;
             b0 -= st;  // entry e of the warp's pieces is adj[b0 + e] for its owner's b0
+            // the pieces that have entries, in order, for the entries to look up
+            const uint32_t nz = __ballot_sync(kFullMask, len != 0);
+            const uint32_t mypos = __popc(nz & lanemask_lt());
+            uint4* const own = sm.own[tid >> 5];
+            __syncwarp();
+            if (len) own[mypos] = make_uint4((uint32_t)b0, (uint32_t)(b0 >> 32), kc, 0u);
+            __syncwarp();
             for (uint32_t e0 = lane; e0 < ((total + 31u) & ~31u); e0 += 32 * kBatch) {
                 uint32_t u[kBatch], kk[kBatch], ow[kBatch], ku[kBatch], old[kBatch];
+                // an entry's piece: the one whose start is the last at or before it, by counting the
+                // starts in a map of the step's positions
+                const uint32_t E = e0 - lane;
+                uint32_t before = __popc(__ballot_sync(kFullMask, len != 0 && st < E));
+                const uint32_t rel = len != 0 && st >= E ? st - E : 0xffffffffu;
 #pragma unroll
                 for (uint32_t j = 0; j < kBatch; ++j) {
                     const uint32_t e = e0 + 32 * j;
-                    uint32_t o = 0;
-                    if (G > 1) {
-#pragma unroll
-                        for (uint32_t step = 16; step > 0; step >>= 1) {
-                            const uint32_t s = __shfl_sync(kFullMask, st, o + step);
-                            if (o + step < 32 && s <= e) o += step;
-                        }
-                    }
-                    const uint64_t ob = __shfl_sync(kFullMask, b0, o);
-                    kk[j] = __shfl_sync(kFullMask, kc, o);
+                    const uint32_t m = __reduce_or_sync(kFullMask, (rel >> 5) == j ? 1u << (rel & 31u) : 0u);
+                    const uint32_t o = before + __popc(m & (0xffffffffu >> (31u - lane))) - 1u;
+                    before += __popc(m);
+                    const uint4 p = own[o];
+                    kk[j] = p.z;
                     ow[j] = o;
-                    u[j] = e < total ? __ldg(a.adj + ob + e) : 0xffffffffu;
+                    u[j] = e < total ? __ldg(a.adj + ((uint64_t)p.y << 32 | p.x) + e) : 0xffffffffu;
                 }
 #pragma unroll
                 for (uint32_t j = 0; j < kBatch; ++j) ku[j] = u[j] < r ? __ldca(key + u[j]) : ~kk[j];
@@ -309,8 +321,8 @@ __device__ __forceinline__ void split_body(const SplitArgs& a, Team<CL> team, Sp
             }
             if (pull) {
                 __syncwarp();
-                const uint32_t take = cnt[lane];
-                cnt[lane] = 0;
+                const uint32_t take = len ? cnt[mypos] : 0u;
+                if (len) cnt[mypos] = 0;
                 const uint32_t v1[1] = {v}, c1[1] = {kc >> 1};
                 uint32_t np1[1] = {kv >> kKeyBits};
                 uint32_t hit = 0;
