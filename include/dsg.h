@@ -239,7 +239,8 @@ void dsg_peel_free(dsg_peel_state* st);
 dsg_status dsg_kcore(const dsg_graph* g, uint32_t* out_core);
 
 /* As dsg_kcore, also writing up to nstats counters of the run into stats:
- *   [0] levels (core numbers that occur)
+ *   [0] levels (those run, and of the vertices left to the search the core
+ *       numbers that occur)
  *   [1] row pieces queued to the level-wide work queue
  *   [2] remaining vertices scanned (sum over levels; for the vertices that
  *       dsg_set_kcore_tail leaves to the search, what its levels would scan)

@@ -126,6 +126,7 @@ struct PeelSmem {
     unsigned long long base[2];    // the tile's first piece and first survivor
     unsigned long long cursor[2];  // block 0 alone: the two lists' cursors
     unsigned long long add[4];     // this block's part of failed, xsum, rows, dec in the running phase
+    uint64_t own[TB / 32][32];     // phase 2, a warp's pieces: row position to add an entry to
     unsigned long long cum[5];     // failed, xsum, rows, dec and the candidate cursor after the round
     MeetSmem meet;
 };
@@ -445,20 +446,32 @@ __device__ __forceinline__ PeelOut peel_body(const PeelArgs& a, Team<CL> team, P
                 const uint32_t total = __shfl_sync(kFullMask, inc, 31);
                 const uint32_t begin = inc - len;
                 const uint64_t b0 = (it >> kLenBits) - begin;  // entry e of the group is adj[b0 + e] for its owner's b0
+                uint64_t* const own = sm.own[warp];
+                if (G > 1) {
+                    __syncwarp();
+                    const uint32_t nz = __ballot_sync(kFullMask, len != 0);
+                    if (len) own[__popc(nz & lanemask_lt())] = b0;
+                    __syncwarp();
+                }
                 for (uint32_t e0 = lane; e0 < ((total + 31u) & ~31u); e0 += 32 * kBatch) {
                     uint32_t u[kBatch], w[kBatch];
+                    // owner: the last piece that starts at or before e, by counting the pieces' starts in a
+                    // map of the step's positions (a five-step shuffle search per entry before: 1,500
+                    // graphs in one batch 2.52 -> 2.37 ms, 3 10^6 vertices 689 -> 681 us)
+                    const uint32_t e_lo = e0 - lane;
+                    uint32_t before = G > 1 ? __popc(__ballot_sync(kFullMask, len != 0 && begin < e_lo)) : 0u;
+                    const uint32_t rel = len != 0 && begin >= e_lo ? begin - e_lo : 0xffffffffu;
 #pragma unroll
                     for (uint32_t j = 0; j < kBatch; ++j) {
                         const uint32_t e = e0 + 32 * j;
-                        uint32_t o = 0;
-                        if (G > 1) {  // owner: last piece that starts at or before e
-#pragma unroll
-                            for (uint32_t step = 16; step > 0; step >>= 1) {
-                                const uint32_t s = __shfl_sync(kFullMask, begin, o + step);
-                                if (o + step < 32 && s <= e) o += step;
-                            }
+                        uint64_t ob;
+                        if (G > 1) {
+                            const uint32_t m = __reduce_or_sync(kFullMask, (rel >> 5) == j ? 1u << (rel & 31u) : 0u);
+                            ob = own[before + __popc(m & (0xffffffffu >> (31u - lane))) - 1u];
+                            before += __popc(m);
+                        } else {
+                            ob = __shfl_sync(kFullMask, b0, 0);
                         }
-                        const uint64_t ob = __shfl_sync(kFullMask, b0, o);
                         u[j] = e < total ? ld_stream(a.adj + ob + e) : 0xffffffffu;
                     }
 #pragma unroll
