@@ -151,11 +151,11 @@ struct BatchSmem {
 // each other's registers.
 template <int TB, uint32_t size>
 __device__ __noinline__ PeelOut team_peel(const PeelArgs& a, PeelSmem<TB>& sm, uint32_t rank) {
-    return peel_body<TB, (size > 1)>(a, Team<(size > 1)>{rank, size, a.ctl->bar, &a.ctl->err, 0, {}}, sm);
+    return peel_body<TB, (size > 1)>(a, Team<(size > 1)>{rank, size, a.ctl->bar, &a.ctl->err, 0}, sm);
 }
 template <int TB, uint32_t size>
 __device__ __noinline__ void team_split(const SplitArgs& a, SplitSmem<TB>& sm, uint32_t rank) {
-    split_body<TB, (size > 1)>(a, Team<(size > 1)>{rank, size, a.ctl->bar, &a.ctl->err, 0, {}}, sm);
+    split_body<TB, (size > 1)>(a, Team<(size > 1)>{rank, size, a.ctl->bar, &a.ctl->err, 0}, sm);
 }
 
 // A team -- one block, or (CL) a cluster -- takes graphs from
@@ -214,7 +214,7 @@ __global__ void __launch_bounds__(TB, 1024 / TB) batch_kernel(BatchKernelArgs c)
             a.hot_deg = b.hot_deg;
             a.trace = nullptr;
             a.trace_cap = 0;
-            a.r0 = a.S0 = a.E0 = a.best_round0 = a.best_E0 = a.best_V0 = a.max_rounds = 0;
+            a.r0 = a.S0 = a.E0 = a.best_round0 = a.best_E0 = a.best_V0 = a.max_rounds = a.arrivals0 = 0;
         }
         __syncthreads();
         {

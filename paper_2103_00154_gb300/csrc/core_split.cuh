@@ -201,7 +201,7 @@ __device__ __forceinline__ void split_body(const SplitArgs& a, Team<CL> team, Sp
     if (tid < 32) sm.above[tid] = 0;
     if (tid == 0) {
         sm.pushed = 0;
-        sm.meet.ok = 1;
+        meet_init(sm.meet);
     }
     sm.cnt[tid >> 5][lane] = 0;
     __syncthreads();

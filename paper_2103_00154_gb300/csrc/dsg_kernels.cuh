@@ -207,12 +207,27 @@ __device__ __forceinline__ T* at_block0(T* p) {
 // zero.  Every thread of the block calls it; thread 0's `mine` counts.  A wait
 // above limit_ns records ERR_TIMEOUT and clears sm.ok, as does seeing the
 // error of another block.  With one block (size == 1) it is a block barrier.
-struct MeetState {
-    uint32_t epoch = 0, seen0 = 0, seen1 = 0;
-};
+// The low half is never reset and carries into the high one after 2^32
+// arrivals (a path of 2^24 vertices at eps = 0 has 2^23 rounds, each an
+// arrival of every block on each word): meet_sum takes the arrivals, counted
+// in 64 bits, off the whole word.
+
+// The sum, modulo 2^32, of the counts on a word that `arrivals` blocks have arrived on.
+__host__ __device__ __forceinline__ uint32_t meet_sum(uint64_t word, uint64_t arrivals) {
+    return (uint32_t)((word - arrivals) >> 32);
+}
+// A block's view of the meetings, kept by its thread 0 (the others read got and ok).
 struct MeetSmem {
+    uint64_t arrivals[2];  // by word: arrivals when its last meeting was over ...
+    uint32_t seen[2];      // ... and the sums handed out so far
+    uint32_t par;          // the next meeting's word
     uint32_t got, ok;
 };
+__device__ __forceinline__ void meet_init(MeetSmem& sm, uint64_t arrivals = 0) {
+    sm.arrivals[0] = sm.arrivals[1] = arrivals;
+    sm.seen[0] = sm.seen[1] = sm.par = 0;
+    sm.ok = 1;
+}
 
 // The blocks that work on one graph: a co-resident grid (CL = false), or one
 // thread-block cluster (CL = true: the words are in a block's shared memory,
@@ -223,16 +238,26 @@ struct Team {
     unsigned long long (*bar)[16];
     uint32_t* err;
     uint64_t limit_ns;
-    MeetState st;
 
     __device__ __forceinline__ uint32_t meet(uint32_t mine, MeetSmem& sm) {
-        const uint32_t par = st.epoch & 1u;
-        ++st.epoch;
+        // what the wait is over with is read before it: nothing depends on shared memory after it
+        uint32_t par = 0, seen = 0;
+        uint64_t arrivals = 0;
+        if (threadIdx.x == 0) {
+            par = sm.par;
+            seen = sm.seen[par];
+            arrivals = sm.arrivals[par] + size;
+        }
         if constexpr (CL) {
             unsigned long long* word = &bar[par][0];
             if (threadIdx.x == 0 && mine) atomicAdd(word, (unsigned long long)mine);
             cluster_sync();
-            if (threadIdx.x == 0) sm.got = (uint32_t)ld_volatile_u64((const uint64_t*)word) - (par ? st.seen1 : st.seen0);
+            if (threadIdx.x == 0) {
+                const uint32_t sum = (uint32_t)ld_volatile_u64((const uint64_t*)word);
+                sm.got = sum - seen;
+                sm.seen[par] = sum;
+                sm.par = par ^ 1u;
+            }
         } else {
             __syncthreads();
             if (threadIdx.x == 0) {
@@ -240,12 +265,11 @@ struct Team {
                     sm.got = mine;
                 } else {
                     unsigned long long* word = &bar[par][0];
-                    const uint32_t target = ((st.epoch + 1) >> 1) * size;  // odd and even meetings have a word each
                     red_add_release_u64(word, (uint64_t)mine << 32 | 1ull);
                     uint64_t w;
                     uint32_t polls = 0;
                     const uint64_t t0 = global_ns();
-                    while ((int32_t)((uint32_t)(w = ld_acquire_u64(word)) - target) < 0) {
+                    while ((int32_t)((uint32_t)(w = ld_acquire_u64(word)) - (uint32_t)arrivals) < 0) {
                         if ((++polls & 63u) == 0) {
                             if (global_ns() - t0 > limit_ns) atomicOr(err, ERR_TIMEOUT);
                             if (ld_volatile_u32(err) & ERR_TIMEOUT) {
@@ -254,14 +278,16 @@ struct Team {
                             }
                         }
                     }
-                    sm.got = (uint32_t)(w >> 32) - (par ? st.seen1 : st.seen0);
+                    const uint32_t sum = meet_sum(w, arrivals);
+                    sm.got = sum - seen;
+                    sm.seen[par] = sum;
+                    sm.arrivals[par] = arrivals;
+                    sm.par = par ^ 1u;
                 }
             }
         }
         __syncthreads();
-        const uint32_t got = sm.got;
-        if (par) st.seen1 += got; else st.seen0 += got;
-        return got;
+        return sm.got;
     }
 };
 

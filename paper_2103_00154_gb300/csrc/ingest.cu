@@ -1458,14 +1458,14 @@ __global__ void __launch_bounds__(kDirectTB, 1) direct_kernel(DirectArgs a) {
     DirectSmem& sm = *reinterpret_cast<DirectSmem*>(direct_smem_raw);
     const uint32_t tid = threadIdx.x, lane = tid & 31u, n = a.n;
     DirectCtl* const ctl = CL ? at_block0(&sm.ctl) : a.ctl;
-    Team<CL> team{CL ? cluster_rank() : blockIdx.x, gridDim.x, ctl->bar, &ctl->err, a.limit_ns, {}};
+    Team<CL> team{CL ? cluster_rank() : blockIdx.x, gridDim.x, ctl->bar, &ctl->err, a.limit_ns};
     const uint32_t gt = team.rank * kDirectTB + tid, nt = team.size * kDirectTB;
     const uint32_t gw = gt >> 5, nw = nt >> 5;
     // no block of a cluster leaves while another reads block 0's shared memory
     auto leave = [&]() {
         if constexpr (CL) cluster_sync();
     };
-    if (tid == 0) sm.meet.ok = 1;
+    if (tid == 0) meet_init(sm.meet);
     if (CL && team.rank == 0)
         for (uint32_t i = tid; i < sizeof(DirectCtl) / 4; i += kDirectTB) reinterpret_cast<uint32_t*>(&sm.ctl)[i] = 0;
     for (uint32_t i = gt; i < n; i += nt) a.cnt[i] = 0;

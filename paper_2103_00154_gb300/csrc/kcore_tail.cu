@@ -10,7 +10,7 @@ namespace dsg {
 
 __global__ void __launch_bounds__(kSplitTB, 1) core_split_kernel(SplitArgs a) {
     __shared__ SplitSmem<kSplitTB> sm;
-    Team<false> team{blockIdx.x, gridDim.x, a.ctl->bar, &a.ctl->err, a.limit_ns, {}};
+    Team<false> team{blockIdx.x, gridDim.x, a.ctl->bar, &a.ctl->err, a.limit_ns};
     split_body<kSplitTB, false>(a, team, sm);
 }
 
@@ -26,7 +26,7 @@ __global__ void __launch_bounds__(kSplitTB, 1) core_split_cluster_kernel(SplitAr
     if (rank == 0)
         for (uint32_t i = threadIdx.x; i < sizeof(SplitCtl) / 4; i += kSplitTB) words[i] = 0;
     cluster_sync();
-    split_body<kSplitTB, true>(a, Team<true>{rank, kSmallBlocks, a.ctl->bar, &a.ctl->err, 0, {}}, sm);
+    split_body<kSplitTB, true>(a, Team<true>{rank, kSmallBlocks, a.ctl->bar, &a.ctl->err, 0}, sm);
     cluster_sync();  // every block's counts are in; no block leaves while another reads block 0's shared memory
     if (rank == 0)
         for (uint32_t i = threadIdx.x; i < sizeof(SplitCtl) / 4; i += kSplitTB)

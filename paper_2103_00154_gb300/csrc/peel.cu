@@ -16,7 +16,7 @@ namespace dsg {
 template <int TB>
 __global__ void __launch_bounds__(TB, 1024 / TB) peel_kernel(PeelArgs a) {
     __shared__ PeelSmem<TB> sm;
-    Team<false> team{blockIdx.x, gridDim.x, a.ctl->bar, &a.ctl->err, a.limit_ns, {}};
+    Team<false> team{blockIdx.x, gridDim.x, a.ctl->bar, &a.ctl->err, a.limit_ns};
     peel_body<TB, false>(a, team, sm);
 }
 
@@ -37,7 +37,7 @@ __global__ void __launch_bounds__(kSmallTB, 1) peel_cluster_kernel(PeelArgs a, u
         for (uint32_t i = tid; i < sizeof(PeelCtl) / 4; i += kSmallTB) words[i] = 0;
     cluster_sync();
     const PeelOut o =
-        peel_body<kSmallTB, true>(a, Team<true>{rank, kSmallBlocks, a.ctl->bar, &a.ctl->err, 0, {}}, sm);
+        peel_body<kSmallTB, true>(a, Team<true>{rank, kSmallBlocks, a.ctl->bar, &a.ctl->err, 0}, sm);
     for (uint32_t v = rank * kSmallTB + tid; v < a.n; v += kSmallBlocks * kSmallTB) {
         const uint32_t pr = __ldcg(a.st + v) & ~kDead;
         if (peel_round) peel_round[v] = pr;
@@ -65,11 +65,21 @@ __global__ void peel_finish_kernel(uint32_t n, const uint32_t* __restrict__ st, 
     }
 }
 
+// wrap_in (0: off): the meeting words start as if so many blocks had arrived
+// that they pass 2^32 arrivals after that many rounds.
 template <int TB>
-static cudaError_t launch_peel(PeelArgs& a, uint32_t blocks_per_sm, cudaStream_t s, uint32_t max_grid) {
+static cudaError_t launch_peel(PeelArgs& a, uint32_t blocks_per_sm, cudaStream_t s, uint32_t max_grid,
+                               uint32_t wrap_in = 0) {
     uint32_t grid = 1;
     cudaError_t e = coop_grid(peel_kernel<TB>, TB, 0, a.n, blocks_per_sm, &grid, max_grid);
     if (e != cudaSuccess) return e;
+    if (wrap_in) {
+        a.arrivals0 = ((1ull << 32) / grid - wrap_in) * grid;
+        const unsigned long long before = a.arrivals0;
+        for (int w = 0; w < 2 && e == cudaSuccess; ++w)
+            e = cudaMemcpyAsync(&a.ctl->bar[w][0], &before, sizeof(before), cudaMemcpyHostToDevice, s);
+        if (e != cudaSuccess) return e;
+    }
     void* params[] = {&a};
     LaunchScope ls("peel_rounds", s);
     return cudaLaunchCooperativeKernel((const void*)peel_kernel<TB>, dim3(grid), dim3(TB), params, 0, s);
@@ -82,7 +92,7 @@ static uint32_t piece_len(const Tuning& tu) { return std::min<uint32_t>(tu.chunk
 // in hist / peel_round / set (device pointers).
 static dsg_status run_peel(const dsg_graph* g, uint32_t p, uint32_t q, uint64_t* hist_S_out, uint64_t* hist_E_out,
                            uint64_t hist_cap_out, uint32_t* peel_round_out, uint8_t* set_out, PeelCtl* ctl_host,
-                           uint64_t* trace_dev = nullptr, uint64_t trace_cap = 0);
+                           uint64_t* trace_dev = nullptr, uint64_t trace_cap = 0, uint32_t wrap_in = 0);
 
 dsg_status peel_into(const dsg_graph* g, uint32_t p, uint32_t q, uint8_t* set_dev, uint64_t out4[4],
                      uint64_t* extra2) {
@@ -111,7 +121,7 @@ dsg_status peel_into(const dsg_graph* g, uint32_t p, uint32_t q, uint8_t* set_de
 
 static dsg_status run_peel(const dsg_graph* g, uint32_t p, uint32_t q, uint64_t* hist_S_out, uint64_t* hist_E_out,
                            uint64_t hist_cap_out, uint32_t* peel_round_out, uint8_t* set_out, PeelCtl* ctl_host,
-                           uint64_t* trace_dev, uint64_t trace_cap) {
+                           uint64_t* trace_dev, uint64_t trace_cap, uint32_t wrap_in) {
     cudaStream_t s = g->stream;
     const uint32_t n = g->n;
     Tuning tu = tuning_for(g, 0);
@@ -140,7 +150,7 @@ static dsg_status run_peel(const dsg_graph* g, uint32_t p, uint32_t q, uint64_t*
     a.hot_deg = tu.hot_deg;
     a.trace = trace_dev;
     a.trace_cap = trace_cap;
-    a.r0 = a.S0 = a.E0 = a.best_round0 = a.best_E0 = a.best_V0 = a.max_rounds = 0;
+    a.r0 = a.S0 = a.E0 = a.best_round0 = a.best_E0 = a.best_V0 = a.max_rounds = a.arrivals0 = 0;
     const bool lazy = current_tuning().peel_lazy != 0;
     const bool pr_direct = peel_round_out && is_device_ptr(peel_round_out);
     const bool set_direct = set_out && is_device_ptr(set_out);
@@ -171,7 +181,7 @@ static dsg_status run_peel(const dsg_graph* g, uint32_t p, uint32_t q, uint64_t*
         if (peel_round_out && !pr_direct) pr_dev = reinterpret_cast<uint32_t*>(w + o_pr);
         if (set_out && !set_direct) set_dev = w + o_set;
     }
-    const bool small = n + 2 * g->m <= kSmallPeel && (g->max_blocks == 0 || g->max_blocks >= kSmallBlocks) &&
+    const bool small = !wrap_in && n + 2 * g->m <= kSmallPeel && (g->max_blocks == 0 || g->max_blocks >= kSmallBlocks) &&
                        cudaFuncSetAttribute(peel_cluster_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) ==
                            cudaSuccess;
     if (small) {
@@ -181,9 +191,9 @@ static dsg_status run_peel(const dsg_graph* g, uint32_t p, uint32_t q, uint64_t*
         DSG_TRY_CUDA(cudaMemsetAsync(a.ctl, 0, sizeof(PeelCtl), s));
         cudaError_t e;
         switch (tu.block) {
-            case 256: e = launch_peel<256>(a, tu.blocks_per_sm, s, g->max_blocks); break;
-            case 1024: e = launch_peel<1024>(a, tu.blocks_per_sm, s, g->max_blocks); break;
-            default: e = launch_peel<512>(a, tu.blocks_per_sm, s, g->max_blocks); break;
+            case 256: e = launch_peel<256>(a, tu.blocks_per_sm, s, g->max_blocks, wrap_in); break;
+            case 1024: e = launch_peel<1024>(a, tu.blocks_per_sm, s, g->max_blocks, wrap_in); break;
+            default: e = launch_peel<512>(a, tu.blocks_per_sm, s, g->max_blocks, wrap_in); break;
         }
         DSG_TRY_CUDA(e);
         if (pr_dev || set_dev) {
@@ -377,6 +387,25 @@ dsg_status dsg_debug_peel_trace(const dsg_graph* g, uint32_t eps_num, uint32_t e
     return DSG_OK;
 }
 
+uint32_t dsg_debug_meet_sum(uint64_t word, uint64_t arrivals) { return meet_sum(word, arrivals); }
+
+dsg_status dsg_debug_peel_wrap(const dsg_graph* g, uint32_t eps_num, uint32_t eps_den, uint32_t wrap_in,
+                               uint32_t* peel_round, uint8_t* out_set, uint64_t out4[4]) {
+    clear_error();
+    DSG_CHECK_ARG(g && out4, "graph / out4 is NULL");
+    DSG_CHECK_ARG(eps_den != 0, "eps_den must be positive");
+    DSG_CHECK_ARG(wrap_in >= 1 && wrap_in <= 1u << 20, "wrap_in must be in [1, 2^20]");
+    DSG_TRY_CUDA(cudaSetDevice(g->device));
+    PeelCtl c;
+    dsg_status st = run_peel(g, eps_num, eps_den, nullptr, nullptr, 0, peel_round, out_set, &c, nullptr, 0, wrap_in);
+    if (st != DSG_OK) return st;
+    out4[0] = g->n ? c.best_E : 0;
+    out4[1] = g->n ? c.best_V : 0;
+    out4[2] = c.rounds;
+    out4[3] = c.best_round;
+    return DSG_OK;
+}
+
 }  // extern "C"
 
 // ===================================================== no-allocation variant
@@ -536,7 +565,7 @@ extern "C" dsg_status dsg_bahmani_noalloc(uint32_t n, const uint64_t* off, const
     a.hot_deg = tu.hot_deg;
     a.trace = nullptr;
     a.trace_cap = 0;
-    a.r0 = a.S0 = a.E0 = a.best_round0 = a.best_E0 = a.best_V0 = a.max_rounds = 0;
+    a.r0 = a.S0 = a.E0 = a.best_round0 = a.best_E0 = a.best_V0 = a.max_rounds = a.arrivals0 = 0;
     // The buffer keeps whatever the previous call left; only the control
     // block must start at zero (every other array is written before it is read).
     DSG_TRY_CUDA(cudaMemsetAsync(a.ctl, 0, sizeof(PeelCtl), s));
@@ -675,6 +704,7 @@ static dsg_status peel_state_run(dsg_peel_state* ps, uint64_t max_rounds) {
     a.best_E0 = ps->best_E;
     a.best_V0 = ps->best_V;
     a.max_rounds = max_rounds;
+    a.arrivals0 = 0;
     PeelCtl init;
     memset(&init, 0, sizeof(init));
     init.failed = (uint64_t)g->n - ps->S;  // the counters the kernel derives S and E from

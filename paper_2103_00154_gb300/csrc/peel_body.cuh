@@ -94,6 +94,7 @@ struct PeelArgs {
     // skipping those already failed; max_rounds > 0 pauses after that many rounds
     uint64_t r0, S0, E0, best_round0, best_E0, best_V0;
     uint64_t max_rounds;
+    uint64_t arrivals0;   // that each word of ctl->bar already counts (0 but for the test of their wrap)
 };
 
 constexpr uint32_t kLenBits = 24;         // of a piece: entries (chunk_len is kept below 2^24)
@@ -188,7 +189,7 @@ __device__ __forceinline__ PeelOut peel_body(const PeelArgs& a, Team<CL> team, P
         sm.cum[tid] = 0;
     }
     if (tid == 0) {
-        sm.meet.ok = 1;
+        meet_init(sm.meet, a.arrivals0);
         sm.cum[0] = resume ? (uint64_t)a.n - a.S0 : 0;
         sm.cum[1] = resume ? 2 * (a.m - a.E0) : 0;
         sm.cum[4] = 0;
