@@ -288,6 +288,11 @@ typedef struct {
  * next graph largest first (cluster and block barriers instead of grid
  * barriers).  Results equal those of dsg_bahmani / dsg_kcore on each graph
  * alone.  DSG_EINVAL on malformed offsets or eps_den == 0.
+ * Device scratch: a slab per block (about 20 bytes a vertex and 1/32 byte an
+ * entry) and per cluster (at most 112 bytes a vertex and 1/4 byte an entry
+ * with core numbers), each for the largest graph it can still meet; in all at
+ * most 80 bytes a vertex and 8 an entry of the batch, and fewer blocks or
+ * clusters where even that cannot be had.
  */
 dsg_status dsg_batch_solve(const dsg_batch* b, dsg_batch_result* r, void* stream);
 /* Which graphs of a batch the grid-wide kernels solve (before the other

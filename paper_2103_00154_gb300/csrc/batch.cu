@@ -13,6 +13,8 @@
 // body of the grid-wide peel, the clusters that of the bitwise core-number
 // search too, with the block's or the cluster's barrier between rounds and
 // waves, on a slab of scratch per team.
+#include <string.h>
+
 #include <algorithm>
 #include <vector>
 
@@ -120,15 +122,37 @@ __device__ void kcore_block(uint32_t n, const uint64_t* off, const uint32_t* adj
 constexpr uint32_t kClusterBlocks = 8, kClusterBlocksFew = 16, kFewGraphs = 14;
 constexpr uint32_t kClusterTB = 1024;
 
+// A team's scratch for a graph of n vertices and e row entries: offsets and
+// size.  The peel's arrays, a block's level lists (the peel's first three) and
+// the search's share the space.  Larger graphs need no less of anything.
+constexpr uint32_t kBatchChunk = 256;  // entries of a row piece of the peel
+struct SlabLayout {
+    uint64_t at;  // the slab's own place
+    uint64_t listA, listB, items, map, peel_end;
+    uint64_t ds, key, pieces, queue, search_end;
+    uint64_t cap;  // row pieces of the search
+};
+static SlabLayout slab_layout(uint64_t n, uint64_t e) {
+    auto up = [](uint64_t bytes) { return (bytes + 255) & ~uint64_t(255); };
+    SlabLayout l = {};
+    l.listA = up(4 * n);  // after the states
+    l.listB = 2 * l.listA;
+    l.items = 3 * l.listA;
+    l.map = l.items + up(8 * (n + e / kBatchChunk + 1));
+    l.peel_end = l.map + up((n + 15) / 16 * 4);
+    l.cap = n + e / kPiece + 1;
+    l.ds = l.listA;  // after the degrees
+    l.key = l.listB;
+    l.pieces = l.key + up(4 * ((n + 63) & ~uint64_t(63)) * split_key_buffers(e));
+    l.queue = l.pieces + up(16 * l.cap);
+    l.search_end = l.queue + up(16 * l.cap);
+    return l;
+}
+
 struct BatchKernelArgs {
     BatchArgs b;
-    unsigned char* slabs;  // after the error word, one slab per team
-    uint64_t slab;         // bytes of one
-    // offsets inside a slab (the peel's arrays and the search's share the space)
-    uint64_t o_listA, o_listB, o_items, o_map;
-    uint64_t o_ds, o_key, o_pieces, o_queue;
-    uint64_t cap;          // row pieces of the largest graph
-    uint32_t chunk_len;
+    unsigned char* scratch;  // the error word, the slabs' layouts, the slabs
+    const SlabLayout* slabs;  // by the order in which the teams start
 };
 
 template <int TB>
@@ -144,7 +168,8 @@ struct BatchSmem {
     };
     PeelCtl pctl;
     SplitCtl sctl;
-    uint32_t item;
+    uint32_t item, slot;
+    const SlabLayout* slab;  // the team's, once it has taken a graph
 };
 
 // The two bodies as functions of their own: inlined into one kernel they spill
@@ -172,8 +197,9 @@ __global__ void __launch_bounds__(TB, 1024 / TB) batch_kernel(BatchKernelArgs c)
     PeelCtl* const pctl = CL ? at_block0(&sm.pctl) : &sm.pctl;
     SplitCtl* const sctl = CL ? at_block0(&sm.sctl) : &sm.sctl;
     uint32_t* const item0 = CL ? at_block0(&sm.item) : &sm.item;
-    unsigned char* const slab = c.slabs + 256 + (uint64_t)(blockIdx.x / size) * c.slab;
-    uint32_t* const err = reinterpret_cast<uint32_t*>(c.slabs);
+    uint32_t* const slot0 = CL ? at_block0(&sm.slot) : &sm.slot;
+    if (tid == 0) sm.slab = nullptr;
+    uint32_t* const err = reinterpret_cast<uint32_t*>(c.scratch);
     auto sync = [] {
         if constexpr (CL) cluster_sync();
         else __syncthreads();
@@ -183,7 +209,14 @@ __global__ void __launch_bounds__(TB, 1024 / TB) batch_kernel(BatchKernelArgs c)
             static_assert(sizeof(PeelCtl) % 4 == 0 && sizeof(SplitCtl) % 4 == 0, "cleared word by word");
             for (uint32_t i = tid; i < sizeof(PeelCtl) / 4; i += TB) reinterpret_cast<uint32_t*>(&sm.pctl)[i] = 0;
             for (uint32_t i = tid; i < sizeof(SplitCtl) / 4; i += TB) reinterpret_cast<uint32_t*>(&sm.sctl)[i] = 0;
-            if (tid == 0) sm.item = (uint32_t)min(atomicAdd(b.next, 1ull), (unsigned long long)b.G);
+            if (tid == 0) {
+                // a team's first graph comes with its place among the teams that have started: no more
+                // have than graphs are taken, so this graph and all it takes later are no earlier in the
+                // order than that place, which the slab is sized for
+                const unsigned long long t = atomicAdd(b.next, sm.slab ? 1ull : 1ull << 32 | 1ull);
+                sm.item = min((uint32_t)t, b.G);
+                sm.slot = (uint32_t)(t >> 32);
+            }
         }
         sync();
         const uint32_t item = ld_volatile_u32(item0);
@@ -194,6 +227,9 @@ __global__ void __launch_bounds__(TB, 1024 / TB) batch_kernel(BatchKernelArgs c)
         const uint64_t* off = b.goff[g];
         if (tid == 0) {
             PeelArgs& a = sm.pargs;
+            if (!sm.slab) sm.slab = c.slabs + ld_volatile_u32(slot0);
+            const SlabLayout& l = *sm.slab;
+            unsigned char* const slab = c.scratch + l.at;
             a.n = n;
             a.m = n ? (off[n] - off[0]) / 2 : 0;
             a.p = b.p[g];
@@ -201,16 +237,16 @@ __global__ void __launch_bounds__(TB, 1024 / TB) batch_kernel(BatchKernelArgs c)
             a.off = off;
             a.adj = b.gadj[g];
             a.st = reinterpret_cast<uint32_t*>(slab);
-            a.listA = reinterpret_cast<uint32_t*>(slab + c.o_listA);
-            a.listB = reinterpret_cast<uint32_t*>(slab + c.o_listB);
-            a.items = reinterpret_cast<uint64_t*>(slab + c.o_items);
-            a.map = reinterpret_cast<uint32_t*>(slab + c.o_map);
+            a.listA = reinterpret_cast<uint32_t*>(slab + l.listA);
+            a.listB = reinterpret_cast<uint32_t*>(slab + l.listB);
+            a.items = reinterpret_cast<uint64_t*>(slab + l.items);
+            a.map = reinterpret_cast<uint32_t*>(slab + l.map);
             a.candA = a.candB = nullptr;
             a.hist_S = a.hist_E = nullptr;
             a.hist_cap = ~0ull;
             a.ctl = pctl;
             a.limit_ns = 0;
-            a.chunk_len = c.chunk_len;
+            a.chunk_len = kBatchChunk;
             a.hot_deg = b.hot_deg;
             a.trace = nullptr;
             a.trace_cap = 0;
@@ -232,7 +268,7 @@ __global__ void __launch_bounds__(TB, 1024 / TB) batch_kernel(BatchKernelArgs c)
                 if (pctl->err) atomicOr(err, pctl->err);
             }
             if (b.out_set) {
-                const uint32_t* st = reinterpret_cast<const uint32_t*>(slab);
+                const uint32_t* st = reinterpret_cast<const uint32_t*>(c.scratch + sm.slab->at);
                 for (uint32_t v = rank * TB + tid; v < n; v += size * TB)
                     b.out_set[vb + v] = (__ldcg(st + v) & ~kDead) > o.best_round ? 1 : 0;
             }
@@ -242,18 +278,20 @@ __global__ void __launch_bounds__(TB, 1024 / TB) batch_kernel(BatchKernelArgs c)
             if constexpr (CL) {
                 if (tid == 0) {
                     SplitArgs& a = sm.sargs;
+                    const SlabLayout& l = *sm.slab;
+                    unsigned char* const slab = c.scratch + l.at;
                     a.r = n;
                     a.lo = 0;
                     a.off = off;
                     a.adj = b.gadj[g];
                     a.rid = nullptr;
                     a.d = reinterpret_cast<uint32_t*>(slab);
-                    a.ds = reinterpret_cast<uint32_t*>(slab + c.o_ds);
-                    a.key = reinterpret_cast<uint32_t*>(slab + c.o_key);
+                    a.ds = reinterpret_cast<uint32_t*>(slab + l.ds);
+                    a.key = reinterpret_cast<uint32_t*>(slab + l.key);
                     a.kstride = ((uint64_t)n + 63) & ~uint64_t(63);
-                    a.pieces = reinterpret_cast<uint4*>(slab + c.o_pieces);
-                    a.queue = reinterpret_cast<uint4*>(slab + c.o_queue);
-                    a.cap = c.cap;
+                    a.pieces = reinterpret_cast<uint4*>(slab + l.pieces);
+                    a.queue = reinterpret_cast<uint4*>(slab + l.queue);
+                    a.cap = l.cap;
                     a.core = b.core + vb;
                     a.ctl = sctl;
                     a.limit_ns = 0;
@@ -266,52 +304,58 @@ __global__ void __launch_bounds__(TB, 1024 / TB) batch_kernel(BatchKernelArgs c)
                 if (rank == 0 && tid == 0 && sctl->err) atomicOr(err, sctl->err);
                 __syncthreads();
             } else {
+                const SlabLayout& l = *sm.slab;
+                unsigned char* const slab = c.scratch + l.at;
                 kcore_block<TB>(n, off, b.gadj[g], b.core + vb, reinterpret_cast<uint32_t*>(slab),
-                                reinterpret_cast<uint32_t*>(slab + c.o_listA),
-                                reinterpret_cast<uint32_t*>(slab + c.o_listB), sm.level);
+                                reinterpret_cast<uint32_t*>(slab + l.listA),
+                                reinterpret_cast<uint32_t*>(slab + l.listB), sm.level);
             }
         }
     }
     sync();  // no block leaves while another reads block 0's shared memory
 }
 
-// The slab layout for graphs of at most n_max vertices and e_max row entries.
-static BatchKernelArgs batch_layout(const BatchArgs& b, uint32_t n_max, uint64_t e_max, bool search) {
-    BatchKernelArgs c = {};
-    c.b = b;
-    c.chunk_len = 256;
-    uint64_t o = 0;
-    auto carve = [&](uint64_t bytes) { const uint64_t at = o; o += (bytes + 255) & ~uint64_t(255); return at; };
-    const uint64_t n = n_max;
-    carve(4 * n);  // the peel's states (a block's level lists: this and the two after it)
-    c.o_listA = carve(4 * n);
-    c.o_listB = carve(4 * n);
-    c.o_items = carve(8 * (n + e_max / c.chunk_len + 1));
-    c.o_map = carve((n + 15) / 16 * 4);
-    c.slab = o;
-    if (b.core && search) {
-        o = 0;
-        c.cap = n + e_max / kPiece + 1;
-        carve(4 * n);  // the search's degrees
-        c.o_ds = carve(4 * n);
-        c.o_key = carve(4 * ((n + 63) & ~uint64_t(63)) * split_key_buffers(e_max));
-        c.o_pieces = carve(16 * c.cap);
-        c.o_queue = carve(16 * c.cap);
-        c.slab = std::max(c.slab, o);
+// Scratch for `teams` teams over the graphs of the launch (fewer if theirs
+// would take more than scratch_max bytes or cannot be had), cleared error word.
+static cudaError_t batch_slabs(BatchKernelArgs& c, const BatchSizes& sizes, bool search, uint64_t* teams,
+                               size_t scratch_max, cudaStream_t s, void** slabs) {
+    const uint32_t G = c.b.G;
+    std::vector<SlabLayout> all(*teams);  // by place: for the most vertices and the most entries from there on
+    std::vector<uint64_t> bytes(*teams);
+    uint32_t n = 0;
+    uint64_t e = 0;
+    for (uint32_t k = G; k-- > 0;) {
+        n = std::max(n, sizes.n[k]);
+        e = std::max(e, sizes.e[k]);
+        if (k < *teams) {
+            all[k] = slab_layout(n, e);
+            bytes[k] = c.b.core && search ? std::max(all[k].peel_end, all[k].search_end) : all[k].peel_end;
+            // (the kernel's time depends on the addresses by a few percent; over seven places of the
+            // allocation each, 1,500 graphs of up to 100,000 vertices took 2.11 ms with slabs packed
+            // tightly, 2.07 in steps of 64 KB and 2.11 in steps of 2 MB)
+            if (bytes[k] >= 1u << 16) bytes[k] = (bytes[k] + 0xffff) & ~uint64_t(0xffff);
+        }
     }
-    c.slab = std::max<uint64_t>(c.slab, 256);
-    return c;
-}
-
-// Scratch for `teams` teams (fewer if they would take more than scratch_max bytes), cleared error word.
-static cudaError_t batch_slabs(BatchKernelArgs& c, uint64_t* teams, size_t scratch_max, cudaStream_t s, void** slabs) {
-    *teams = std::max<uint64_t>(1, std::min<uint64_t>(*teams, scratch_max / c.slab));
+    uint64_t t = 1, total = bytes[0];
+    while (t < *teams && total + bytes[t] <= scratch_max) total += bytes[t++];
+    constexpr uint64_t kHead = 256;  // the error word's share
     void* p = nullptr;
-    cudaError_t e = dev_alloc(&p, 256 + *teams * c.slab, s);
-    if (e != cudaSuccess) return e;
+    for (;;) {
+        uint64_t at = (kHead + t * sizeof(SlabLayout) + 255) & ~uint64_t(255);
+        for (uint64_t k = 0; k < t; at += bytes[k++]) all[k].at = at;
+        const cudaError_t err = dev_alloc(&p, at, s);
+        if (err == cudaSuccess) break;
+        if (err != cudaErrorMemoryAllocation || t == 1) return err;
+        cudaGetLastError();  // handled here
+        t = (t + 1) / 2;
+    }
     *slabs = p;
-    c.slabs = static_cast<unsigned char*>(p);
-    return cudaMemsetAsync(p, 0, 256, s);
+    *teams = t;
+    c.scratch = static_cast<unsigned char*>(p);
+    c.slabs = reinterpret_cast<const SlabLayout*>(c.scratch + kHead);
+    std::vector<unsigned char> head(kHead + t * sizeof(SlabLayout), 0);
+    memcpy(head.data() + kHead, all.data(), t * sizeof(SlabLayout));
+    return cudaMemcpyAsync(p, head.data(), head.size(), cudaMemcpyHostToDevice, s);
 }
 
 template <int TB>
@@ -334,12 +378,13 @@ static uint32_t batch_slots(uint32_t block) {
 
 uint32_t batch_slots_for(uint32_t block) { return batch_slots(block); }
 
-cudaError_t batch_launch(const BatchArgs& a, uint32_t n_max, uint64_t e_max, size_t scratch_max, cudaStream_t s,
-                         void** slabs, uint32_t block, uint32_t max_grid) {
-    BatchKernelArgs c = batch_layout(a, n_max, e_max, false);
+cudaError_t batch_launch(const BatchArgs& a, const BatchSizes& sizes, size_t scratch_max, cudaStream_t s, void** slabs,
+                         uint32_t block, uint32_t max_grid) {
+    BatchKernelArgs c = {};
+    c.b = a;
     uint64_t teams = std::min<uint64_t>(batch_slots(block), a.G);
     if (max_grid) teams = std::min<uint64_t>(teams, max_grid);
-    cudaError_t e = batch_slabs(c, &teams, scratch_max, s, slabs);
+    cudaError_t e = batch_slabs(c, sizes, false, &teams, scratch_max, s, slabs);
     if (e != cudaSuccess) return e;
     const uint32_t grid = (uint32_t)teams;
     LaunchScope ls("batch_solve", s);
@@ -351,9 +396,10 @@ cudaError_t batch_launch(const BatchArgs& a, uint32_t n_max, uint64_t e_max, siz
     return cudaGetLastError();
 }
 
-cudaError_t batch_cluster_launch(const BatchArgs& a, uint32_t n_max, uint64_t e_max, size_t scratch_max, cudaStream_t s,
+cudaError_t batch_cluster_launch(const BatchArgs& a, const BatchSizes& sizes, size_t scratch_max, cudaStream_t s,
                                  void** slabs, uint32_t max_sms) {
-    BatchKernelArgs c = batch_layout(a, n_max, e_max, true);
+    BatchKernelArgs c = {};
+    c.b = a;
     // (16 blocks need leave of the device; without it 8 do)
     const bool few = a.G <= kFewGraphs && cudaFuncSetAttribute(batch_kernel<kClusterTB, kClusterBlocksFew>,
                                                               cudaFuncAttributeNonPortableClusterSizeAllowed,
@@ -376,7 +422,7 @@ cudaError_t batch_cluster_launch(const BatchArgs& a, uint32_t n_max, uint64_t e_
     if (e != cudaSuccess) return e;
     uint64_t teams = std::min<uint64_t>(fit > 0 ? fit : 1, a.G);
     if (max_sms) teams = std::min<uint64_t>(teams, std::max<uint32_t>(1, max_sms / size));
-    e = batch_slabs(c, &teams, scratch_max, s, slabs);
+    e = batch_slabs(c, sizes, true, &teams, scratch_max, s, slabs);
     if (e != cudaSuccess) return e;
     cfg.gridDim = dim3((uint32_t)teams * size);
     LaunchScope ls("batch_clusters", s);
@@ -582,6 +628,12 @@ extern "C" dsg_status dsg_batch_solve(const dsg_batch* b, dsg_batch_result* r, v
     }
     a.stats = d_stats;
     uint64_t big_sum_S = 0, big_dec = 0, big_entries = 0;
+    std::vector<uint32_t> on(G);  // vertices and row entries, in the order of the launches
+    std::vector<uint64_t> oe(G);
+    for (uint32_t i = 0; i < G; ++i) {
+        on[i] = (uint32_t)(vb[order[i] + 1] - vb[order[i]]);
+        oe[i] = hoff_ends[order[i] + 1] - hoff_ends[order[i]];
+    }
     // which graphs run on the whole GPU one after the other, which get a cluster, which a block
     uint32_t nbig = 0, ncl = 0;
     if (tu.batch_split) {
@@ -589,12 +641,8 @@ extern "C" dsg_status dsg_batch_solve(const dsg_batch* b, dsg_batch_result* r, v
         ncl = nbig;
     } else {
         std::vector<uint64_t> w(G);
-        std::vector<uint32_t> wn(G);
-        for (uint32_t i = 0; i < G; ++i) {
-            w[i] = work(order[i]);
-            wn[i] = (uint32_t)(vb[order[i] + 1] - vb[order[i]]);
-        }
-        batch_classes(w.data(), wn.data(), G, &nbig, &ncl);
+        for (uint32_t i = 0; i < G; ++i) w[i] = on[i] + oe[i];
+        batch_classes(w.data(), on.data(), G, &nbig, &ncl);
     }
     std::vector<uint64_t> res(4 * (size_t)G, 0);
     for (uint32_t i = 0; i < nbig; ++i) {
@@ -621,17 +669,14 @@ extern "C" dsg_status dsg_batch_solve(const dsg_batch* b, dsg_batch_result* r, v
         }
     }
     // clusters and blocks run side by side: the blocks fill the SMs the clusters leave
-    auto largest = [&](uint32_t lo, uint32_t hi, uint32_t* n_max, uint64_t* e_max) {
-        *n_max = 0;
-        *e_max = 0;
-        for (uint32_t i = lo; i < hi; ++i) {
-            const uint32_t g = order[i];
-            *n_max = std::max<uint32_t>(*n_max, (uint32_t)(vb[g + 1] - vb[g]));
-            *e_max = std::max<uint64_t>(*e_max, hoff_ends[g + 1] - hoff_ends[g]);
-        }
+    uint32_t h_err[2] = {0, 0};
+    // what a launch may take for its slabs: a few times the graphs' own size, so that small graphs
+    // among large ones do not hold memory in proportion to the large ones
+    auto scratch_max = [&](uint32_t lo, uint32_t hi) {
+        uint64_t bytes = 0;
+        for (uint32_t i = lo; i < hi; ++i) bytes += 80 * (uint64_t)on[i] + 8 * oe[i] + 4096;
+        return (size_t)bytes;
     };
-    uint32_t n_max = 0, h_err[2] = {0, 0};
-    uint64_t e_max = 0;
     BatchSide* side = nullptr;
     void *slabs_cl = nullptr, *slabs_bl = nullptr;
     if (ncl > nbig) {
@@ -640,22 +685,21 @@ extern "C" dsg_status dsg_batch_solve(const dsg_batch* b, dsg_batch_result* r, v
         ca.G = ncl - nbig;
         DSG_TRY_CUDA(sc.get(&ca.next, 1));
         DSG_TRY_CUDA(cudaMemsetAsync(ca.next, 0, sizeof(unsigned long long), s));
-        largest(nbig, ncl, &n_max, &e_max);
         if (ncl < G) {
             DSG_TRY_CUDA(batch_side(&side));
             DSG_TRY_CUDA(cudaEventRecord(side->fork, s));
             DSG_TRY_CUDA(cudaStreamWaitEvent(side->s, side->fork, 0));
         }
-        const cudaError_t e = batch_cluster_launch(ca, n_max, e_max, SIZE_MAX, s, &slabs_cl);
+        const cudaError_t e = batch_cluster_launch(ca, {on.data() + nbig, oe.data() + nbig},
+                                                   scratch_max(nbig, ncl), s, &slabs_cl);
         if (slabs_cl) sc.adopt(slabs_cl);
         DSG_TRY_CUDA(e);
     }
     a.order = d_order + ncl;
     a.G = G - ncl;
     if (a.G) {
-        largest(ncl, G, &n_max, &e_max);
         cudaStream_t sb = side ? side->s : s;
-        cudaError_t e = batch_launch(a, n_max, e_max, SIZE_MAX, sb, &slabs_bl, block);
+        cudaError_t e = batch_launch(a, {on.data() + ncl, oe.data() + ncl}, scratch_max(ncl, G), sb, &slabs_bl, block);
         if (slabs_bl && e == cudaSuccess)
             e = cudaMemcpyAsync(&h_err[1], slabs_bl, sizeof(uint32_t), cudaMemcpyDeviceToHost, sb);
         if (slabs_bl) dev_free(slabs_bl, sb);

@@ -412,7 +412,7 @@ __device__ __forceinline__ void split_body(const SplitArgs& a, Team<CL> team, Sp
 
 // Key buffers for a graph of `entries` row entries: the bits searched, since
 // (lo + 2^b)^2 stays below the entries.
-inline uint64_t split_key_buffers(uint64_t entries) {
+__host__ __device__ inline uint64_t split_key_buffers(uint64_t entries) {
     uint64_t nbuf = 1;
     while (nbuf < kSplitBits && (1ull << (2 * nbuf)) <= entries) ++nbuf;
     return nbuf;

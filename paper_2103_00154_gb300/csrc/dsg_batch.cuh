@@ -20,28 +20,34 @@ struct BatchArgs {
     uint32_t* core;         // core numbers per vertex slot (nullable)
     uint8_t* out_set;       // membership in the densest set found (nullable)
     uint64_t* res;          // 4 per graph: E, V, rounds, best_round
-    unsigned long long* next;
+    unsigned long long* next;   // low half: graphs taken, high half: teams that have taken one
     uint32_t hot_deg;
     unsigned long long* stats;  // nullable, 3 counters summed over the batch: sum over graphs and rounds of
                                 // |S_r|, alive-neighbour decrements of the peels, adjacency entries scanned
 };
 
+// The graphs of a launch in its order (host): vertices and row entries.
+struct BatchSizes {
+    const uint32_t* n;
+    const uint64_t* e;
+};
 
 // Launch the block-per-graph kernel over a.order[0, a.G) on stream s
 // (asynchronous) with `block` threads per block (256, 512 or 1024; 0: 512),
 // at most max_grid blocks (0: as many as fit).  a.next must be zeroed and
-// every table filled.  The kernel works on slabs of scratch, one per block,
-// sized by the largest graph (n_max vertices, e_max row entries); at most
-// scratch_max bytes of them, at least one.  *slabs gets them, to be freed by
-// the caller in stream order; the first word is an error word to read when
-// the launch is done.
-cudaError_t batch_launch(const BatchArgs& a, uint32_t n_max, uint64_t e_max, size_t scratch_max, cudaStream_t s,
-                         void** slabs, uint32_t block = 0, uint32_t max_grid = 0);
+// every table filled.  The kernel works on slabs of scratch, one per block:
+// the k-th block to start gets one for the largest of the graphs from the
+// k-th on, which are all it can meet.  At most scratch_max bytes of them, and
+// half as many while there is no memory for them, but at least one.  *slabs
+// gets them, to be freed by the caller in stream order; the first word is an
+// error word to read when the launch is done.
+cudaError_t batch_launch(const BatchArgs& a, const BatchSizes& sizes, size_t scratch_max, cudaStream_t s, void** slabs,
+                         uint32_t block = 0, uint32_t max_grid = 0);
 
 // The same with a thread-block cluster per graph (on at most max_sms SMs; 0:
 // all), for the graphs too large for a block of their own to keep the launch
 // short.
-cudaError_t batch_cluster_launch(const BatchArgs& a, uint32_t n_max, uint64_t e_max, size_t scratch_max, cudaStream_t s,
+cudaError_t batch_cluster_launch(const BatchArgs& a, const BatchSizes& sizes, size_t scratch_max, cudaStream_t s,
                                  void** slabs, uint32_t max_sms = 0);
 
 // Which graphs of a batch, sorted largest first by work (2m + n), go where:

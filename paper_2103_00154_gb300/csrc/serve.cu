@@ -104,6 +104,12 @@ static size_t request_charge(uint32_t n, uint64_t m_raw) {
     return (size_t)m_raw * 64 + (size_t)n * 96 + (64u << 10);
 }
 
+// of these, what a request in a batch holds beside the batch's scratch: its
+// rows (room for every raw pair both ways), its outputs, its table entries
+static size_t resident_bytes(uint32_t n, uint64_t m_raw) {
+    return (size_t)m_raw * 8 + (size_t)n * 13 + 2048;
+}
+
 struct Inflight {
     std::vector<ServeReq*> reqs;
     BatchArgs a;
@@ -265,12 +271,14 @@ static dsg_status launch_batch(dsg_server* s, Inflight& f, cudaStream_t ss, cuda
     std::vector<const uint64_t*> goff(G);
     std::vector<const uint32_t*> gadj(G);
     std::vector<uint32_t> gn(G), gp(G), gq(G), order(G);
+    std::vector<uint64_t> ge(G);
     std::vector<uint8_t> wc(G);
     for (uint32_t i = 0; i < G; ++i) {
         ServeReq* r = f.reqs[i];
         goff[i] = r->g->off;
         gadj[i] = r->g->adj;
         gn[i] = r->n;
+        ge[i] = 2 * r->m;
         gp[i] = r->p;
         gq[i] = r->q;
         wc[i] = r->want_core ? 1 : 0;
@@ -312,26 +320,21 @@ static dsg_status launch_batch(dsg_server* s, Inflight& f, cudaStream_t ss, cuda
     uint32_t grid = 0, ncl = 0;
     {
         std::vector<uint64_t> w(G);
-        for (uint32_t i = 0; i < G; ++i) w[i] = 2 * f.reqs[i]->m + f.reqs[i]->n;
+        for (uint32_t i = 0; i < G; ++i) w[i] = ge[i] + gn[i];
         batch_classes(w.data(), gn.data(), G, &grid, &ncl);  // (none runs on the whole GPU here)
     }
-    // a launch's scratch stays within what its requests were admitted with
+    // a launch's scratch stays within what its requests were admitted with, less what they hold already
     auto launch = [&](uint32_t lo, uint32_t hi, bool clusters, cudaStream_t st) {
         BatchArgs b = a;
         b.order = a.order + lo;
         b.G = hi - lo;
         b.next = a.next + (clusters ? 1 : 0);
-        uint32_t n_max = 0;
-        uint64_t e_max = 0;
         size_t room = 0;
-        for (uint32_t i = lo; i < hi; ++i) {
-            n_max = std::max(n_max, f.reqs[i]->n);
-            e_max = std::max<uint64_t>(e_max, 2 * f.reqs[i]->m);
-            room += f.reqs[i]->charge;
-        }
-        if (clusters) return batch_cluster_launch(b, n_max, e_max, room, st, &f.slabs_cl, std::max(1u, sms - big_sms));
+        for (uint32_t i = lo; i < hi; ++i) room += f.reqs[i]->charge - resident_bytes(f.reqs[i]->n, f.reqs[i]->m_raw);
+        const BatchSizes sizes = {gn.data() + lo, ge.data() + lo};
+        if (clusters) return batch_cluster_launch(b, sizes, room, st, &f.slabs_cl, std::max(1u, sms - big_sms));
         const uint32_t cap = (uint32_t)((uint64_t)batch_slots_for(512) * (sms - big_sms) / sms);
-        return batch_launch(b, n_max, e_max, room, st, &f.slabs_bl, 512, cap ? cap : 1);
+        return batch_launch(b, sizes, room, st, &f.slabs_bl, 512, cap ? cap : 1);
     };
     cudaError_t e = cudaSuccess;
     if (ncl == 0 || ncl == G) {
