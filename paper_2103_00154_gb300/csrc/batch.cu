@@ -429,23 +429,23 @@ cudaError_t batch_cluster_launch(const BatchArgs& a, const BatchSizes& sizes, si
     return cudaLaunchKernelEx(&cfg, kernel, c);
 }
 
-// A cluster for a graph of more than twice a block's share of the batch (it
-// would be the last to end; at one share the clusters hold SMs that the blocks
-// use better: 600 graphs with core numbers 7.2 against 9.2 ms) and of more than
-// 2^17 units of work (40 graphs of 3,000 to 35,000 vertices: 0.44 ms against
-// 0.53 from 2^15 and 0.69 from 2^18).  The whole GPU for one that is more than
-// a quarter of the batch (8 graphs of 100,000 to 300,000 vertices: all in
-// clusters 4.4 ms, three of them on the whole GPU first 5.7) or too large for
-// the search to take it whole.
-void batch_classes(const uint64_t* work, const uint32_t* n, uint32_t G, uint32_t* grid, uint32_t* cluster) {
-    uint64_t total = 0;
-    for (uint32_t i = 0; i < G; ++i) total += work[i];
+// More than a quarter of the batch (8 graphs of 100,000 to 300,000 vertices: all
+// in clusters 4.4 ms, three of them on the whole GPU first 5.7), or too large
+// for the search to take it whole.
+bool batch_takes_grid(uint64_t work, uint32_t n, uint64_t total) {
+    return (work > (1u << 20) && work > total / 4) || n > kTailWhole * 65536;
+}
+
+// More than twice a block's share of the batch (it would be the last to end; at
+// one share the clusters hold SMs that the blocks use better: 600 graphs with
+// core numbers 7.2 against 9.2 ms) and more than 2^17 units of work (40 graphs
+// of 3,000 to 35,000 vertices: 0.44 ms against 0.53 from 2^15 and 0.69 from
+// 2^18).
+uint32_t batch_clusters(const uint64_t* work, uint32_t G, uint64_t total) {
     const uint64_t share = total / batch_slots(512);
     uint32_t k = 0;
-    while (k < G && ((work[k] > (1u << 20) && work[k] > total / 4) || n[k] > kTailWhole * 65536)) ++k;
-    *grid = k;
     while (k < G && work[k] > (1u << 17) && work[k] > 2 * share) ++k;
-    *cluster = k;
+    return k;
 }
 
 // want_core[g] read from host or device memory.
@@ -592,10 +592,6 @@ extern "C" dsg_status dsg_batch_solve(const dsg_batch* b, dsg_batch_result* r, v
         // the tables live in stream-ordered scratch: keep the host vectors alive until the copies ran
         DSG_TRY_CUDA(cudaStreamSynchronize(s));
     }
-    uint32_t* d_order;
-    DSG_TRY_CUDA(sc.get(&d_order, G));
-    DSG_TRY_CUDA(copy_any(d_order, order.data(), G * sizeof(uint32_t), s));
-    a.order = d_order;
     bool core_direct = r->core && is_device_ptr(r->core);
     bool set_direct = r->out_set && is_device_ptr(r->out_set);
     a.core = nullptr;
@@ -628,22 +624,30 @@ extern "C" dsg_status dsg_batch_solve(const dsg_batch* b, dsg_batch_result* r, v
     }
     a.stats = d_stats;
     uint64_t big_sum_S = 0, big_dec = 0, big_entries = 0;
-    std::vector<uint32_t> on(G);  // vertices and row entries, in the order of the launches
-    std::vector<uint64_t> oe(G);
-    for (uint32_t i = 0; i < G; ++i) {
-        on[i] = (uint32_t)(vb[order[i] + 1] - vb[order[i]]);
-        oe[i] = hoff_ends[order[i] + 1] - hoff_ends[order[i]];
-    }
     // which graphs run on the whole GPU one after the other, which get a cluster, which a block
     uint32_t nbig = 0, ncl = 0;
     if (tu.batch_split) {
         while (nbig < G && work(order[nbig]) > tu.batch_split) ++nbig;
-        ncl = nbig;
     } else {
-        std::vector<uint64_t> w(G);
-        for (uint32_t i = 0; i < G; ++i) w[i] = on[i] + oe[i];
-        batch_classes(w.data(), on.data(), G, &nbig, &ncl);
+        // (one of many vertices may stand anywhere in the order)
+        nbig = (uint32_t)(std::stable_partition(order.begin(), order.end(),
+                                                [&](uint32_t x) {
+                                                    return batch_takes_grid(work(x), (uint32_t)(vb[x + 1] - vb[x]),
+                                                                            total_work);
+                                                }) -
+                          order.begin());
     }
+    std::vector<uint32_t> on(G);  // vertices and row entries, in the order of the launches
+    std::vector<uint64_t> oe(G), ow(G);
+    for (uint32_t i = 0; i < G; ++i) {
+        on[i] = (uint32_t)(vb[order[i] + 1] - vb[order[i]]);
+        oe[i] = hoff_ends[order[i] + 1] - hoff_ends[order[i]];
+        ow[i] = on[i] + oe[i];
+    }
+    ncl = nbig + (tu.batch_split ? 0 : batch_clusters(ow.data() + nbig, G - nbig, total_work));
+    uint32_t* d_order;
+    DSG_TRY_CUDA(sc.get(&d_order, G));
+    DSG_TRY_CUDA(copy_any(d_order, order.data(), G * sizeof(uint32_t), s));
     std::vector<uint64_t> res(4 * (size_t)G, 0);
     for (uint32_t i = 0; i < nbig; ++i) {
         const uint32_t g = order[i];

@@ -50,10 +50,12 @@ cudaError_t batch_launch(const BatchArgs& a, const BatchSizes& sizes, size_t scr
 cudaError_t batch_cluster_launch(const BatchArgs& a, const BatchSizes& sizes, size_t scratch_max, cudaStream_t s,
                                  void** slabs, uint32_t max_sms = 0);
 
-// Which graphs of a batch, sorted largest first by work (2m + n), go where:
-// [0, *grid) one at a time on the whole GPU, [*grid, *cluster) a cluster each,
-// the rest a block each.
-void batch_classes(const uint64_t* work, const uint32_t* n, uint32_t G, uint32_t* grid, uint32_t* cluster);
+// Whether a graph of a batch of `total` work (2m + n, summed) is solved by the
+// whole GPU, before the others.
+bool batch_takes_grid(uint64_t work, uint32_t n, uint64_t total);
+// How many of the others, given largest first, get a cluster each; the rest
+// get a block each.
+uint32_t batch_clusters(const uint64_t* work, uint32_t G, uint64_t total);
 
 // Blocks of `block` threads the block-per-graph kernel can keep resident on the GPU.
 uint32_t batch_slots_for(uint32_t block);

@@ -29,7 +29,7 @@ struct Tuning {
     uint32_t tail_max = 65536;   // k-core: scale of the graphs and remaining graphs whose core numbers are searched
                                  // bit by bit instead of level by level (kTailHandOver, kTailWhole; 0: never)
     uint32_t batch_split = 0;    // batches: a graph whose work (2m + n) exceeds this is solved by the
-                                 // grid-wide kernels, the others by a block each (0: batch_classes)
+                                 // grid-wide kernels, the others by a block each (0: batch_takes_grid)
     uint32_t batch_block = 512;  // batches: threads per block of the block-per-graph kernel
     uint32_t peel_lazy = 1;      // peel: thin-tail rounds test only the candidate list (0: every round
                                  // tests the whole alive list); read from the global tuning only

@@ -317,12 +317,10 @@ static dsg_status launch_batch(dsg_server* s, Inflight& f, cudaStream_t ss, cuda
     const uint32_t sms = (uint32_t)dev_info().sms;
     const uint32_t big_sms =
         s->cfg.big_work == UINT64_MAX ? 0 : (uint32_t)std::min<uint64_t>((uint64_t)s->cfg.big_sms * s->cfg.big_threads, sms - 1);
-    uint32_t grid = 0, ncl = 0;
-    {
-        std::vector<uint64_t> w(G);
-        for (uint32_t i = 0; i < G; ++i) w[i] = ge[i] + gn[i];
-        batch_classes(w.data(), gn.data(), G, &grid, &ncl);  // (none runs on the whole GPU here)
-    }
+    std::vector<uint64_t> work(G);
+    uint64_t total = 0;
+    for (uint32_t i = 0; i < G; ++i) total += work[i] = ge[i] + gn[i];
+    const uint32_t ncl = batch_clusters(work.data(), G, total);  // (none runs on the whole GPU here)
     // a launch's scratch stays within what its requests were admitted with, less what they hold already
     auto launch = [&](uint32_t lo, uint32_t hi, bool clusters, cudaStream_t st) {
         BatchArgs b = a;
