@@ -1366,8 +1366,16 @@ constexpr uint32_t kDirectRow = 16 * 1024;  // longest row (repeats counted) a b
 // 524,288 217 / 565, 2^21 925 / 865, 2^22 1371 / 1185).
 constexpr uint64_t kDirectPairs = 1500000;
 // Up to here one cluster, above a grid of a block per 1,024 pairs (12,000
-// pairs: 63 against 74 us; 50,000: 96 against 73 us).
+// pairs: 63 against 74 us; 50,000: 96 against 73 us) and per 2,048 vertices:
+// counts, scans and row sweeps walk every vertex, however few pairs there are
+// (us for 10^4 pairs, cluster / grid: 20,000 vertices 71 / 86, 50,000 78 / 79,
+// 100,000 87 / 80, 10^6 300 / 126, 6 10^6 1542 / 359 -- 2101 with blocks by the
+// pairs alone, 604 on the other path; a block per 8,192 vertices: 10^5 111
+// instead of 80, 10^6 135 instead of 126).
 constexpr uint64_t kDirectClusterPairs = 16384;
+constexpr uint32_t kDirectClusterVertices = 65536;
+constexpr uint64_t kDirectBlockPairs = 1024, kDirectBlockVertices = 2048;
+constexpr uint64_t kDirectShared = 16;  // times that beside other work
 
 struct DirectArgs {
     uint32_t n, m;
@@ -1692,7 +1700,7 @@ static dsg_status ingest_direct(uint32_t n, uint32_t m, const uint32_t* src, con
                                 cudaStream_t s, dsg_graph** out) {
     int dev = 0;
     DSG_TRY_CUDA(cudaGetDevice(&dev));
-    const bool cluster = m <= kDirectClusterPairs;
+    const bool cluster = m <= kDirectClusterPairs && n <= kDirectClusterVertices;
     static std::atomic<bool> ready[64] = {};  // the attributes are per function and device, set once (idempotent)
     if (!ready[dev & 63]) {
         for (auto* k : {direct_kernel<true>, direct_kernel<false>})
@@ -1738,12 +1746,13 @@ static dsg_status ingest_direct(uint32_t n, uint32_t m, const uint32_t* src, con
                 e = launch_cluster(direct_kernel<true>, kDirectBlocks, kDirectTB, sizeof(DirectSmem), s, a);
         } else {
             uint32_t grid = 1;
-            const uint64_t pairs_per_block = shared ? 16384 : 1024;
+            const uint64_t per = shared ? kDirectShared : 1;
+            const uint64_t blocks = std::max(m / (kDirectBlockPairs * per), n / (kDirectBlockVertices * per));
             e = cudaMemsetAsync(a.ctl, 0, sizeof(DirectCtl), s);
             if (e == cudaSuccess) e = cudaMemcpyAsync(a.out, h, sizeof(h), cudaMemcpyHostToDevice, s);
             if (e == cudaSuccess)
-                e = coop_grid(direct_kernel<false>, kDirectTB, sizeof(DirectSmem), (uint64_t)m * kDirectTB / pairs_per_block, 1,
-                              &grid, kDirectGridMax);
+                e = coop_grid(direct_kernel<false>, kDirectTB, sizeof(DirectSmem), blocks * kDirectTB, 1, &grid,
+                              kDirectGridMax);
             if (e == cudaSuccess) {
                 void* params[] = {&a};
                 LaunchScope ls("ingest_direct", s);
