@@ -403,6 +403,8 @@ void dsg_serve_destroy(dsg_server* s);
  *   chunk_len      rows are cut into pieces of at most this many entries, >= 32
  * Process-wide; also read from DSG_BLOCK, DSG_BLOCKS_PER_SM, DSG_SHORT_MAX and
  * DSG_CHUNK_LEN at first use.  Results never depend on these.
+ * DSG_CLUSTERS=0 (read at first use): no thread-block clusters; grids and
+ * blocks do their work, as they do where a GPU has no room for a cluster.
  */
 dsg_status dsg_set_tuning(uint32_t block, uint32_t blocks_per_sm, uint32_t short_max, uint32_t chunk_len);
 dsg_status dsg_get_tuning(uint32_t* block, uint32_t* blocks_per_sm, uint32_t* short_max, uint32_t* chunk_len);

@@ -8,6 +8,7 @@
 
 #include <mutex>
 #include <unordered_map>
+#include <vector>
 
 #include "dsg_common.cuh"
 #include "dsg_kernels.cuh"
@@ -118,6 +119,63 @@ bool is_device_ptr(const void* p) {
 cudaError_t copy_any(void* dst, const void* src, size_t bytes, cudaStream_t s) {
     if (bytes == 0) return cudaSuccess;
     return cudaMemcpyAsync(dst, src, bytes, cudaMemcpyDefault, s);
+}
+
+typedef int (*CtxGetCurrentFn)(void**);
+typedef int (*CtxGetIdFn)(void*, unsigned long long*);
+
+unsigned long long current_ctx_id() {
+    static CtxGetCurrentFn get_current = nullptr;
+    static CtxGetIdFn get_id = nullptr;
+    static std::once_flag once;
+    std::call_once(once, [] {
+        void* f = nullptr;
+        cudaDriverEntryPointQueryResult q;
+        if (cudaGetDriverEntryPointByVersion("cuCtxGetCurrent", &f, 12000, cudaEnableDefault, &q) == cudaSuccess &&
+            q == cudaDriverEntryPointSuccess)
+            get_current = reinterpret_cast<CtxGetCurrentFn>(f);
+        f = nullptr;
+        if (cudaGetDriverEntryPointByVersion("cuCtxGetId", &f, 12000, cudaEnableDefault, &q) == cudaSuccess &&
+            q == cudaDriverEntryPointSuccess)
+            get_id = reinterpret_cast<CtxGetIdFn>(f);
+    });
+    void* ctx = nullptr;
+    unsigned long long id = 0;
+    if (!get_current || !get_id || get_current(&ctx) != 0 || !ctx || get_id(ctx, &id) != 0) return 0;
+    return id;
+}
+
+uint32_t clusters_fit(const void* kernel, uint32_t blocks, uint32_t threads, size_t smem) {
+    static const bool allowed = [] {
+        const char* e = getenv("DSG_CLUSTERS");
+        return !(e && e[0] == '0' && !e[1]);
+    }();
+    if (!allowed) return 0;
+    struct Known {
+        unsigned long long ctx;
+        const void* kernel;
+        uint32_t fit;
+    };
+    static thread_local std::vector<Known> known;
+    const unsigned long long ctx = current_ctx_id();
+    for (const Known& k : known)
+        if (ctx && k.ctx == ctx && k.kernel == kernel) return k.fit;
+    int fit = 0;
+    cudaError_t e = cudaSuccess;
+    if (smem) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e == cudaSuccess && blocks > 8) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    if (e == cudaSuccess) {
+        cudaLaunchAttribute attr;
+        const cudaLaunchConfig_t cfg = cluster_config(blocks, blocks, threads, smem, nullptr, &attr);
+        e = cudaOccupancyMaxActiveClusters(&fit, kernel, &cfg);
+    }
+    if (e != cudaSuccess) {
+        cudaGetLastError();  // not to be found by the next launch's check
+        fit = 0;
+    }
+    if (known.size() >= 64) known.clear();  // (contexts that came and went)
+    known.push_back({ctx, kernel, fit > 0 ? (uint32_t)fit : 0u});
+    return known.back().fit;
 }
 
 const DevInfo& dev_info() {

@@ -400,31 +400,18 @@ cudaError_t batch_cluster_launch(const BatchArgs& a, const BatchSizes& sizes, si
                                  void** slabs, uint32_t max_sms) {
     BatchKernelArgs c = {};
     c.b = a;
-    // (16 blocks need leave of the device; without it 8 do)
-    const bool few = a.G <= kFewGraphs && cudaFuncSetAttribute(batch_kernel<kClusterTB, kClusterBlocksFew>,
-                                                              cudaFuncAttributeNonPortableClusterSizeAllowed,
-                                                              1) == cudaSuccess;
-    const uint32_t size = few ? kClusterBlocksFew : kClusterBlocks;
-    auto* const kernel = few ? batch_kernel<kClusterTB, kClusterBlocksFew> : batch_kernel<kClusterTB, kClusterBlocks>;
-    cudaLaunchConfig_t cfg = {};
-    cfg.blockDim = dim3(kClusterTB);
-    cfg.stream = s;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = size;
-    attr[0].val.clusterDim.y = 1;
-    attr[0].val.clusterDim.z = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    cfg.gridDim = dim3(size);
-    int fit = 0;
-    cudaError_t e = cudaOccupancyMaxActiveClusters(&fit, kernel, &cfg);
-    if (e != cudaSuccess) return e;
-    uint64_t teams = std::min<uint64_t>(fit > 0 ? fit : 1, a.G);
+    const uint32_t fit_few =
+        a.G <= kFewGraphs ? clusters_fit(batch_kernel<kClusterTB, kClusterBlocksFew>, kClusterBlocksFew, kClusterTB, 0) : 0;
+    const uint32_t size = fit_few ? kClusterBlocksFew : kClusterBlocks;
+    auto* const kernel = fit_few ? batch_kernel<kClusterTB, kClusterBlocksFew> : batch_kernel<kClusterTB, kClusterBlocks>;
+    uint64_t teams = fit_few ? fit_few : clusters_fit(batch_kernel<kClusterTB, kClusterBlocks>, kClusterBlocks, kClusterTB, 0);
+    if (teams == 0) return cudaErrorInvalidConfiguration;  // (batch_clusters gives no graph to clusters then)
+    teams = std::min<uint64_t>(teams, a.G);
     if (max_sms) teams = std::min<uint64_t>(teams, std::max<uint32_t>(1, max_sms / size));
-    e = batch_slabs(c, sizes, true, &teams, scratch_max, s, slabs);
+    const cudaError_t e = batch_slabs(c, sizes, true, &teams, scratch_max, s, slabs);
     if (e != cudaSuccess) return e;
-    cfg.gridDim = dim3((uint32_t)teams * size);
+    cudaLaunchAttribute attr;
+    const cudaLaunchConfig_t cfg = cluster_config((uint32_t)teams * size, size, kClusterTB, 0, s, &attr);
     LaunchScope ls("batch_clusters", s);
     return cudaLaunchKernelEx(&cfg, kernel, c);
 }
@@ -444,6 +431,7 @@ bool batch_takes_grid(uint64_t work, uint32_t n, uint64_t total) {
 uint32_t batch_clusters(const uint64_t* work, uint32_t G, uint64_t total) {
     const uint64_t share = total / batch_slots(512);
     uint32_t k = 0;
+    if (G == 0 || !clusters_fit(batch_kernel<kClusterTB, kClusterBlocks>, kClusterBlocks, kClusterTB, 0)) return 0;
     while (k < G && work[k] > (1u << 17) && work[k] > 2 * share) ++k;
     return k;
 }

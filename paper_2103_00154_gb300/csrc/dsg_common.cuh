@@ -55,6 +55,10 @@ struct DevInfo {
 };
 const DevInfo& dev_info();
 
+// Id of the current context (0 when the driver cannot tell); never used again
+// by another one.
+unsigned long long current_ctx_id();
+
 // Upper bound on device-side waits (ns); 0 = library default.
 uint64_t wait_limit_ns();
 

@@ -148,23 +148,40 @@ cudaError_t coop_grid(K kernel, uint32_t block, size_t smem, uint64_t work_items
     return cudaSuccess;
 }
 
-// A launch of one thread-block cluster of `blocks` blocks (16 need the
-// kernel's non-portable attribute).
-template <class... P, class... A>
-cudaError_t launch_cluster(void (*kernel)(P...), uint32_t blocks, uint32_t threads, size_t smem, cudaStream_t s,
-                           A... args) {
+// A launch of thread-block clusters of `blocks` blocks, `grid` blocks in all.
+inline cudaLaunchConfig_t cluster_config(uint32_t grid, uint32_t blocks, uint32_t threads, size_t smem, cudaStream_t s,
+                                         cudaLaunchAttribute* attr) {
+    attr->id = cudaLaunchAttributeClusterDimension;
+    attr->val.clusterDim.x = blocks;
+    attr->val.clusterDim.y = 1;
+    attr->val.clusterDim.z = 1;
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(blocks);
+    cfg.gridDim = dim3(grid);
     cfg.blockDim = dim3(threads);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = s;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = blocks;
-    attr[0].val.clusterDim.y = 1;
-    attr[0].val.clusterDim.z = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
+    return cfg;
+}
+
+// How many such clusters of a kernel the current context can hold at once, the
+// kernel's attributes for them set: 0 where a cluster of that size has no
+// place (a partitioned or capped GPU) or DSG_CLUSTERS is 0; the grid or the
+// blocks beside it do the work then.  Asked once per thread, context and
+// kernel (always the same blocks, threads and shared memory).
+uint32_t clusters_fit(const void* kernel, uint32_t blocks, uint32_t threads, size_t smem);
+template <class... P>
+uint32_t clusters_fit(void (*kernel)(P...), uint32_t blocks, uint32_t threads, size_t smem) {
+    return clusters_fit(reinterpret_cast<const void*>(kernel), blocks, threads, smem);
+}
+
+// One cluster.
+template <class... P, class... A>
+cudaError_t launch_cluster(void (*kernel)(P...), uint32_t blocks, uint32_t threads, size_t smem, cudaStream_t s,
+                           A... args) {
+    cudaLaunchAttribute attr;
+    const cudaLaunchConfig_t cfg = cluster_config(blocks, blocks, threads, smem, s, &attr);
     return cudaLaunchKernelEx(&cfg, kernel, args...);
 }
 

@@ -24,7 +24,6 @@
 #include <cooperative_groups.h>
 
 #include <algorithm>
-#include <atomic>
 
 #include "dsg_common.cuh"
 #include "dsg_kernels.cuh"
@@ -1700,14 +1699,8 @@ static dsg_status ingest_direct(uint32_t n, uint32_t m, const uint32_t* src, con
                                 cudaStream_t s, dsg_graph** out) {
     int dev = 0;
     DSG_TRY_CUDA(cudaGetDevice(&dev));
-    const bool cluster = m <= kDirectClusterPairs && n <= kDirectClusterVertices;
-    static std::atomic<bool> ready[64] = {};  // the attributes are per function and device, set once (idempotent)
-    if (!ready[dev & 63]) {
-        for (auto* k : {direct_kernel<true>, direct_kernel<false>})
-            DSG_TRY_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(DirectSmem)));
-        DSG_TRY_CUDA(cudaFuncSetAttribute(direct_kernel<true>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
-        ready[dev & 63] = true;
-    }
+    const bool cluster = m <= kDirectClusterPairs && n <= kDirectClusterVertices &&
+                         clusters_fit(direct_kernel<true>, kDirectBlocks, kDirectTB, sizeof(DirectSmem)) > 0;
     Scratch sc(s);
     DirectArgs a;
     a.n = n;
@@ -1750,6 +1743,9 @@ static dsg_status ingest_direct(uint32_t n, uint32_t m, const uint32_t* src, con
             const uint64_t blocks = std::max(m / (kDirectBlockPairs * per), n / (kDirectBlockVertices * per));
             e = cudaMemsetAsync(a.ctl, 0, sizeof(DirectCtl), s);
             if (e == cudaSuccess) e = cudaMemcpyAsync(a.out, h, sizeof(h), cudaMemcpyHostToDevice, s);
+            if (e == cudaSuccess)
+                e = cudaFuncSetAttribute(direct_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)sizeof(DirectSmem));
             if (e == cudaSuccess)
                 e = coop_grid(direct_kernel<false>, kDirectTB, sizeof(DirectSmem), blocks * kDirectTB, 1, &grid,
                               kDirectGridMax);

@@ -195,8 +195,7 @@ dsg_status core_split(uint32_t r, uint32_t lo, const uint64_t* off, const uint32
     a.pieces = reinterpret_cast<uint4*>(w + words);
     a.queue = a.pieces + a.cap;
     const bool small = r + entries <= kSmallCore && (g->max_blocks == 0 || g->max_blocks >= kSmallBlocks) &&
-                       cudaFuncSetAttribute(core_split_cluster_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed,
-                                            1) == cudaSuccess;
+                       clusters_fit(core_split_cluster_kernel, kSmallBlocks, kSplitTB, 0) > 0;
     if (small) {
         LaunchScope ls("kcore_split", s);
         DSG_TRY_CUDA(launch_cluster(core_split_cluster_kernel, kSmallBlocks, kSplitTB, 0, s, a));

@@ -182,8 +182,7 @@ static dsg_status run_peel(const dsg_graph* g, uint32_t p, uint32_t q, uint64_t*
         if (set_out && !set_direct) set_dev = w + o_set;
     }
     const bool small = !wrap_in && n + 2 * g->m <= kSmallPeel && (g->max_blocks == 0 || g->max_blocks >= kSmallBlocks) &&
-                       cudaFuncSetAttribute(peel_cluster_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) ==
-                           cudaSuccess;
+                       clusters_fit(peel_cluster_kernel, kSmallBlocks, kSmallTB, 0) > 0;
     if (small) {
         LaunchScope ls("peel_rounds", s);
         DSG_TRY_CUDA(launch_cluster(peel_cluster_kernel, kSmallBlocks, kSmallTB, 0, s, a, pr_dev, set_dev));
@@ -435,38 +434,12 @@ static __device__ __align__(256) unsigned char g_noalloc_scratch[kNoAllocScratch
 // made again (cudaDeviceReset, a released primary context) the module is
 // loaded again and the array may sit elsewhere, so the new context looks it
 // up afresh.
-typedef int (*CtxGetCurrentFn)(void**);
-typedef int (*CtxGetIdFn)(void*, unsigned long long*);
-
 struct NoAllocSlot {
     unsigned long long ctx_id = 0;  // 0: empty
     unsigned char* addr = nullptr;
 };
 static std::mutex g_noalloc_mu;
 static NoAllocSlot g_noalloc_slots[64];
-
-// Id of the current context (0 when the driver cannot tell: the address is
-// then looked up on every call).
-static unsigned long long current_ctx_id() {
-    static CtxGetCurrentFn get_current = nullptr;
-    static CtxGetIdFn get_id = nullptr;
-    static std::once_flag once;
-    std::call_once(once, [] {
-        void* f = nullptr;
-        cudaDriverEntryPointQueryResult q;
-        if (cudaGetDriverEntryPointByVersion("cuCtxGetCurrent", &f, 12000, cudaEnableDefault, &q) == cudaSuccess &&
-            q == cudaDriverEntryPointSuccess)
-            get_current = reinterpret_cast<CtxGetCurrentFn>(f);
-        f = nullptr;
-        if (cudaGetDriverEntryPointByVersion("cuCtxGetId", &f, 12000, cudaEnableDefault, &q) == cudaSuccess &&
-            q == cudaDriverEntryPointSuccess)
-            get_id = reinterpret_cast<CtxGetIdFn>(f);
-    });
-    void* ctx = nullptr;
-    unsigned long long id = 0;
-    if (!get_current || !get_id || get_current(&ctx) != 0 || !ctx || get_id(ctx, &id) != 0) return 0;
-    return id;
-}
 
 static dsg_status noalloc_scratch(unsigned char** out) {
     int dev = 0;
