@@ -394,10 +394,10 @@ void dsg_serve_destroy(dsg_server* s);
 
 /*
  * Launch parameters of the round kernels (not part of the method):
- *   block          threads per block of the persistent kernels: 256, 512, 1024
+ *   block          threads per block of the persistent kernels: 256, 512,
+ *                  1024, or 0 (the default): picked by the graph's size and
+ *                  the kernel (dsg_tune_lookup tells; dsg_get_tuning says 512)
  *   blocks_per_sm  resident blocks per SM (0 = as many as fit)
- *                  (until this call or DSG_BLOCK gives it, it is picked by
- *                  the graph's size and the kernel)
  *   short_max      has no effect any more (rows of all lengths are walked
  *                  edge-balanced)
  *   chunk_len      rows are cut into pieces of at most this many entries, >= 32

@@ -31,9 +31,11 @@ def round_bound(n: int, p: int, q: int) -> int:
     return int(lib().dsg_round_bound(n, p, q))
 
 
-def set_tuning(block: int = 512, blocks_per_sm: int = 0, short_max: int = 32, chunk_len: int = 256,
+def set_tuning(block: int = 0, blocks_per_sm: int = 0, short_max: int = 32, chunk_len: int = 256,
                hot_deg: int = 0, local_max: int = 1024, local_work: int = 16384, inline_max: int = 256,
                kcore_tail: int = 65536, batch_split: int = 0, peel_lazy: bool = True, peel_vec: bool = False):
+    """Launch parameters of every later solve, all of them; set_tuning() sets the
+    defaults again (block = 0: by graph size and kernel)."""
     N.check(lib().dsg_set_tuning(block, blocks_per_sm, short_max, chunk_len), "set_tuning")
     N.check(lib().dsg_set_hot_degree(hot_deg), "set_hot_degree")
     N.check(lib().dsg_set_local_max(local_max, local_work), "set_local_max")

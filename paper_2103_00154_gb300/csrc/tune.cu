@@ -14,7 +14,7 @@ namespace dsg {
 static std::mutex g_tune_mu;
 static Tuning g_tune;
 static bool g_tune_set = false;
-static bool g_block_given = false;  // by dsg_set_tuning or DSG_BLOCK: then no rule of its own picks the block size
+static bool g_block_given = false;  // by dsg_set_tuning or DSG_BLOCK; else default_block picks the block size
 
 static uint32_t env_u32(const char* name, uint32_t dflt) {
     const char* e = getenv(name);
@@ -56,12 +56,12 @@ using namespace dsg;
 
 extern "C" dsg_status dsg_set_tuning(uint32_t block, uint32_t blocks_per_sm, uint32_t short_max, uint32_t chunk_len) {
     clear_error();
-    DSG_CHECK_ARG(block == 256 || block == 512 || block == 1024, "block must be 256, 512 or 1024");
+    DSG_CHECK_ARG(block == 0 || block == 256 || block == 512 || block == 1024, "block must be 0, 256, 512 or 1024");
     DSG_CHECK_ARG(chunk_len >= 32 && chunk_len <= (1u << 20), "chunk_len must be in [32, 2^20]");
     DSG_CHECK_ARG(short_max >= 1 && short_max <= 4096, "short_max must be in [1, 4096]");
     std::lock_guard<std::mutex> lk(g_tune_mu);
-    g_tune.block = block;
-    g_block_given = true;
+    g_tune.block = block ? block : Tuning().block;
+    g_block_given = block != 0;
     g_tune.blocks_per_sm = blocks_per_sm;
     g_tune.short_max = short_max;
     g_tune.chunk_len = chunk_len;
