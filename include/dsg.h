@@ -134,7 +134,8 @@ typedef struct {
     uint64_t* hist_E;     /* out, nullable: |E(S_r)| for r = 0..R */
     uint32_t* peel_round; /* out, nullable, n entries: round (1-based) in which v failed */
     uint8_t* out_set;     /* out, nullable, n entries: membership in S~ */
-    uint64_t edges_scanned; /* out: adjacency entries read by the neighbour scans (= 2m) */
+    uint64_t edges_scanned; /* out: adjacency entries read by the neighbour scans (2m, less the rows of a
+                               last round of at most 2^16 vertices, which are not read) */
     uint64_t decrements;    /* out: degree decrements of surviving neighbours (edges whose
                                ends failed in different rounds) */
     uint64_t tested;        /* out: vertex tests of the threshold passes, summed over the rounds */

@@ -353,7 +353,7 @@ dsg_status dsg_bahmani_trace(const dsg_graph* g, uint32_t eps_num, uint32_t eps_
     t->best_round = c.best_round;
     t->best_E = g->n ? c.best_E : 0;
     t->best_V = g->n ? c.best_V : 0;
-    t->edges_scanned = 2 * g->m;
+    t->edges_scanned = g->n ? c.scanned : 0;
     t->decrements = g->n ? c.dec : 0;
     t->tested = g->n ? c.tested : 0;
     t->lazy_rounds = g->n ? c.lazy_rounds : 0;

@@ -11,8 +11,9 @@
 //     summed (X);
 //   the blocks meet (Algorithm 1's synchronisation between its two parts),
 //     on a word that also sums the pieces queued;
-//   phase 2 (Alg. 1 part 2): every adjacency entry u of every failed v is read
-//     once, the pieces dealt to the warps in groups as large as spread them
+//   phase 2 (Alg. 1 part 2; not where every vertex left has failed and there
+//     are at most kLastMax of them): every adjacency entry u of every failed v
+//     is read once, the pieces dealt to the warps in groups as large as spread them
 //     over all warps and a group's entries to the warp's lanes; u's bits in
 //     the status map say whether it is still alive (and whether it is a hub);
 //     an alive u loses one degree (atomicSub, combined per block for hubs) and
@@ -65,6 +66,7 @@ struct __align__(128) PeelCtl {
     unsigned long long rounds, best_round, best_E, best_V;
     unsigned long long stamps;
     unsigned long long cur_S, cur_E;  // |S_r| and |E(S_r)| where the launch stopped
+    unsigned long long scanned;       // row entries read by the neighbour scans
 };
 
 struct PeelArgs {
@@ -129,6 +131,7 @@ struct PeelSmem {
     unsigned long long add[4];     // this block's part of failed, xsum, rows, dec in the running phase
     uint64_t own[TB / 32][32];     // phase 2, a warp's pieces: row position to add an entry to
     unsigned long long cum[5];     // failed, xsum, rows, dec and the candidate cursor after the round
+    unsigned long long scanned;    // rows after the last round that was scanned
     MeetSmem meet;
 };
 
@@ -191,6 +194,7 @@ __device__ __forceinline__ PeelOut peel_body(const PeelArgs& a, Team<CL> team, P
         sm.cum[1] = resume ? 2 * (a.m - a.E0) : 0;
         sm.cum[2] = sm.cum[3] = sm.cum[4] = 0;
         sm.agg_used = 0;
+        sm.scanned = 0;
     }
     if (team.rank == 0 && tid == 0 && !resume && a.hist_S) {
         a.hist_S[0] = S;
@@ -546,6 +550,7 @@ __device__ __forceinline__ PeelOut peel_body(const PeelArgs& a, Team<CL> team, P
         const uint64_t rows_left = 2 * a.m - sm.cum[2], cand_hi = sm.cum[4];
         ++r;
         if (team.rank == 0 && tid == 0) {
+            sm.scanned = sm.cum[2];
             if (!a.hist_S) {
             } else if (r < a.hist_cap) {
                 a.hist_S[r] = S1;
@@ -613,6 +618,7 @@ __device__ __forceinline__ PeelOut peel_body(const PeelArgs& a, Team<CL> team, P
         ctl->dec = sm.cum[3];
         ctl->tested = tested;
         ctl->lazy_rounds = lazy_rounds;
+        ctl->scanned = sm.scanned;
     }
     return {r, best_round, best_E, best_V};
 }
