@@ -335,7 +335,7 @@ typedef struct {
                               grid-wide kernels on big_sms SMs, not in a block-per-graph batch
                               (0: 2^23; UINT64_MAX: never) */
     uint32_t big_sms;      /* SMs each grid-wide solve of a big request uses (0: a quarter of them
-                              divided by big_threads); the block-per-graph batches use the rest */
+                              divided by big_threads); each launch of a batch leaves them free */
     uint64_t max_batch_work; /* a launch closes before the next ready request would take its summed
                                 work (2m + n of its graphs) past this, so one launch's run time, and
                                 the wait of the requests behind it, stays bounded (0: no limit) */

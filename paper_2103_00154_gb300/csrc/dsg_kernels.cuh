@@ -4,6 +4,10 @@
 // between translation units.
 #pragma once
 
+#include <algorithm>
+#include <condition_variable>
+#include <mutex>
+
 #include "dsg_common.cuh"
 
 namespace dsg {
@@ -69,9 +73,42 @@ class LaunchScope {
 dsg_status ingest_from_csr_entries(uint32_t n, const uint64_t* off, const uint32_t* adj, uint64_t total,
                                    uint32_t flags, cudaStream_t s, dsg_graph** out);
 
-// dsg_graph_from_edges; shared: other work is on the GPU, take few blocks.
+// Room on the GPU, in blocks of an SM each, for the grids of several host
+// threads whose blocks wait for one another: as long as all that run at once
+// fit side by side, none depends on another's leaving.
+class GridRoom {
+  public:
+    // least: what a thread that wants that much waits for
+    void set(uint32_t blocks, uint32_t least) {
+        free_ = blocks;
+        least_ = least;
+    }
+    // Up to `want` blocks, as many as are free once there are min(want, least).
+    uint32_t take(uint32_t want) {
+        std::unique_lock<std::mutex> lk(mu_);
+        cv_.wait(lk, [&] { return free_ >= std::min(want, least_); });
+        const uint32_t got = std::min(want, free_);
+        free_ -= got;
+        return got;
+    }
+    void give(uint32_t blocks) {
+        {
+            std::lock_guard<std::mutex> lk(mu_);
+            free_ += blocks;
+        }
+        cv_.notify_all();
+    }
+
+  private:
+    std::mutex mu_;
+    std::condition_variable cv_;
+    uint32_t free_ = 1, least_ = 1;
+};
+
+// dsg_graph_from_edges; room (nullable): other work is on the GPU, take few
+// blocks, and those that wait for one another from there.
 dsg_status graph_from_edges(uint32_t n, uint64_t m_raw, const uint32_t* src, const uint32_t* dst, uint32_t flags,
-                            bool shared, void* stream, dsg_graph** out);
+                            GridRoom* room, void* stream, dsg_graph** out);
 
 // One peel on a graph (any dsg_graph, including a view into a packed batch):
 // set_dev (device, nullable) gets the densest-set mask; out4 = E, V, rounds,

@@ -1693,9 +1693,9 @@ static dsg_status finish_rows(uint32_t n, const uint64_t* start, const uint32_t*
     return DSG_OK;
 }
 
-// The small-input path.  shared: other work is on the GPU (the server's
-// ingest threads): few blocks, which find room beside it.
-static dsg_status ingest_direct(uint32_t n, uint32_t m, const uint32_t* src, const uint32_t* dst, bool shared,
+// The small-input path.  room: other work is on the GPU (the server's ingest
+// threads): few blocks, which find room beside it.
+static dsg_status ingest_direct(uint32_t n, uint32_t m, const uint32_t* src, const uint32_t* dst, GridRoom* room,
                                 cudaStream_t s, dsg_graph** out) {
     int dev = 0;
     DSG_TRY_CUDA(cudaGetDevice(&dev));
@@ -1726,6 +1726,15 @@ static dsg_status ingest_direct(uint32_t n, uint32_t m, const uint32_t* src, con
     g->n = n;
     g->device = dev;
     g->stream = s;
+    struct Share {  // of the room, until the launch is over
+        GridRoom* room;
+        uint32_t blocks = 0;
+        void give() {
+            if (blocks) room->give(blocks);
+            blocks = 0;
+        }
+        ~Share() { give(); }
+    } share{room};
     uint64_t h[3] = {0, ERR_TIMEOUT, 0};  // (the error stays set if a wait runs out: the kernel leaves before it writes it)
     cudaError_t e = dev_alloc((void**)&g->off, ((size_t)n + 1) * sizeof(uint64_t), s);
     if (e == cudaSuccess) e = dev_alloc((void**)&g->adj, (size_t)(m ? 2 * (uint64_t)m : 1) * sizeof(uint32_t), s);
@@ -1739,7 +1748,7 @@ static dsg_status ingest_direct(uint32_t n, uint32_t m, const uint32_t* src, con
                 e = launch_cluster(direct_kernel<true>, kDirectBlocks, kDirectTB, sizeof(DirectSmem), s, a);
         } else {
             uint32_t grid = 1;
-            const uint64_t per = shared ? kDirectShared : 1;
+            const uint64_t per = room ? kDirectShared : 1;
             const uint64_t blocks = std::max(m / (kDirectBlockPairs * per), n / (kDirectBlockVertices * per));
             e = cudaMemsetAsync(a.ctl, 0, sizeof(DirectCtl), s);
             if (e == cudaSuccess) e = cudaMemcpyAsync(a.out, h, sizeof(h), cudaMemcpyHostToDevice, s);
@@ -1749,6 +1758,7 @@ static dsg_status ingest_direct(uint32_t n, uint32_t m, const uint32_t* src, con
             if (e == cudaSuccess)
                 e = coop_grid(direct_kernel<false>, kDirectTB, sizeof(DirectSmem), blocks * kDirectTB, 1, &grid,
                               kDirectGridMax);
+            if (e == cudaSuccess && room) share.blocks = grid = room->take(grid);
             if (e == cudaSuccess) {
                 void* params[] = {&a};
                 LaunchScope ls("ingest_direct", s);
@@ -1759,6 +1769,7 @@ static dsg_status ingest_direct(uint32_t n, uint32_t m, const uint32_t* src, con
     }
     if (e == cudaSuccess) e = cudaMemcpyAsync(h, a.out, sizeof(h), cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+    share.give();
     if (e == cudaSuccess && !h[1] && !h[2]) {
         g->m = h[0] / 2;
         *out = g;
@@ -1789,10 +1800,10 @@ static uint32_t grid_for(uint64_t work, uint32_t block) {
 }
 
 // Core ingest on device arrays src/dst (m_raw pairs).  Allocates the graph.
-static dsg_status ingest_device(uint32_t n, uint64_t m_raw, const uint32_t* src, const uint32_t* dst, bool shared,
+static dsg_status ingest_device(uint32_t n, uint64_t m_raw, const uint32_t* src, const uint32_t* dst, GridRoom* room,
                                 cudaStream_t s, dsg_graph** out) {
     if (n && m_raw <= kDirectPairs && n <= 4 * kDirectPairs)
-        return ingest_direct(n, (uint32_t)m_raw, src, dst, shared, s, out);
+        return ingest_direct(n, (uint32_t)m_raw, src, dst, room, s, out);
     int dev = 0;
     DSG_TRY_CUDA(cudaGetDevice(&dev));
     Scratch sc(s);
@@ -2008,7 +2019,7 @@ dsg_status ingest_from_csr_entries(uint32_t n, const uint64_t* off, const uint32
     DSG_TRY_CUDA(sc.get(&src, total ? total : 1));
     { LaunchScope ls_("ingest_expand_rows", s); expand_rows<<<grid_for((uint64_t)n * 32, 256), 256, 0, s>>>(n, doff, src); }
     DSG_TRY_CUDA(cudaGetLastError());
-    dsg_status st = ingest_device(n, total, src, dadj, false, s, out);
+    dsg_status st = ingest_device(n, total, src, dadj, nullptr, s, out);
     if (st == DSG_OK && (flags & DSG_CSR_VALIDATE)) {
         st = validate_csr(*out);
         if (st != DSG_OK) {
@@ -2085,7 +2096,7 @@ dsg_status validate_csr(const dsg_graph* g) {
 using namespace dsg;
 
 dsg_status dsg::graph_from_edges(uint32_t n, uint64_t m_raw, const uint32_t* src, const uint32_t* dst, uint32_t flags,
-                                 bool shared, void* stream, dsg_graph** out) {
+                                 GridRoom* room, void* stream, dsg_graph** out) {
     clear_error();
     DSG_CHECK_ARG(out, "out is NULL");
     DSG_CHECK_ARG(n < 0x80000000u, "n must be below 2^31");
@@ -2106,7 +2117,7 @@ dsg_status dsg::graph_from_edges(uint32_t n, uint64_t m_raw, const uint32_t* src
         dsrc = a;
         ddst = b;
     }
-    dsg_status st = ingest_device(n, m_raw, dsrc, ddst, shared, s, out);
+    dsg_status st = ingest_device(n, m_raw, dsrc, ddst, room, s, out);
     if (st == DSG_OK && (flags & DSG_CSR_VALIDATE)) {
         st = validate_csr(*out);
         if (st != DSG_OK) {
@@ -2119,5 +2130,5 @@ dsg_status dsg::graph_from_edges(uint32_t n, uint64_t m_raw, const uint32_t* src
 
 extern "C" dsg_status dsg_graph_from_edges(uint32_t n, uint64_t m_raw, const uint32_t* src, const uint32_t* dst,
                                            uint32_t flags, void* stream, dsg_graph** out) {
-    return graph_from_edges(n, m_raw, src, dst, flags, false, stream, out);
+    return graph_from_edges(n, m_raw, src, dst, flags, nullptr, stream, out);
 }

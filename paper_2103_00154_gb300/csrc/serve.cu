@@ -87,6 +87,8 @@ struct dsg_server {
     std::vector<cudaStream_t> s_ingest;
     std::vector<std::thread> big_workers;
     std::vector<cudaStream_t> s_big;
+    uint32_t big_total = 0;  // SMs that the big-request threads' grids may take together
+    dsg::GridRoom room;      // the others, for the ingest threads' grids
     bool stop_helpers = false;
     // statistics
     uint64_t submitted = 0, admitted = 0, completed = 0, rejected = 0, batches = 0, big_done = 0;
@@ -160,7 +162,7 @@ static bool is_big(const dsg_server* s, const ServeReq* r) {
 static void ingest_one(dsg_server* s, ServeReq* r, cudaStream_t st_ing) {
     const double t_in = now_us();
     dsg_graph* g = nullptr;
-    dsg_status st = graph_from_edges(r->n, r->m_raw, r->src, r->dst, 0, true, st_ing, &g);
+    dsg_status st = graph_from_edges(r->n, r->m_raw, r->src, r->dst, 0, &s->room, st_ing, &g);
     if (r->owned) {
         free(r->src);
         free(r->dst);
@@ -313,10 +315,8 @@ static dsg_status launch_batch(dsg_server* s, Inflight& f, cudaStream_t ss, cuda
     a.hot_deg = 0;
     a.stats = nullptr;
     f.d_res = a.res;
-    // the batches leave the big-request threads' share of the SMs free
-    const uint32_t sms = (uint32_t)dev_info().sms;
-    const uint32_t big_sms =
-        s->cfg.big_work == UINT64_MAX ? 0 : (uint32_t)std::min<uint64_t>((uint64_t)s->cfg.big_sms * s->cfg.big_threads, sms - 1);
+    // each launch alone leaves the big-request threads' share of the SMs free
+    const uint32_t sms = (uint32_t)dev_info().sms, big_sms = s->big_total;
     std::vector<uint64_t> work(G);
     uint64_t total = 0;
     for (uint32_t i = 0; i < G; ++i) total += work[i] = ge[i] + gn[i];
@@ -499,6 +499,13 @@ dsg_status dsg_serve_create(const dsg_serve_config* cfg, dsg_server** out) {
     }
     if (e == cudaSuccess && !s->cfg.big_sms)
         s->cfg.big_sms = std::max<uint32_t>(1, (uint32_t)dev_info().sms / (4 * s->cfg.big_threads));
+    if (e == cudaSuccess) {
+        const uint32_t sms = (uint32_t)dev_info().sms;
+        s->big_total = s->cfg.big_work == UINT64_MAX
+                           ? 0
+                           : (uint32_t)std::min<uint64_t>((uint64_t)s->cfg.big_sms * s->cfg.big_threads, sms - 1);
+        s->room.set(sms - s->big_total, std::max<uint32_t>(1, (sms - s->big_total) / s->cfg.ingest_threads));
+    }
     s->s_ingest.assign(s->cfg.ingest_threads, nullptr);
     for (uint32_t k = 0; k < s->cfg.ingest_threads && e == cudaSuccess; ++k)
         e = cudaStreamCreateWithFlags(&s->s_ingest[k], cudaStreamNonBlocking);
