@@ -16,6 +16,7 @@
 #include <string.h>
 
 #include <algorithm>
+#include <mutex>
 #include <vector>
 
 #include "core_split.cuh"
@@ -470,28 +471,56 @@ __global__ void gather_ends_kernel(const uint64_t* __restrict__ off, const uint6
     if (g < G1) ends[g] = off[vb[g]];
 }
 
-// A second stream and two events per calling thread and device, made once.
+// A second stream and two events for a call, taken from those that calls of the
+// same context have given back: as many exist as calls ran at once, however
+// many threads made them.
 struct BatchSide {
-    int device = -1;
+    unsigned long long ctx = 0;
     cudaStream_t s = nullptr;
     cudaEvent_t fork = nullptr, join = nullptr;
 };
+static std::mutex g_side_mu;
+static std::vector<BatchSide> g_sides;  // not in use
 
-static cudaError_t batch_side(BatchSide** out) {
-    static thread_local BatchSide cache[16];
-    int dev = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e != cudaSuccess) return e;
-    BatchSide& b = cache[dev & 15];
-    if (b.device != dev) {
-        if ((e = cudaStreamCreateWithFlags(&b.s, cudaStreamNonBlocking)) != cudaSuccess) return e;
-        if ((e = cudaEventCreateWithFlags(&b.fork, cudaEventDisableTiming)) != cudaSuccess) return e;
-        if ((e = cudaEventCreateWithFlags(&b.join, cudaEventDisableTiming)) != cudaSuccess) return e;
-        b.device = dev;
+class SideGuard {
+  public:
+    ~SideGuard() {
+        if (!b_.s) return;
+        std::lock_guard<std::mutex> lk(g_side_mu);
+        g_sides.push_back(b_);
     }
-    *out = &b;
-    return cudaSuccess;
-}
+    cudaError_t take() {
+        unsigned long long ctx = current_ctx_id();
+        int dev = 0;
+        if (!ctx && cudaGetDevice(&dev) == cudaSuccess) ctx = ~(unsigned long long)dev;  // no ids: one context a device
+        {
+            std::lock_guard<std::mutex> lk(g_side_mu);
+            for (size_t i = 0; i < g_sides.size(); ++i) {
+                if (g_sides[i].ctx != ctx) continue;
+                b_ = g_sides[i];
+                g_sides.erase(g_sides.begin() + i);
+                return cudaSuccess;
+            }
+        }
+        BatchSide b;
+        b.ctx = ctx;
+        cudaError_t e = cudaStreamCreateWithFlags(&b.s, cudaStreamNonBlocking);
+        if (e == cudaSuccess) e = cudaEventCreateWithFlags(&b.fork, cudaEventDisableTiming);
+        if (e == cudaSuccess) e = cudaEventCreateWithFlags(&b.join, cudaEventDisableTiming);
+        if (e == cudaSuccess) {
+            b_ = b;
+            return e;
+        }
+        if (b.fork) cudaEventDestroy(b.fork);
+        if (b.s) cudaStreamDestroy(b.s);
+        return e;
+    }
+    explicit operator bool() const { return b_.s != nullptr; }
+    const BatchSide* operator->() const { return &b_; }
+
+  private:
+    BatchSide b_;
+};
 
 }  // namespace dsg
 
@@ -669,7 +698,7 @@ extern "C" dsg_status dsg_batch_solve(const dsg_batch* b, dsg_batch_result* r, v
         for (uint32_t i = lo; i < hi; ++i) bytes += 80 * (uint64_t)on[i] + 8 * oe[i] + 4096;
         return (size_t)bytes;
     };
-    BatchSide* side = nullptr;
+    SideGuard side;
     void *slabs_cl = nullptr, *slabs_bl = nullptr;
     if (ncl > nbig) {
         BatchArgs ca = a;
@@ -678,7 +707,7 @@ extern "C" dsg_status dsg_batch_solve(const dsg_batch* b, dsg_batch_result* r, v
         DSG_TRY_CUDA(sc.get(&ca.next, 1));
         DSG_TRY_CUDA(cudaMemsetAsync(ca.next, 0, sizeof(unsigned long long), s));
         if (ncl < G) {
-            DSG_TRY_CUDA(batch_side(&side));
+            DSG_TRY_CUDA(side.take());
             DSG_TRY_CUDA(cudaEventRecord(side->fork, s));
             DSG_TRY_CUDA(cudaStreamWaitEvent(side->s, side->fork, 0));
         }
