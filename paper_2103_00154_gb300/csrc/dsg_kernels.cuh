@@ -390,13 +390,6 @@ __device__ __forceinline__ bool agg_add(AggTable& t, uint32_t u) {
     return false;
 }
 
-// Shared scratch of the block-wide scans and reductions of the round kernels.
-template <int TB>
-struct TileSmem {
-    uint32_t scan_tmp[33];
-    uint64_t scan_tmp64[33];
-};
-
 constexpr uint32_t kBatch = 4;  // entries handed to a visitor per thread and call
 
 // Shared memory of the block-wide walker below.

@@ -216,10 +216,9 @@ __global__ void __launch_bounds__(1024) range_hist_kernel(uint32_t n, uint64_t m
 // different multiples of the target, or when r is a multiple of span_cut.
 // Writes range_bucket[r], the first vertex and the entry base of every
 // bucket (bucket_v0[F] = n, bucket_base[F] = total entries), start[n] =
-// total, *nb = F and *maxb = the largest bucket's entries.  A thread's ranges
-// are consecutive; their counts come and their buckets go through shared
-// memory, so that global memory is read and written in lines (32,768 ranges:
-// 98 us before, 35 now).
+// total, *nb = F.  A thread's ranges are consecutive; their counts come and
+// their buckets go through shared memory, so that global memory is read and
+// written in lines (32,768 ranges: 98 us before, 35 now).
 constexpr uint32_t kPlanPer = kRangesMax / 1024;  // ranges per thread
 constexpr size_t kPlanSmem = (size_t)kRangesMax / 32 * 33 * 4;
 __device__ __forceinline__ uint32_t plan_at(uint32_t r) { return r + (r >> 5); }  // a word of padding per 32
@@ -228,8 +227,7 @@ __global__ void __launch_bounds__(1024) bucket_plan_kernel(uint32_t n, const uin
                                                            BucketPlan pl, uint16_t* __restrict__ range_bucket,
                                                            uint32_t* __restrict__ bucket_v0,
                                                            uint64_t* __restrict__ bucket_base,
-                                                           uint64_t* __restrict__ start, uint32_t* __restrict__ nb,
-                                                           unsigned long long* __restrict__ maxb) {
+                                                           uint64_t* __restrict__ start, uint32_t* __restrict__ nb) {
     extern __shared__ uint32_t cs[];  // the ranges' counts, then their buckets
     __shared__ uint64_t tmp64[33];
     __shared__ uint32_t tmp32[33];
@@ -261,8 +259,7 @@ __global__ void __launch_bounds__(1024) bucket_plan_kernel(uint32_t n, const uin
         p += cj;
     }
     uint32_t nf_total;
-    const uint32_t id0 = block_excl_scan<uint32_t>(nf, tmp32, &nf_total);
-    uint32_t id = id0;
+    uint32_t id = block_excl_scan<uint32_t>(nf, tmp32, &nf_total);
     p = pre;
     for (uint32_t j = 0; j < kPlanPer; ++j) {
         const uint32_t r = r0 + j;
@@ -283,11 +280,8 @@ __global__ void __launch_bounds__(1024) bucket_plan_kernel(uint32_t n, const uin
         start[n] = total;
         *nb = nf_total;
     }
-    __syncthreads();  // every bucket base is written (and visible to the block)
+    __syncthreads();
     for (uint32_t r = threadIdx.x; r < pl.nranges; r += 1024) range_bucket[r] = (uint16_t)cs[plan_at(r)];
-    uint64_t big = 0;
-    for (uint32_t b = id0; b < id; ++b) big = max(big, bucket_base[b + 1] - bucket_base[b]);
-    if (big) atomicMax(maxb, (unsigned long long)big);
 }
 
 // The buckets are reached in two partition passes of small fan-out, so that a
@@ -1825,7 +1819,7 @@ static dsg_status ingest_device(uint32_t n, uint64_t m_raw, const uint32_t* src,
     uint32_t *range_cnt, *bucket_v0, *nb, *ticket, *b_pre, *r_pre, *big_list, *fill;
     uint16_t* range_bucket;
     uint64_t *bucket_base, *group_base, *E1, *E2;
-    unsigned long long *bucket_fill, *group_fill, *maxb;
+    unsigned long long *bucket_fill, *group_fill;
     PartPlan* pp;
     DSG_TRY_CUDA(sc.get(&range_cnt, pl.nranges ? pl.nranges : 1));
     DSG_TRY_CUDA(sc.get(&range_bucket, pl.nranges ? pl.nranges : 1));
@@ -1842,7 +1836,6 @@ static dsg_status ingest_device(uint32_t n, uint64_t m_raw, const uint32_t* src,
     DSG_TRY_CUDA(sc.get(&big_list, fcap));
     DSG_TRY_CUDA(sc.get(&pp, 1));
     DSG_TRY_CUDA(sc.get(&nb, 2));
-    DSG_TRY_CUDA(sc.get(&maxb, 1));
     ticket = nb + 1;
     DSG_TRY_CUDA(sc.get(&E1, cap ? cap : 1));
     DSG_TRY_CUDA(sc.get(&E2, cap ? cap : 1));
@@ -1852,7 +1845,6 @@ static dsg_status ingest_device(uint32_t n, uint64_t m_raw, const uint32_t* src,
     DSG_TRY_CUDA(cudaMemsetAsync(bucket_fill, 0, fcap * 8, s));
     DSG_TRY_CUDA(cudaMemsetAsync(group_fill, 0, gcap * 8, s));
     DSG_TRY_CUDA(cudaMemsetAsync(nb, 0, 2 * sizeof(uint32_t), s));
-    DSG_TRY_CUDA(cudaMemsetAsync(maxb, 0, sizeof(unsigned long long), s));
     DSG_TRY_CUDA(cudaMemsetAsync(cnt, 0, ((size_t)n + 1) * 4, s));  // big buckets add their counts into it
     const size_t hist_smem = (size_t)pl.nranges * 4;
     const size_t part_smem = sizeof(PartSmem) + (((size_t)pl.nranges * 2 + 15) & ~size_t(15));
@@ -1883,8 +1875,7 @@ static dsg_status ingest_device(uint32_t n, uint64_t m_raw, const uint32_t* src,
     DSG_TRY_CUDA(cudaGetLastError());
     {
         LaunchScope ls_("ingest_bucket_plan", s);
-        bucket_plan_kernel<<<1, 1024, kPlanSmem, s>>>(n, range_cnt, pl, range_bucket, bucket_v0, bucket_base, start, nb,
-                                              maxb);
+        bucket_plan_kernel<<<1, 1024, kPlanSmem, s>>>(n, range_cnt, pl, range_bucket, bucket_v0, bucket_base, start, nb);
     }
     DSG_TRY_CUDA(cudaGetLastError());
     {

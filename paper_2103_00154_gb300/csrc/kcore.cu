@@ -159,7 +159,6 @@ static_assert(kTakeSlots >= 1 && kTakeSlots <= 32, "a block takes 1..32 queue sl
 
 template <int TB>
 struct CoreSmem {
-    TileSmem<TB> tile;
     BlockTile<TB> btile;
     uint32_t lq[kLocalQ];   // vertices that reached k, not yet claimed
     uint32_t lq_tail;
