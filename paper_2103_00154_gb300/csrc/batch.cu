@@ -714,7 +714,12 @@ extern "C" dsg_status dsg_batch_solve(const dsg_batch* b, dsg_batch_result* r, v
         const cudaError_t e = batch_cluster_launch(ca, {on.data() + nbig, oe.data() + nbig},
                                                    scratch_max(nbig, ncl), s, &slabs_cl);
         if (slabs_cl) sc.adopt(slabs_cl);
-        DSG_TRY_CUDA(e);
+        if (e == cudaErrorMemoryAllocation && !slabs_cl) {
+            cudaGetLastError();
+            ncl = nbig;  // not even one cluster's scratch: a block each, which takes a quarter of it
+        } else {
+            DSG_TRY_CUDA(e);
+        }
     }
     a.order = d_order + ncl;
     a.G = G - ncl;

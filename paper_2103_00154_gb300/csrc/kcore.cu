@@ -635,8 +635,9 @@ static cudaError_t launch_kcore(CoreArgs& a, uint32_t grid, cudaStream_t s) {
     return cudaLaunchCooperativeKernel((const void*)kcore_kernel<TB>, dim3(grid), dim3(TB), params, 0, s);
 }
 
-dsg_status run_kcore(const dsg_graph* g, uint32_t* core_out, uint64_t* stats, uint32_t nstats,
-                     uint64_t* trace_dev, uint64_t trace_cap, uint64_t* stamps) {
+// search: false keeps the levels to the end.
+static dsg_status kcore_with(bool search, const dsg_graph* g, uint32_t* core_out, uint64_t* stats, uint32_t nstats,
+                             uint64_t* trace_dev, uint64_t trace_cap, uint64_t* stamps) {
     cudaStream_t s = g->stream;
     const uint32_t n = g->n;
     if (n == 0) return DSG_OK;
@@ -652,7 +653,7 @@ dsg_status run_kcore(const dsg_graph* g, uint32_t* core_out, uint64_t* stats, ui
     a.local_max = tu.local_max;
     a.local_work = tu.local_work;
     a.inline_max = tu.inline_max;
-    const uint64_t tail = 2 * g->m < kTailMaxEntries ? tu.tail_max : 0;
+    const uint64_t tail = search && 2 * g->m < kTailMaxEntries ? tu.tail_max : 0;
     a.tail_max = (uint32_t)(kTailHandOver * std::min<uint64_t>(tail, kTailMaxVertices));
     a.trace = trace_dev;
     a.trace_cap = trace_cap;
@@ -740,6 +741,19 @@ dsg_status run_kcore(const dsg_graph* g, uint32_t* core_out, uint64_t* stats, ui
     DSG_TRY_CUDA(cudaStreamSynchronize(s));
     for (uint32_t i = 0; stats && i < nstats && i < 5; ++i) stats[i] = vals[i];
     return DSG_OK;
+}
+
+dsg_status run_kcore(const dsg_graph* g, uint32_t* core_out, uint64_t* stats, uint32_t nstats, uint64_t* trace_dev,
+                     uint64_t trace_cap, uint64_t* stamps) {
+    dsg_status st = kcore_with(true, g, core_out, stats, nstats, trace_dev, trace_cap, stamps);
+    if (st == DSG_ENOMEM) {
+        // the search's arrays (about 90 bytes a vertex and 1/4 an entry of what it takes over) cannot be
+        // had; the levels alone need 32 and 1/13
+        cudaGetLastError();
+        clear_error();
+        st = kcore_with(false, g, core_out, stats, nstats, trace_dev, trace_cap, stamps);
+    }
+    return st;
 }
 
 }  // namespace dsg

@@ -330,9 +330,13 @@ static dsg_status launch_batch(dsg_server* s, Inflight& f, cudaStream_t ss, cuda
         size_t room = 0;
         for (uint32_t i = lo; i < hi; ++i) room += f.reqs[i]->charge - resident_bytes(f.reqs[i]->n, f.reqs[i]->m_raw);
         const BatchSizes sizes = {gn.data() + lo, ge.data() + lo};
-        if (clusters) return batch_cluster_launch(b, sizes, room, st, &f.slabs_cl, std::max(1u, sms - big_sms));
+        if (clusters) {
+            const cudaError_t e = batch_cluster_launch(b, sizes, room, st, &f.slabs_cl, std::max(1u, sms - big_sms));
+            if (e != cudaErrorMemoryAllocation || f.slabs_cl) return e;
+            cudaGetLastError();  // not even one cluster's scratch: a block each, which takes a quarter of it
+        }
         const uint32_t cap = (uint32_t)((uint64_t)batch_slots_for(512) * (sms - big_sms) / sms);
-        return batch_launch(b, sizes, room, st, &f.slabs_bl, 512, cap ? cap : 1);
+        return batch_launch(b, sizes, room, st, clusters ? &f.slabs_cl : &f.slabs_bl, 512, cap ? cap : 1);
     };
     cudaError_t e = cudaSuccess;
     if (ncl == 0 || ncl == G) {
