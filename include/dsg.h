@@ -170,7 +170,7 @@ uint64_t dsg_round_bound(uint32_t n, uint32_t eps_num, uint32_t eps_den);
  * bytes: four of 4n bytes (vertex state, two alive lists, one spare), the row
  * pieces 8(n + 2m/chunk_len + 1) bytes, the status map 4 ceil(n/16)
  * bytes, two round histories of 8(dsg_round_bound(n, p, q) + 1) bytes, and a
- * control block of about 1 KB; chunk_len is the current tuning's
+ * control block of 1,280 bytes; chunk_len is the current tuning's
  * (dsg_set_tuning; 256 by default).  A graph whose scratch exceeds 64 MiB is
  * rejected with DSG_EINVAL before any GPU work (with eps > 0 and the default
  * chunk_len that admits n up to about 2.7 million at m = 8n).

@@ -503,7 +503,8 @@ extern "C" dsg_status dsg_bahmani_noalloc(uint32_t n, const uint64_t* off, const
     const size_t b_list = align256((size_t)n * 4);
     const size_t b_chunk = align256((size_t)chunk_cap * 8);
     const size_t b_hist = align256((size_t)cap * 8);
-    const size_t b_ctl = align256(sizeof(PeelCtl));
+    constexpr size_t b_ctl = 1280;  // the control block's share (a part of the documented limit)
+    static_assert(sizeof(PeelCtl) <= b_ctl, "the control block's share");
     const size_t b_map = align256(((size_t)n + 15) / 16 * 4);
     const size_t need = 4 * b_list + b_chunk + b_map + 2 * b_hist + b_ctl;
     if (need > kNoAllocScratchBytes) {
