@@ -497,10 +497,9 @@ dsg_status dsg_cbds(const dsg_graph* g, const uint32_t* core, uint32_t* out_core
 /*
  * Autotuner.  dsg_autotune times candidate launch parameters for the peel
  * (what bit 0, at eps_num/eps_den) and/or the core numbers (bit 1) on graph g
- * by coordinate descent over block size, hub threshold, chunk length and
- * short-row limit (peel) or block size, hub threshold, the local-drain
- * limits and the inline-drain limit (core numbers), keeping a change only
- * when it is at least 2%
+ * by coordinate descent over block size, hub threshold and chunk length (peel)
+ * or block size, the local-drain limits, the inline-drain limit, chunk length
+ * and kcore_tail (core numbers), keeping a change only when it is at least 2%
  * faster.  The winner is recorded for g's size class (floor log2 n,
  * floor log2 2m) on this device and used by every later solve of a graph of
  * that class; *trials gets the number of timed solves.  The table is saved
@@ -538,9 +537,9 @@ void dsg_set_allocator(dsg_alloc_fn alloc, dsg_free_fn free_fn, void* ctx);
  * calls plus one dsg_kcore call (out_sets[i], out_E[i], out_V[i]; out_core),
  * with the peels and the core decomposition running side by side on two
  * internal streams, the peels on the share of the SMs that their autotuned
- * time has in the summed time (within 1/4 and 3/4; half when the graph's size
- * class is not tuned; the environment variable DSG_SOLVE_PEEL_PERMILLE, 1..999,
- * overrides it) -- unless the autotuned times show the core numbers taking
+ * time has in the summed time (within 1/4 and 3/4; count / (count + 8), within
+ * 0.15 and 1/2, when the graph's size class is not tuned; the environment
+ * variable DSG_SOLVE_PEEL_PERMILLE, 1..999, overrides it) -- unless the autotuned times show the core numbers taking
  * over four times as long as the peels, in which case they run one after the
  * other on the whole GPU.  Results never depend on the choice.  out_sets (and its entries),
  * out_E, out_V nullable; out_core NULL runs the peels only.  Work starts
@@ -551,7 +550,8 @@ void dsg_set_allocator(dsg_alloc_fn alloc, dsg_free_fn free_fn, void* ctx);
 dsg_status dsg_solve(const dsg_graph* g, uint32_t count, const uint32_t* eps_num, const uint32_t* eps_den,
                      uint8_t* const* out_sets, uint64_t* out_E, uint64_t* out_V, uint32_t* out_core);
 
-/* Upper bound (ns) on every device-side wait (grid barriers, queue polls).
+/* Upper bound (ns) on every device-side wait of a grid (meetings of its blocks,
+ * queue polls; the barrier of a thread-block cluster is the hardware's own).
  * A wait that runs out makes its kernel return and the call report
  * DSG_ETIMEOUT.  0 restores the default (10 s, or DSG_WAIT_LIMIT_NS). */
 void dsg_set_wait_limit_ns(uint64_t ns);
@@ -570,8 +570,9 @@ dsg_status dsg_debug_wait_timeout(uint32_t which, uint64_t limit_ns);
  * Analysis probes (no counterpart in the paper; used to measure the round
  * machinery, not part of the method).
  *   dsg_debug_peel_trace   one Algorithm 1 run recording %globaltimer (ns)
- *                          at kernel start and after every grid barrier
- *                          (2 per round) into ts[cap]; *count = stamps taken
+ *                          at kernel start and after every meeting of the
+ *                          blocks (2 per round) into ts[cap]; *count = stamps
+ *                          taken
  *   dsg_debug_kcore_trace  one core decomposition recording pairs
  *                          (ns, kind << 32 | k): kind 0 start, 1 degrees
  *                          initialised, 2 level over (block 0), 3/4/5 block
@@ -579,7 +580,11 @@ dsg_status dsg_debug_wait_timeout(uint32_t which, uint64_t limit_ns);
  *                          each level five (value, kind << 32 | k) pairs:
  *                          6/7 latest own / queue phase end over the blocks
  *                          (ns, as block 0 sees them), 8 claims, 9 claims by
- *                          the scan, 10 queued row pieces; *count = pairs
+ *                          the scan, 10 queued row pieces; of the bitwise
+ *                          search, with the bit in the place of k: 11 a bit's
+ *                          keys written, 12 / 13 its first / a later wave
+ *                          over, 14 (value) the pieces that wave queued;
+ *                          *count = pairs
  */
 dsg_status dsg_debug_peel_trace(const dsg_graph* g, uint32_t eps_num, uint32_t eps_den, uint64_t* ts, uint64_t cap,
                                 uint64_t* count);

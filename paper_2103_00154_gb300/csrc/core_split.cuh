@@ -40,8 +40,8 @@
 // cached in L1 although the kernel rewrites it while it runs.
 //
 // The blocks meet after every wave (Team::meet: the pieces that the wave queued
-// come back with the wait).
-// Every wait is bounded (ERR_TIMEOUT).
+// come back with the wait).  A grid's wait is bounded (ERR_TIMEOUT); a cluster's
+// is the hardware's barrier over blocks that were launched together.
 //
 // What bounds it: the wide waves, L2 gathers (a bit's first wave on Chung-Lu
 // 2^24, 65,287 vertices and about 45 M row entries read: 60 us); the thin ones,

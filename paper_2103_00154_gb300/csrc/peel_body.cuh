@@ -22,9 +22,11 @@
 //     monotone counters and keeps the densest set (strict ">": a later round
 //     replaces the best only when strictly denser, as in Algorithm 1); block 0
 //     records the history.
-// Once the alive rows hold at most kSoloEntries entries (dead ones counted),
-// block 0 runs the remaining rounds alone and the others leave: a round then
-// costs block barriers and shared-memory cursors only.
+// Once the alive rows hold at most kSoloEntries entries and the alive list
+// kSoloList vertices, block 0 of a grid runs the remaining rounds alone and the
+// others leave: a round then costs block barriers and shared-memory cursors
+// only.  (Lazy rounds leave the list as it is, so a lazy tail stays with the
+// grid until a round tests everyone again.)
 // The edges removed in round r (Algorithm 1's reduction) are (X + D) / 2: the
 // failures' degrees count every edge between two failures twice and every
 // edge from a failure to a survivor once, and D counts the latter once more.
