@@ -593,15 +593,17 @@ dsg_status dsg_debug_kcore_trace(const dsg_graph* g, uint64_t* ts, uint64_t cap,
 /*
  * Probes of the word the blocks of a peel meet on (arrivals in its low half,
  * the sum of their counts in its high half), for the tests of its wrap.
- *   dsg_debug_meet_sum   the sum, modulo 2^32, on a word that so many blocks
- *                        have arrived on; needs no GPU
+ *   dsg_debug_meet_count what `blocks` blocks handed in at the meeting after
+ *                        which the word has had `arrivals` arrivals (modulo
+ *                        2^32); high: its high half after the meeting before
+ *                        it; needs no GPU
  *   dsg_debug_peel_wrap  one Algorithm 1 run by the grid-wide kernel whose
  *                        words start so many arrivals on that they pass 2^32
  *                        after wrap_in rounds (1 .. 2^20); peel_round and
  *                        out_set as in dsg_trace, out4 = E, V, rounds, best
  *                        round
  */
-uint32_t dsg_debug_meet_sum(uint64_t word, uint64_t arrivals);
+uint32_t dsg_debug_meet_count(uint64_t word, uint32_t high, uint32_t arrivals, uint32_t blocks);
 dsg_status dsg_debug_peel_wrap(const dsg_graph* g, uint32_t eps_num, uint32_t eps_den, uint32_t wrap_in,
                                uint32_t* peel_round, uint8_t* out_set, uint64_t out4[4]);
 

@@ -138,7 +138,7 @@ _SIGS = [
     ("dsg_set_allocator", None, [ALLOC_FN, FREE_FN, _VP]),
     ("dsg_debug_wait_timeout", c.c_int, [c.c_uint32, c.c_uint64]),
     ("dsg_debug_peel_trace", c.c_int, [_VP, c.c_uint32, c.c_uint32, _U64P, c.c_uint64, _U64P]),
-    ("dsg_debug_meet_sum", c.c_uint32, [c.c_uint64, c.c_uint64]),
+    ("dsg_debug_meet_count", c.c_uint32, [c.c_uint64, c.c_uint32, c.c_uint32, c.c_uint32]),
     ("dsg_debug_peel_wrap", c.c_int, [_VP, c.c_uint32, c.c_uint32, c.c_uint32, _VP, _VP, _U64P]),
     ("dsg_debug_kcore_trace", c.c_int, [_VP, _U64P, c.c_uint64, _U64P]),
     ("dsg_launch_count", c.c_ulonglong, []),

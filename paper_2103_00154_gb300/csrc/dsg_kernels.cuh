@@ -261,25 +261,27 @@ __device__ __forceinline__ T* at_block0(T* p) {
 // zero.  Every thread of the block calls it; thread 0's `mine` counts.  A wait
 // above limit_ns records ERR_TIMEOUT and clears sm.ok, as does seeing the
 // error of another block.  With one block (size == 1) it is a block barrier.
-// The low half is never reset and carries into the high one after 2^32
+// The low half is never reset and carries into the high one every 2^32
 // arrivals (a path of 2^24 vertices at eps = 0 has 2^23 rounds, each an
-// arrival of every block on each word): meet_sum takes the arrivals, counted
-// in 64 bits, off the whole word.
+// arrival of every block on each word): a block that counts them modulo 2^32
+// knows at which meeting that is, and takes it off.
 
-// The sum, modulo 2^32, of the counts on a word that `arrivals` blocks have arrived on.
-__host__ __device__ __forceinline__ uint32_t meet_sum(uint64_t word, uint64_t arrivals) {
-    return (uint32_t)((word - arrivals) >> 32);
+// The counts handed in at the meeting after which a word of `blocks` blocks has
+// had `arrivals` arrivals (modulo 2^32); high: the word's high half after the
+// meeting before it.
+__host__ __device__ __forceinline__ uint32_t meet_count(uint64_t word, uint32_t high, uint32_t arrivals,
+                                                        uint32_t blocks) {
+    return (uint32_t)(word >> 32) - (high + (arrivals < blocks ? 1u : 0u));
 }
 // A block's view of the meetings, kept by its thread 0 (the others read got and ok).
 struct MeetSmem {
-    uint64_t arrivals[2];  // by word: arrivals when its last meeting was over ...
-    uint32_t seen[2];      // ... and the sums handed out so far
-    uint32_t par;          // the next meeting's word
+    uint32_t arrivals[2], high[2];  // by word, after its last meeting
+    uint32_t par;                   // the next meeting's word
     uint32_t got, ok;
 };
-__device__ __forceinline__ void meet_init(MeetSmem& sm, uint64_t arrivals = 0) {
+__device__ __forceinline__ void meet_init(MeetSmem& sm, uint32_t arrivals = 0) {
     sm.arrivals[0] = sm.arrivals[1] = arrivals;
-    sm.seen[0] = sm.seen[1] = sm.par = 0;
+    sm.high[0] = sm.high[1] = sm.par = 0;
     sm.ok = 1;
 }
 
@@ -294,12 +296,12 @@ struct Team {
     uint64_t limit_ns;
 
     __device__ __forceinline__ uint32_t meet(uint32_t mine, MeetSmem& sm) {
-        // what the wait is over with is read before it: nothing depends on shared memory after it
-        uint32_t par = 0, seen = 0;
-        uint64_t arrivals = 0;
+        // read before the wait, written after the others may go on: the chain from the word's arrival
+        // to the block's release is a subtraction and one store
+        uint32_t par = 0, high = 0, arrivals = 0;
         if (threadIdx.x == 0) {
             par = sm.par;
-            seen = sm.seen[par];
+            high = sm.high[par];
             arrivals = sm.arrivals[par] + size;
         }
         if constexpr (CL) {
@@ -308,9 +310,8 @@ struct Team {
             cluster_sync();
             if (threadIdx.x == 0) {
                 const uint32_t sum = (uint32_t)ld_volatile_u64((const uint64_t*)word);
-                sm.got = sum - seen;
-                sm.seen[par] = sum;
-                sm.par = par ^ 1u;
+                sm.got = sum - high;
+                high = sum;
             }
         } else {
             __syncthreads();
@@ -323,7 +324,7 @@ struct Team {
                     uint64_t w;
                     uint32_t polls = 0;
                     const uint64_t t0 = global_ns();
-                    while ((int32_t)((uint32_t)(w = ld_acquire_u64(word)) - (uint32_t)arrivals) < 0) {
+                    while ((int32_t)((uint32_t)(w = ld_acquire_u64(word)) - arrivals) < 0) {
                         if ((++polls & 63u) == 0) {
                             if (global_ns() - t0 > limit_ns) atomicOr(err, ERR_TIMEOUT);
                             if (ld_volatile_u32(err) & ERR_TIMEOUT) {
@@ -332,16 +333,19 @@ struct Team {
                             }
                         }
                     }
-                    const uint32_t sum = meet_sum(w, arrivals);
-                    sm.got = sum - seen;
-                    sm.seen[par] = sum;
-                    sm.arrivals[par] = arrivals;
-                    sm.par = par ^ 1u;
+                    sm.got = meet_count(w, high, arrivals, size);
+                    high = (uint32_t)(w >> 32);
                 }
             }
         }
         __syncthreads();
-        return sm.got;
+        const uint32_t got = sm.got;
+        if (threadIdx.x == 0) {
+            sm.par = par ^ 1u;
+            sm.high[par] = high;
+            sm.arrivals[par] = arrivals;
+        }
+        return got;
     }
 };
 

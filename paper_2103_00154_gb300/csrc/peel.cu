@@ -74,7 +74,7 @@ static cudaError_t launch_peel(PeelArgs& a, uint32_t blocks_per_sm, cudaStream_t
     cudaError_t e = coop_grid(peel_kernel<TB>, TB, 0, a.n, blocks_per_sm, &grid, max_grid);
     if (e != cudaSuccess) return e;
     if (wrap_in) {
-        a.arrivals0 = ((1ull << 32) / grid - wrap_in) * grid;
+        a.arrivals0 = (uint32_t)(((1ull << 32) / grid - wrap_in) * grid);
         const unsigned long long before = a.arrivals0;
         for (int w = 0; w < 2 && e == cudaSuccess; ++w)
             e = cudaMemcpyAsync(&a.ctl->bar[w][0], &before, sizeof(before), cudaMemcpyHostToDevice, s);
@@ -386,7 +386,9 @@ dsg_status dsg_debug_peel_trace(const dsg_graph* g, uint32_t eps_num, uint32_t e
     return DSG_OK;
 }
 
-uint32_t dsg_debug_meet_sum(uint64_t word, uint64_t arrivals) { return meet_sum(word, arrivals); }
+uint32_t dsg_debug_meet_count(uint64_t word, uint32_t high, uint32_t arrivals, uint32_t blocks) {
+    return meet_count(word, high, arrivals, blocks);
+}
 
 dsg_status dsg_debug_peel_wrap(const dsg_graph* g, uint32_t eps_num, uint32_t eps_den, uint32_t wrap_in,
                                uint32_t* peel_round, uint8_t* out_set, uint64_t out4[4]) {

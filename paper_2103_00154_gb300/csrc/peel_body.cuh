@@ -98,7 +98,7 @@ struct PeelArgs {
     // skipping those already failed; max_rounds > 0 pauses after that many rounds
     uint64_t r0, S0, E0, best_round0, best_E0, best_V0;
     uint64_t max_rounds;
-    uint64_t arrivals0;   // that each word of ctl->bar already counts (0 but for the test of their wrap)
+    uint32_t arrivals0;   // that each word of ctl->bar already counts (0 but for the test of their wrap)
 };
 
 constexpr uint32_t kLenBits = 24;         // of a piece: entries (chunk_len is kept below 2^24)
