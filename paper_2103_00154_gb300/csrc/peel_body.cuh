@@ -189,12 +189,16 @@ __device__ __forceinline__ PeelOut peel_body(const PeelArgs& a, Team<CL> team, P
     bool solo = team.size == 1;
     uint32_t size = team.size;  // blocks at work
     if (tid < 2) sm.cursor[tid] = 0;
-    if (tid < 4) sm.add[tid] = 0;
+    if (tid < 4) {
+        sm.add[tid] = 0;
+        sm.cum[tid] = 0;
+    }
+    __syncwarp();
     if (tid == 0) {
         meet_init(sm.meet, a.arrivals0);
         sm.cum[0] = resume ? (uint64_t)a.n - a.S0 : 0;
         sm.cum[1] = resume ? 2 * (a.m - a.E0) : 0;
-        sm.cum[2] = sm.cum[3] = sm.cum[4] = 0;
+        sm.cum[4] = 0;
         sm.agg_used = 0;
         sm.scanned = 0;
     }
