@@ -128,12 +128,11 @@ constexpr uint32_t kClusterTB = 1024;
 // the search's share the space.  Larger graphs need no less of anything.
 constexpr uint32_t kBatchChunk = 256;  // entries of a row piece of the peel
 struct SlabLayout {
-    uint64_t at;  // the slab's own place
     uint64_t listA, listB, items, map, peel_end;
     uint64_t ds, key, pieces, queue, search_end;
     uint64_t cap;  // row pieces of the search
 };
-static SlabLayout slab_layout(uint64_t n, uint64_t e) {
+__host__ __device__ inline SlabLayout slab_layout(uint64_t n, uint64_t e) {
     auto up = [](uint64_t bytes) { return (bytes + 255) & ~uint64_t(255); };
     SlabLayout l = {};
     l.listA = up(4 * n);  // after the states
@@ -150,10 +149,15 @@ static SlabLayout slab_layout(uint64_t n, uint64_t e) {
     return l;
 }
 
+struct Slab {
+    uint64_t at;    // its place in the scratch
+    uint64_t n, e;  // the graphs it is for
+};
+
 struct BatchKernelArgs {
     BatchArgs b;
-    unsigned char* scratch;  // the error word, the slabs' layouts, the slabs
-    const SlabLayout* slabs;  // by the order in which the teams start
+    unsigned char* scratch;  // the error word, the table of the slabs, the slabs
+    const Slab* slabs;       // by the order in which the teams start
 };
 
 template <int TB>
@@ -170,7 +174,8 @@ struct BatchSmem {
     PeelCtl pctl;
     SplitCtl sctl;
     uint32_t item, slot;
-    const SlabLayout* slab;  // the team's, once it has taken a graph
+    unsigned char* slab;  // the team's, once it has taken a graph ...
+    SlabLayout lay;       // ... and its layout
 };
 
 // The two bodies as functions of their own: inlined into one kernel they spill
@@ -228,9 +233,13 @@ __global__ void __launch_bounds__(TB, 1024 / TB) batch_kernel(BatchKernelArgs c)
         const uint64_t* off = b.goff[g];
         if (tid == 0) {
             PeelArgs& a = sm.pargs;
-            if (!sm.slab) sm.slab = c.slabs + ld_volatile_u32(slot0);
-            const SlabLayout& l = *sm.slab;
-            unsigned char* const slab = c.scratch + l.at;
+            if (!sm.slab) {
+                const Slab z = c.slabs[ld_volatile_u32(slot0)];
+                sm.slab = c.scratch + z.at;
+                sm.lay = slab_layout(z.n, z.e);
+            }
+            const SlabLayout& l = sm.lay;
+            unsigned char* const slab = sm.slab;
             a.n = n;
             a.m = n ? (off[n] - off[0]) / 2 : 0;
             a.p = b.p[g];
@@ -269,7 +278,7 @@ __global__ void __launch_bounds__(TB, 1024 / TB) batch_kernel(BatchKernelArgs c)
                 if (pctl->err) atomicOr(err, pctl->err);
             }
             if (b.out_set) {
-                const uint32_t* st = reinterpret_cast<const uint32_t*>(c.scratch + sm.slab->at);
+                const uint32_t* st = sm.pargs.st;
                 for (uint32_t v = rank * TB + tid; v < n; v += size * TB)
                     b.out_set[vb + v] = (__ldcg(st + v) & ~kDead) > o.best_round ? 1 : 0;
             }
@@ -279,8 +288,8 @@ __global__ void __launch_bounds__(TB, 1024 / TB) batch_kernel(BatchKernelArgs c)
             if constexpr (CL) {
                 if (tid == 0) {
                     SplitArgs& a = sm.sargs;
-                    const SlabLayout& l = *sm.slab;
-                    unsigned char* const slab = c.scratch + l.at;
+                    const SlabLayout& l = sm.lay;
+                    unsigned char* const slab = sm.slab;
                     a.r = n;
                     a.lo = 0;
                     a.off = off;
@@ -305,8 +314,8 @@ __global__ void __launch_bounds__(TB, 1024 / TB) batch_kernel(BatchKernelArgs c)
                 if (rank == 0 && tid == 0 && sctl->err) atomicOr(err, sctl->err);
                 __syncthreads();
             } else {
-                const SlabLayout& l = *sm.slab;
-                unsigned char* const slab = c.scratch + l.at;
+                const SlabLayout& l = sm.lay;
+                unsigned char* const slab = sm.slab;
                 kcore_block<TB>(n, off, b.gadj[g], b.core + vb, reinterpret_cast<uint32_t*>(slab),
                                 reinterpret_cast<uint32_t*>(slab + l.listA),
                                 reinterpret_cast<uint32_t*>(slab + l.listB), sm.level);
@@ -321,7 +330,7 @@ __global__ void __launch_bounds__(TB, 1024 / TB) batch_kernel(BatchKernelArgs c)
 static cudaError_t batch_slabs(BatchKernelArgs& c, const BatchSizes& sizes, bool search, uint64_t* teams,
                                size_t scratch_max, cudaStream_t s, void** slabs) {
     const uint32_t G = c.b.G;
-    std::vector<SlabLayout> all(*teams);  // by place: for the most vertices and the most entries from there on
+    std::vector<Slab> all(*teams);  // by place: for the most vertices and the most entries from there on
     std::vector<uint64_t> bytes(*teams);
     uint32_t n = 0;
     uint64_t e = 0;
@@ -329,8 +338,9 @@ static cudaError_t batch_slabs(BatchKernelArgs& c, const BatchSizes& sizes, bool
         n = std::max(n, sizes.n[k]);
         e = std::max(e, sizes.e[k]);
         if (k < *teams) {
-            all[k] = slab_layout(n, e);
-            bytes[k] = c.b.core && search ? std::max(all[k].peel_end, all[k].search_end) : all[k].peel_end;
+            all[k] = {0, n, e};
+            const SlabLayout l = slab_layout(n, e);
+            bytes[k] = c.b.core && search ? std::max(l.peel_end, l.search_end) : l.peel_end;
             // (the kernel's time depends on the addresses by a few percent; over seven places of the
             // allocation each, 1,500 graphs of up to 100,000 vertices took 2.11 ms with slabs packed
             // tightly, 2.07 in steps of 64 KB and 2.11 in steps of 2 MB)
@@ -342,7 +352,7 @@ static cudaError_t batch_slabs(BatchKernelArgs& c, const BatchSizes& sizes, bool
     constexpr uint64_t kHead = 256;  // the error word's share
     void* p = nullptr;
     for (;;) {
-        uint64_t at = (kHead + t * sizeof(SlabLayout) + 255) & ~uint64_t(255);
+        uint64_t at = (kHead + t * sizeof(Slab) + 255) & ~uint64_t(255);
         for (uint64_t k = 0; k < t; at += bytes[k++]) all[k].at = at;
         const cudaError_t err = dev_alloc(&p, at, s);
         if (err == cudaSuccess) break;
@@ -353,9 +363,9 @@ static cudaError_t batch_slabs(BatchKernelArgs& c, const BatchSizes& sizes, bool
     *slabs = p;
     *teams = t;
     c.scratch = static_cast<unsigned char*>(p);
-    c.slabs = reinterpret_cast<const SlabLayout*>(c.scratch + kHead);
-    std::vector<unsigned char> head(kHead + t * sizeof(SlabLayout), 0);
-    memcpy(head.data() + kHead, all.data(), t * sizeof(SlabLayout));
+    c.slabs = reinterpret_cast<const Slab*>(c.scratch + kHead);
+    std::vector<unsigned char> head(kHead + t * sizeof(Slab), 0);
+    memcpy(head.data() + kHead, all.data(), t * sizeof(Slab));
     return cudaMemcpyAsync(p, head.data(), head.size(), cudaMemcpyHostToDevice, s);
 }
 
