@@ -193,7 +193,7 @@ __device__ __forceinline__ PeelOut peel_body(const PeelArgs& a, Team<CL> team, P
         sm.add[tid] = 0;
         sm.cum[tid] = 0;
     }
-    __syncwarp();
+    __syncwarp();  // cleared by four threads, then set by one of them
     if (tid == 0) {
         meet_init(sm.meet, a.arrivals0);
         sm.cum[0] = resume ? (uint64_t)a.n - a.S0 : 0;
